@@ -90,7 +90,9 @@ __global__ void __launch_bounds__(kScanBlock) scan_onepass_kernel(const uint32_t
     const size_t base = (size_t)b * kScanChunk + (size_t)tid * kScanItems;
     uint32_t c[kScanItems];
     uint64_t sum = 0;
-    if (base + kScanItems <= (size_t)n && perm) {
+    // 16-byte loads where perm allows them (a batch camera's order starts at a
+    // multiple of n records, which need not be one of four)
+    if (base + kScanItems <= (size_t)n && perm && (reinterpret_cast<uintptr_t>(perm) & 15) == 0) {
         uint32_t g[kScanItems];
 #pragma unroll
         for (int q = 0; q < kScanItems / 4; ++q) {
