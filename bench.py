@@ -468,9 +468,9 @@ def kernel_work(P, n, evals, packed=False):
         "preprocess_kernel": ("hbm", n * PREPROCESS_BYTES),
         "sort_hist_kernel": ("hbm", n * 4),              # the depth keys once
         "onesweep_kernel": ("hbm", n * 16),              # a depth-sort pass: key + value read and written
-        "scan_onepass_kernel": ("hbm", n * 12),        # depth order read, counts gathered, offsets written
-        "emit_warp_kernel": ("hbm", P * 8 + n * 28),     # pairs written; depth order, offset, count, segments
-        "tile_count_kernel": ("hbm", P * 4),             # the tile ids once
+        "scan_onepass_kernel": ("hbm", n * 20),        # depth order read, counts gathered, both offsets written
+        "cell_expand_kernel": ("hbm", P * 4),            # the sorted values written (the entries are few)
+        "emit_warp_kernel": ("hbm", P * 8 + n * 28),     # full-key emit: pairs written; offsets, counts, rectangles
         # key + value read, and written (packed: one word written)
         "tile_sort_pass": ("hbm", P * (12 if packed else 16)),
         # key + value (packed: one word) read, value written
@@ -489,9 +489,6 @@ TRAFFIC_PER_UNIT = {
     "render_kernel": ("eval", (13.032192e6 + 0.436224e6) / 398728138),
     "tile_sort_pass": ("pair", (165.526528e6 + 34.277120e6) / 20633099),
     "tile_sort_pass_values": ("pair", (82.809600e6 + 35.105536e6) / 20633099),
-    "emit_warp_kernel": ("pair", (52.036864e6 + 118.226176e6) / 20633099),
-    "preprocess_kernel": ("gaussian", (147.195648e6 + 41.842176e6) / 600000),
-    "tile_count_kernel": ("pair", (82.591232e6 + 1.410816e6) / 20633099),
 }
 
 

@@ -72,9 +72,9 @@ typedef enum {
 /* How qb_bin_emit/qb_sort order the pairs by (tile, depth, index).  Both give
  * identical sorted values and ranges.
  *  DEPTH_FIRST  (default) sort the n Gaussians by (depth, index) once, emit
- *               each Gaussian's pairs in that order with 32-bit tile keys, then
- *               stable-sort the pairs on the tile bits only (with emit_fused
- *               the emit runs the first digit pass itself).
+ *               in that order one entry per Gaussian and cell of 8 x 4 tiles
+ *               (the cell's tiles as bits), stable-sort the entries by cell and
+ *               expand them to the tiles' lists.
  *  FULL_KEY     emit in index order with 64-bit keys (tile << 31) | depth
  *               bits and stable-sort on all 31 + tile bits (SortPairs, Sec. 2). */
 typedef enum { QB_SORT_DEPTH_FIRST = 0, QB_SORT_FULL_KEY = 1 } qb_sort_mode;
@@ -142,15 +142,8 @@ typedef struct {
     int32_t sorted_in_alt;    /* internal: sorted pairs live in buffer 1    */
     int32_t sort_mode;        /* qb_sort_mode; set before qb_preprocess     */
     int32_t depth_in_alt;     /* internal: depth order lives in buffer 1    */
-    int32_t emit_fused;       /* DEPTH_FIRST: 1 = the emit performs the tile
-                                 sort's first digit pass (per-tile counts from
-                                 the preprocess); 0 (default) = plain emit, the
-                                 per-tile counts from a histogram of the
-                                 emitted tile ids in qb_sort.  Frames of more
-                                 than 24576 tiles (beyond the histogram's
-                                 shared memory, e.g. 3840 x 2160) always take
-                                 the fused emit; 1 selects it on any frame.
-                                 Set before qb_preprocess                    */
+    int32_t emit_fused;       /* accepted, without effect: DEPTH_FIRST has one
+                                 emit for every frame size                   */
     int32_t reserved[3];      /* internal */
 } qb_frame;
 
@@ -168,7 +161,7 @@ typedef struct {
     uint32_t *offsets;  /* [n]     exclusive prefix of counts in emission order
                                    (index order, or depth order in DEPTH_FIRST) */
     uint64_t *keys;     /* [P]     FULL_KEY: (tile << 31) | depth bits, sorted after qb_sort */
-    uint32_t *tile_keys;/* [P]     DEPTH_FIRST: scratch of the tile sort; the sorted
+    uint32_t *tile_keys;/* [P]     DEPTH_FIRST: scratch of the cell sort; the sorted
                                    tile ids are given by the ranges (qb_frame_tile_keys) */
     uint32_t *vals;     /* [P]     Gaussian index, in sorted order after qb_sort */
     uint32_t *depth_order; /* [n]  DEPTH_FIRST: Gaussians by (depth, index) */
@@ -182,8 +175,8 @@ typedef struct {
     uint32_t *err_flags;/* [2]     [0]: bit0 capacity, bit1 timeout.  [1]:
                                    test-only, zero after qb_frame_init; a test
                                    may set it to k > 0 to exercise a bounded
-                                   spin-wait: the second block of the last
-                                   (values-only) tile-sort pass then finds its
+                                   spin-wait: the second tile of the last
+                                   (values-only) cell-sort pass then finds its
                                    predecessor unpublished, gives up after k
                                    polls and raises TIMEOUT; the sorted values
                                    are then undefined (do not render them)  */
@@ -252,28 +245,24 @@ qb_status qb_preprocess(qb_frame *frame, const qb_scene *scene, const qb_camera 
                         qb_stream_t stream);
 
 /* Stage 2 (Sec. 2 "DuplicateWithKeys", Sec. 3.2 QPass): exclusive scan of the
- * tile counts, then one (key, value) pair per Gaussian-tile overlap with
- * key = (tile << 31) | float bits of the depth (FULL_KEY) or the tile id
- * (DEPTH_FIRST, after sorting the Gaussians by depth), value = Gaussian
- * index, in emission order (each Gaussian's pairs at its scan offset).  In
- * DEPTH_FIRST with emit_fused the per-tile counts (from the preprocess) give
- * the ranges here, and in the QPass modes the emit also performs the first
- * digit pass of the tile sort, so the pairs leave it bucketed by their lowest
- * tile digit rather than in emission order; without emit_fused (the default)
- * qb_sort counts the emitted tile ids.
+ * tile counts in emission order, then the emit.  FULL_KEY: one (key, value)
+ * pair per Gaussian-tile overlap, key = (tile << 31) | float bits of the
+ * depth, value = Gaussian index, each Gaussian's pairs at its scan offset.
+ * DEPTH_FIRST: after sorting the Gaussians by depth, one entry per Gaussian
+ * and cell of 8 x 4 tiles (the QPass traversal on the cells), which qb_sort
+ * turns into the sorted values; vals holds them after qb_sort only.
  * If n_pairs_out is non-NULL the host synchronises once to read P, stores it
  * in *n_pairs_out and frame->n_pairs, and returns CAPACITY (writing no pairs)
  * when P > pair_capacity.  With NULL nothing synchronises; an overflow is
  * then flagged on the device and reported by qb_frame_check. */
 qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream);
 
-/* Stage 3 (Sec. 2 "SortPairs"): stable LSD radix sort of the pairs with the
- * library's onesweep sort on the key bits [0, 31 + tile bits) (FULL_KEY),
- * then the per-tile [start, end) ranges; or (DEPTH_FIRST) a histogram of
- * the emitted tile ids giving the ranges and every pass's bucket offsets
- * (unless the fused emit already did), then the remaining digit passes on
- * the tile bits, whose last pass writes only the values (in vals,
- * sorted_in_alt = 0). */
+/* Stage 3 (Sec. 2 "SortPairs"): the values by (tile, depth, index) in vals and
+ * the per-tile [start, end) ranges.  FULL_KEY: stable LSD radix sort of the
+ * pairs with the library's onesweep sort on the key bits [0, 31 + tile bits),
+ * then the ranges of the sorted keys.  DEPTH_FIRST: stable sort of the entries
+ * by cell (digits of at most sort_digit_bits), the tiles' counts and ranges,
+ * and the expansion to the tiles' lists (in vals, sorted_in_alt = 0). */
 qb_status qb_sort(qb_frame *frame, qb_stream_t stream);
 
 /* Stage 4 (Sec. 2 "Render", Eq. 2): front-to-back compositing per pixel.

@@ -58,9 +58,10 @@ bool make_layout(int n, int W, int H, uint64_t cap, Layout &L) {
     L.meta = take(4 * N);
     L.counts = take(4 * N);
     L.offsets = take(4 * N);
-    L.counts_e = take(4 * N);
+    L.cc = take(8 * N);
+    L.coff = take(4 * N);
     L.chunk_first = take(4 * chunk_table_size(cap));
-    L.segs = take(64 * N);
+    L.rects = take(32 * N);
     L.scan_part = take(8 * scan_partials_count(n));
     L.keys0 = take(8 * cap);
     L.keys1 = take(8 * cap);
@@ -84,9 +85,13 @@ bool make_layout(int n, int W, int H, uint64_t cap, Layout &L) {
     }
     L.dsort_scratch = take(db);
     L.ranges = take(8 * (size_t)tiles);
-    L.tile_counts = take(4 * ((size_t)tiles + 1));  // + the tile histogram's block counter
-    L.tile_diff = take(4 * (size_t)(tx + 1) * (ty + 1));
-    L.tile_single = take(4 * (size_t)tiles);
+    const int ncells = cell_geo(W, H, 8).ncells;
+    L.cell_zero = take(4 * cell_zero_words(ncells));
+    L.cell_start = take(4 * ((size_t)ncells + 1));
+    L.row_start = take(4 * ((size_t)ncells + 1));
+    L.row_cell = take(4 * cell_rows_max(cap, ncells));
+    L.row_counts = take(128 * cell_rows_max(cap, ncells));
+    L.tile_total = take(4 * (size_t)tiles);
     L.order_cnt = take(4 * 2 * (size_t)kOrderBuckets);
     L.order_list = take(4 * 2 * (size_t)kOrderBuckets * tiles);
     L.tfinal = take(4 * (size_t)W * H);
@@ -134,6 +139,34 @@ TileSet frame_tileset(const qb_frame *f) {
     ts.cam[0].tile_base = 0;
     ts.cam[0].pix_base = 0;
     return ts;
+}
+
+// The depth-first binning of a frame.  The cell entries' buffers are those
+// that the full-key path uses for its pairs: there are at most as many entries
+// as pairs, and vals0 receives the sorted values after the last entry is read.
+CellBin frame_cells(const qb_frame *f, const Layout &L) {
+    CellBin b;
+    std::memset(&b, 0, sizeof(b));
+    b.n = f->n;
+    b.perm = at<uint32_t>(f, f->depth_in_alt ? L.dvals1 : L.dvals0);
+    b.coff = at<uint32_t>(f, L.coff);
+    b.chunk_first = at<uint32_t>(f, L.chunk_first);
+    b.rects = at<uint4>(f, L.rects);
+    b.n_pairs = at<uint64_t>(f, L.state);
+    b.n_cells = at<uint64_t>(f, L.state + 16);
+    b.n_cells_max = f->n_pairs != UINT64_MAX ? f->n_pairs : f->pair_capacity;
+    b.capacity = f->pair_capacity;
+    b.naive = (f->bin_mode & 0xff) == QB_BIN_QUADBOX_NAIVE;
+    b.err = at<uint32_t>(f, L.state + 8);
+    b.sort_scratch = at<void>(f, L.sort_scratch);
+    b.geo = cell_geo(f->width, f->height, f->sort_digit_bits);
+    b.arr = CellArrays{at<uint32_t>(f, L.cell_zero), at<uint32_t>(f, L.cell_start), at<uint32_t>(f, L.row_start),
+                       at<uint32_t>(f, L.row_cell),  at<uint32_t>(f, L.row_counts), at<uint32_t>(f, L.tile_total),
+                       at<uint32_t>(f, L.vals1),     at<uint32_t>(f, L.vals0),      at<uint64_t>(f, L.keys0),
+                       at<uint64_t>(f, L.keys1)};
+    b.ranges = at<uint2>(f, L.ranges);
+    b.vals = at<uint32_t>(f, L.vals0);
+    return b;
 }
 
 CamSet frame_camset(const qb_camera &c) {
@@ -333,33 +366,17 @@ qb_status qb_preprocess(qb_frame *frame, const qb_scene *scene, const qb_camera 
     a.r3 = at<float>(frame, L.r3);
     a.meta = at<int>(frame, L.meta);
     a.counts = at<uint32_t>(frame, L.counts);
-    a.tile_diff = nullptr;
-    a.tile_single = nullptr;
-    a.segs = at<uint4>(frame, L.segs);
-    std::memset(a.diff_off, 0, sizeof(a.diff_off));
-    std::memset(a.single_off, 0, sizeof(a.single_off));
+    a.cc = at<uint2>(frame, L.cc);
+    a.rects = at<uint4>(frame, L.rects);
     if (frame->sort_mode < QB_SORT_DEPTH_FIRST || frame->sort_mode > QB_SORT_FULL_KEY)
         return fail(QB_ERR_INVALID_ARG, "invalid sort_mode %d", frame->sort_mode);
     const int eff = frame->sort_mode;
-    // the fused emit needs the per-tile counts before it runs: from the
-    // preprocess's difference arrays (also when the grid is too large for the
-    // histogram of the unfused path)
-    const bool fused = eff == QB_SORT_DEPTH_FIRST &&
-                       (frame->emit_fused != 0 || frame->tiles_x * frame->tiles_y > kTileCountMax);
-    if (fused) {
-        a.tile_diff = at<int>(frame, L.tile_diff);
-        a.tile_single = at<int>(frame, L.tile_single);
-        // the two count arrays are adjacent in the workspace: clear them together
-        QB_CUDA(cudaMemsetAsync(a.tile_diff, 0, L.tile_single - L.tile_diff + 4 * (size_t)frame->tiles_x * frame->tiles_y,
-                                (cudaStream_t)stream));
-    }
     if (eff != QB_SORT_FULL_KEY) {  // the depth-order sort's keys, written by the preprocess
         a.depth_keys = at<uint32_t>(frame, L.dkeys0);
         a.depth_vals = at<uint32_t>(frame, L.dvals0);
     }
     QB_CUDA(launch_preprocess(a, scene->sh_degree, (cudaStream_t)stream));
-    // requested sort | effective sort << 8 | fused emit << 16, as the counts were made for
-    frame->reserved[0] = frame->sort_mode | (eff << 8) | ((fused ? 1 : 0) << 16);
+    frame->reserved[0] = frame->sort_mode;  // the sort that the preprocess was made for
     frame->bin_mode = mode;
     frame->sh_degree = scene->sh_degree;
     frame->stage = 1;
@@ -374,17 +391,17 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
     if (frame->stage < 1) return fail(QB_ERR_STATE, "qb_bin_emit before qb_preprocess");
     if (frame->sort_mode < QB_SORT_DEPTH_FIRST || frame->sort_mode > QB_SORT_FULL_KEY)
         return fail(QB_ERR_INVALID_ARG, "invalid sort_mode %d", frame->sort_mode);
-    if (frame->sort_mode != (frame->reserved[0] & 0xff))
+    if (frame->sort_mode != frame->reserved[0])
         return fail(QB_ERR_STATE, "sort_mode changed between qb_preprocess and qb_bin_emit");
-    const int eff = (frame->reserved[0] >> 8) & 0xff;
-    const bool fused = (frame->reserved[0] >> 16) & 1;
     if (frame->sort_digit_bits < 8 || frame->sort_digit_bits > kMaxDigitBits)
         return fail(QB_ERR_INVALID_ARG, "sort_digit_bits must be 8..11");
     cudaStream_t s = (cudaStream_t)stream;
     uint64_t *d_np = at<uint64_t>(frame, L.state);
     uint32_t *err = at<uint32_t>(frame, L.state + 8);
-    const bool depth_first = eff != QB_SORT_FULL_KEY;  // Gaussians emitted in depth order
-    const uint32_t *perm = nullptr;
+    const bool depth_first = frame->sort_mode != QB_SORT_FULL_KEY;  // Gaussians emitted in depth order
+    uint64_t *partials = at<uint64_t>(frame, L.scan_part);
+    uint32_t *chunk_first = at<uint32_t>(frame, L.chunk_first);
+    const uint32_t chunk_cap = (uint32_t)chunk_table_size(frame->pair_capacity);
     if (depth_first) {
         // emission order = Gaussians sorted by (depth, index)
         uint32_t *dk0 = at<uint32_t>(frame, L.dkeys0), *dk1 = at<uint32_t>(frame, L.dkeys1);
@@ -395,20 +412,13 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
             QB_CUDA(sort_pairs(dk0, dv0, dk1, dv1, (uint64_t)frame->n, nullptr, kDepthBits, kDepthDigitBits,
                                at<void>(frame, L.dsort_scratch), err, s, &passes));
         frame->depth_in_alt = passes & 1;
-        perm = frame->depth_in_alt ? dv1 : dv0;
-    }
-    QB_CUDA(launch_scan(at<uint32_t>(frame, L.counts), perm, frame->n, at<uint32_t>(frame, L.offsets),
-                        at<uint64_t>(frame, L.scan_part), d_np, err, s, at<uint32_t>(frame, L.counts_e),
-                        at<uint32_t>(frame, L.chunk_first), (uint32_t)chunk_table_size(frame->pair_capacity)));
-    if (eff == QB_SORT_DEPTH_FIRST && fused) {
-        // per-tile counts -> ranges and the tile sort's bucket offsets
-        const int tile_bits = frame->key_bits - kDepthBits;
-        const uint32_t zero_off[1] = {0u};
-        QB_CUDA(launch_tile_prep(at<int>(frame, L.tile_diff), at<int>(frame, L.tile_single), frame_tileset(frame),
-                                 zero_off, zero_off,
-                                 at<uint2>(frame, L.ranges), sort_hist_table(at<void>(frame, L.sort_scratch)),
-                                 sort_hist_stride(), frame->sort_digit_bits, tile_bits, frame->pair_capacity, s));
-        frame->reserved[1] = frame->sort_digit_bits;  // digit width the offsets were made for
+        QB_CUDA(launch_scan_cells(at<uint2>(frame, L.cc), frame->depth_in_alt ? dv1 : dv0, frame->n,
+                                  at<uint32_t>(frame, L.offsets), at<uint32_t>(frame, L.coff), partials, d_np,
+                                  at<uint64_t>(frame, L.state + 16), frame->pair_capacity, err, chunk_first, chunk_cap,
+                                  s));
+    } else {
+        QB_CUDA(launch_scan(at<uint32_t>(frame, L.counts), frame->n, at<uint32_t>(frame, L.offsets),
+                            at<uint32_t>(frame, L.coff), partials, d_np, err, chunk_first, chunk_cap, s));
     }
     frame->n_pairs = UINT64_MAX;
     if (n_pairs_out) {
@@ -423,56 +433,26 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
         }
         frame->n_pairs = P;
     }
-    EmitArgs a;
-    std::memset(&a, 0, sizeof(a));
-    a.n = frame->n;
-    a.n_per_cam = frame->n > 0 ? frame->n : 1;
-    a.ts = frame_tileset(frame);
-    a.perm = perm;
-    a.xy = at<float2>(frame, L.xy);
-    a.box = at<float4>(frame, L.box);
-    a.r3 = at<float>(frame, L.r3);
-    a.meta = at<int>(frame, L.meta);
-    a.rgbd = at<float4>(frame, L.rgbd);
-    a.counts = at<uint32_t>(frame, L.counts);
-    a.offsets = at<uint32_t>(frame, L.offsets);
-    a.counts_e = at<uint32_t>(frame, L.counts_e);
-    a.chunk_first = at<uint32_t>(frame, L.chunk_first);
-    a.vals = at<uint32_t>(frame, L.vals0);
-    a.n_pairs = d_np;
-    a.n_pairs_host = frame->n_pairs;
-    a.capacity = frame->pair_capacity;
-    a.mode = frame->bin_mode & 0xff;
-    a.clamp3s = (frame->bin_mode & QB_BIN_NO_CLAMP) == 0;
-    a.err = err;
-    a.segs = at<uint4>(frame, L.segs);
     if (depth_first) {
-        // QPass emit in depth order; in the QPass modes it also performs the
-        // tile sort's first digit pass (qb_sort runs the remaining ones)
-        void *scratch = at<void>(frame, L.sort_scratch);
-        const int rb = frame->sort_digit_bits;
-        const int tile_bits = frame->key_bits - kDepthBits;
-        const int passes = tile_bits > 0 ? (tile_bits + rb - 1) / rb : 0;
-        uint32_t *kA = at<uint32_t>(frame, L.keys0), *vA = at<uint32_t>(frame, L.vals0);
-        uint32_t *kB = at<uint32_t>(frame, L.keys1), *vB = at<uint32_t>(frame, L.vals1);
-        if (fused && passes > 0 && a.mode != QB_BIN_QUADBOX_NAIVE) {
-            const bool to_a = pass_writes_a(passes, 0);
-            QB_CUDA(sort_clear(scratch, frame->pair_capacity, rb, 0, 1, s));
-            QB_CUDA(launch_emit_sweep(a, pass_geo(tile_bits, rb).bits[0], passes > 1, to_a ? kA : kB, to_a ? vA : vB,
-                                      sort_hist_table(scratch),
-                                      sort_lookback(scratch, frame->pair_capacity, rb, 0), sort_counter(scratch, 0),
-                                      s));
-            frame->reserved[2] = 1;  // first pass left to qb_sort
-        } else {
-            // plain emit into the buffer the first pass reads (or the final one)
-            const bool into_a = passes == 0 || !pass_writes_a(passes, 0);
-            a.vals = into_a ? vA : vB;
-            QB_CUDA(launch_emit<uint32_t>(a, into_a ? kA : kB, s));
-            frame->reserved[2] = 0;
-        }
-        frame->reserved[1] = frame->sort_digit_bits;  // digit width the buffers were chosen for
+        QB_CUDA(launch_cell_emit(frame_cells(frame, L), s));
+        frame->reserved[1] = frame->sort_digit_bits;  // digit width the bucket offsets were made for
     } else {
-        QB_CUDA(launch_emit<uint64_t>(a, at<uint64_t>(frame, L.keys0), s));
+        EmitArgs a;
+        std::memset(&a, 0, sizeof(a));
+        a.n = frame->n;
+        a.rgbd = at<float4>(frame, L.rgbd);
+        a.counts = at<uint32_t>(frame, L.counts);
+        a.offsets = at<uint32_t>(frame, L.offsets);
+        a.chunk_first = chunk_first;
+        a.rects = at<uint4>(frame, L.rects);
+        a.vals = at<uint32_t>(frame, L.vals0);
+        a.n_pairs = d_np;
+        a.n_pairs_host = frame->n_pairs;
+        a.capacity = frame->pair_capacity;
+        a.mode = frame->bin_mode & 0xff;
+        a.err = err;
+        a.tiles_x = (uint32_t)frame->tiles_x;
+        QB_CUDA(launch_emit(a, at<uint64_t>(frame, L.keys0), s));
     }
     frame->stage = 2;
     return QB_OK;
@@ -489,42 +469,21 @@ qb_status qb_sort(qb_frame *frame, qb_stream_t stream) {
     const bool known = frame->n_pairs != UINT64_MAX;
     const uint64_t n_max = known ? frame->n_pairs : frame->pair_capacity;
     const uint64_t *n_dev = known ? nullptr : at<uint64_t>(frame, L.state);
-    int passes = 0;
-    const int ntiles = frame->tiles_x * frame->tiles_y;
-    uint32_t *err = at<uint32_t>(frame, L.state + 8);
-    const int eff = (frame->reserved[0] >> 8) & 0xff;
-    const bool fused = (frame->reserved[0] >> 16) & 1;
-    if (eff == QB_SORT_DEPTH_FIRST) {
-        // pairs were emitted in depth order: a stable sort on the tile id alone
-        // (bucket offsets and ranges came from the per-tile counts in qb_bin_emit)
+    if (frame->reserved[0] != QB_SORT_FULL_KEY) {
+        // entries were emitted in depth order: a stable sort by cell, then the
+        // expansion to the tiles' lists
         if (frame->sort_digit_bits != frame->reserved[1])
             return fail(QB_ERR_STATE, "sort_digit_bits changed between qb_bin_emit and qb_sort");
-        const int tile_bits = frame->key_bits - kDepthBits;
-        const int rb = frame->sort_digit_bits;
-        passes = tile_bits > 0 ? (tile_bits + rb - 1) / rb : 0;
-        if (!fused) {
-            // per-tile counts from the emitted tile ids -> ranges and every
-            // pass's bucket offsets
-            const uint32_t *src = at<uint32_t>(frame, passes > 0 && pass_writes_a(passes, 0) ? L.keys1 : L.keys0);
-            uint32_t *counts = at<uint32_t>(frame, L.tile_counts);
-            QB_CUDA(launch_tile_count(src, n_max, n_dev, ntiles, counts, at<uint2>(frame, L.ranges),
-                                      sort_hist_table(at<void>(frame, L.sort_scratch)), sort_hist_stride(), rb,
-                                      tile_bits, s));
-        }
-        if (passes > 0)
-            QB_CUDA(tile_sort_passes(at<uint32_t>(frame, L.keys0), at<uint32_t>(frame, L.vals0),
-                                     at<uint32_t>(frame, L.keys1), at<uint32_t>(frame, L.vals1), frame->pair_capacity,
-                                     n_max, n_dev, tile_bits, frame->reserved[2], rb, at<void>(frame, L.sort_scratch),
-                                     err, s, (uint64_t)frame->n));
+        QB_CUDA(launch_cell_sort(frame_cells(frame, L), s));
         frame->sorted_in_alt = 0;  // the values end in vals0; the tile of each is given by the ranges
-        (void)ntiles;
     } else {
+        int passes = 0;
         QB_CUDA(sort_pairs(at<uint64_t>(frame, L.keys0), at<uint32_t>(frame, L.vals0), at<uint64_t>(frame, L.keys1),
                            at<uint32_t>(frame, L.vals1), n_max, n_dev, frame->key_bits, frame->sort_digit_bits,
-                           at<void>(frame, L.sort_scratch), err, s, &passes));
+                           at<void>(frame, L.sort_scratch), at<uint32_t>(frame, L.state + 8), s, &passes));
         frame->sorted_in_alt = passes & 1;
         const uint64_t *sorted = at<uint64_t>(frame, frame->sorted_in_alt ? L.keys1 : L.keys0);
-        QB_CUDA(launch_ranges<uint64_t>(sorted, n_max, n_dev, at<uint2>(frame, L.ranges), ntiles, s));
+        QB_CUDA(launch_ranges(sorted, n_max, n_dev, at<uint2>(frame, L.ranges), frame->tiles_x * frame->tiles_y, s));
     }
     frame->stage = 3;
     return QB_OK;

@@ -3,9 +3,8 @@
 // launch projects the scene into every camera of a group (one grid row per
 // camera), so the scene's parameters and SH coefficients are read once per
 // group.  Each camera's pairs are then binned like a single frame -- depth
-// order of its records, scan, QPass emit with camera-local tile ids, the
-// shared-memory tile histogram (ranges and bucket offsets) and the two-pass
-// tile sort -- into the camera's own slot of sorted values.  Last, one
+// order of its records, scan, and the cell binning (qb_cells.cu) with
+// camera-local ids -- into the camera's own slot of sorted values.  Last, one
 // persistent render takes tiles of every camera of the batch from one global
 // work queue, so cameras of uneven resolution balance across the whole GPU
 // and no camera's tail leaves SMs idle before the next one starts.
@@ -43,32 +42,28 @@ struct Geo {  // per-camera geometry of a batch
     int tx[QB_MAX_CAMERAS], ty[QB_MAX_CAMERAS];
     uint64_t tile_base[QB_MAX_CAMERAS + 1];
     uint64_t pix_base[QB_MAX_CAMERAS + 1];
-    int max_tile_bits, max_tiles;
+    int max_tiles, max_cells;
 };
 
-int bits_for(uint64_t v) {  // bits to hold values < v
-    int b = 0;
-    while ((1ull << b) < v) ++b;
-    return b;
-}
+constexpr int kMaxCameraTiles = 24576;  // accepted tiles of one camera
 
 bool make_geo(int n_cams, const int32_t *W, const int32_t *H, Geo &g) {
     if (n_cams < 1 || n_cams > QB_MAX_CAMERAS || !W || !H) return false;
     g.tile_base[0] = 0;
     g.pix_base[0] = 0;
-    g.max_tile_bits = 1;
     g.max_tiles = 1;
+    g.max_cells = 1;
     for (int k = 0; k < n_cams; ++k) {
         if (W[k] <= 0 || H[k] <= 0 || W[k] > (1 << 15) || H[k] > (1 << 15)) return false;
         g.tx[k] = (W[k] + kTile - 1) / kTile;
         g.ty[k] = (H[k] + kTile - 1) / kTile;
         const int tiles = g.tx[k] * g.ty[k];
-        if (tiles > kTileCountMax) return false;  // beyond the tile histogram's shared memory
+        if (tiles > kMaxCameraTiles) return false;
         g.tile_base[k + 1] = g.tile_base[k] + (uint64_t)tiles;
         g.pix_base[k + 1] = g.pix_base[k] + (uint64_t)W[k] * H[k];
         g.max_tiles = tiles > g.max_tiles ? tiles : g.max_tiles;
-        const int tb = bits_for((uint64_t)tiles);
-        g.max_tile_bits = tb > g.max_tile_bits ? tb : g.max_tile_bits;
+        const int cells = cell_geo(W[k], H[k], 8).ncells;
+        g.max_cells = cells > g.max_cells ? cells : g.max_cells;
     }
     return g.tile_base[n_cams] < (1ull << 32);
 }
@@ -85,10 +80,11 @@ struct BLayout {
     size_t slots;                                     // [n_cams][cap] sorted values per camera
     size_t ranges;                                    // [total tiles]
     size_t tfinal, ncontrib, neval;                   // [total pixels]
-    size_t segs, dk0, dk1, dv0, dv1;                  // [group * n] group scratch
+    size_t rects, cc, dk0, dk1, dv0, dv1;             // [group * n] group scratch
     // one camera's binning scratch, kBatchStreams sets set_stride bytes apart:
-    size_t keysA, keysB, valsT;                       // [cap] pairs
-    size_t offsets, counts_e, chunk_first, scan_part, dsort, sort, tile_counts;
+    size_t keysA, valsA, valsB;                       // [cap] cell entries
+    size_t offsets, coff, chunk_first, scan_part, dsort, sort, n_cells;
+    size_t cell_zero, cell_start, row_start, row_cell, row_counts, tile_total;
     size_t set_stride;
     size_t gscreen;                                   // [n_cams * n][9]
     size_t queue, state;
@@ -119,29 +115,36 @@ bool make_blayout(int n, int n_cams, int group, uint64_t cap, const Geo &g, BLay
     L.tfinal = take(4 * g.pix_base[n_cams]);
     L.ncontrib = take(4 * g.pix_base[n_cams]);
     L.neval = take(4 * g.pix_base[n_cams]);
-    L.segs = take(64 * grecs);
+    L.rects = take(32 * grecs);
+    L.cc = take(8 * grecs);
     L.dk0 = take(4 * grecs);
     L.dk1 = take(4 * grecs);
     L.dv0 = take(4 * grecs);
     L.dv1 = take(4 * grecs);
     const size_t set0 = off;
     L.keysA = take(4 * cap);
-    L.keysB = take(4 * cap);
-    L.valsT = take(4 * cap);
+    L.valsA = take(8 * cap);
+    L.valsB = take(8 * cap);
     L.offsets = take(4 * (size_t)n);
-    L.counts_e = take(4 * (size_t)n);
+    L.coff = take(4 * (size_t)n);
     L.chunk_first = take(4 * chunk_table_size(cap));
     L.scan_part = take(8 * scan_partials_count(n));
     size_t db = 0, sb = 0;
     for (int d = 8; d <= kMaxDigitBits; ++d) {
         const size_t b1 = sort_scratch_bytes((uint64_t)n, kDepthBits, d);
-        const size_t b2 = sort_scratch_bytes(cap, g.max_tile_bits, d);
+        const size_t b2 = cell_sort_scratch_bytes(cap, g.max_cells, d);
         db = b1 > db ? b1 : db;
         sb = b2 > sb ? b2 : sb;
     }
     L.dsort = take(db);
     L.sort = take(sb);
-    L.tile_counts = take(4 * ((size_t)g.max_tiles + 1));
+    L.n_cells = take(8);
+    L.cell_zero = take(4 * cell_zero_words(g.max_cells));
+    L.cell_start = take(4 * ((size_t)g.max_cells + 1));
+    L.row_start = take(4 * ((size_t)g.max_cells + 1));
+    L.row_cell = take(4 * cell_rows_max(cap, g.max_cells));
+    L.row_counts = take(128 * cell_rows_max(cap, g.max_cells));
+    L.tile_total = take(4 * (size_t)g.max_tiles);
     L.set_stride = off - set0;
     off += (kBatchStreams - 1) * L.set_stride;  // the other sets
     L.gscreen = take(72 * recs);
@@ -434,7 +437,8 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
         a.r3 = bat<float>(b, L.r3) + v.rec0;
         a.meta = bat<int>(b, L.meta) + v.rec0;
         a.counts = bat<uint32_t>(b, L.counts) + v.rec0;
-        a.segs = bat<uint4>(b, L.segs);
+        a.rects = bat<uint4>(b, L.rects);
+        a.cc = bat<uint2>(b, L.cc);
         a.depth_keys = bat<uint32_t>(b, L.dk0);  // the depth-order sort's keys and record indices
         a.depth_vals = bat<uint32_t>(b, L.dv0);
         QB_BCUDA(launch_preprocess(a, scene->sh_degree, s));
@@ -450,9 +454,6 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
             const int set = nside > 0 ? c % nside : 0;
             const cudaStream_t cs = nside > 0 ? ss.side[set] : s;
             const size_t so = (size_t)set * L.set_stride;
-            uint32_t *keysA = bat<uint32_t>(b, L.keysA + so), *keysB = bat<uint32_t>(b, L.keysB + so);
-            uint32_t *valsT = bat<uint32_t>(b, L.valsT + so);
-            void *sort_scratch = bat<void>(b, L.sort + so);
             const size_t r0 = (size_t)c * n;  // the camera's records within the group
             uint32_t *dk0 = bat<uint32_t>(b, L.dk0) + r0, *dk1 = bat<uint32_t>(b, L.dk1) + r0;
             uint32_t *dv0 = bat<uint32_t>(b, L.dv0) + r0, *dv1 = bat<uint32_t>(b, L.dv1) + r0;
@@ -461,49 +462,37 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
                 QB_BCUDA(sort_pairs(dk0, dv0, dk1, dv1, (uint64_t)n, nullptr, kDepthBits, kDepthDigitBits,
                                     bat<void>(b, L.dsort + so), err, cs, &passes));
             const uint32_t *perm = (passes & 1) ? dv1 : dv0;  // group record indices in depth order
-            QB_BCUDA(launch_scan(a.counts, perm, n, bat<uint32_t>(b, L.offsets + so),
-                                 bat<uint64_t>(b, L.scan_part + so), npairs + k, err, cs,
-                                 bat<uint32_t>(b, L.counts_e + so), bat<uint32_t>(b, L.chunk_first + so),
-                                 (uint32_t)chunk_table_size(cap)));
-            const int ntiles = geo.tx[k] * geo.ty[k];
-            const int tile_bits = bits_for((uint64_t)ntiles);
-            const int tpasses = tile_bits > 0 ? (tile_bits + rb - 1) / rb : 0;
-            uint32_t *slot = bat<uint32_t>(b, L.slots) + (size_t)k * cap;
-            // plain emit into the buffer pair the first pass reads (or the final one)
-            const bool into_a = tpasses == 0 || !pass_writes_a(tpasses, 0);
-            EmitArgs e;
+            uint64_t *n_cells = bat<uint64_t>(b, L.n_cells + so);
+            uint32_t *coff = bat<uint32_t>(b, L.coff + so), *chunk_first = bat<uint32_t>(b, L.chunk_first + so);
+            QB_BCUDA(launch_scan_cells(a.cc, perm, n, bat<uint32_t>(b, L.offsets + so), coff,
+                                       bat<uint64_t>(b, L.scan_part + so), npairs + k, n_cells, cap, err, chunk_first,
+                                       (uint32_t)chunk_table_size(cap), cs));
+            CellBin e;
             std::memset(&e, 0, sizeof(e));
             e.n = n;
-            e.n_per_cam = n > 0 ? n : 1;
             e.perm = perm;
-            e.xy = a.xy;
-            e.box = a.box;
-            e.r3 = a.r3;
-            e.meta = a.meta;
-            e.rgbd = a.rgbd;
-            e.counts = a.counts;
-            e.offsets = bat<uint32_t>(b, L.offsets + so);
-            e.counts_e = bat<uint32_t>(b, L.counts_e + so);
-            e.chunk_first = bat<uint32_t>(b, L.chunk_first + so);
-            e.segs = bat<uint4>(b, L.segs);
-            e.vals = into_a ? slot : valsT;
+            e.coff = coff;
+            e.chunk_first = chunk_first;
+            e.rects = a.rects;
             e.n_pairs = npairs + k;
-            e.n_pairs_host = UINT64_MAX;
+            e.n_cells = n_cells;
+            e.n_cells_max = cap;
             e.capacity = cap;
-            e.mode = base_mode;
-            e.clamp3s = a.clamp3s;
+            e.naive = base_mode == QB_BIN_QUADBOX_NAIVE;
             e.err = err;
-            e.ts = v.ts;
-            QB_BCUDA(launch_emit<uint32_t>(e, into_a ? keysA : keysB, cs));
-            // per-tile counts -> the camera's ranges and every pass's bucket
-            // offsets; then the tile sort, whose last pass writes the slot
-            uint2 *ranges = bat<uint2>(b, L.ranges) + geo.tile_base[k];
-            QB_BCUDA(launch_tile_count(into_a ? keysA : keysB, cap, npairs + k, ntiles,
-                                       bat<uint32_t>(b, L.tile_counts + so), ranges, sort_hist_table(sort_scratch),
-                                       sort_hist_stride(), rb, tile_bits, cs));
-            if (tpasses > 0)
-                QB_BCUDA(tile_sort_passes(keysA, slot, keysB, valsT, cap, cap, npairs + k, tile_bits, 0, rb,
-                                          sort_scratch, err, cs, (uint64_t)b->group * (uint64_t)b->n));
+            e.sort_scratch = bat<void>(b, L.sort + so);
+            e.geo = cell_geo(b->widths[k], b->heights[k], rb);
+            // (the slot holds the cell ids of a second pass until the expansion writes the values)
+            uint32_t *slot = bat<uint32_t>(b, L.slots) + (size_t)k * cap;
+            e.arr = CellArrays{bat<uint32_t>(b, L.cell_zero + so), bat<uint32_t>(b, L.cell_start + so),
+                               bat<uint32_t>(b, L.row_start + so), bat<uint32_t>(b, L.row_cell + so),
+                               bat<uint32_t>(b, L.row_counts + so), bat<uint32_t>(b, L.tile_total + so),
+                               bat<uint32_t>(b, L.keysA + so), slot, bat<uint64_t>(b, L.valsA + so),
+                               bat<uint64_t>(b, L.valsB + so)};
+            e.ranges = bat<uint2>(b, L.ranges) + geo.tile_base[k];
+            e.vals = slot;
+            QB_BCUDA(launch_cell_emit(e, cs));
+            QB_BCUDA(launch_cell_sort(e, cs));
         }
         for (int i = 0; i < nside; ++i) {  // join before the next group's preprocess reuses the group scratch
             QB_BCUDA(cudaEventRecord(ss.join[i], ss.side[i]));

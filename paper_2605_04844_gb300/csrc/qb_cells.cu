@@ -1,0 +1,540 @@
+// qb_cells.cu -- K3-K5 of the depth-first path (DuplicateWithKeys with QPass
+// traversal, SortPairs and the tile ranges of Sec. 2 and 3.2), through cells
+// of 8 x 4 tiles.
+//
+// Sorting every (tile, Gaussian) pair moves each pair through memory several
+// times (emit, histogram, two digit passes: about 40 bytes and a dozen
+// instructions per pair).  A Gaussian's tiles lie in few cells, 8 to 24 tiles
+// of it per cell on the frames measured, so here one entry stands for all its tiles in a
+// cell: (cell id; Gaussian | tile bits << 32).  The entries are emitted in
+// depth order and sorted by cell, one digit pass at 1080p over a twelfth of
+// the elements, and only then expanded:
+//   cell_count    per row (at most kCellRow consecutive entries of one cell) the number of
+//                 entries of each of the cell's 32 tiles: the tile bits of 32
+//                 entries, transposed across a warp, are one word per tile;
+//   cell_prefix   per cell the exclusive prefix over its rows, the tiles'
+//                 totals, and from these the ranges of all tiles;
+//   cell_expand   per row, each tile's Gaussians to the tile's list, 32
+//                 entries at a time: a ballot per tile gives the compacted
+//                 positions, so a tile's stores are contiguous.
+// The result (values in tile order, depth order within a tile; the ranges)
+// is the one of the stable sort of all pairs by tile id.
+// One GB300, start of the frame to its sorted values without the depth order:
+// 1M Gaussians at 1080p (34.8M pairs, 2.7M entries), emit + histogram + two
+// pair passes 0.54 ms, now 0.23; 3-sigma boxes (100.8M pairs, 5.0M entries)
+// 1.36 -> 0.39 ms; 3840 x 2160 (126M pairs, 6.4M entries) 1.9 -> 0.54 ms.
+#include <algorithm>
+
+#include "qb_scan.cuh"
+#include "qb_sweep.cuh"
+
+namespace qb {
+
+constexpr int kCellWarps = 8;             // warps per emit block
+constexpr uint32_t kCellChunk = 512;      // emitted entries per warp and step
+constexpr int kCellHistMax = 4096;        // cells a block's histogram holds in shared memory
+static_assert(kCellChunk % kEmitStride == 0, "a warp's range starts on the scan's chunk table");
+
+CellGeo cell_geo(int W, int H, int digit_bits) {
+    CellGeo g;
+    g.tiles_x = (W + kTile - 1) / kTile;
+    g.tiles_y = (H + kTile - 1) / kTile;
+    g.ntiles = g.tiles_x * g.tiles_y;
+    g.cells_x = (g.tiles_x + kCellX - 1) / kCellX;
+    g.cells_y = (g.tiles_y + kCellY - 1) / kCellY;
+    g.ncells = g.cells_x * g.cells_y;
+    g.cell_bits = 0;
+    while ((1 << g.cell_bits) < g.ncells) ++g.cell_bits;
+    g.digit_bits = digit_bits;
+    g.passes = pass_geo(g.cell_bits, g.digit_bits);
+    return g;
+}
+
+size_t cell_sort_scratch_bytes(uint64_t pair_capacity, int ncells, int digit_bits) {
+    int bits = 1;
+    while ((1 << bits) < ncells) ++bits;
+    return sort_scratch_bytes(pair_capacity, bits, digit_bits);
+}
+
+// A warp's table of the cell-level QPass segments of 32 Gaussians, and their
+// tile rectangles.
+struct CellTable {
+    int32_t start[32 * 7];  // range position of the segment's first entry
+    uint32_t geo[32 * 7];   // first line | first cell << 16
+    uint32_t len[32 * 7];   // cells per line | owner lane << 16 | column flag << 24
+    float inv[32 * 7];      // 1 / cells per line
+    uint32_t gid[32];
+    uint4 rects[32][2];
+};
+
+__device__ __forceinline__ uint64_t cell_value(uint32_t gid, uint32_t bits) { return ((uint64_t)bits << 32) | gid; }
+
+__device__ __forceinline__ uint32_t tiles_in_cell(const uint4 &w0, const uint4 &w1, int cx, int cy) {
+    return cell_bits_of(unpack_rect(w0.x, w0.y), cx, cy) | cell_bits_of(unpack_rect(w0.z, w0.w), cx, cy) |
+           cell_bits_of(unpack_rect(w1.x, w1.y), cx, cy) | cell_bits_of(unpack_rect(w1.z, w1.w), cx, cy);
+}
+
+// Entries [C, C + L) in emission order, by one warp: the Gaussian whose run
+// holds entry C comes from the scan's table; the following ones are taken 32
+// at a time, each lane decomposing its Gaussian's cells into runs, and the
+// range is produced 32 consecutive entries at a time (lane q finds its run
+// from a ballot of the run starts in its group).
+__device__ __forceinline__ void cell_emit_range(const CellBin &b, uint64_t E, uint64_t C, int32_t L, CellTable &S,
+                                                uint32_t *hist) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t le_mask = lanemask_le();
+    int64_t j0 = b.chunk_first[C / kEmitStride];
+    int32_t done_to = 0;  // range positions [0, done_to) produced
+    while (done_to < L && j0 < b.n) {
+        const int64_t j = j0 + lane;
+        uint32_t gid = 0;
+        int64_t rel = (int64_t)1 << 40;
+        if (j < b.n) {
+            gid = b.perm[j];
+            rel = (int64_t)b.coff[j] - (int64_t)C;
+        }
+        // the run ends where the next one begins
+        int64_t end = __shfl_down_sync(0xffffffffu, rel, 1);
+        if (lane == 31) end = j + 1 < b.n ? (int64_t)b.coff[j + 1] - (int64_t)C : (int64_t)E - (int64_t)C;
+        if (end == (int64_t)1 << 40) end = (int64_t)E - (int64_t)C;
+        if (j >= b.n) rel = end = (int64_t)E - (int64_t)C;
+        const bool relevant = end > rel && rel < L && end > 0;
+        QSeg seg[7];
+#pragma unroll
+        for (int q = 0; q < 7; ++q) seg[q] = QSeg{0, 0, 0, 0};
+        bool columns = false;
+        __syncwarp();
+        if (relevant) {
+            const uint4 w0 = b.rects[2 * (size_t)gid], w1 = b.rects[2 * (size_t)gid + 1];
+            S.rects[lane][0] = w0;
+            S.rects[lane][1] = w1;
+            const Rect r[4] = {cell_rect(unpack_rect(w0.x, w0.y)), cell_rect(unpack_rect(w0.z, w0.w)),
+                               cell_rect(unpack_rect(w1.x, w1.y)), cell_rect(unpack_rect(w1.z, w1.w))};
+            QPass qp;
+            if (qpass_setup(r, qp)) {
+                qpass_segments(qp, seg);
+                columns = qp.columns;
+            }
+        }
+        int ns = 0;
+#pragma unroll
+        for (int q = 0; q < 7; ++q) ns += seg_empty(seg[q]) ? 0 : 1;
+        S.gid[lane] = gid;
+        const int sincl = warp_incl_scan(ns);
+        const int nseg = __shfl_sync(0xffffffffu, sincl, 31);
+        int32_t r0 = (int32_t)(rel > -((int64_t)1 << 30) ? rel : -((int64_t)1 << 30));
+        int k = sincl - ns;  // this lane's first table entry
+#pragma unroll
+        for (int q = 0; q < 7; ++q) {
+            if (seg_empty(seg[q])) continue;
+            S.start[k] = r0;
+            S.geo[k] = (uint32_t)seg[q].s0 | ((uint32_t)seg[q].lo << 16);
+            S.len[k] = (uint32_t)seg[q].len | ((uint32_t)lane << 16) | ((uint32_t)columns << 24);
+            S.inv[k] = 1.0f / (float)seg[q].len;
+            r0 += seg[q].nl * seg[q].len;
+            ++k;
+        }
+        const int64_t last_end = __shfl_sync(0xffffffffu, end, 31);
+        const int32_t batch_end = (int32_t)(last_end < (int64_t)L ? last_end : (int64_t)L);
+        __syncwarp();
+        // cur: last segment starting at or before done_to
+        int cur = -1;
+        for (int q = 0; q < nseg; q += 32) {
+            const bool le = q + lane < nseg && S.start[q + lane] <= done_to;
+            cur += __popc(__ballot_sync(0xffffffffu, le));
+        }
+        for (int32_t c0 = done_to; c0 < batch_end; c0 += 32) {
+            const int cand = cur + 1 + lane;
+            uint32_t bit = 0u;
+            if (cand < nseg) {
+                const int32_t st = S.start[cand];
+                if (st < c0 + 32) bit = 1u << (st - c0);
+            }
+            const uint32_t M = __reduce_or_sync(0xffffffffu, bit);
+            const int32_t p = c0 + lane;
+            if (p < batch_end) {
+                const int idx = cur + __popc(M & le_mask);
+                const uint32_t geo = S.geo[idx], ln = S.len[idx];
+                uint32_t q, r;
+                seg_divide((uint32_t)(p - S.start[idx]), ln & 0xffffu, S.inv[idx], q, r);
+                const uint32_t line = (geo & 0xffffu) + q, u = (geo >> 16) + r;
+                const bool cols = (ln >> 24) & 1u;
+                const uint32_t owner = (ln >> 16) & 0xffu;
+                const uint32_t cx = cols ? line : u, cy = cols ? u : line;
+                const uint32_t cell = cy * (uint32_t)b.geo.cells_x + cx;
+                b.arr.keys_a[C + p] = cell;
+                b.arr.vals_a[C + p] =
+                    cell_value(S.gid[owner], tiles_in_cell(S.rects[owner][0], S.rects[owner][1], (int)cx, (int)cy));
+                atomicAdd(hist + cell, 1u);
+            }
+            cur += __popc(M);
+        }
+        done_to = max(done_to, batch_end);
+        j0 += 32;
+    }
+}
+
+// The same for QuadBox-dagger (no QPass): one thread per Gaussian runs nested
+// loops over the cells of each sub-box and skips those an earlier one holds.
+__device__ __forceinline__ void cell_emit_naive(const CellBin &b, int64_t j, uint32_t *hist) {
+    const uint32_t gid = b.perm[j];
+    const uint32_t off = b.coff[j];
+    const uint32_t end = j + 1 < b.n ? b.coff[j + 1] : (uint32_t)*b.n_cells;
+    if (end == off) return;
+    const uint4 w0 = b.rects[2 * (size_t)gid], w1 = b.rects[2 * (size_t)gid + 1];
+    const Rect r[4] = {cell_rect(unpack_rect(w0.x, w0.y)), cell_rect(unpack_rect(w0.z, w0.w)),
+                       cell_rect(unpack_rect(w1.x, w1.y)), cell_rect(unpack_rect(w1.z, w1.w))};
+    uint32_t at = off;
+    for (int q = 0; q < 4; ++q) {
+        if (rect_empty(r[q])) continue;
+        for (int cy = r[q].y0; cy <= r[q].y1; ++cy)
+            for (int cx = r[q].x0; cx <= r[q].x1; ++cx) {
+                bool seen = false;
+                for (int p = 0; p < q; ++p) seen |= in_rect(r[p], cx, cy);
+                if (seen || at >= end) continue;
+                const uint32_t cell = (uint32_t)(cy * b.geo.cells_x + cx);
+                b.arr.keys_a[at] = cell;
+                b.arr.vals_a[at] = cell_value(gid, tiles_in_cell(w0, w1, cx, cy));
+                atomicAdd(hist + cell, 1u);
+                ++at;
+            }
+    }
+}
+
+// From the cells' entry counts, run by one block: the first entry and first
+// row of each cell, and every sort pass's exclusive bucket offsets.  A digit
+// d of pass p (width b, shift h) covers the runs of 2^h consecutive cells
+// that start at u 2^(b+h) + d 2^h; each run's sum is a difference of two
+// offsets.  s_dsum has room for 2^kMaxDigitBits digit sums.
+__device__ __forceinline__ void cell_prepare(const CellBin &b, uint32_t *s_dsum) {
+    constexpr int U = 4;
+    const int ncells = b.geo.ncells;
+    uint32_t entries = 0, rows = 0;  // before this step's cells
+    for (int c0 = 0; c0 < ncells; c0 += U * (int)blockDim.x) {
+        uint32_t v[U], sum = 0, rsum = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int c = c0 + (int)threadIdx.x * U + u;
+            v[u] = c < ncells ? __ldcg(b.arr.count + c) : 0u;
+            sum += v[u];
+            rsum += (v[u] + kCellRow - 1) / kCellRow;
+        }
+        uint32_t total, rtotal;
+        uint32_t e = entries + block_incl_scan<uint32_t>(sum, &total) - sum;
+        uint32_t r = rows + block_incl_scan<uint32_t>(rsum, &rtotal) - rsum;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int c = c0 + (int)threadIdx.x * U + u;
+            if (c < ncells) {
+                b.arr.start[c] = e;
+                b.arr.row_start[c] = r;
+            }
+            e += v[u];
+            r += (v[u] + kCellRow - 1) / kCellRow;
+        }
+        entries += total;
+        rows += rtotal;
+    }
+    if (threadIdx.x == 0) {
+        b.arr.start[ncells] = entries;
+        b.arr.row_start[ncells] = rows;
+    }
+    __threadfence_block();
+    __syncthreads();
+    uint32_t *table = sort_hist_at(b.sort_scratch);
+    const volatile uint32_t *start = b.arr.start;
+    for (int p = 0; p < b.geo.passes.passes; ++p) {
+        const int bits = b.geo.passes.bits[p], sh = b.geo.passes.shift[p];
+        const int Rp = 1 << bits, period = Rp << sh;
+        const int runs = Rp * ((ncells + period - 1) / period);
+        for (int d = threadIdx.x; d < Rp; d += blockDim.x) s_dsum[d] = 0u;
+        __syncthreads();
+        for (int i = threadIdx.x; i < runs; i += blockDim.x) {
+            const int d = i & (Rp - 1), u = i >> bits;
+            const int c = u * period + (d << sh);
+            if (c >= ncells) continue;
+            const uint32_t v = start[min(ncells, c + (1 << sh))] - start[c];
+            if (v) atomicAdd(&s_dsum[d], v);
+        }
+        __syncthreads();
+        const int per = (Rp + (int)blockDim.x - 1) / (int)blockDim.x;
+        const int d0 = (int)threadIdx.x * per, d1 = min(Rp, d0 + per);
+        uint32_t sum = 0;
+        for (int d = d0; d < d1; ++d) sum += s_dsum[d];
+        uint32_t tot;
+        uint32_t r = block_incl_scan<uint32_t>(sum, &tot) - sum;
+        for (int d = d0; d < d1; ++d) {
+            table[p * kHistStride + d] = r;
+            r += s_dsum[d];
+        }
+        __syncthreads();
+    }
+}
+
+// The emit, balanced over the entries (warp w takes the ranges [w C, (w+1) C),
+// w + warps, ...), with a histogram of the cells (in shared memory up to
+// kCellHistMax cells) whose last block makes the cells' offsets.  It also
+// zeroes the look-back words and counters of the sort's passes, sized by the
+// entries there are and not by the capacity.
+template <bool NAIVE>
+__global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    CellTable *s_tab = reinterpret_cast<CellTable *>(smem);
+    uint32_t *s_hist = reinterpret_cast<uint32_t *>(smem + (NAIVE ? 0 : kCellWarps * sizeof(CellTable)));
+    __shared__ bool s_last;
+    const int tid = threadIdx.x, wid = tid >> 5;
+    const bool in_smem = b.geo.ncells <= kCellHistMax;
+    const uint64_t E = *b.n_cells;
+    if (blockIdx.x == 0 && tid == 0) {
+        const uint64_t P = *b.n_pairs;
+        if (P > b.capacity || (P > 0 && E == 0)) atomicOr(b.err, kErrCapacity);
+    }
+    if (in_smem)
+        for (int c = tid; c < b.geo.ncells; c += blockDim.x) s_hist[c] = 0u;
+    const uint64_t threads = (uint64_t)gridDim.x * blockDim.x, gt = (uint64_t)blockIdx.x * blockDim.x + tid;
+    for (int p = 0; p < b.geo.passes.passes; ++p) {
+        uint32_t *lb = sort_lookback_at(b.sort_scratch, b.capacity, b.geo.digit_bits, p);
+        // (a pass of fewer than 4 bits still runs with 16 digits)
+        const uint64_t words = ((E + kSortTile - 1) / kSortTile) << max(b.geo.passes.bits[p], 4);
+        for (uint64_t i = gt; i < words; i += threads) lb[i] = 0u;
+        if (gt == 0) *sort_counter_at(b.sort_scratch, p) = 0u;
+    }
+    __syncthreads();
+    uint32_t *hist = in_smem ? s_hist : b.arr.count;
+    if constexpr (NAIVE) {
+        if (E > 0)
+            for (uint64_t j = gt; j < (uint64_t)b.n; j += threads) cell_emit_naive(b, (int64_t)j, hist);
+    } else {
+        const uint64_t step = (uint64_t)gridDim.x * kCellWarps * kCellChunk;
+        for (uint64_t C = ((uint64_t)blockIdx.x * kCellWarps + wid) * kCellChunk; C < E; C += step)
+            cell_emit_range(b, E, C, (int32_t)min((uint64_t)kCellChunk, E - C), s_tab[wid], hist);
+    }
+    if (in_smem) {
+        __syncthreads();
+        for (int c = tid; c < b.geo.ncells; c += blockDim.x) {
+            const uint32_t v = s_hist[c];
+            if (v) atomicAdd(b.arr.count + c, v);
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(b.arr.count + b.geo.ncells, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    cell_prepare(b, reinterpret_cast<uint32_t *>(smem));  // the table and histogram are no longer needed
+}
+
+cudaError_t launch_cell_emit(const CellBin &b, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(b.arr.count, 0, 4 * cell_zero_words(b.geo.ncells), s);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const size_t hist = b.geo.ncells <= kCellHistMax ? 4 * (size_t)b.geo.ncells : 0;
+    const size_t dsum = (size_t)4 << kMaxDigitBits;
+    if (b.naive) {
+        const size_t smem = std::max(hist, dsum);
+        const uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>(((uint64_t)b.n + 255) / 256, (uint64_t)sms * 8));
+        note_launch("cell_emit_naive_kernel", s),
+            cell_emit_kernel<true><<<(unsigned)blocks, kCellWarps * 32, smem, s>>>(b);
+        return cudaGetLastError();
+    }
+    const size_t smem = std::max(kCellWarps * sizeof(CellTable) + hist, dsum);
+    e = ensure_dyn_smem((const void *)cell_emit_kernel<false>, kCellWarps * sizeof(CellTable) + 4 * (size_t)kCellHistMax);
+    if (e != cudaSuccess) return e;
+    const uint64_t want = (b.n_cells_max + kCellWarps * kCellChunk - 1) / (kCellWarps * kCellChunk);
+    const uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * 4));
+    note_launch("cell_emit_kernel", s), cell_emit_kernel<false><<<(unsigned)blocks, kCellWarps * 32, smem, s>>>(b);
+    return cudaGetLastError();
+}
+
+// Bit i of lane t's result is bit t of lane i's x (a 32 x 32 bit transpose).
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        // columns whose index has bit j clear
+        const uint32_t m = j == 16 ? 0x0000ffffu : j == 8 ? 0x00ff00ffu : j == 4 ? 0x0f0f0f0fu
+                                                          : j == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+        x = (lane & j) ? (x & ~m) | ((y >> j) & m) : (x & m) | ((y & m) << j);
+    }
+    return x;
+}
+
+// The cell that owns row r, found by one warp (32-ary search of row_start).
+__device__ __forceinline__ int cell_of_row(const uint32_t *row_start, int ncells, uint32_t r, int lane) {
+    int lo = 0, hi = ncells - 1;  // row_start[lo] <= r, answer in [lo, hi]: the last cell with row_start <= r
+    while (hi > lo) {
+        const int span = hi - lo;
+        const int probe = lo + (int)(((int64_t)span * (lane + 1) + 31) / 32);  // 32 probes in (lo, hi]
+        const uint32_t m = __ballot_sync(0xffffffffu, row_start[probe] <= r);
+        const int k = m ? 31 - __clz(m) : -1;  // highest probe at or below r
+        const int new_lo = k >= 0 ? lo + (int)(((int64_t)span * (k + 1) + 31) / 32) : lo;
+        const int new_hi = k < 31 ? lo + (int)(((int64_t)span * (k + 2) + 31) / 32) - 1 : hi;
+        lo = new_lo;
+        hi = max(new_lo, new_hi);
+    }
+    return lo;
+}
+
+// The tile of bit `lane` of a cell, or -1 beyond the image.
+__device__ __forceinline__ int tile_of_lane(const CellGeo &g, int cell, int lane) {
+    const int cy = cell / g.cells_x, cx = cell - cy * g.cells_x;
+    const int tx = (cx << kCellXShift) + (lane & (kCellX - 1)), ty = (cy << kCellYShift) + (lane >> kCellXShift);
+    return tx < g.tiles_x && ty < g.tiles_y ? ty * g.tiles_x + tx : -1;
+}
+
+constexpr int kRowWarps = 8;  // warps per block of the row kernels
+
+__global__ void __launch_bounds__(kRowWarps * 32) cell_count_kernel(CellGeo g, CellArrays a,
+                                                                    const uint64_t *__restrict__ vals) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t rows = a.row_start[g.ncells];
+    for (uint32_t r = blockIdx.x * kRowWarps + (threadIdx.x >> 5); r < rows; r += gridDim.x * kRowWarps) {
+        const int cell = cell_of_row(a.row_start, g.ncells, r, lane);
+        const uint32_t first = a.start[cell] + (r - a.row_start[cell]) * kCellRow;
+        const uint32_t end = min(first + kCellRow, a.start[cell + 1]);
+        uint32_t bits[kCellRow / 32];
+#pragma unroll
+        for (int k = 0; k < (int)kCellRow / 32; ++k) {
+            const uint32_t i = first + 32 * k + lane;
+            bits[k] = i < end ? (uint32_t)(vals[i] >> 32) : 0u;
+        }
+        uint32_t c = 0;
+#pragma unroll
+        for (int k = 0; k < (int)kCellRow / 32; ++k) c += __popc(warp_transpose(bits[k], lane));
+        a.row_counts[(size_t)r * 32 + lane] = tile_of_lane(g, cell, lane) >= 0 ? c : 0u;
+        if (lane == 0) a.row_cell[r] = (uint32_t)cell;
+    }
+}
+
+// Block c turns cell c's rows into their exclusive prefix (a warp takes a
+// contiguous part of the rows) and writes the totals of its tiles; the last
+// block scans the totals into the ranges ([0, 0) for an empty tile).
+__global__ void __launch_bounds__(1024) cell_prefix_kernel(CellGeo g, CellArrays a, uint2 *__restrict__ ranges,
+                                                           const uint64_t *n_pairs, const uint64_t *n_cells) {
+    __shared__ uint32_t s_part[32][32];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int cell = blockIdx.x;
+    const uint32_t r0 = a.row_start[cell], nr = a.row_start[cell + 1] - r0;
+    const uint32_t per = (nr + nw - 1) / nw;
+    const uint32_t w0 = min(nr, wid * per), w1 = min(nr, w0 + per);
+    uint32_t *rows = a.row_counts + (size_t)r0 * 32 + lane;
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (uint32_t r = w0; r < w1; ++r) sum += __ldcg(rows + (size_t)r * 32);
+    s_part[wid][lane] = sum;
+    __syncthreads();
+    uint32_t run = 0, total = 0;
+    for (int w = 0; w < nw; ++w) {
+        const uint32_t v = s_part[w][lane];
+        run += w < wid ? v : 0u;
+        total += v;
+    }
+    for (uint32_t r = w0; r < w1; r += 8) {
+        uint32_t v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = r + k < w1 ? __ldcg(rows + (size_t)(r + k) * 32) : 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (r + k < w1) rows[(size_t)(r + k) * 32] = run;
+            run += v[k];
+        }
+    }
+    if (wid == 0) {
+        const int t = tile_of_lane(g, cell, lane);
+        if (t >= 0) a.tile_total[t] = total;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(a.count + g.ncells + 1, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // exclusive scan over the tiles, eight consecutive ones per thread
+    uint64_t before = 0;
+    for (int t0 = 0; t0 < g.ntiles; t0 += 8 * (int)blockDim.x) {
+        const int t = t0 + 8 * (int)threadIdx.x;
+        uint32_t v[8], s = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = t + k < g.ntiles ? __ldcg(a.tile_total + t + k) : 0u;
+            s += v[k];
+        }
+        uint32_t tot;
+        uint32_t e = (uint32_t)before + block_incl_scan<uint32_t>(s, &tot) - s;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (t + k < g.ntiles) ranges[t + k] = v[k] ? make_uint2(e, e + v[k]) : make_uint2(0u, 0u);
+            e += v[k];
+        }
+        before += tot;
+    }
+    // After a look-back time-out the sorted entries are undefined: unless the
+    // tiles' totals add up to the pairs there are, nothing is expanded.
+    if (*n_cells > 0 && before != *n_pairs) {
+        for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) ranges[t] = make_uint2(0u, 0u);
+        if (threadIdx.x == 0) a.row_start[g.ncells] = 0u;
+    }
+}
+
+__global__ void __launch_bounds__(kRowWarps * 32) cell_expand_kernel(CellGeo g, CellArrays a,
+                                                                     const uint64_t *__restrict__ in,
+                                                                     const uint2 *__restrict__ ranges,
+                                                                     uint32_t *__restrict__ vals) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = lanemask_lt();
+    const uint32_t rows = a.row_start[g.ncells];
+    for (uint32_t r = blockIdx.x * kRowWarps + (threadIdx.x >> 5); r < rows; r += gridDim.x * kRowWarps) {
+        const int cell = (int)a.row_cell[r];
+        const uint32_t first = a.start[cell] + (r - a.row_start[cell]) * kCellRow;
+        const uint32_t end = min(first + kCellRow, a.start[cell + 1]);
+        uint64_t e[kCellRow / 32];
+#pragma unroll
+        for (int k = 0; k < (int)kCellRow / 32; ++k) {
+            const uint32_t i = first + 32 * k + lane;
+            e[k] = i < end ? in[i] : 0ull;
+        }
+        const int t = tile_of_lane(g, cell, lane);
+        const uint32_t have = __ballot_sync(0xffffffffu, t >= 0);
+        uint32_t base = t >= 0 ? ranges[t].x + a.row_counts[(size_t)r * 32 + lane] : 0u;
+#pragma unroll
+        for (int k = 0; k < (int)kCellRow / 32; ++k) {
+            if (first + 32 * k >= end) break;  // warp-uniform
+            const uint32_t gid = (uint32_t)e[k], bits = (uint32_t)(e[k] >> 32) & have;
+#pragma unroll
+            for (int q = 0; q < 32; ++q) {
+                const bool on = (bits >> q) & 1u;
+                const uint32_t m = __ballot_sync(0xffffffffu, on);
+                const uint32_t at = __shfl_sync(0xffffffffu, base, q) + __popc(m & lt);
+                if (on) vals[at] = gid;
+            }
+            base += __popc(warp_transpose(bits, lane));
+        }
+    }
+}
+
+cudaError_t launch_cell_sort(const CellBin &b, cudaStream_t s) {
+    bool in_b = false;
+    cudaError_t e = cell_sort_passes(b, s, &in_b);
+    if (e != cudaSuccess) return e;
+    const uint64_t *sorted = in_b ? b.arr.vals_b : b.arr.vals_a;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint64_t rows = cell_rows_max(b.n_cells_max, b.geo.ncells);
+    const uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>((rows + kRowWarps - 1) / kRowWarps, (uint64_t)sms * 8));
+    note_launch("cell_count_kernel", s),
+        cell_count_kernel<<<(unsigned)blocks, kRowWarps * 32, 0, s>>>(b.geo, b.arr, sorted);
+    // enough warps for the rows of a crowded cell, fewer where there are many cells
+    const unsigned threads = b.geo.ncells <= 2048 ? 1024 : 256;
+    note_launch("cell_prefix_kernel", s),
+        cell_prefix_kernel<<<b.geo.ncells, threads, 0, s>>>(b.geo, b.arr, b.ranges, b.n_pairs, b.n_cells);
+    note_launch("cell_expand_kernel", s),
+        cell_expand_kernel<<<(unsigned)blocks, kRowWarps * 32, 0, s>>>(b.geo, b.arr, sorted, b.ranges, b.vals);
+    return cudaGetLastError();
+}
+
+}  // namespace qb

@@ -38,16 +38,18 @@ struct CamDev {
 
 // Workspace offsets (bytes) of a frame; all 256-byte aligned.
 struct Layout {
-    size_t xy, shape, conic_o, rgbd, box, r3, meta, counts, offsets, segs;
-    size_t counts_e, chunk_first;  // counts in emission order; the emit's chunk table
+    size_t xy, shape, conic_o, rgbd, box, r3, meta, counts, offsets;
+    size_t rects;  // [n] packed sub-box tile rectangles (pack_rects)
+    size_t cc;     // [n] (tile count, cell count)
+    size_t coff;   // [n] counts (FULL_KEY) or cell offsets (DEPTH_FIRST) in emission order
+    size_t chunk_first;  // the emit's chunk table
     size_t scan_part;
     size_t keys0, keys1, vals0, vals1;
     size_t sort_scratch, sort_scratch_bytes;
     size_t dkeys0, dkeys1, dvals0, dvals1, dsort_scratch;  // depth order of the Gaussians
     size_t ranges, tfinal, ncontrib, neval;
-    size_t tile_counts;  // per-tile pair counts of the tile histogram (+ its block counter)
-    size_t tile_diff;  // (tiles_y+1) x (tiles_x+1) int difference array
-    size_t tile_single;  // tiles ints: pair counts of single-tile Gaussians
+    size_t cell_zero;    // cell counts and finished-block counters (CellLayout)
+    size_t cell_start, row_start, row_cell, row_counts, tile_total;  // CellArrays
     size_t order_cnt;   // [2][kOrderBuckets]: the render's and the backward's tile orders (TileOrder)
     size_t order_list;  // [2][kOrderBuckets][tiles]
     size_t gscreen;  // [n][9] screen-space gradients
@@ -96,33 +98,10 @@ size_t sort_scratch_bytes(uint64_t n, int end_bit, int digit_bits);
 cudaError_t sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt,
                        uint64_t n_max, const uint64_t *n_dev, int end_bit, int digit_bits,
                        void *scratch, uint32_t *err_flags, cudaStream_t stream, int *passes_out);
-// The same sort on 32-bit keys (end_bit <= 32).  With hist_ready the
-// exclusive bucket offsets of every pass are already in the scratch's
-// histogram table (sort_hist_table, stride sort_hist_stride per pass).
+// The same sort on 32-bit keys (end_bit <= 32).
 cudaError_t sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
                        uint64_t n_max, const uint64_t *n_dev, int end_bit, int digit_bits,
-                       void *scratch, uint32_t *err_flags, cudaStream_t stream, int *passes_out,
-                       bool hist_ready = false);
-uint32_t *sort_hist_table(void *scratch);
-int sort_hist_stride();
-// Pieces of the depth-first tile sort.  The look-back words of pass p are laid
-// out for n_cap pairs; sort_clear zeroes the tile counters and look-back words
-// of passes [first_pass, end_pass).
-uint32_t *sort_lookback(void *scratch, uint64_t n_cap, int digit_bits, int pass);
-uint32_t *sort_counter(void *scratch, int pass);
-cudaError_t sort_clear(void *scratch, uint64_t n_cap, int digit_bits, int first_pass, int end_pass,
-                       cudaStream_t s);
-// Passes [first_pass, passes) of the tile sort on bits [0, end_bit) (pass
-// widths from pass_geo): pass p writes buffer A when passes - 1 - p is even,
-// else B, reading the other; the last pass writes values only (into A).
-// Values are below val_bound; a two-pass sort from pass 0 whose values fit
-// beside the second digit in one word carries packed words between its
-// passes and leaves vB unused.
-cudaError_t tile_sort_passes(uint32_t *kA, uint32_t *vA, uint32_t *kB, uint32_t *vB, uint64_t n_cap, uint64_t n_max,
-                             const uint64_t *n_dev, int end_bit, int first_pass, int digit_bits, void *scratch,
-                             uint32_t *err, cudaStream_t s, uint64_t val_bound);
-inline bool pass_writes_a(int passes, int p) { return ((passes - 1 - p) & 1) == 0; }
-
+                       void *scratch, uint32_t *err_flags, cudaStream_t stream, int *passes_out);
 // ---- device helpers -----------------------------------------------------------
 // Gaussians whose stretching factor f (Eq. f-closed) has f^2 below this take
 // the render's exact power form: with r = b / a = -Sigma12 / Sigma22 and
@@ -334,16 +313,68 @@ __device__ __forceinline__ int qpass_segments(const QPass &qp, QSeg seg[7]) {
 
 __device__ __forceinline__ bool seg_empty(const QSeg &g) { return g.nl <= 0 || g.len <= 0; }
 
-__device__ __forceinline__ uint32_t qpass_count(const Rect rects[4]) {
-    QPass qp;
-    if (!qpass_setup(rects, qp)) return 0;
-    uint32_t c = 0;
-    for (int s = qp.s0; s <= qp.s1; ++s) {
-        int lo, hi;
-        qpass_line(qp, s, lo, hi);
-        c += (hi >= lo) ? (uint32_t)(hi - lo + 1) : 0u;
+__device__ __forceinline__ Rect both(const Rect &a, const Rect &b) {
+    return Rect{max(a.x0, b.x0), max(a.y0, b.y0), min(a.x1, b.x1), min(a.y1, b.y1)};
+}
+
+__device__ __forceinline__ int rect_area(const Rect &r) { return max(r.x1 - r.x0 + 1, 0) * max(r.y1 - r.y0 + 1, 0); }
+
+// Tiles (or cells) in the union of the sub-box rectangles, by inclusion and
+// exclusion: what a QPass traversal counts (its merged line intervals hold no
+// tile outside the union, because the sub-boxes share the corner mu^2D), in
+// about 130 branch-free integer operations where the run decomposition
+// (qpass_segments) takes several hundred.
+__device__ __forceinline__ uint32_t union_count(const Rect r[4]) {
+    const Rect r01 = both(r[0], r[1]), r02 = both(r[0], r[2]), r03 = both(r[0], r[3]);
+    const Rect r12 = both(r[1], r[2]), r13 = both(r[1], r[3]), r23 = both(r[2], r[3]);
+    const int one = rect_area(r[0]) + rect_area(r[1]) + rect_area(r[2]) + rect_area(r[3]);
+    const int two = rect_area(r01) + rect_area(r02) + rect_area(r03) + rect_area(r12) + rect_area(r13) + rect_area(r23);
+    const int three = rect_area(both(r01, r[2])) + rect_area(both(r01, r[3])) + rect_area(both(r23, r[0])) +
+                      rect_area(both(r23, r[1]));
+    return (uint32_t)(one - two + three - rect_area(both(r01, r23)));
+}
+
+// The depth-first path bins Gaussians into cells of kCellX x kCellY tiles
+// first (qb_cells.cu): the cells a Gaussian's tiles lie in, and per cell one
+// bit per tile.
+constexpr int kCellXShift = 3, kCellYShift = 2;
+constexpr int kCellX = 1 << kCellXShift, kCellY = 1 << kCellYShift;
+static_assert(kCellX * kCellY == 32, "a cell's tiles are the bits of one word");
+
+// The cells a tile rectangle touches.  An empty rectangle stays empty:
+// intersections are stored as empty_rect() (1, 1, 0, 0), whose corners would
+// meet after the shift, so it is kept apart.
+__device__ __forceinline__ Rect cell_rect(const Rect &r) {
+    if (rect_empty(r)) return empty_rect();
+    return Rect{r.x0 >> kCellXShift, r.y0 >> kCellYShift, r.x1 >> kCellXShift, r.y1 >> kCellYShift};
+}
+
+// The tiles of rectangle r inside cell (cx, cy), bit (ty % kCellY) kCellX +
+// tx % kCellX.
+__device__ __forceinline__ uint32_t cell_bits_of(const Rect &r, int cx, int cy) {
+    const int x0 = max(r.x0 - (cx << kCellXShift), 0), x1 = min(r.x1 - (cx << kCellXShift), kCellX - 1);
+    const int y0 = max(r.y0 - (cy << kCellYShift), 0), y1 = min(r.y1 - (cy << kCellYShift), kCellY - 1);
+    if (x0 > x1 || y0 > y1) return 0u;
+    const uint32_t row = ((2u << (x1 - x0)) - 1u) << x0;                    // the columns of one row
+    const uint32_t rows = (0x01010101u >> (kCellX * (kCellY - 1 - (y1 - y0)))) << (kCellX * y0);
+    return row * rows;
+}
+
+// A Gaussian's four sub-box rectangles in two uint4 (tile coordinates below
+// 2^16), rectangle q in words 2q (x0 | y0 << 16) and 2q + 1 (x1 | y1 << 16).
+__device__ __forceinline__ void pack_rects(const Rect r[4], uint4 out[2]) {
+    uint32_t w[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        w[2 * q] = (uint32_t)r[q].x0 | ((uint32_t)r[q].y0 << 16);
+        w[2 * q + 1] = (uint32_t)r[q].x1 | ((uint32_t)r[q].y1 << 16);
     }
-    return c;
+    out[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    out[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
+__device__ __forceinline__ Rect unpack_rect(uint32_t lo, uint32_t hi) {
+    return Rect{(int)(lo & 0xffffu), (int)(lo >> 16), (int)(hi & 0xffffu), (int)(hi >> 16)};
 }
 
 // Naive traversal (QuadBox-dagger, Table 3): nested loops over each

@@ -28,19 +28,10 @@ struct PreArgs {
     float *r3;
     int *meta;
     uint32_t *counts;
-    int *tile_diff;    // per camera [(tiles_y+1)][(tiles_x+1)] difference array of pair counts, or null
-    int *tile_single;  // per camera [tiles] pair counts of single-tile Gaussians
-    uint32_t diff_off[kMaxGroupCams], single_off[kMaxGroupCams];
-    uint4 *segs;       // [records][4] QPass segment records (pack_segments), or null
+    uint2 *cc;         // [records] (tiles, cells)
+    uint4 *rects;      // [records][2] packed sub-box rectangles (pack_rects), written where there are tiles
     uint32_t *depth_keys, *depth_vals;  // [records] depth-sort keys and record indices, or null
 };
-
-// A Gaussian's QPass traversal as at most seven segments, packed in 16 words
-// (four uint4): word 0 = segment count | column flag << 3 | first tile row
-// << 4 | last tile row << 18; segment k in words 1 + 2k (first line | first
-// cell << 16) and 2 + 2k (lines | cells << 16).
-// Only the first ceil((1 + 2 ns) / 4) uint4 are written and read.
-__device__ __forceinline__ int seg_chunks(int ns) { return (1 + 2 * ns + 3) >> 2; }
 
 // Image geometry of one camera in a set of cameras rendered together.  Tile
 // ids are global over the set (camera c owns [tile_base, tile_base + tiles));
@@ -81,32 +72,63 @@ __device__ __forceinline__ int camera_of(const TileSet &ts, uint32_t gtile) {
     return c;
 }
 
-struct TileOffsets {
-    uint32_t diff[kMaxGroupCams], single[kMaxGroupCams];
-};
-
+// The full-key emit (a single frame, index order).
 struct EmitArgs {
-    int n;                 // records (cameras x Gaussians)
-    int n_per_cam;         // Gaussians per camera
-    const uint32_t *perm;  // emission order -> record (null: index order)
-    const float2 *xy;
-    const float4 *box;
-    const float *r3;
-    const int *meta;
+    int n;
     const float4 *rgbd;
-    const uint32_t *counts;   // by Gaussian
-    const uint32_t *offsets;  // by emission position
-    const uint32_t *counts_e;     // the counts by emission position, or null (read through perm)
-    const uint32_t *chunk_first;  // emission position holding output position c kEmitStride, or null
-    const uint4 *segs;        // QPass segment records from the preprocess, or null (recomputed)
+    const uint32_t *counts, *offsets;
+    const uint32_t *chunk_first;  // Gaussian holding output position c kEmitStride
+    const uint4 *rects;
     uint32_t *vals;
     const uint64_t *n_pairs;
     uint64_t n_pairs_host;  // P when the host knows it, else UINT64_MAX
     uint64_t capacity;
     int mode;
-    bool clamp3s;
     uint32_t *err;
-    TileSet ts;  // camera of record r is r / n_per_cam
+    uint32_t tiles_x;
+};
+
+// Geometry of the cells of one image, and the widths of the passes that sort
+// their ids.
+struct CellGeo {
+    int tiles_x, tiles_y, cells_x, cells_y, ncells, ntiles;
+    int cell_bits, digit_bits;  // digit_bits: of a pass at most (sort scratch layout)
+    PassGeo passes;
+};
+
+// Device arrays of the cell binning (qb_cells.cu).
+struct CellArrays {
+    uint32_t *count;       // [ncells] entries per cell, then the two finished-block counters
+    uint32_t *start;       // [ncells + 1] first sorted entry of each cell
+    uint32_t *row_start;   // [ncells + 1] first row of each cell
+    uint32_t *row_cell;    // [rows]
+    uint32_t *row_counts;  // [rows][32] entries per tile; after the prefix, those of the cell's earlier rows
+    uint32_t *tile_total;  // [ntiles rounded up to 8]
+    // entries (cell id; Gaussian | tile bits << 32), two buffers; keys_b is read
+    // and written by sorts of two passes or more only
+    uint32_t *keys_a, *keys_b;
+    uint64_t *vals_a, *vals_b;
+};
+constexpr uint32_t kCellRow = 128;  // sorted entries per row
+inline size_t cell_zero_words(int ncells) { return (size_t)ncells + 2; }
+inline size_t cell_rows_max(uint64_t pair_capacity, int ncells) { return (size_t)(pair_capacity / kCellRow) + ncells; }
+
+struct CellBin {
+    int n;
+    const uint32_t *perm;   // record of each emission position
+    const uint32_t *coff;   // cell offset of each emission position
+    const uint32_t *chunk_first;
+    const uint4 *rects;     // by record
+    const uint64_t *n_pairs, *n_cells;
+    uint64_t n_cells_max;   // bound on *n_cells (the capacity, or P where the host knows it)
+    uint64_t capacity;
+    bool naive;             // emit by nested loops (QB_BIN_QUADBOX_NAIVE)
+    uint32_t *err;
+    void *sort_scratch;
+    CellGeo geo;
+    CellArrays arr;
+    uint2 *ranges;          // [ntiles]
+    uint32_t *vals;         // [P] sorted values
 };
 
 // Tiles filed by work into kOrderBuckets buckets, heaviest first: bucket
@@ -210,40 +232,35 @@ struct PreBwdArgs {
 
 cudaError_t launch_preprocess(const PreArgs &a, int deg, cudaStream_t s);
 // partials: scan_partials_count(n) words of scratch (block status words and
-// the block counter), cleared by the launch; a look-back that waits too long
-// raises kErrTimeout in *err.
-cudaError_t launch_scan(const uint32_t *counts, const uint32_t *perm, int n, uint32_t *offsets, uint64_t *partials,
-                        uint64_t *n_pairs, uint32_t *err, cudaStream_t s, uint32_t *counts_e = nullptr,
-                        uint32_t *chunk_first = nullptr, uint32_t chunk_cap = 0);
+// the block counter), 16-byte aligned, cleared by the launch; a look-back that
+// waits too long raises kErrTimeout in *err.  launch_scan: the counts in index
+// order (full-key path).  launch_scan_cells: (tiles, cells) in the order perm;
+// *n_cells becomes 0 when the pairs exceed the capacity.
+cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32_t *counts_e, uint64_t *partials,
+                        uint64_t *n_pairs, uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s);
+cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint32_t *offsets, uint32_t *coff,
+                              uint64_t *partials, uint64_t *n_pairs, uint64_t *n_cells, uint64_t capacity,
+                              uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s);
 // Output positions per entry of the scan's chunk table (a divisor of every
 // emit kernel's per-warp output range).
 constexpr uint32_t kEmitStride = 256;
 inline uint64_t chunk_table_size(uint64_t pair_capacity) { return pair_capacity / kEmitStride + 1; }
 size_t scan_partials_count(int n);
-template <typename KeyT>
-cudaError_t launch_emit(const EmitArgs &a, KeyT *keys, cudaStream_t s);
-// K3 fused with the first pass of the depth-first tile sort (digit bits
-// [0, digit_bits) of the tile id); write_keys false when it is the only pass.
-cudaError_t launch_emit_sweep(const EmitArgs &a, int digit_bits, bool write_keys, uint32_t *kout, uint32_t *vout,
-                              const uint32_t *bin_off, uint32_t *lookback, uint32_t *counter, cudaStream_t s);
-// Counts, scans and places the pairs (writes e.vals and the ranges).
+cudaError_t launch_emit(const EmitArgs &a, uint64_t *keys, cudaStream_t s);
 cudaError_t launch_expand_ranges(const uint2 *ranges, int ntiles, uint32_t *out, uint64_t n_out, cudaStream_t s);
-template <typename KeyT>
-cudaError_t launch_ranges(const KeyT *keys, uint64_t n_max, const uint64_t *n_dev, uint2 *ranges, int ntiles,
+cudaError_t launch_ranges(const uint64_t *keys, uint64_t n_max, const uint64_t *n_dev, uint2 *ranges, int ntiles,
                           cudaStream_t s);
-// Ranges and every tile-sort pass's bucket offsets from the per-tile counts
-// in the preprocess's difference arrays (the fused-emit frame path).
-cudaError_t launch_tile_prep(int *tile_diff, const int *tile_single, const TileSet &ts,
-                             const uint32_t *diff_off, const uint32_t *single_off, uint2 *ranges, uint32_t *hist,
-                             int hist_stride, int digit_bits, int tile_bits, uint64_t capacity, cudaStream_t s);
-// Per-tile counts of n tile ids into counts[0, ntiles) (counts and the
-// block counter at counts[ntiles] zeroed here); ntiles <= kTileCountMax.
-// With ranges non-null the last block also writes the ranges and every
-// tile-sort pass's exclusive bucket offsets (hist, stride hist_stride).
-constexpr int kTileCountMax = 24576;
-cudaError_t launch_tile_count(const uint32_t *keys, uint64_t n_max, const uint64_t *n_dev, int ntiles,
-                              uint32_t *counts, uint2 *ranges, uint32_t *hist, int hist_stride, int digit_bits,
-                              int tile_bits, cudaStream_t s);
+// The depth-first binning after the depth order and the scan: the emit of
+// (cell, Gaussian, tile bits) entries; then their sort by cell and the
+// expansion to the sorted values and ranges.
+CellGeo cell_geo(int W, int H, int digit_bits);
+size_t cell_sort_scratch_bytes(uint64_t pair_capacity, int ncells, int digit_bits);
+cudaError_t launch_cell_emit(const CellBin &b, cudaStream_t s);
+cudaError_t launch_cell_sort(const CellBin &b, cudaStream_t s);
+// Sorts b's entries by cell (bucket offsets already in the scratch's table,
+// look-back words and counters cleared); values only from the last pass.
+// *in_b: the sorted values lie in vals_b.
+cudaError_t cell_sort_passes(const CellBin &b, cudaStream_t s, bool *in_b);
 cudaError_t launch_render(const RenderArgs &a, int batch, cudaStream_t s);
 // Files every tile of a single frame (a.ts.cam[0]) into a.order by an
 // estimate of the render's work: the entries composited until four sample

@@ -3,8 +3,9 @@
 //
 // One thread per Gaussian.  Reads the raw parameters (44 B + 12 (deg+1)^2 B),
 // writes mu^2D, conic+opacity, colour+depth, the box record, the 3-sigma
-// radius, a meta word and the tile count (68 B).  Culled Gaussians write only
-// their count and meta word and skip the SH read.
+// radius, a meta word, the tile and cell counts, the sub-boxes' tile
+// rectangles and the depth-sort pair.  Culled Gaussians write only their
+// counts and meta word and skip the SH read.
 #include "qb_kernels.cuh"
 #include "qb_project.cuh"
 
@@ -34,6 +35,7 @@ __global__ void __launch_bounds__(256, 3) preprocess_kernel(PreArgs a) {
     }
     if (!ok) {
         a.counts[o] = 0u;
+        a.cc[o] = make_uint2(0u, 0u);
         a.meta[o] = 0;
         a.shape[o] = make_float2(0.f, 0.f);
         if (a.depth_keys) {  // no tiles: sorts after every Gaussian that has some
@@ -89,68 +91,27 @@ __global__ void __launch_bounds__(256, 3) preprocess_kernel(PreArgs a) {
 
     Rect rects[4];
     box_rects(p.mx, p.my, bt.box, bt.r3, bt.orient, a.mode, a.clamp3s, cam.W, cam.H, rects);
-    uint32_t cnt = 0;
-    QPass qp;
-    if (qpass_setup(rects, qp)) {
-        QSeg seg[7];
-        const int ns = qpass_segments(qp, seg);
-        // QPass count: the lines of each run of equal intervals times its length
+    // tiles, and cells of 8 x 4 tiles, of the QPass traversal
+    uint32_t cnt, ccnt;
+    Rect crects[4];
 #pragma unroll
-        for (int q = 0; q < 7; ++q) cnt += (uint32_t)(seg[q].nl * seg[q].len);
-        if (a.segs && cnt > 0u) {
-            // the segments, for the emit (which then skips the box and QPass setup)
-            uint32_t w[16];
-            int ylo = 1 << 14, yhi = -1;  // tile rows the segments cover
-#pragma unroll
-            for (int q = 0; q < 7; ++q) {
-                if (seg_empty(seg[q])) continue;
-                const int a0 = qp.columns ? seg[q].lo : seg[q].s0;
-                const int a1 = a0 + (qp.columns ? seg[q].len : seg[q].nl) - 1;
-                ylo = min(ylo, a0);
-                yhi = max(yhi, a1);
-            }
-            w[0] = (uint32_t)ns | ((uint32_t)qp.columns << 3) | ((uint32_t)ylo << 4) | ((uint32_t)yhi << 18);
-#pragma unroll
-            for (int q = 0; q < 7; ++q) {
-                w[1 + 2 * q] = q < ns ? (uint32_t)seg[q].s0 | ((uint32_t)seg[q].lo << 16) : 0u;
-                w[2 + 2 * q] = q < ns ? (uint32_t)seg[q].nl | ((uint32_t)seg[q].len << 16) : 0u;
-            }
-            w[15] = 0u;
-            uint4 *dst = a.segs + 4 * o;
-            const int nc = seg_chunks(ns);
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (c < nc) dst[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-        }
-        const int tiles_x = (cam.W + kTile - 1) >> kTileShift;
-        if (a.tile_diff && cnt == 1u) {
-            // one tile (the common case): count it directly
-            int t = 0;
-#pragma unroll
-            for (int q = 0; q < 7; ++q)
-                if (!seg_empty(seg[q]))
-                    t = qp.columns ? seg[q].lo * tiles_x + seg[q].s0 : seg[q].s0 * tiles_x + seg[q].lo;
-            atomicAdd(a.tile_single + a.single_off[ci] + t, 1);
-        } else if (a.tile_diff) {
-            // per-tile pair counts as a 2D difference array: +1/-1 at the corners
-            // of every rectangle of the Gaussian's tile set
-            const int stride = tiles_x + 1;
-            int *D = a.tile_diff + a.diff_off[ci];
-#pragma unroll
-            for (int q = 0; q < 7; ++q) {
-                if (seg_empty(seg[q])) continue;
-                const int l0 = seg[q].s0, l1 = seg[q].s0 + seg[q].nl - 1;
-                const int u0 = seg[q].lo, u1 = seg[q].lo + seg[q].len - 1;
-                const int x0 = qp.columns ? l0 : u0, x1 = qp.columns ? l1 : u1;
-                const int y0 = qp.columns ? u0 : l0, y1 = qp.columns ? u1 : l1;
-                atomicAdd(D + y0 * stride + x0, 1);
-                atomicAdd(D + y0 * stride + x1 + 1, -1);
-                atomicAdd(D + (y1 + 1) * stride + x0, -1);
-                atomicAdd(D + (y1 + 1) * stride + x1 + 1, 1);
-            }
-        }
+    for (int q = 0; q < 4; ++q) crects[q] = cell_rect(rects[q]);
+    if (a.mode == QB_BIN_AABB3S || a.mode == QB_BIN_ADR) {  // a single box
+        cnt = (uint32_t)rect_area(rects[0]);
+        ccnt = (uint32_t)rect_area(crects[0]);
+    } else if (a.mode == QB_BIN_QUADBOX_NAIVE) {  // the same sets, counted the naive way
+        cnt = naive_count(rects);
+        ccnt = naive_count(crects);
+    } else {
+        cnt = union_count(rects);
+        ccnt = union_count(crects);
     }
-    if (a.mode == QB_BIN_QUADBOX_NAIVE) cnt = naive_count(rects);  // the same set, counted the naive way
+    if (cnt > 0u) {
+        uint4 pk[2];
+        pack_rects(rects, pk);
+        a.rects[2 * o] = pk[0];
+        a.rects[2 * o + 1] = pk[1];
+    }
 
     a.xy[o] = make_float2(p.mx, p.my);
     // the exact power form's terms (qb_internal.cuh), for elongated Gaussians only
@@ -166,6 +127,7 @@ __global__ void __launch_bounds__(256, 3) preprocess_kernel(PreArgs a) {
     a.r3[o] = bt.r3;
     a.meta[o] = meta;
     a.counts[o] = cnt;
+    a.cc[o] = make_uint2(cnt, ccnt);
     if (a.depth_keys) {
         // the depth-order sort's input: positive float depths order like their
         // bits; Gaussians without tiles sort last

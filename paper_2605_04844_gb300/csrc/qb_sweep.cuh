@@ -1,6 +1,5 @@
 // qb_sweep.cuh -- the body of one digit pass of the onesweep radix sort
-// (SortPairs, Sec. 2), shared by the plain pass kernel (qb_sort.cu) and the
-// QPass emit that performs the tile sort's first pass itself (qb_binning.cu).
+// (SortPairs, Sec. 2) of the pair sort and of the cell sort (qb_sort.cu).
 //
 // A block owns one tile of kSortTile consecutive input positions; its keys arrive
 // in registers, warp-striped (item k of lane l of warp w is position
@@ -35,6 +34,22 @@ constexpr int kHistStride = 1 << kMaxDigitBits;  // per-pass stride of the histo
 // kMaxPasses u32, padded to 256 B][look-back words: passes x tiles x 2^RB u32]
 constexpr size_t kSortCounters = (size_t)kMaxPasses * kHistStride * 4;
 constexpr size_t kSortHeader = kSortCounters + 256;
+
+// Pieces of a sort's scratch (qb_internal.cuh).
+__host__ __device__ inline uint64_t sort_tiles(uint64_t n) { return (n + kSortTile - 1) / kSortTile; }
+
+__host__ __device__ inline uint32_t *sort_hist_at(void *scratch) { return static_cast<uint32_t *>(scratch); }
+
+// Look-back words of pass p: laid out for n_cap pairs and digits of at most
+// digit_bits (a pass with fewer bits uses the start of each tile's row).
+__host__ __device__ inline uint32_t *sort_lookback_at(void *scratch, uint64_t n_cap, int digit_bits, int pass) {
+    return reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(scratch) + kSortHeader) +
+           (size_t)pass * sort_tiles(n_cap) * ((size_t)1 << digit_bits);
+}
+
+__host__ __device__ inline uint32_t *sort_counter_at(void *scratch, int pass) {
+    return reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(scratch) + kSortCounters) + pass;
+}
 
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t *p) {
     uint32_t v;
@@ -99,39 +114,36 @@ __device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t v, uint32_t *to
 }
 
 // Shared memory of one pass: the scatter buffer ((key, value) pairs for 32-bit
-// keys; keys, then values, for 64-bit keys), per-warp digit counters, and
-// per-digit global base, local start and tile count.
-template <int RB, typename KeyT>
-constexpr size_t sweep_smem() {
-    return (size_t)kSortTile * 8 + (size_t)kSortWarps * (1 << RB) * 2 + (size_t)3 * (1 << RB) * 4;
+// keys; keys, then values, for 64-bit keys; values and keys side by side for
+// 64-bit values), per-warp digit counters, and per-digit global base, local
+// start and tile count.
+template <typename ValT>
+constexpr size_t sweep_stage() {
+    return (size_t)kSortTile * (sizeof(ValT) == 8 ? 12 : 8);
 }
 
-// What a pass writes at each output position.
-enum SweepOut : int {
-    kOutPairs = 0,   // the key to kout and the value to vout
-    kOutValues = 1,  // the value only (the last pass, whose keys the per-tile ranges imply)
-    kOutPacked = 2,  // one word to kout: (key >> pack_shift) << vbits | value
-};
+template <int RB, typename ValT = uint32_t>
+constexpr size_t sweep_smem() {
+    return sweep_stage<ValT>() + (size_t)kSortWarps * (1 << RB) * 2 + (size_t)3 * (1 << RB) * 4;
+}
 
 // One pass over the tile `tile` (positions [tbase, tbase + kSortTile) of n) on the
 // digit (key >> shift) & mask, mask < 2^RB.  val(k) gives item k's value; it
 // is asked for only at the scatter, after the ranking (so a caller can load
 // values late and keep fewer registers live).  bin_off: the pass's exclusive
-// bucket offsets; lookback: the pass's status words [tiles][2^RB].  OUT
-// (SweepOut) says what is written; kOutPacked (32-bit keys) needs values
-// below 2^vbits and keys below 2^(pack_shift + 32 - vbits).
-template <int RB, typename KeyT, int OUT, class ValFn>
+// bucket offsets; lookback: the pass's status words [tiles][2^RB].  Without
+// WRITE_KEYS (the last pass of a sort whose keys its ranges imply) only the
+// values are written.  64-bit values go with 32-bit keys.
+template <int RB, typename KeyT, typename ValT, bool WRITE_KEYS, class ValFn>
 __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn &&val,
                                            uint32_t n, uint32_t tbase, uint32_t tile,
                                            const uint32_t *__restrict__ bin_off, uint32_t *lookback, int shift,
                                            uint32_t mask, uint32_t *err, KeyT *__restrict__ kout,
-                                           uint32_t *__restrict__ vout, uint8_t *smem, int pack_shift = 0,
-                                           int vbits = 0) {
-    static_assert(OUT != kOutPacked || sizeof(KeyT) == 4, "packed output is for 32-bit keys");
-    constexpr bool WRITE_KEYS = OUT != kOutValues;
+                                           ValT *__restrict__ vout, uint8_t *smem) {
+    static_assert(sizeof(ValT) == 4 || sizeof(KeyT) == 4, "64-bit values go with 32-bit keys");
     constexpr int R = 1 << RB;
     constexpr int PER = (R + kSortBlock - 1) / kSortBlock;
-    uint16_t *s_whist = reinterpret_cast<uint16_t *>(smem + (size_t)kSortTile * 8);
+    uint16_t *s_whist = reinterpret_cast<uint16_t *>(smem + sweep_stage<ValT>());
     uint32_t *s_gbase = reinterpret_cast<uint32_t *>(s_whist + kSortWarps * R);
     uint32_t *s_lstart = s_gbase + R;
     uint32_t *s_bcount = s_lstart + R;
@@ -279,7 +291,33 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
     __syncthreads();
 
     const uint32_t tcount = min(n - tbase, (uint32_t)kSortTile);
-    if constexpr (sizeof(KeyT) == 4) {
+    if constexpr (sizeof(ValT) == 8) {
+        // ---- values and keys to block order in shared memory, then out ----
+        ValT *s_val = reinterpret_cast<ValT *>(smem);
+        uint32_t *s_key = reinterpret_cast<uint32_t *>(smem + (size_t)kSortTile * 8);
+#pragma unroll
+        for (int k = 0; k < kSortItems; ++k) {
+            if (32 * k + lane < wcount) {
+                const uint32_t d = dig(k);
+                const uint32_t j = s_lstart[d] + s_whist[wid * R + d] + rank[k];
+                s_key[j] = (uint32_t)key[k];
+                s_val[j] = val(k);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kSortItems; ++k) {
+            const uint32_t j = tid + k * kSortBlock;
+            if (j < tcount) {
+                const uint32_t kk = s_key[j];
+                const uint32_t dest = s_gbase[(kk >> shift) & mask] + j;
+                if (dest < n) {  // dest >= n only after a look-back timeout
+                    if (WRITE_KEYS) kout[dest] = (KeyT)kk;
+                    vout[dest] = s_val[j];
+                }
+            }
+        }
+    } else if constexpr (sizeof(KeyT) == 4) {
         // ---- (key, value) pairs to block order in shared memory, then out ----
         uint2 *s_pairs = reinterpret_cast<uint2 *>(smem);
 #pragma unroll
@@ -298,12 +336,8 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
                 const uint32_t d = (kv.x >> shift) & mask;
                 const uint32_t dest = s_gbase[d] + j;
                 if (dest < n) {  // dest >= n only after a look-back timeout
-                    if (OUT == kOutPacked) {
-                        kout[dest] = (KeyT)(((kv.x >> pack_shift) << vbits) | kv.y);
-                    } else {
-                        if (WRITE_KEYS) kout[dest] = (KeyT)kv.x;
-                        vout[dest] = kv.y;
-                    }
+                    if (WRITE_KEYS) kout[dest] = (KeyT)kv.x;
+                    vout[dest] = kv.y;
                 }
             }
         }
