@@ -138,7 +138,8 @@ typedef struct {
     int32_t stage;          /* 0 init, 1 preprocessed, 2 emitted, 3 sorted */
     uint64_t n_pairs;       /* host copy of P when known, else UINT64_MAX  */
     int32_t sort_digit_bits;  /* 8..11, radix digit width of qb_sort        */
-    int32_t render_batch;     /* Gaussians staged per shared-memory batch   */
+    int32_t render_batch;     /* accepted, without effect (a warp stages 32
+                                 entries at a time)                          */
     int32_t sorted_in_alt;    /* internal: sorted pairs live in buffer 1    */
     int32_t sort_mode;        /* qb_sort_mode; set before qb_preprocess     */
     int32_t depth_in_alt;     /* internal: depth order lives in buffer 1    */
@@ -340,8 +341,8 @@ qb_status qb_sort_pairs(uint64_t *d_keys, uint32_t *d_vals, uint64_t *d_keys_alt
 /* Launch parameters of the batched path (picked by the autotuner).
  *  tiles_per_fetch  tiles a persistent render block takes from the global
  *                   tile-work queue at a time (1..8)
- *  render_batch     Gaussians staged per shared-memory batch (64, 128, 256)
- *  sort_digit_bits  radix digit width of each camera's tile sort (8..11)
+ *  render_batch     accepted, without effect
+ *  sort_digit_bits  largest radix digit width of each camera's cell sort (8..11)
  *  blocks_per_sm    persistent render blocks per SM (0: as many as fit) */
 typedef struct {
     int32_t tiles_per_fetch;

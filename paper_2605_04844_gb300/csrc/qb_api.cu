@@ -523,7 +523,7 @@ static qb_status render_fwd_impl(qb_frame *frame, const float *bg, float *d_img,
     a.order_out = TileOrder{cnt + kOrderBuckets, list + (size_t)kOrderBuckets * ntiles};
     QB_CUDA(cudaMemsetAsync(cnt, 0, 4 * 2 * (size_t)kOrderBuckets, (cudaStream_t)stream));
     QB_CUDA(launch_tile_work(a, (cudaStream_t)stream));
-    QB_CUDA(launch_render(a, frame->render_batch, (cudaStream_t)stream));
+    QB_CUDA(launch_render(a, (cudaStream_t)stream));
     frame->stage = 4;
     return QB_OK;
 }

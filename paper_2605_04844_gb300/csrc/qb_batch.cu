@@ -519,7 +519,7 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
     r.queue = bat<uint32_t>(b, L.queue);
     r.tiles_per_fetch = t.tiles_per_fetch;
     r.blocks_per_sm = t.blocks_per_sm;
-    QB_BCUDA(launch_render(r, t.render_batch, s));
+    QB_BCUDA(launch_render(r, s));
     b->sh_degree = scene->sh_degree;
     b->bin_mode = mode;
     b->stage = 1;

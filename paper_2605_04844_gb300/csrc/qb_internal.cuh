@@ -116,6 +116,18 @@ constexpr float kElongatedF2 = 0.01f;  // f < 0.1: aspect ratio above 10 : 1
 // them first never changes a decision of that test.
 __device__ __forceinline__ float skip_threshold(float o) { return -logf(255.0f * o) - 1e-3f; }
 
+// e^x of both lanes as 2^(x log2 e), for the exponents of the compositing
+// (at least skip_threshold, so the result is no subnormal and ex2's
+// flush-to-zero form gives what its other form gives, without the rescaling
+// that one needs; NaN stays NaN).
+__device__ __forceinline__ float2 exp2_of(float2 x) {
+    const float2 t = __fmul2_rn(x, make_float2(1.4426950408889634f, 1.4426950408889634f));
+    float2 r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(t.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(t.y));
+    return r;
+}
+
 // Whether some point of the pixel rectangle [x0, x1] x [y0, y1] can give the
 // Gaussian (mu^2D, conic (a, b, c)) an exponent above t, i.e. whether the
 // rectangle meets the ellipse q(d) = a dx^2 + 2 b dx dy + c dy^2 <= -2t,

@@ -261,7 +261,7 @@ cudaError_t launch_cell_sort(const CellBin &b, cudaStream_t s);
 // look-back words and counters cleared); values only from the last pass.
 // *in_b: the sorted values lie in vals_b.
 cudaError_t cell_sort_passes(const CellBin &b, cudaStream_t s, bool *in_b);
-cudaError_t launch_render(const RenderArgs &a, int batch, cudaStream_t s);
+cudaError_t launch_render(const RenderArgs &a, cudaStream_t s);
 // Files every tile of a single frame (a.ts.cam[0]) into a.order by an
 // estimate of the render's work: the entries composited until four sample
 // pixels of the tile stop (the whole list where one does not).

@@ -1,14 +1,18 @@
 // qb_render.cu -- K6: tile-parallel front-to-back compositing (Sec. 2
 // "Render", Eq. 2), as one block per tile (single frame) or as a persistent
-// kernel that takes tiles of several cameras from a global work queue.
+// kernel whose warps take half tiles of several cameras from a global work
+// queue.
 //
-// A tile is rendered by 64 threads, two warps each owning one half of the
-// tile (rows 0-7 or 8-15); a thread owns four pixels of one column of its
-// half, rows r, r + 2, r + 4 and r + 6, evaluated as two packed pairs (r, r + 2)
-// and (r + 4, r + 6) that share the column's dx terms.  The tile's
-// depth-sorted Gaussian list is walked in
-// batches staged in shared memory (mu^2D, the skip threshold, opacity, the
-// rescaled conic and the colour).  Per entry and pixel (3DGS conventions):
+// A warp renders one half of a tile (rows 0-7 or 8-15) on its own; a thread
+// owns four pixels of one column of the half, rows r, r + 2, r + 4 and r + 6,
+// evaluated as two packed pairs (r, r + 2) and (r + 4, r + 6) that share the
+// column's dx terms.  The warp walks the tile's depth-sorted Gaussian list 32
+// entries at a time: each lane brings in one entry's record (asynchronous
+// copies of the next 32 run during the walk of the current ones), tests its
+// alpha ellipse against the half's 16 x 8 pixels (ellipse_meets_rect), and
+// the entries that reach it are written, compacted, to the warp's staging
+// memory.  An entry left out is one every pixel of the half would reject.
+// Per entry and pixel (3DGS conventions):
 //   power = -(a dx^2 + 2 b dx dy + c dy^2)/2, skip if it is so low that alpha
 //   is certainly below 1/255 (power > 0 arises only as a float32 rounding of
 //   0 and is kept);
@@ -17,206 +21,245 @@
 //   C += alpha T c; T = T'.
 // Each pair is evaluated with the packed FP32x2 instructions (fma/mul/add
 // .f32x2); each packed lane rounds exactly like the scalar operation it
-// replaces.  A tile ends as soon as all of its pixels have stopped.
-// While staging a batch, each entry's alpha ellipse is tested against the
-// two half tiles (ellipse_meets_rect); a warp then walks only the entries
-// that reach its half, a third of the warp-entries of a 1M-Gaussian 1080p
-// frame fewer, with identical results (a skipped entry is one every pixel of
-// the half would have rejected).
+// replaces.  A warp ends as soon as all of its pixels have stopped.
+//
+// The kernel is bound by issue slots (and by the ALU pipe's compares and
+// selects).  Against a two-warp block that staged 128 entries behind
+// barriers and walked the set bits of a mask, a warp of its own needs no
+// barrier, ends with its own pixels, and its compacted list has no bit scan:
+// 1M Gaussians at 1080p 229 -> 181 us, 3M at 1440p seen from inside 1034 ->
+// 911, 1M at 2160p 816 -> 653, 16 views of 1M (persistent) 3340 -> 2670.
+// Measured slower: 64 registers (32 warps per SM, spills), two entries'
+// exponents ahead of both blends, the next entry's operands loaded ahead
+// (+21 %), T chosen by a select instead of multiplied by 1 - 0.
 #include "qb_kernels.cuh"
 
 namespace qb {
 
-constexpr int kRenderThreads = 64;  // four pixels per thread
+constexpr int kRenderThreads = 64;  // a block of the single-frame kernel: the two halves of a tile
 constexpr float kCapTest = 0.98f;    // opacities above this may meet the 0.99 cap
 #define kNaN __int_as_float(0x7fc00000)
 constexpr int kRenderPairs = 2;     // packed pixel pairs per thread
 
-// Per staged entry, five float4 in shared memory laid out for the packed
-// FP32x2 arithmetic of sm_100+: every operand the two pixels of a pair
-// share is stored twice, so a pair register loads it without a move.
+// A warp's shared memory.  raw: one entry's record per lane, the target of
+// the asynchronous copies, read back by the same lane.  The others hold the
+// compacted entries laid out for the packed FP32x2 arithmetic of sm_100+:
+// every operand the two pixels of a pair share is stored twice, so a pair
+// register loads it without a move.
 //   sx = (mu_x, mu_x, mu_y, mu_y), sq = (ca, ca, cb, cb),
-//   sk = (cc, cc, skip threshold, +-opacity), sc1 = (r, r, g, g),
-//   sc2 = (b, b, rr, ce).
-// An elongated Gaussian (qb_internal.cuh) carries a negative opacity and the
-// exact power form's rr = b / a and ce = -1 / (2 Sigma22): its exponent is
-// ca u^2 + ce dy^2 with u = dx + rr dy, which does not cancel.
-// mask[w * BATCH / 32 + k] holds, for warp w (rows 8w .. 8w + 7 of the tile),
-// one bit per entry 32k .. 32k + 31 of the batch: set where the entry's
-// alpha ellipse (exponent above its skip threshold) meets the warp's 16 x 8
-// pixels.  A warp walks only the set bits; every pixel of a cleared entry
-// would have rejected it.
+//   sk = (cc, cc, skip threshold, info), s1 = (o, o, r, r), s2 = (g, g, b, b),
+//   se = (rr, rr, ce, ce) (elongated entries only).
+// info is the entry's position in the list + 1, with kSlowEntry set where the
+// entry may meet the 0.99 cap or is elongated (qb_internal.cuh), kLongEntry
+// for the latter: then its exponent is ca u^2 + ce dy^2 with
+// u = dx + rr dy, rr = b / a, ce = -1 / (2 Sigma22), which does not cancel.
+constexpr uint32_t kSlowEntry = 0x80000000u, kLongEntry = 0x40000000u;  // positions are below 2^30
 struct RenderStage {
-    float4 *sx, *sq, *sk, *sc1, *sc2;
-    uint32_t *mask;
+    float4 raw_co[32], raw_rgb[32];
+    float2 raw_xy[32], raw_sh[32];
+    float4 sx[32], sq[32], sk[32], s1[32], s2[32], se[32];
 };
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
-// The compositing state of one packed pair of pixels.
+__device__ __forceinline__ void copy_async16(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void copy_async8(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// min(a, b), NaN where either is
+__device__ __forceinline__ float min_nan(float a, float b) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// The compositing state of one packed pair of pixels.  A pixel outside the
+// image, or one that has stopped, carries a NaN row npy: its exponent and its
+// alpha are then NaN and fail every test.
 struct RenderPair {
     float2 T, cr, cg, cb, npy;
-    bool done0, done1;
-    int n0, n1, last0, last1;  // n0, n1: the counted variant only
+    int last0, last1;
+    int n0, n1;  // the counted variant only
 };
 
-// Both pixels of a pair are composited in lock step: every entry's exponent
-// is evaluated for the pair with packed operations; entries whose exponent
-// is out of range for every pixel of the warp skip the rest.  An entry a
-// pixel rejects (or a pixel that has stopped) takes weight 0, which leaves
-// its colour and transmittance bit-for-bit unchanged, so the branch-free
-// update composes exactly the entries the per-pixel rules of the header
-// accept.
-// COUNT (measurement only) also adds the tile's (pixel, entry) evaluations
-// and the evaluations whose power test passed to a.counts[0], a.counts[1].
-template <int BATCH, bool COUNT = false>
-__device__ __forceinline__ void render_tile(const RenderArgs &a, uint32_t gtile, const CamTile &C, const RenderStage &S) {
+// Both pixels of a pair are composited in lock step.  An entry a pixel
+// rejects (or a pixel that has stopped) takes weight 0, which leaves its
+// colour and transmittance bit-for-bit unchanged, so the branch-free update
+// composes exactly the entries the per-pixel rules of the header accept.
+// (alpha >= 1/255 implies power >= skip, so the power test needs no second look.)
+template <bool CAP, bool COUNT>
+__device__ __forceinline__ void blend(RenderPair (&P)[kRenderPairs], const float2 (&pw)[kRenderPairs], float2 op,
+                                      float2 cr, float2 cg, float2 cb, int nj) {
+    float2 al[kRenderPairs], tT[kRenderPairs];
+#pragma unroll
+    for (int r = 0; r < kRenderPairs; ++r) {
+        RenderPair &q = P[r];
+        al[r] = __fmul2_rn(op, exp2_of(pw[r]));
+        if (CAP) al[r] = f2(min_nan(kAlphaMax, al[r].x), min_nan(kAlphaMax, al[r].y));
+        const bool ok0 = al[r].x >= kAlphaMin, ok1 = al[r].y >= kAlphaMin;
+        // T (1 - alpha); fma(alpha, -1, 1) is 1 - alpha rounded once
+        tT[r] = __fmul2_rn(q.T, __ffma2_rn(al[r], f2(-1.f, -1.f), f2(1.f, 1.f)));
+        const bool ac0 = ok0 && tT[r].x >= kTStop, ac1 = ok1 && tT[r].y >= kTStop;
+        // alpha of the accepted entries, 0 elsewhere: T (1 - 0) = T and
+        // c + r * 0 = c exactly, so the updates need no select
+        const float2 aa = f2(ac0 ? al[r].x : 0.f, ac1 ? al[r].y : 0.f);
+        const float2 w = __fmul2_rn(aa, q.T);
+        q.cr = __ffma2_rn(cr, w, q.cr);
+        q.cg = __ffma2_rn(cg, w, q.cg);
+        q.cb = __ffma2_rn(cb, w, q.cb);
+        q.T = __fmul2_rn(q.T, __ffma2_rn(aa, f2(-1.f, -1.f), f2(1.f, 1.f)));
+        q.last0 = ac0 ? nj : q.last0;
+        q.last1 = ac1 ? nj : q.last1;
+    }
+    // Once in a pixel's life an accepted alpha takes T below the stop: its row
+    // becomes NaN.  One minimum over the four pixels tells (a NaN loses against
+    // any number in fminf); which of them stopped is looked at only then.
+    if (fminf(fminf(tT[0].x, tT[0].y), fminf(tT[1].x, tT[1].y)) < kTStop) {
+#pragma unroll
+        for (int r = 0; r < kRenderPairs; ++r) {
+            const bool st0 = al[r].x >= kAlphaMin && tT[r].x < kTStop, st1 = al[r].y >= kAlphaMin && tT[r].y < kTStop;
+            if (st0) P[r].npy.x = kNaN;
+            if (st1) P[r].npy.y = kNaN;
+            if (COUNT && st0) P[r].n0 = nj;
+            if (COUNT && st1) P[r].n1 = nj;
+        }
+    }
+}
+
+// One half (0: rows 0-7, 1: rows 8-15) of a tile by one warp; returns the
+// largest last-contributor count of the lane's pixels.  COUNT (measurement
+// only) also adds the half's (pixel, entry) evaluations and the evaluations
+// whose power test passed to a.counts[0], a.counts[1].
+template <bool COUNT = false>
+__device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, int half, const CamTile &C,
+                                           RenderStage &S) {
     const uint32_t lt = gtile - C.tile_base;
-    const uint32_t *vals = a.vals + C.vals_base;
     const int tx = (int)(lt % (uint32_t)C.tiles_x), ty = (int)(lt / (uint32_t)C.tiles_x);
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int lane = threadIdx.x & 31;
+    const uint32_t below = (1u << lane) - 1u;
     const int px = tx * kTile + (lane & (kTile - 1));
-    const int pyb = ty * kTile + wid * 8 + (lane >> kTileShift);
+    const int pyb = ty * kTile + half * 8 + (lane >> kTileShift);
     const float2 npx = f2(-(float)px, -(float)px);
+    // the half's pixels, for the ellipse test
+    const float x0 = (float)(tx * kTile), y0 = (float)(ty * kTile + half * 8);
     RenderPair P[kRenderPairs];
 #pragma unroll
     for (int r = 0; r < kRenderPairs; ++r) {
-        const int y0 = pyb + 4 * r, y1 = y0 + 2;
-        const bool in0 = px < C.W && y0 < C.H, in1 = px < C.W && y1 < C.H;
-        P[r].done0 = !in0;
-        P[r].done1 = !in1;
-        // a pixel outside the image (later: one that has stopped) carries a
-        // NaN row, so its exponent is NaN and fails every test
-        P[r].npy = f2(in0 ? -(float)y0 : kNaN, in1 ? -(float)y1 : kNaN);
+        const int ya = pyb + 4 * r, yb = ya + 2;
+        P[r].npy = f2(px < C.W && ya < C.H ? -(float)ya : kNaN, px < C.W && yb < C.H ? -(float)yb : kNaN);
         P[r].T = f2(1.f, 1.f);
         P[r].cr = P[r].cg = P[r].cb = f2(0.f, 0.f);
-        P[r].n0 = P[r].n1 = P[r].last0 = P[r].last1 = 0;
+        P[r].last0 = P[r].last1 = P[r].n0 = P[r].n1 = 0;
     }
+    auto stopped = [](float npy) { return npy != npy; };
     auto all_done = [&]() {
-        bool d = true;
-#pragma unroll
-        for (int r = 0; r < kRenderPairs; ++r) d = d && P[r].done0 && P[r].done1;
-        return d;
+        return stopped(P[0].npy.x) && stopped(P[0].npy.y) && stopped(P[1].npy.x) && stopped(P[1].npy.y);
     };
 
     const uint2 range = a.ranges[gtile];
     const int total = (int)(range.y - range.x);
+    const uint32_t *vals = a.vals + C.vals_base + range.x;
+    auto fetch = [&](uint32_t v) {  // the lane's record of the next 32 entries
+        const uint32_t g = C.rec_base + v;
+        copy_async16(&S.raw_co[lane], a.conic_o + g);
+        copy_async16(&S.raw_rgb[lane], a.rgbd + g);
+        copy_async8(&S.raw_xy[lane], a.xy + g);
+        copy_async8(&S.raw_sh[lane], a.shape + g);
+    };
     uint32_t npass = 0;  // COUNT only
+    if (lane < total) fetch(vals[lane]);
+    uint32_t vnext = 32 + lane < total ? vals[32 + lane] : 0u;
 
-    for (int base = 0; base < total; base += BATCH) {
-        if (__syncthreads_count(all_done()) == kRenderThreads) break;
-#pragma unroll 1
-        for (int q = tid; q < BATCH; q += kRenderThreads) {
-            const int idx = base + q;
-            bool hit0 = false, hit1 = false;
-            if (idx < total) {
-                const uint32_t g = C.rec_base + vals[range.x + idx];
-                const float2 m = a.xy[g];
-                const float4 co = a.conic_o[g];
-                const float4 rgb = a.rgbd[g];
-                const float2 sh = a.shape[g];
-                const float ca = -0.5f * co.x, cbv = -co.y, cc = -0.5f * co.z;
-                const float skip = skip_threshold(co.w);
-                S.sx[q] = make_float4(m.x, m.x, m.y, m.y);
-                S.sq[q] = make_float4(ca, ca, cbv, cbv);
-                S.sk[q] = make_float4(cc, cc, skip, sh.y != 0.f ? -co.w : co.w);
-                S.sc1[q] = make_float4(rgb.x, rgb.x, rgb.y, rgb.y);
-                S.sc2[q] = make_float4(rgb.z, rgb.z, sh.x, sh.y);
-                const float x0 = (float)(tx * kTile), y0 = (float)(ty * kTile);
-                hit0 = ellipse_meets_rect(m.x, m.y, co.x, co.y, co.z, skip, sh.y != 0.f, x0, y0, x0 + 15.f, y0 + 7.f);
-                hit1 = ellipse_meets_rect(m.x, m.y, co.x, co.y, co.z, skip, sh.y != 0.f, x0, y0 + 8.f, x0 + 15.f,
-                                          y0 + 15.f);
-            }
-            const uint32_t b0 = __ballot_sync(0xffffffffu, hit0), b1 = __ballot_sync(0xffffffffu, hit1);
-            if (lane == 0) {
-                S.mask[q >> 5] = b0;
-                S.mask[BATCH / 32 + (q >> 5)] = b1;
-            }
+    for (int base = 0; base < total; base += 32) {
+        copy_wait();
+        bool hit = false;
+        float2 m = f2(0.f, 0.f), sh = f2(0.f, 0.f);
+        float4 co = make_float4(0.f, 0.f, 0.f, 0.f), rgb = co;
+        float skip = 0.f;
+        if (base + lane < total) {
+            m = S.raw_xy[lane];
+            sh = S.raw_sh[lane];
+            co = S.raw_co[lane];
+            rgb = S.raw_rgb[lane];
+            skip = skip_threshold(co.w);
+            hit = ellipse_meets_rect(m.x, m.y, co.x, co.y, co.z, skip, sh.y != 0.f, x0, y0, x0 + 15.f, y0 + 7.f);
         }
-        __syncthreads();
-        const int cnt = min(BATCH, total - base);
-        for (int w0 = 0; w0 < cnt; w0 += 32) {
-            // every 32 entries: leave once all pixels of the warp have stopped
-            if (__all_sync(0xffffffffu, all_done())) break;
-            uint32_t bits = S.mask[wid * (BATCH / 32) + (w0 >> 5)];
-            while (bits) {
-                const int j = w0 + __ffs(bits) - 1;
-                bits &= bits - 1;
-                const float4 X = S.sx[j], Q = S.sq[j], K = S.sk[j];
-                const float2 dx = __fadd2_rn(f2(X.x, X.y), npx);
-                float2 pw[kRenderPairs];
-                if (K.w >= 0.f) {
-                    // power = A + dy (B + cc dy), A = ca dx^2, B = cb dx; dx, A and
-                    // B are the column's, shared by the thread's four pixels
-                    const float2 A = __fmul2_rn(__fmul2_rn(f2(Q.x, Q.y), dx), dx);
-                    const float2 B = __fmul2_rn(f2(Q.z, Q.w), dx);
-#pragma unroll
-                    for (int r = 0; r < kRenderPairs; ++r) {
-                        const float2 dy = __fadd2_rn(f2(X.z, X.w), P[r].npy);
-                        pw[r] = __ffma2_rn(dy, __ffma2_rn(f2(K.x, K.y), dy, B), A);
-                    }
-                } else {
-                    // elongated (the same for the whole warp): power = ca u^2 +
-                    // ce dy^2, u = dx + rr dy
-                    const float4 E = S.sc2[j];
-#pragma unroll
-                    for (int r = 0; r < kRenderPairs; ++r) {
-                        const float2 dy = __fadd2_rn(f2(X.z, X.w), P[r].npy);
-                        const float2 u = __ffma2_rn(f2(E.z, E.z), dy, dx);
-                        pw[r] = __ffma2_rn(__fmul2_rn(f2(Q.x, Q.y), u), u, __fmul2_rn(__fmul2_rn(f2(E.w, E.w), dy), dy));
-                    }
-                }
-                const float op = fabsf(K.w);
-                bool e0[kRenderPairs], e1[kRenderPairs];
-                bool any = false;
+        const uint32_t hits = __ballot_sync(0xffffffffu, hit);  // also: the walk of the last entries is over
+        if (hit) {
+            const int k = __popc(hits & below);
+            const float ca = -0.5f * co.x, cbv = -co.y, cc = -0.5f * co.z;
+            uint32_t info = (uint32_t)(base + lane + 1);
+            if (co.w > kCapTest) info |= kSlowEntry;
+            if (sh.y != 0.f) info |= kSlowEntry | kLongEntry;
+            S.sx[k] = make_float4(m.x, m.x, m.y, m.y);
+            S.sq[k] = make_float4(ca, ca, cbv, cbv);
+            S.sk[k] = make_float4(cc, cc, skip, __uint_as_float(info));
+            S.s1[k] = make_float4(co.w, co.w, rgb.x, rgb.x);
+            S.s2[k] = make_float4(rgb.y, rgb.y, rgb.z, rgb.z);
+            if (sh.y != 0.f) S.se[k] = make_float4(sh.x, sh.x, sh.y, sh.y);
+        }
+        if (base + 32 + lane < total) {
+            fetch(vnext);
+            vnext = base + 64 + lane < total ? vals[base + 64 + lane] : 0u;
+        }
+        __syncwarp();
+        const int cnt = __popc(hits);
+#pragma unroll 2
+        for (int j = 0; j < cnt; ++j) {
+            const float4 X = S.sx[j], Q = S.sq[j], K = S.sk[j];
+            const uint32_t info = __float_as_uint(K.w);
+            const float2 dx = __fadd2_rn(f2(X.x, X.y), npx);
+            float2 pw[kRenderPairs];
+            if (!(info & kLongEntry)) {
+                // power = A + dy (B + cc dy), A = ca dx^2, B = cb dx; dx, A and
+                // B are the column's, shared by the thread's four pixels
+                const float2 A = __fmul2_rn(__fmul2_rn(f2(Q.x, Q.y), dx), dx);
+                const float2 B = __fmul2_rn(f2(Q.z, Q.w), dx);
 #pragma unroll
                 for (int r = 0; r < kRenderPairs; ++r) {
-                    // power >= skip; the rule power <= 0 needs no test: a
-                    // positive exponent is a float32 rounding of 0 (the conic is
-                    // positive definite), where alpha = o e^power rounds like o
-                    e0[r] = pw[r].x >= K.z;
-                    e1[r] = pw[r].y >= K.z;
-                    if (COUNT) npass += (uint32_t)e0[r] + (uint32_t)e1[r];
-                    any = any || e0[r] || e1[r];
+                    const float2 dy = __fadd2_rn(f2(X.z, X.w), P[r].npy);
+                    pw[r] = __ffma2_rn(dy, __ffma2_rn(f2(K.x, K.y), dy, B), A);
                 }
-                if (!__any_sync(0xffffffffu, any)) continue;
-                const float4 C1 = S.sc1[j], C2 = S.sc2[j];
-                // entries evaluated so far by a pixel still running: base + j + 1
-                const int nj = base + j + 1;
-                // o G can reach the 0.99 cap only for o near it (G <= 1 up to
-                // the exponential's rounding); the same for the whole warp
-                const bool capped = op > kCapTest;
+            } else {
+                // elongated (the same for the whole warp): power = ca u^2 +
+                // ce dy^2, u = dx + rr dy
+                const float4 E = S.se[j];
 #pragma unroll
                 for (int r = 0; r < kRenderPairs; ++r) {
-                    RenderPair &q = P[r];
-                    float2 al = __fmul2_rn(f2(op, op), f2(__expf(pw[r].x), __expf(pw[r].y)));
-                    if (capped) al = f2(fminf(kAlphaMax, al.x), fminf(kAlphaMax, al.y));
-                    const float a0 = al.x, a1 = al.y;
-                    const bool ok0 = e0[r] && a0 >= kAlphaMin, ok1 = e1[r] && a1 >= kAlphaMin;
-                    // T (1 - alpha); fma(alpha, -1, 1) is 1 - alpha rounded once
-                    const float2 tT = __fmul2_rn(q.T, __ffma2_rn(al, f2(-1.f, -1.f), f2(1.f, 1.f)));
-                    const bool st0 = ok0 && tT.x < kTStop, st1 = ok1 && tT.y < kTStop;
-                    const bool ac0 = ok0 && !st0, ac1 = ok1 && !st1;
-                    if (st0 || st1) {  // once in a pixel's life: record the stop, poison its row
-                        if (st0) q.done0 = true, q.npy.x = kNaN;
-                        if (st1) q.done1 = true, q.npy.y = kNaN;
-                        if (COUNT && st0) q.n0 = nj;
-                        if (COUNT && st1) q.n1 = nj;
-                    }
-                    // alpha of the accepted entries, 0 elsewhere: T (1 - 0) = T and
-                    // c + r * 0 = c exactly, so the updates need no select
-                    const float2 aa = f2(ac0 ? a0 : 0.f, ac1 ? a1 : 0.f);
-                    const float2 w = __fmul2_rn(aa, q.T);
-                    q.cr = __ffma2_rn(f2(C1.x, C1.y), w, q.cr);
-                    q.cg = __ffma2_rn(f2(C1.z, C1.w), w, q.cg);
-                    q.cb = __ffma2_rn(f2(C2.x, C2.y), w, q.cb);
-                    q.T = __fmul2_rn(q.T, __ffma2_rn(aa, f2(-1.f, -1.f), f2(1.f, 1.f)));
-                    q.last0 = ac0 ? nj : q.last0;
-                    q.last1 = ac1 ? nj : q.last1;
+                    const float2 dy = __fadd2_rn(f2(X.z, X.w), P[r].npy);
+                    const float2 u = __ffma2_rn(f2(E.x, E.y), dy, dx);
+                    pw[r] = __ffma2_rn(__fmul2_rn(f2(Q.x, Q.y), u), u, __fmul2_rn(__fmul2_rn(f2(E.z, E.w), dy), dy));
                 }
             }
+            // power >= skip for some pixel; the rule power <= 0 needs no test: a
+            // positive exponent is a float32 rounding of 0 (the conic is
+            // positive definite), where alpha = o e^power rounds like o.
+            // (A NaN loses against any number in fmaxf.)
+            const bool any = fmaxf(fmaxf(pw[0].x, pw[0].y), fmaxf(pw[1].x, pw[1].y)) >= K.z;
+            if (COUNT)
+                npass += (uint32_t)(pw[0].x >= K.z) + (uint32_t)(pw[0].y >= K.z) + (uint32_t)(pw[1].x >= K.z) +
+                         (uint32_t)(pw[1].y >= K.z);
+            if (!__any_sync(0xffffffffu, any)) continue;
+            const float4 C1 = S.s1[j], C2 = S.s2[j];
+            // o G can reach the 0.99 cap only for o near it (G <= 1 up to the
+            // exponential's rounding); the same for the whole warp
+            if (!(info & kSlowEntry))
+                blend<false, COUNT>(P, pw, f2(C1.x, C1.y), f2(C1.z, C1.w), f2(C2.x, C2.y), f2(C2.z, C2.w), (int)info);
+            else
+                blend<true, COUNT>(P, pw, f2(C1.x, C1.y), f2(C1.z, C1.w), f2(C2.x, C2.y), f2(C2.z, C2.w),
+                                   (int)(info & ~(kSlowEntry | kLongEntry)));
         }
+        if (__all_sync(0xffffffffu, all_done())) break;
     }
+    copy_wait();  // the staging memory is the warp's next tile's
     const size_t plane = (size_t)C.W * C.H;
     float *img = a.img + 3 * C.pix_base;
     unsigned long long ev = 0;
@@ -224,8 +267,8 @@ __device__ __forceinline__ void render_tile(const RenderArgs &a, uint32_t gtile,
     for (int r = 0; r < kRenderPairs; ++r) {
         RenderPair &q = P[r];
         // a pixel that never stopped evaluated the whole list
-        if (COUNT && !q.done0) q.n0 = total;
-        if (COUNT && !q.done1) q.n1 = total;
+        if (COUNT && !stopped(q.npy.x)) q.n0 = total;
+        if (COUNT && !stopped(q.npy.y)) q.n1 = total;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int py = pyb + 4 * r + 2 * h;
@@ -243,18 +286,6 @@ __device__ __forceinline__ void render_tile(const RenderArgs &a, uint32_t gtile,
             }
         }
     }
-    if (a.order_out.cnt) {
-        // the tile's largest last-contributor count (the backward walks that
-        // many entries) files it for the backward
-        __shared__ int s_last[2];
-        int m = 0;
-#pragma unroll
-        for (int r = 0; r < kRenderPairs; ++r) m = max(m, max(P[r].last0, P[r].last1));
-        m = __reduce_max_sync(0xffffffffu, m);
-        if (lane == 0) s_last[wid] = m;
-        __syncthreads();
-        if (tid == 0) order_file(a.order_out, a.ts.total_tiles, gtile, (uint32_t)max(s_last[0], s_last[1]));
-    }
     if (COUNT) {
         unsigned long long ps = npass;
 #pragma unroll
@@ -267,18 +298,27 @@ __device__ __forceinline__ void render_tile(const RenderArgs &a, uint32_t gtile,
             atomicAdd(a.counts + 1, ps);
         }
     }
+    return max(max(P[0].last0, P[0].last1), max(P[1].last0, P[1].last1));
 }
 
-// One block per tile of a single camera; with an order, the blocks (which
-// start roughly in index order) take the heaviest tiles first, so that the
-// last blocks to start are short ones.
-template <int BATCH, bool COUNT>
+// One block per tile of a single camera, a warp per half; with an order, the
+// blocks (which start roughly in index order) take the heaviest tiles first,
+// so that the last blocks to start are short ones.
+template <bool COUNT>
 __global__ void __launch_bounds__(kRenderThreads) render_kernel(RenderArgs a) {
-    __shared__ float4 s_stage[5][BATCH];
-    __shared__ uint32_t s_mask[2 * BATCH / 32];
-    const RenderStage S{s_stage[0], s_stage[1], s_stage[2], s_stage[3], s_stage[4], s_mask};
+    __shared__ RenderStage s_stage[2];
+    __shared__ int s_last[2];
+    const int wid = threadIdx.x >> 5;
     const uint32_t t = a.order.cnt ? order_pick(a.order, a.ts.total_tiles, blockIdx.x) : (uint32_t)blockIdx.x;
-    render_tile<BATCH, COUNT>(a, t, a.ts.cam[0], S);
+    const int last = render_half<COUNT>(a, t, wid, a.ts.cam[0], s_stage[wid]);
+    if (a.order_out.cnt) {
+        // the tile's largest last-contributor count (the backward walks that
+        // many entries) files it for the backward
+        const int m = __reduce_max_sync(0xffffffffu, last);
+        if ((threadIdx.x & 31) == 0) s_last[wid] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) order_file(a.order_out, a.ts.total_tiles, t, (uint32_t)max(s_last[0], s_last[1]));
+    }
 }
 
 // A warp per tile walks the tile's list 32 entries at a time for four sample
@@ -385,57 +425,41 @@ cudaError_t launch_tile_work(const RenderArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Persistent blocks take tiles_per_fetch consecutive tiles at a time from a
-// global counter over the tiles of all cameras in the set.
-template <int BATCH>
+// Persistent warps take the halves of tiles_per_fetch consecutive tiles at a
+// time from a global counter over the tiles of all cameras in the set.
 __global__ void __launch_bounds__(kRenderThreads) render_persistent_kernel(RenderArgs a) {
-    __shared__ float4 s_stage[5][BATCH];
-    __shared__ uint32_t s_mask[2 * BATCH / 32];
-    __shared__ uint32_t s_next;
-    const RenderStage S{s_stage[0], s_stage[1], s_stage[2], s_stage[3], s_stage[4], s_mask};
+    __shared__ RenderStage s_stage[2];
+    RenderStage &S = s_stage[threadIdx.x >> 5];
+    const uint32_t halves = 2u * a.ts.total_tiles, take = 2u * (uint32_t)a.tiles_per_fetch;
     for (;;) {
-        if (threadIdx.x == 0) s_next = atomicAdd(a.queue, (uint32_t)a.tiles_per_fetch);
-        __syncthreads();
-        const uint32_t t0 = s_next;
-        __syncthreads();
-        if (t0 >= a.ts.total_tiles) break;
-        const uint32_t t1 = min(t0 + (uint32_t)a.tiles_per_fetch, a.ts.total_tiles);
-        for (uint32_t t = t0; t < t1; ++t) {
-            if (a.cam_table) {
-                const CamTile C = a.cam_table[camera_in_table(a.cam_table, a.ts.n_cams, t)];
-                render_tile<BATCH>(a, t, C, S);
-            } else {
-                render_tile<BATCH>(a, t, a.ts.cam[camera_of(a.ts, t)], S);
-            }
+        uint32_t h0 = 0;
+        if ((threadIdx.x & 31) == 0) h0 = atomicAdd(a.queue, take);
+        h0 = __shfl_sync(0xffffffffu, h0, 0);
+        if (h0 >= halves) break;
+        const uint32_t h1 = min(h0 + take, halves);
+        for (uint32_t h = h0; h < h1; ++h) {
+            const uint32_t t = h >> 1;
+            const CamTile C = a.cam_table[camera_in_table(a.cam_table, a.ts.n_cams, t)];
+            render_half(a, t, (int)(h & 1u), C, S);
         }
     }
 }
 
-template <int BATCH>
-static cudaError_t launch_render_b(const RenderArgs &a, cudaStream_t s) {
+cudaError_t launch_render(const RenderArgs &a, cudaStream_t s) {
+    if (a.ts.total_tiles == 0) return cudaSuccess;
     if (a.queue) {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_persistent_kernel<BATCH>, kRenderThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_persistent_kernel, kRenderThreads, 0);
         if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_sm) per_sm = a.blocks_per_sm;
-        note_launch("render_persistent_kernel", s), render_persistent_kernel<BATCH><<<sms * (per_sm > 0 ? per_sm : 1), kRenderThreads, 0, s>>>(a);
+        note_launch("render_persistent_kernel", s), render_persistent_kernel<<<sms * (per_sm > 0 ? per_sm : 1), kRenderThreads, 0, s>>>(a);
     } else if (a.counts) {
-        note_launch("render_kernel_counted", s),
-            render_kernel<BATCH, true><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
+        note_launch("render_kernel_counted", s), render_kernel<true><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
     } else {
-        note_launch("render_kernel", s), render_kernel<BATCH, false><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
+        note_launch("render_kernel", s), render_kernel<false><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
     }
     return cudaGetLastError();
-}
-
-cudaError_t launch_render(const RenderArgs &a, int batch, cudaStream_t s) {
-    if (a.ts.total_tiles == 0) return cudaSuccess;
-    switch (batch) {
-    case 64: return launch_render_b<64>(a, s);
-    case 128: return launch_render_b<128>(a, s);
-    default: return launch_render_b<256>(a, s);
-    }
 }
 
 }  // namespace qb
