@@ -2,13 +2,14 @@
 // differentiable rasteriser (Sec. 4.1 states the rasteriser is differentiable;
 // the gradients below differentiate Eq. 2 and the Sec. 2 projection).
 //
-// K7: a 64-thread block per tile (each warp a half tile, four pixels of a
-// column per thread, rows r, r+2, r+4, r+6 of the half, evaluated as two
-// pairs with the packed FP32x2 instructions) walks the tile list in reverse,
-// from the largest last-contributor position of its pixels down to 0; the
-// blocks take the tiles by decreasing walk length, the order the forward
-// render filed.  Each pixel recomputes
-// alpha exactly as the forward did and the transmittance by division,
+// K7: a warp per half tile (16 x 8 pixels, four pixels of a column per lane,
+// rows r, r+2, r+4, r+6 of the half, evaluated as two pairs with the packed
+// FP32x2 instructions) walks the tile list in reverse, from the largest
+// last-contributor position of its own pixels down to 0, staging the entries
+// that reach its pixels like the forward (qb_stage.cuh); the blocks take the
+// tiles by decreasing walk length, the order the forward render filed.  Each
+// pixel recomputes alpha exactly as the forward did and the transmittance by
+// division,
 // T_k = T_{k+1} / (1 - alpha_k); with B_k = sum_{i>k} T_i alpha_i c_i + T_final bg
 // the colour behind entry k,
 //   dC/dc_k     = T_k alpha_k
@@ -18,23 +19,29 @@
 // derivative where the cap binds.
 // The 9 per-Gaussian sums (mu_x, mu_y, Sigma11, Sigma12, Sigma22, o, r, g, b;
 // the covariance entries are the well-conditioned parametrisation, with
-// dL/dLambda = -Sigma dL/dSigma Sigma) are reduced over the warp by a
-// transpose-reduction (12 shuffles) that leaves one sum on each of 9 lanes,
-// which add them to float64 accumulators in parallel.  The same tile routine
-// serves one block per tile and a persistent kernel over several cameras.
+// dL/dLambda = -Sigma dL/dSigma Sigma) are summed over the warp three entries
+// at a time: every lane puts its 9 values in a row of shared memory each, and
+// 27 lanes then sum a row of 32 with eight 16-byte loads and add it to its
+// float64 accumulator: 19 instructions per entry where a 12-shuffle transpose
+// reduction with its selects took about 70.  (The chain to the scale and
+// rotation of a thin Gaussian amplifies the rounding of these sums, so they
+// keep the order of the butterfly.)  The same routine serves one block per tile
+// and a persistent kernel over several cameras.
+//
+// The kernel is bound by latency between dependent packed operations at 20
+// warps per SM (96 registers; issue 65 %, FMA pipe 52 %).  1M Gaussians at
+// 1080p 461 -> 357 us, 5 views of 200k (persistent) 2023 -> 1710; 80 or 88
+// registers (12 or 11 blocks per SM) measured 3 to 6 % slower.
 //
 // K8: one thread per Gaussian chains the (mu^2D, Sigma2D, o, colour)
 // gradients of every camera of the set to means, (log-)scales, quaternions,
 // opacity (logits) and SH, summing over cameras in registers.
-#include "qb_kernels.cuh"
 #include "qb_project.cuh"
+#include "qb_stage.cuh"
 
 namespace qb {
 
-constexpr int kBwdPix = 4;                            // pixels per thread (one column)
-constexpr int kBwdThreads = kTile * kTile / kBwdPix;  // threads per tile
-static_assert(kBwdThreads == 64 && kBwdPix == 4, "two warps per tile, each a half tile of 16 x 8 pixels");
-constexpr int kBwdBatch = 128;  // entries staged per shared-memory batch
+constexpr int kBwdThreads = 64;  // a block of the single-frame kernel: the two halves of a tile
 
 // float -> double by rebuilding the IEEE-754 bit pattern with integer
 // operations (exponent rebias 127 -> 1023, mantissa 23 -> 52 bits), so the
@@ -49,74 +56,77 @@ __device__ __forceinline__ double widen(float v) {
     return __longlong_as_double((long long)bits);
 }
 
-// Sum g[0..8] over the warp and add the 9 totals to dst[0..8].  Each butterfly
-// step halves the vector every lane carries (9 -> 5 -> 3 -> 2 -> 1): lanes on
-// the lower side of a step keep the first half, those on the upper side the
-// second half.  Afterwards lane l (bit 0 clear) holds element
-// 5 b4 + 3 b3 + 2 b2 + b1 of the original vector, when that index is real.
-__device__ __forceinline__ void warp_reduce9_add(const float g[9], double *dst, int lane) {
-    const unsigned F = 0xffffffffu;
-    float w[5];
-    const bool u4 = lane & 16;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const float lo = g[i], hi = (i + 5 < 9) ? g[i + 5] : 0.f;
-        w[i] = (u4 ? hi : lo) + __shfl_xor_sync(F, u4 ? lo : hi, 16);
-    }
-    float x[3];
-    const bool u3 = lane & 8;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const float lo = w[i], hi = (i + 3 < 5) ? w[i + 3] : 0.f;
-        x[i] = (u3 ? hi : lo) + __shfl_xor_sync(F, u3 ? lo : hi, 8);
-    }
-    float y[2];
-    const bool u2 = lane & 4;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const float lo = x[i], hi = (i + 2 < 3) ? x[i + 2] : 0.f;
-        y[i] = (u2 ? hi : lo) + __shfl_xor_sync(F, u2 ? lo : hi, 4);
-    }
-    const bool u1 = lane & 2;
-    float z = (u1 ? y[1] : y[0]) + __shfl_xor_sync(F, u1 ? y[0] : y[1], 2);
-    z += __shfl_xor_sync(F, z, 1);
-    const int ix = 2 * ((lane >> 2) & 1) + ((lane >> 1) & 1);
-    const int iw = 3 * ((lane >> 3) & 1) + ix;
-    const int iv = 5 * ((lane >> 4) & 1) + iw;
-    if (!(lane & 1) && ix < 3 && iw < 5 && iv < 9 && z != 0.f) atomicAdd(dst + iv, widen(z));
+// 1 / x for x in [0.01, 1].
+__device__ __forceinline__ float reciprocal(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
-// Staged entries of a backward batch, laid out for the packed FP32x2
-// arithmetic (operands the pixels of a thread share are stored twice):
-//   s0 = (mu_x, mu_x, mu_y, mu_y), s1 = (ca, ca, cb, cb),
-//   s2 = (cc, cc, skip threshold, elongated), s3 = (r, r, g, g), s4 = (b, b, o, o),
-//   s5 = (rr, rr, ce, ce),
-// with (ca, cb, cc) = (-a/2, -b, -c/2) the rescaled conic of the forward and,
-// for an elongated Gaussian (s2.w = 1), the exact power form's terms
-// (qb_render.cu): power = ca u^2 + ce dy^2, u = dx + rr dy.
+// The warp sums of up to kRedEntries entries: row 9 e + i holds, per lane, value
+// i of the e-th waiting entry.  Rows of 36 floats put the 16-byte loads of
+// eight neighbouring lanes (each summing a row of its own) on distinct banks.
+constexpr int kRedEntries = 3, kRedStride = 36;
 struct BwdStage {
-    uint32_t *id;
-    float4 *s0, *s1, *s2, *s3, *s4, *s5;
-    int *maxlast;
+    RenderStage in;
+    float red[9 * kRedEntries * kRedStride];
+    uint32_t ids[32];             // record of each staged entry
+    uint32_t red_id[kRedEntries];  // record of each waiting entry
 };
 
-__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+// Adds the waiting entries' sums to the accumulators (all lanes; the rows and
+// ids are written by then up to a warp synchronisation, done here).  The
+// staged values carry the sign and factor that are applied to the sums here:
+// -1 for 0..4 and 6..8, and 1/2 for the squares 2 and 4.
+__device__ __forceinline__ void bwd_flush(const BwdStage &S, int waiting, double *g_screen, int lane) {
+    __syncwarp();
+    if (lane < 9 * waiting) {
+        const float4 *row = reinterpret_cast<const float4 *>(S.red + lane * kRedStride);
+        // lanes l and l + 16, then l and l + 8, + 4, + 2, + 1: the tree of a
+        // butterfly over the warp
+        float2 v[16];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float4 q = row[k];
+            v[2 * k] = f2(q.x, q.y);
+            v[2 * k + 1] = f2(q.z, q.w);
+        }
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1)
+#pragma unroll
+            for (int k = 0; k < d; ++k) v[k] = __fadd2_rn(v[k], v[k + d]);
+        const float2 s = v[0];
+        const int e = lane / 9, i = lane - 9 * e;
+        const float z = (s.x + s.y) * (i == 5 ? 1.f : i == 2 || i == 4 ? -0.5f : -1.f);
+        if (z != 0.f) atomicAdd(g_screen + (size_t)S.red_id[e] * 9 + i, widen(z));
+    }
+    __syncwarp();
+}
 
 // The per-pixel state of a pair of pixels (one packed lane each): the
 // transmittance in front of the current entry, T; -S2 with
 // S2 = sum_c dL/dC_c B_c (the colour behind the entry, B_c, only enters the
 // gradient through this sum, which is updated as S2 += w S1 when an entry of
-// weight w = alpha T is passed); and dL/dC per channel.
+// weight w = alpha T is passed); and dL/dC per channel.  npy is kFar until the
+// walk reaches the 32 entries that hold the pixel's last contributor: at that
+// distance the exponent is hugely negative and every term finite.
+constexpr float kFar = 1e15f;
 struct BwdPair {
     float2 T, nS2, g0, g1, g2, npy;
     int last0, last1;
 };
 
-// A tile by kBwdThreads threads: two warps, each owning one half of the tile
-// (rows 0-7 or 8-15, a compact footprint, so a small ellipse reaches one
-// warp more often than both); a thread owns kBwdPix pixels of one column of
-// its half (rows r, r + 2, r + 4, r + 6) as two packed pairs (r, r + 2) and
-// (r + 4, r + 6).  Per entry, for every pixel:
+// Operands of an entry that all pixels of a column share.
+struct BwdEntry {
+    float2 dx, cadx2, B, cb;       // dx; 2 ca dx, cb dx, cb
+    float2 no, cr, cg, cbl;        // -opacity, colour
+};
+
+// One entry for the thread's four pixels: updates their state and returns
+// their summed contributions (each pair's two pixels packed) in X.  An entry a
+// pixel does not composite takes alpha = 0 (T, S2 unchanged, no contribution),
+// so the pairs run in lock step without branches.  CAP: the entry may meet
+// the 0.99 cap; LONG: vx, vy come from the exact form.
 //   T <- T / (1 - alpha)                       (T in front of the entry)
 //   dL/dc_k     += alpha T dL/dC
 //   dL/dalpha    = T S1 - S2 / (1 - alpha),    S1 = sum_c dL/dC_c c_k,c
@@ -125,23 +135,85 @@ struct BwdPair {
 // v = -dpower/dmu = (2 ca dx + cb dy, cb dx + 2 cc dy):
 //   dL/do += G dL/dalpha, dpower = o G dL/dalpha,
 //   dL/dmu += dpower v, dL/dSigma += dpower (vx^2/2, vx vy, vy^2/2).
-// An entry a pixel does not composite takes alpha = 0 (T, S2 unchanged, no
-// contribution), so the pairs run in lock step without branches.
-__device__ __forceinline__ void render_bwd_tile(const BwdArgs &a, uint32_t gtile, const CamTile &C, const BwdStage &S) {
+// X0..X4 and X6..X8 come with the opposite sign, X2 and X4 without the 1/2
+// (bwd_flush).
+template <bool CAP>
+__device__ __forceinline__ bool bwd_entry(BwdPair (&P)[2], const float2 (&pw)[2], const float2 (&vx)[2],
+                                          const float2 (&vy)[2], const BwdEntry &E, int nj, float2 (&X)[9]) {
+    bool contrib = false;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        BwdPair &q = P[r];
+        const float2 G = exp2_of(pw[r]);
+        const float2 noG = __fmul2_rn(E.no, G);  // -o G
+        bool c0, c1;
+        float2 na, Gm;
+        if constexpr (CAP) {
+            const float a0 = min_nan(kAlphaMax, -noG.x), a1 = min_nan(kAlphaMax, -noG.y);
+            c0 = nj <= q.last0 && a0 >= kAlphaMin;
+            c1 = nj <= q.last1 && a1 >= kAlphaMin;
+            na = f2(c0 ? -a0 : 0.f, c1 ? -a1 : 0.f);
+            // derivative through o G where the cap does not bind
+            Gm = f2(c0 && -noG.x < kAlphaMax ? G.x : 0.f, c1 && -noG.y < kAlphaMax ? G.y : 0.f);
+        } else {
+            c0 = nj <= q.last0 && noG.x <= -kAlphaMin;
+            c1 = nj <= q.last1 && noG.y <= -kAlphaMin;
+            Gm = f2(c0 ? G.x : 0.f, c1 ? G.y : 0.f);
+            na = __fmul2_rn(E.no, Gm);  // -alpha of the composited, 0 elsewhere
+        }
+        contrib = contrib || c0 || c1;
+        const float2 om = __fadd2_rn(f2(1.f, 1.f), na);  // 1 - alpha (1 where not composited)
+        const float2 inv = f2(reciprocal(om.x), reciprocal(om.y));  // exactly 1 where om is
+        q.T = __fmul2_rn(q.T, inv);
+        const float2 nw = __fmul2_rn(na, q.T);  // -alpha T
+        const float2 S1 = __ffma2_rn(q.g0, E.cr, __ffma2_rn(q.g1, E.cg, __fmul2_rn(q.g2, E.cbl)));
+        const float2 dal = __ffma2_rn(inv, q.nS2, __fmul2_rn(q.T, S1));
+        q.nS2 = __ffma2_rn(nw, S1, q.nS2);
+        // -dpower; o Gm is alpha where the cap does not bind
+        const float2 ndp = __fmul2_rn(dal, CAP ? __fmul2_rn(E.no, Gm) : na);
+        const float2 dpvx = __fmul2_rn(ndp, vx[r]), dpvy = __fmul2_rn(ndp, vy[r]);
+        if (r == 0) {
+            X[0] = dpvx;
+            X[1] = dpvy;
+            X[2] = __fmul2_rn(dpvx, vx[r]);
+            X[3] = __fmul2_rn(dpvx, vy[r]);
+            X[4] = __fmul2_rn(dpvy, vy[r]);
+            X[5] = __fmul2_rn(Gm, dal);
+            X[6] = __fmul2_rn(nw, q.g0);
+            X[7] = __fmul2_rn(nw, q.g1);
+            X[8] = __fmul2_rn(nw, q.g2);
+        } else {
+            X[0] = __fadd2_rn(X[0], dpvx);
+            X[1] = __fadd2_rn(X[1], dpvy);
+            X[2] = __ffma2_rn(dpvx, vx[r], X[2]);
+            X[3] = __ffma2_rn(dpvx, vy[r], X[3]);
+            X[4] = __ffma2_rn(dpvy, vy[r], X[4]);
+            X[5] = __ffma2_rn(Gm, dal, X[5]);
+            X[6] = __ffma2_rn(nw, q.g0, X[6]);
+            X[7] = __ffma2_rn(nw, q.g1, X[7]);
+            X[8] = __ffma2_rn(nw, q.g2, X[8]);
+        }
+    }
+    return contrib;
+}
+
+// One half (0: rows 0-7, 1: rows 8-15) of a tile by one warp.
+__device__ __forceinline__ void render_bwd_half(const BwdArgs &a, uint32_t gtile, int half, const CamTile &C,
+                                                BwdStage &S) {
     const uint32_t lt = gtile - C.tile_base;
-    const uint32_t *vals = a.vals + C.vals_base;
     const int tx = (int)(lt % (uint32_t)C.tiles_x), ty = (int)(lt / (uint32_t)C.tiles_x);
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int lane = threadIdx.x & 31;
     const int px = tx * kTile + (lane & (kTile - 1));
-    const int py_first = ty * kTile + (tid >> 5) * 8 + (lane >> kTileShift);
+    const int py_first = ty * kTile + half * 8 + (lane >> kTileShift);
     const float2 npx = f2(-(float)px, -(float)px);
+    const float x0 = (float)(tx * kTile), y0 = (float)(ty * kTile + half * 8);
     const size_t plane = (size_t)C.W * C.H;
     const float *dl = a.dL_dimg + 3 * C.pix_base;
 
     BwdPair P[2];
     int mylast = 0;
 #pragma unroll
-    for (int h = 0; h < kBwdPix; ++h) {
+    for (int h = 0; h < 4; ++h) {
         const int py = py_first + 2 * h;
         float T = 0.f, g0 = 0.f, g1 = 0.f, g2 = 0.f;
         int last = 0;
@@ -157,174 +229,139 @@ __device__ __forceinline__ void render_bwd_tile(const BwdArgs &a, uint32_t gtile
         const float nS2 = -(g0 * (T * a.bg[0]) + g1 * (T * a.bg[1]) + g2 * (T * a.bg[2]));
         BwdPair &q = P[h >> 1];
         if (h & 1) {
-            q.T.y = T, q.nS2.y = nS2, q.g0.y = g0, q.g1.y = g1, q.g2.y = g2, q.npy.y = -(float)py, q.last1 = last;
+            q.T.y = T, q.nS2.y = nS2, q.g0.y = g0, q.g1.y = g1, q.g2.y = g2, q.last1 = last;
         } else {
-            q.T.x = T, q.nS2.x = nS2, q.g0.x = g0, q.g1.x = g1, q.g2.x = g2, q.npy.x = -(float)py, q.last0 = last;
+            q.T.x = T, q.nS2.x = nS2, q.g0.x = g0, q.g1.x = g1, q.g2.x = g2, q.last0 = last;
         }
         mylast = max(mylast, last);
     }
-    if (tid == 0) *S.maxlast = 0;
-    __syncthreads();
-    if (mylast > 0) atomicMax(S.maxlast, mylast);
-    __syncthreads();
-    const int maxlast = *S.maxlast;
-    const uint32_t rstart = a.ranges[gtile].x;
-    const float2 one = f2(1.f, 1.f), two = f2(2.f, 2.f);
+    const int maxlast = __reduce_max_sync(0xffffffffu, mylast);
+    if (maxlast == 0) return;
+    const uint32_t *vals = a.vals + C.vals_base + a.ranges[gtile].x;
+    const StageSource src{a.xy, a.shape, a.conic_o, a.rgbd};
+    // lane l takes position end - 1 - l of the 32 entries before `end`, so the
+    // staged entries run from the back to the front
+    uint32_t rec = 0u, vnext = 0u;
+    if (lane < maxlast) {
+        rec = C.rec_base + vals[maxlast - 1 - lane];
+        stage_copy(S.in, src, rec, lane);
+    }
+    if (lane + 32 < maxlast) vnext = vals[maxlast - 33 - lane];
+    int waiting = 0;  // entries in S.red
 
-    for (int end = maxlast; end > 0; end -= kBwdBatch) {
-        const int cnt = min(kBwdBatch, end);
-        const int start = end - cnt;
-        __syncthreads();
-        for (int k = tid; k < cnt; k += kBwdThreads) {
-            const uint32_t g = C.rec_base + vals[rstart + start + k];
-            S.id[k] = g;
-            const float2 m = a.xy[g];
-            const float4 co = a.conic_o[g];
-            const float4 rgb = a.rgbd[g];
-            const float2 sh = a.shape[g];
-            const float ca = -0.5f * co.x, cb = -co.y, cc = -0.5f * co.z;
-            S.s0[k] = make_float4(m.x, m.x, m.y, m.y);
-            S.s1[k] = make_float4(ca, ca, cb, cb);
-            S.s2[k] = make_float4(cc, cc, skip_threshold(co.w), sh.y != 0.f ? 1.f : 0.f);
-            S.s3[k] = make_float4(rgb.x, rgb.x, rgb.y, rgb.y);
-            S.s4[k] = make_float4(rgb.z, rgb.z, co.w, co.w);
-            if (sh.y != 0.f) S.s5[k] = make_float4(sh.x, sh.x, sh.y, sh.y);  // read for elongated entries only
+    for (int end = maxlast; end > 0; end -= 32) {
+        copy_wait();
+        const int cnt = stage_entries<true>(S.in, lane < end, end - lane, x0, y0, lane, rec, S.ids);
+        if (lane + 32 < end) {
+            rec = C.rec_base + vnext;
+            stage_copy(S.in, src, rec, lane);
+            if (lane + 64 < end) vnext = vals[end - 65 - lane];
         }
-        __syncthreads();
-        for (int j = cnt - 1; j >= 0; --j) {
-            const int p = start + j;
-            const float4 X = S.s0[j], Q = S.s1[j], K = S.s2[j];
-            const float2 dx = __fadd2_rn(f2(X.x, X.y), npx);
-            const float2 cadx = __fmul2_rn(f2(Q.x, Q.y), dx);
-            const float2 A = __fmul2_rn(cadx, dx);
-            const float2 B = __fmul2_rn(f2(Q.z, Q.w), dx);
-            const float2 cc2 = f2(K.x, K.y);
-            const bool elong = K.w != 0.f;  // the same for the whole warp
-            float2 dy[2], pw[2], cau[2];
-            float4 E;
-            if (!elong) {
+        // pixels whose last contributor lies before these entries stay out
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int py = py_first + 4 * r;
+            P[r].npy = f2(P[r].last0 > end - 32 ? -(float)py : kFar, P[r].last1 > end - 32 ? -(float)(py + 2) : kFar);
+        }
+        __syncwarp();
+        for (int j = 0; j < cnt; ++j) {
+            const float4 X4 = S.in.sx[j], Q = S.in.sq[j], K = S.in.sk[j];
+            const uint32_t info = __float_as_uint(K.w);
+            BwdEntry E;
+            E.dx = __fadd2_rn(f2(X4.x, X4.y), npx);
+            const float2 ca = f2(Q.x, Q.y), cc = f2(K.x, K.y);
+            float2 dy[2], pw[2], vx[2], vy[2];
+            if (!(info & kLongEntry)) {
+                const float2 cadx = __fmul2_rn(ca, E.dx);
+                const float2 A = __fmul2_rn(cadx, E.dx);
+                E.cb = f2(Q.z, Q.w);
+                E.B = __fmul2_rn(E.cb, E.dx);
+                E.cadx2 = __fadd2_rn(cadx, cadx);
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
-                    dy[r] = __fadd2_rn(f2(X.z, X.w), P[r].npy);
-                    pw[r] = __ffma2_rn(dy[r], __ffma2_rn(cc2, dy[r], B), A);
+                    dy[r] = __fadd2_rn(f2(X4.z, X4.w), P[r].npy);
+                    pw[r] = __ffma2_rn(dy[r], __ffma2_rn(cc, dy[r], E.B), A);
                 }
             } else {
                 // the forward's exact power form (the same operations)
-                E = S.s5[j];
+                const float4 L = S.in.se[j];
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
-                    dy[r] = __fadd2_rn(f2(X.z, X.w), P[r].npy);
-                    const float2 u = __ffma2_rn(f2(E.x, E.y), dy[r], dx);
-                    cau[r] = __fmul2_rn(f2(Q.x, Q.y), u);
-                    pw[r] = __ffma2_rn(cau[r], u, __fmul2_rn(__fmul2_rn(f2(E.z, E.w), dy[r]), dy[r]));
+                    dy[r] = __fadd2_rn(f2(X4.z, X4.w), P[r].npy);
+                    const float2 u = __ffma2_rn(f2(L.x, L.y), dy[r], E.dx);
+                    vx[r] = __fmul2_rn(ca, u);
+                    pw[r] = __ffma2_rn(vx[r], u, __fmul2_rn(__fmul2_rn(f2(L.z, L.w), dy[r]), dy[r]));
                 }
             }
-            bool e[4];
+            // the forward's power test
+            const bool any = fmaxf(fmaxf(pw[0].x, pw[0].y), fmaxf(pw[1].x, pw[1].y)) >= K.z;
+            if (!__any_sync(0xffffffffu, any)) continue;
+            // v = -dpower/dmu: (2 ca dx + cb dy, cb dx + 2 cc dy), or in the
+            // exact form (2 ca u, 2 ca u rr + 2 ce dy), which does not cancel
+            if (!(info & kLongEntry)) {
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                // the forward's test: power >= skip (a positive power is a
-                // rounding of 0, kept)
-                e[2 * r] = p < P[r].last0 && pw[r].x >= K.z;
-                e[2 * r + 1] = p < P[r].last1 && pw[r].y >= K.z;
-            }
-            if (!__any_sync(0xffffffffu, e[0] || e[1] || e[2] || e[3])) continue;
-            const float4 C1 = S.s3[j], C2 = S.s4[j];
-            const float2 o2 = f2(C2.z, C2.w);
-            float2 X0, X1, X2, X3, X4, X5, X6, X7, X8;
-            bool contrib = false;
+                for (int r = 0; r < 2; ++r) {
+                    vx[r] = __ffma2_rn(E.cb, dy[r], E.cadx2);
+                    vy[r] = __ffma2_rn(f2(2.f, 2.f), __fmul2_rn(cc, dy[r]), E.B);
+                }
+            } else {
+                const float4 L = S.in.se[j];
+                const float2 ce2 = f2(L.z + L.z, L.w + L.w);
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                BwdPair &q = P[r];
-                const float2 G = f2(__expf(pw[r].x), __expf(pw[r].y));
-                const float2 oG = __fmul2_rn(o2, G);
-                const float al0 = fminf(kAlphaMax, oG.x), al1 = fminf(kAlphaMax, oG.y);
-                const bool c0 = e[2 * r] && al0 >= kAlphaMin, c1 = e[2 * r + 1] && al1 >= kAlphaMin;
-                contrib = contrib || c0 || c1;
-                const float2 na = f2(c0 ? -al0 : 0.f, c1 ? -al1 : 0.f);
-                const float2 om = __fadd2_rn(one, na);  // 1 - alpha (1 where not composited)
-                const float2 inv = f2(c0 ? __fdividef(1.f, om.x) : 1.f, c1 ? __fdividef(1.f, om.y) : 1.f);
-                q.T = __fmul2_rn(q.T, inv);
-                const float2 nw = __fmul2_rn(na, q.T);  // -alpha T
-                const float2 S1 = __ffma2_rn(q.g0, f2(C1.x, C1.y),
-                                             __ffma2_rn(q.g1, f2(C1.z, C1.w), __fmul2_rn(q.g2, f2(C2.x, C2.y))));
-                const float2 dal = __ffma2_rn(inv, q.nS2, __fmul2_rn(q.T, S1));
-                q.nS2 = __ffma2_rn(nw, S1, q.nS2);
-                // derivative through o G where the cap does not bind
-                const float2 Gm = f2(c0 && oG.x < kAlphaMax ? G.x : 0.f, c1 && oG.y < kAlphaMax ? G.y : 0.f);
-                const float2 dp = __fmul2_rn(dal, __fmul2_rn(o2, Gm));
-                // dpower/dmu: (2 ca dx + cb dy, cb dx + 2 cc dy), or in the
-                // exact form (2 ca u, 2 ca u rr + 2 ce dy), which does not cancel
-                float2 vx, vy;
-                if (!elong) {
-                    vx = __ffma2_rn(f2(Q.z, Q.w), dy[r], __fmul2_rn(two, cadx));
-                    vy = __ffma2_rn(two, __fmul2_rn(cc2, dy[r]), B);
-                } else {
-                    vx = __fmul2_rn(two, cau[r]);
-                    vy = __ffma2_rn(__fmul2_rn(two, cau[r]), f2(E.x, E.y), __fmul2_rn(two, __fmul2_rn(f2(E.z, E.w), dy[r])));
-                }
-                const float2 dpvx = __fmul2_rn(dp, vx), dpvy = __fmul2_rn(dp, vy);
-                if (r == 0) {
-                    X0 = dpvx;
-                    X1 = dpvy;
-                    X2 = __fmul2_rn(dpvx, vx);
-                    X3 = __fmul2_rn(dpvx, vy);
-                    X4 = __fmul2_rn(dpvy, vy);
-                    X5 = __fmul2_rn(Gm, dal);
-                    X6 = __fmul2_rn(nw, q.g0);
-                    X7 = __fmul2_rn(nw, q.g1);
-                    X8 = __fmul2_rn(nw, q.g2);
-                } else {
-                    X0 = __fadd2_rn(X0, dpvx);
-                    X1 = __fadd2_rn(X1, dpvy);
-                    X2 = __ffma2_rn(dpvx, vx, X2);
-                    X3 = __ffma2_rn(dpvx, vy, X3);
-                    X4 = __ffma2_rn(dpvy, vy, X4);
-                    X5 = __ffma2_rn(Gm, dal, X5);
-                    X6 = __ffma2_rn(nw, q.g0, X6);
-                    X7 = __ffma2_rn(nw, q.g1, X7);
-                    X8 = __ffma2_rn(nw, q.g2, X8);
+                for (int r = 0; r < 2; ++r) {
+                    vx[r] = __fadd2_rn(vx[r], vx[r]);
+                    vy[r] = __ffma2_rn(vx[r], f2(L.x, L.y), __fmul2_rn(ce2, dy[r]));
                 }
             }
-            if (__ballot_sync(0xffffffffu, contrib)) {
-                const float gv[9] = {X0.x + X0.y, X1.x + X1.y, 0.5f * (X2.x + X2.y), X3.x + X3.y,
-                                     0.5f * (X4.x + X4.y), X5.x + X5.y, -(X6.x + X6.y), -(X7.x + X7.y),
-                                     -(X8.x + X8.y)};
-                warp_reduce9_add(gv, a.g_screen + (size_t)S.id[j] * 9, lane);
+            const float4 C1 = S.in.s1[j], C2 = S.in.s2[j];
+            E.no = f2(C1.x, C1.y), E.cr = f2(C1.z, C1.w), E.cg = f2(C2.x, C2.y), E.cbl = f2(C2.z, C2.w);
+            float2 X[9];
+            bool contrib;
+            if (!(info & kSlowEntry)) contrib = bwd_entry<false>(P, pw, vx, vy, E, (int)info, X);
+            else contrib = bwd_entry<true>(P, pw, vx, vy, E, (int)(info & ~(kSlowEntry | kLongEntry)), X);
+            if (__any_sync(0xffffffffu, contrib)) {
+                float *row = S.red + 9 * waiting * kRedStride + lane;
+#pragma unroll
+                for (int i = 0; i < 9; ++i) row[i * kRedStride] = X[i].x + X[i].y;
+                if (lane == 0) S.red_id[waiting] = S.ids[j];
+                if (++waiting == kRedEntries) {
+                    bwd_flush(S, waiting, a.g_screen, lane);
+                    waiting = 0;
+                }
             }
         }
     }
+    if (waiting > 0) bwd_flush(S, waiting, a.g_screen, lane);
+    copy_wait();
+    __syncwarp();
 }
 
 // One block per tile; with an order, the heaviest tiles first (as the forward).
 __global__ void __launch_bounds__(kBwdThreads) render_bwd_kernel(BwdArgs a) {
-    __shared__ uint32_t s_id[kBwdBatch];
-    __shared__ float4 s_st[6][kBwdBatch];
-    __shared__ int s_maxlast;
-    const BwdStage S{s_id, s_st[0], s_st[1], s_st[2], s_st[3], s_st[4], s_st[5], &s_maxlast};
+    __shared__ __align__(16) BwdStage s_stage[2];
+    const int wid = threadIdx.x >> 5;
     const uint32_t t = a.order.cnt ? order_pick(a.order, a.ts.total_tiles, blockIdx.x) : (uint32_t)blockIdx.x;
-    render_bwd_tile(a, t, a.ts.cam[0], S);
+    render_bwd_half(a, t, wid, a.ts.cam[0], s_stage[wid]);
 }
 
-__global__ void __launch_bounds__(kBwdThreads) render_bwd_persistent_kernel(BwdArgs a) {
-    __shared__ uint32_t s_id[kBwdBatch];
-    __shared__ float4 s_st[6][kBwdBatch];
-    __shared__ int s_maxlast;
-    __shared__ uint32_t s_next;
-    const BwdStage S{s_id, s_st[0], s_st[1], s_st[2], s_st[3], s_st[4], s_st[5], &s_maxlast};
+// Persistent warps take the halves of tiles_per_fetch consecutive tiles at a
+// time from a global counter over the tiles of all cameras in the set.  (At
+// most 104 registers: unbounded the compiler takes 112, nine blocks per SM
+// instead of ten, 4 % slower.)
+__global__ void __maxnreg__(104) render_bwd_persistent_kernel(BwdArgs a) {
+    __shared__ __align__(16) BwdStage s_stage[2];
+    BwdStage &S = s_stage[threadIdx.x >> 5];
+    const uint32_t halves = 2u * a.ts.total_tiles, take = 2u * (uint32_t)a.tiles_per_fetch;
     for (;;) {
-        if (threadIdx.x == 0) s_next = atomicAdd(a.queue, (uint32_t)a.tiles_per_fetch);
-        __syncthreads();
-        const uint32_t t0 = s_next;
-        __syncthreads();
-        if (t0 >= a.ts.total_tiles) break;
-        const uint32_t t1 = min(t0 + (uint32_t)a.tiles_per_fetch, a.ts.total_tiles);
-        for (uint32_t t = t0; t < t1; ++t) {
-            if (a.cam_table) {
-                const CamTile C = a.cam_table[camera_in_table(a.cam_table, a.ts.n_cams, t)];
-                render_bwd_tile(a, t, C, S);
-            } else {
-                render_bwd_tile(a, t, a.ts.cam[camera_of(a.ts, t)], S);
-            }
+        uint32_t h0 = 0;
+        if ((threadIdx.x & 31) == 0) h0 = atomicAdd(a.queue, take);
+        h0 = __shfl_sync(0xffffffffu, h0, 0);
+        if (h0 >= halves) break;
+        const uint32_t h1 = min(h0 + take, halves);
+        for (uint32_t h = h0; h < h1; ++h) {
+            const uint32_t t = h >> 1;
+            const CamTile C = a.cam_table[camera_in_table(a.cam_table, a.ts.n_cams, t)];
+            render_bwd_half(a, t, (int)(h & 1u), C, S);
         }
     }
 }

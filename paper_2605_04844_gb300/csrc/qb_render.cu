@@ -32,54 +32,12 @@
 // Measured slower: 64 registers (32 warps per SM, spills), two entries'
 // exponents ahead of both blends, the next entry's operands loaded ahead
 // (+21 %), T chosen by a select instead of multiplied by 1 - 0.
-#include "qb_kernels.cuh"
+#include "qb_stage.cuh"
 
 namespace qb {
 
 constexpr int kRenderThreads = 64;  // a block of the single-frame kernel: the two halves of a tile
-constexpr float kCapTest = 0.98f;    // opacities above this may meet the 0.99 cap
-#define kNaN __int_as_float(0x7fc00000)
 constexpr int kRenderPairs = 2;     // packed pixel pairs per thread
-
-// A warp's shared memory.  raw: one entry's record per lane, the target of
-// the asynchronous copies, read back by the same lane.  The others hold the
-// compacted entries laid out for the packed FP32x2 arithmetic of sm_100+:
-// every operand the two pixels of a pair share is stored twice, so a pair
-// register loads it without a move.
-//   sx = (mu_x, mu_x, mu_y, mu_y), sq = (ca, ca, cb, cb),
-//   sk = (cc, cc, skip threshold, info), s1 = (o, o, r, r), s2 = (g, g, b, b),
-//   se = (rr, rr, ce, ce) (elongated entries only).
-// info is the entry's position in the list + 1, with kSlowEntry set where the
-// entry may meet the 0.99 cap or is elongated (qb_internal.cuh), kLongEntry
-// for the latter: then its exponent is ca u^2 + ce dy^2 with
-// u = dx + rr dy, rr = b / a, ce = -1 / (2 Sigma22), which does not cancel.
-constexpr uint32_t kSlowEntry = 0x80000000u, kLongEntry = 0x40000000u;  // positions are below 2^30
-struct RenderStage {
-    float4 raw_co[32], raw_rgb[32];
-    float2 raw_xy[32], raw_sh[32];
-    float4 sx[32], sq[32], sk[32], s1[32], s2[32], se[32];
-};
-
-__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-
-__device__ __forceinline__ void copy_async16(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
-__device__ __forceinline__ void copy_async8(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
-__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// min(a, b), NaN where either is
-__device__ __forceinline__ float min_nan(float a, float b) {
-    float r;
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
 
 // The compositing state of one packed pair of pixels.  A pixel outside the
 // image, or one that has stopped, carries a NaN row npy: its exponent and its
@@ -144,7 +102,6 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
     const uint32_t lt = gtile - C.tile_base;
     const int tx = (int)(lt % (uint32_t)C.tiles_x), ty = (int)(lt / (uint32_t)C.tiles_x);
     const int lane = threadIdx.x & 31;
-    const uint32_t below = (1u << lane) - 1u;
     const int px = tx * kTile + (lane & (kTile - 1));
     const int pyb = ty * kTile + half * 8 + (lane >> kTileShift);
     const float2 npx = f2(-(float)px, -(float)px);
@@ -167,51 +124,19 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
     const uint2 range = a.ranges[gtile];
     const int total = (int)(range.y - range.x);
     const uint32_t *vals = a.vals + C.vals_base + range.x;
-    auto fetch = [&](uint32_t v) {  // the lane's record of the next 32 entries
-        const uint32_t g = C.rec_base + v;
-        copy_async16(&S.raw_co[lane], a.conic_o + g);
-        copy_async16(&S.raw_rgb[lane], a.rgbd + g);
-        copy_async8(&S.raw_xy[lane], a.xy + g);
-        copy_async8(&S.raw_sh[lane], a.shape + g);
-    };
+    const StageSource src{a.xy, a.shape, a.conic_o, a.rgbd};
     uint32_t npass = 0;  // COUNT only
-    if (lane < total) fetch(vals[lane]);
+    if (lane < total) stage_copy(S, src, C.rec_base + vals[lane], lane);
     uint32_t vnext = 32 + lane < total ? vals[32 + lane] : 0u;
 
     for (int base = 0; base < total; base += 32) {
         copy_wait();
-        bool hit = false;
-        float2 m = f2(0.f, 0.f), sh = f2(0.f, 0.f);
-        float4 co = make_float4(0.f, 0.f, 0.f, 0.f), rgb = co;
-        float skip = 0.f;
-        if (base + lane < total) {
-            m = S.raw_xy[lane];
-            sh = S.raw_sh[lane];
-            co = S.raw_co[lane];
-            rgb = S.raw_rgb[lane];
-            skip = skip_threshold(co.w);
-            hit = ellipse_meets_rect(m.x, m.y, co.x, co.y, co.z, skip, sh.y != 0.f, x0, y0, x0 + 15.f, y0 + 7.f);
-        }
-        const uint32_t hits = __ballot_sync(0xffffffffu, hit);  // also: the walk of the last entries is over
-        if (hit) {
-            const int k = __popc(hits & below);
-            const float ca = -0.5f * co.x, cbv = -co.y, cc = -0.5f * co.z;
-            uint32_t info = (uint32_t)(base + lane + 1);
-            if (co.w > kCapTest) info |= kSlowEntry;
-            if (sh.y != 0.f) info |= kSlowEntry | kLongEntry;
-            S.sx[k] = make_float4(m.x, m.x, m.y, m.y);
-            S.sq[k] = make_float4(ca, ca, cbv, cbv);
-            S.sk[k] = make_float4(cc, cc, skip, __uint_as_float(info));
-            S.s1[k] = make_float4(co.w, co.w, rgb.x, rgb.x);
-            S.s2[k] = make_float4(rgb.y, rgb.y, rgb.z, rgb.z);
-            if (sh.y != 0.f) S.se[k] = make_float4(sh.x, sh.x, sh.y, sh.y);
-        }
+        const int cnt = stage_entries<false>(S, base + lane < total, base + lane + 1, x0, y0, lane);
         if (base + 32 + lane < total) {
-            fetch(vnext);
+            stage_copy(S, src, C.rec_base + vnext, lane);
             vnext = base + 64 + lane < total ? vals[base + 64 + lane] : 0u;
         }
         __syncwarp();
-        const int cnt = __popc(hits);
 #pragma unroll 2
         for (int j = 0; j < cnt; ++j) {
             const float4 X = S.sx[j], Q = S.sq[j], K = S.sk[j];
