@@ -31,16 +31,62 @@ __global__ void __launch_bounds__(256) l1_grad_kernel(const float *__restrict__ 
 
 // Adam, step t (1-based): m = b1 m + (1 - b1) g; v = b2 v + (1 - b2) g^2;
 // p -= lr * (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + eps).
+// One pass over seven arrays' worth of traffic, bound by memory: with VEC
+// (16-byte aligned arrays) a thread has four 16-byte loads of two groups of four
+// parameters in flight, instead of four 4-byte ones.  500k Gaussians of SH
+// degree 3 (five launches, 826 MB): 195 -> 160 us with the launches' gaps.
+__device__ __forceinline__ void adam_one(float &p, float g, float &m, float &v, float lr, float b1, float b2, float eps,
+                                         float c1, float c2) {
+    const float mi = fmaf(b1, m, (1.f - b1) * g);
+    const float vi = fmaf(b2, v, (1.f - b2) * g * g);
+    m = mi;
+    v = vi;
+    p -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
+template <bool VEC>
 __global__ void __launch_bounds__(256) adam_kernel(float *__restrict__ p, const float *__restrict__ g,
                                                    float *__restrict__ m, float *__restrict__ v, uint64_t n, float lr,
                                                    float b1, float b2, float eps, float c1, float c2) {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
-        const float vi = fmaf(b2, v[i], (1.f - b2) * gi * gi);
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, threads = (uint64_t)gridDim.x * blockDim.x;
+    uint64_t i0 = 0;
+    if constexpr (VEC) {
+        const uint64_t n4 = n / 4;
+        constexpr int U = 2;
+        for (uint64_t j = t; j < n4; j += U * threads) {
+            float4 P[U], G[U], M[U], V[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint64_t k = j + u * threads;
+                if (k < n4) {
+                    P[u] = reinterpret_cast<const float4 *>(p)[k];
+                    G[u] = reinterpret_cast<const float4 *>(g)[k];
+                    M[u] = reinterpret_cast<const float4 *>(m)[k];
+                    V[u] = reinterpret_cast<const float4 *>(v)[k];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint64_t k = j + u * threads;
+                if (k < n4) {
+                    adam_one(P[u].x, G[u].x, M[u].x, V[u].x, lr, b1, b2, eps, c1, c2);
+                    adam_one(P[u].y, G[u].y, M[u].y, V[u].y, lr, b1, b2, eps, c1, c2);
+                    adam_one(P[u].z, G[u].z, M[u].z, V[u].z, lr, b1, b2, eps, c1, c2);
+                    adam_one(P[u].w, G[u].w, M[u].w, V[u].w, lr, b1, b2, eps, c1, c2);
+                    reinterpret_cast<float4 *>(p)[k] = P[u];
+                    reinterpret_cast<float4 *>(m)[k] = M[u];
+                    reinterpret_cast<float4 *>(v)[k] = V[u];
+                }
+            }
+        }
+        i0 = 4 * n4;  // at most three are left
+    }
+    for (uint64_t i = i0 + t; i < n; i += threads) {
+        float pi = p[i], mi = m[i], vi = v[i];
+        adam_one(pi, g[i], mi, vi, lr, b1, b2, eps, c1, c2);
+        p[i] = pi;
         m[i] = mi;
         v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     }
 }
 
@@ -63,7 +109,11 @@ cudaError_t launch_adam(float *p, const float *g, float *m, float *v, uint64_t n
                         float eps, int t, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-    note_launch("adam_kernel", s), adam_kernel<<<grid_for(n), 256, 0, s>>>(p, g, m, v, n, lr, b1, b2, eps, c1, c2);
+    const bool vec = ((reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(g) | reinterpret_cast<uintptr_t>(m) |
+                       reinterpret_cast<uintptr_t>(v)) & 15) == 0;
+    note_launch("adam_kernel", s);
+    if (vec) adam_kernel<true><<<grid_for((n + 7) / 8), 256, 0, s>>>(p, g, m, v, n, lr, b1, b2, eps, c1, c2);
+    else adam_kernel<false><<<grid_for(n), 256, 0, s>>>(p, g, m, v, n, lr, b1, b2, eps, c1, c2);
     return cudaGetLastError();
 }
 
