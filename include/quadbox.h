@@ -157,7 +157,8 @@ typedef struct {
     float *box;         /* [n][4]  (x_max, y_max, f x_max, f y_max)         */
     float *r3;          /* [n]     3-sigma radius ceil(3 sqrt(lambda_max))  */
     int32_t *meta;      /* [n]     bit0 visible, bit1 orient (Sigma12 >= 0),
-                                   bits2-4 colour channel clamped at 0      */
+                                   bits2-4 colour channel clamped at 0,
+                                   bit5 a colour channel not finite         */
     uint32_t *counts;   /* [n]     tiles per Gaussian                       */
     uint32_t *offsets;  /* [n]     exclusive prefix of counts in emission order
                                    (index order, or depth order in DEPTH_FIRST) */

@@ -26,6 +26,7 @@ constexpr int kMaxPasses = 8;              // ceil(64 / 8)
 constexpr int kMetaVisible = 1;
 constexpr int kMetaOrient = 2;
 constexpr int kMetaClampShift = 2;
+constexpr int kMetaNonFinite = 32;  // a colour channel is infinite or NaN
 
 struct CamDev {
     float V[12];  // rows 0..2 of the world->view matrix

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(256, 3) preprocess_kernel(PreArgs a) {
         }
     }
     int meta = kMetaVisible | (bt.orient ? kMetaOrient : 0);
+    if (!isfinite(rgb[0]) || !isfinite(rgb[1]) || !isfinite(rgb[2])) meta |= kMetaNonFinite;
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) {
         if (rgb[ch] < 0.f) {
