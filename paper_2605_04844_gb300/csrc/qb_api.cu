@@ -87,7 +87,7 @@ bool make_layout(int n, int W, int H, uint64_t cap, Layout &L) {
     L.ranges = take(8 * (size_t)tiles);
     const int ncells = cell_geo(W, H, 8).ncells;
     L.cell_zero = take(4 * cell_zero_words(ncells));
-    L.cell_start = take(4 * ((size_t)ncells + 1));
+    L.cell_start = take(4 * ((size_t)ncells + 2));
     L.row_start = take(4 * ((size_t)ncells + 1));
     L.row_cell = take(4 * cell_rows_max(cap, ncells));
     L.row_counts = take(128 * cell_rows_max(cap, ncells));

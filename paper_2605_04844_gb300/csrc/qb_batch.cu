@@ -140,7 +140,7 @@ bool make_blayout(int n, int n_cams, int group, uint64_t cap, const Geo &g, BLay
     L.sort = take(sb);
     L.n_cells = take(8);
     L.cell_zero = take(4 * cell_zero_words(g.max_cells));
-    L.cell_start = take(4 * ((size_t)g.max_cells + 1));
+    L.cell_start = take(4 * ((size_t)g.max_cells + 2));
     L.row_start = take(4 * ((size_t)g.max_cells + 1));
     L.row_cell = take(4 * cell_rows_max(cap, g.max_cells));
     L.row_counts = take(128 * cell_rows_max(cap, g.max_cells));

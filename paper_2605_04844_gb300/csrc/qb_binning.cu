@@ -25,9 +25,9 @@ constexpr int kScanChunk = kScanBlock * kScanItems;
 // j-th Gaussian in depth order; offsets gets the tiles' exclusive prefix,
 // coff the cells'.  Otherwise entry j is counts[j], offsets its prefix and
 // coff the count itself (the emit reads it in order).  chunk_first[c] becomes
-// the position whose outputs (cells or pairs) hold output c kEmitStride, so
-// the emit's warps find their first Gaussian with one load instead of a
-// search.  The last block writes P, and for DUAL the number of cell entries,
+// the position whose outputs (cell entries or pairs) hold output c
+// kEmitStride, so the emit's warps find their first Gaussian with one load
+// instead of a search.  The last block writes P, and for DUAL the number of cell entries,
 // 0 when P exceeds the capacity (then nothing downstream writes).
 //
 // Status of a block: two 64-bit words stored and loaded as one 128-bit word,
@@ -35,7 +35,9 @@ constexpr int kScanChunk = kScanBlock * kScanItems;
 // 62-bit count; the first word's flag holds for both.
 //
 // The kernel is bound by latency (gathers, look-back): 8 entries per thread
-// instead of 16 give twice the blocks.
+// instead of 16 give twice the blocks, and all resident blocks reach their
+// look-back at about the same time, so it reads 256 words at once instead of
+// 32 (a chain of two or three loads where there were up to a dozen).
 constexpr uint64_t kScanAgg = 1ull << 63, kScanIncl = 1ull << 62, kScanCount = kScanIncl - 1;
 
 struct ScanWord {
@@ -72,10 +74,10 @@ struct ScanArgs {
 };
 
 template <bool DUAL>
-__global__ void __launch_bounds__(kScanBlock) scan_onepass_kernel(ScanArgs A) {
-    __shared__ uint32_t s_block;
-    __shared__ uint64_t s_prefix[2];
-    const int tid = threadIdx.x, lane = tid & 31;
+__global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A) {
+    __shared__ uint32_t s_block, s_ready[kScanBlock / 32], s_incl[kScanBlock / 32];
+    __shared__ uint64_t s_sum[kScanBlock / 32], s_sumd[kScanBlock / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) s_block = atomicAdd(A.counter, 1u);
     __syncthreads();
     const uint32_t b = s_block;
@@ -117,80 +119,79 @@ __global__ void __launch_bounds__(kScanBlock) scan_onepass_kernel(ScanArgs A) {
     uint64_t ctot, dtot = 0, cincl, dincl = 0;
     cincl = block_incl_scan<uint64_t>(csum, &ctot);
     if (DUAL) dincl = block_incl_scan<uint64_t>(dsum, &dtot);
-    // publish, then look back (warp 0, 32 earlier blocks per step)
+    // Publish, then look back over 256 earlier blocks per step: thread k reads
+    // the word of block t - k, and the sums of those before the first word not
+    // yet published are added, up to and including the first inclusive word,
+    // which ends the walk.  (Before block 0 reads as an inclusive zero.)
     if (tid == 0) st_status(A.status + b, ScanWord{(b == 0 ? kScanIncl : kScanAgg) | ctot, dtot});
-    if (tid < 32) {
-        // The words of blocks t, t - 1, ..., t - 31 are read together; the
-        // sums of the lanes before the first word not yet published are
-        // added, up to and including the first inclusive word, which ends the
-        // walk.  (Before block 0 reads as an inclusive zero.)
-        uint64_t acc = 0, accd = 0;
-        int64_t t = (int64_t)b - 1;
-        int spins = 0;
-        while (t >= 0) {
-            const int64_t mine = t - lane;
-            const ScanWord w = mine >= 0 ? ld_status(A.status + mine) : ScanWord{kScanIncl, 0};
-            const uint32_t ready = __ballot_sync(0xffffffffu, (w.a & (kScanAgg | kScanIncl)) != 0);
-            const uint32_t inclm = __ballot_sync(0xffffffffu, (w.a & kScanIncl) != 0);
-            const int first_unready = ready == 0xffffffffu ? 32 : __ffs(~ready) - 1;
-            const int first_incl = inclm ? __ffs(inclm) - 1 : 32;
-            const bool ends = first_incl < first_unready;
-            const int used = ends ? first_incl + 1 : first_unready;
-            uint64_t v = lane < used ? (w.a & kScanCount) : 0ull, u = lane < used ? w.b : 0ull;
+    uint64_t acc = 0, accd = 0;
+    int spins = 0;
+    for (int64_t t = (int64_t)b - 1; t >= 0;) {
+        const int64_t mine = t - tid;
+        const ScanWord w = mine >= 0 ? ld_status(A.status + mine) : ScanWord{kScanIncl, 0};
+        const uint32_t ready = __ballot_sync(0xffffffffu, (w.a & (kScanAgg | kScanIncl)) != 0);
+        const uint32_t inclm = __ballot_sync(0xffffffffu, (w.a & kScanIncl) != 0);
+        if (lane == 0) s_ready[wid] = ready, s_incl[wid] = inclm;
+        __syncthreads();
+        int first_unready = kScanBlock, first_incl = kScanBlock;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (DUAL) u += __shfl_xor_sync(0xffffffffu, u, o);
-            }
-            acc += v;
-            accd += u;
-            if (ends) break;
-            if (used > 0) {
-                t -= used;
-                continue;
-            }
-            // the nearest earlier block has not published yet
+        for (int k = kScanBlock / 32 - 1; k >= 0; --k) {
+            if (~s_ready[k]) first_unready = 32 * k + __ffs(~s_ready[k]) - 1;
+            if (s_incl[k]) first_incl = 32 * k + __ffs(s_incl[k]) - 1;
+        }
+        const bool ends = first_incl < first_unready;
+        const int used = ends ? first_incl + 1 : first_unready;
+        uint64_t v = tid < used ? (w.a & kScanCount) : 0ull, u = tid < used ? w.b : 0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (DUAL) u += __shfl_xor_sync(0xffffffffu, u, o);
+        }
+        if (lane == 0) s_sum[wid] = v, s_sumd[wid] = u;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kScanBlock / 32; ++k) acc += s_sum[k], accd += s_sumd[k];
+        if (ends) break;  // the same for the whole block
+        t -= used;
+        if (used == 0) {  // the nearest earlier block has not published yet
             if (++spins > kSpinLimit) {
-                if (lane == 0) atomicOr(A.err, kErrTimeout);
+                if (tid == 0) atomicOr(A.err, kErrTimeout);
                 break;
             }
             __nanosleep(64);
         }
-        if (lane == 0) {
-            if (b > 0) st_status(A.status + b, ScanWord{kScanIncl | ((acc + ctot) & kScanCount), accd + dtot});
-            s_prefix[0] = acc;
-            s_prefix[1] = accd;
-            if ((int)b == nb - 1) {
-                const uint64_t P = acc + ctot, E = accd + dtot;
-                *A.n_pairs = P;
-                // (E <= P: every cell of a Gaussian holds one of its tiles)
-                if (DUAL) *A.n_cells = P <= A.capacity && E <= A.capacity ? E : 0ull;
-            }
+    }
+    if (tid == 0) {
+        if (b > 0) st_status(A.status + b, ScanWord{kScanIncl | ((acc + ctot) & kScanCount), accd + dtot});
+        if ((int)b == nb - 1) {
+            const uint64_t P = acc + ctot, E = accd + dtot;
+            *A.n_pairs = P;
+            // (E <= P: cell_entries)
+            if (DUAL) *A.n_cells = P <= A.capacity && E <= A.capacity ? E : 0ull;
         }
     }
-    __syncthreads();
-    uint64_t run = s_prefix[0] + cincl - csum;
-    // outputs of the emit: cells (DUAL) or pairs
-    const uint64_t out0 = DUAL ? s_prefix[1] + dincl - dsum : run;
-    uint64_t r = out0;
+    uint64_t run = acc + cincl - csum;
+    {
+        uint64_t q = DUAL ? accd + dincl - dsum : run;  // outputs of the emit: cell entries or pairs
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        const uint32_t e = DUAL ? d[k] : c[k];
-        if (e > 0u) {
-            // the run [r, r + e) of this Gaussian holds these chunk starts
-            const uint64_t c0 = (r + kEmitStride - 1) / kEmitStride, c1 = (r + e - 1) / kEmitStride;
-            for (uint64_t ch = c0; ch <= c1 && ch < A.chunk_cap; ++ch) A.chunk_first[ch] = (uint32_t)(base + k);
+        for (int k = 0; k < kScanItems; ++k) {
+            const uint32_t e = DUAL ? d[k] : c[k];
+            if (e > 0u) {
+                // the run [q, q + e) of this Gaussian holds these chunk starts
+                const uint64_t c0 = (q + kEmitStride - 1) / kEmitStride, c1 = (q + e - 1) / kEmitStride;
+                for (uint64_t ch = c0; ch <= c1 && ch < A.chunk_cap; ++ch) A.chunk_first[ch] = (uint32_t)(base + k);
+            }
+            q += e;
         }
-        r += e;
     }
-    r = out0;
+    uint32_t r = (uint32_t)(accd + dincl - dsum);
     if (whole) {
         uint32_t o[kScanItems], p[kScanItems];
 #pragma unroll
         for (int k = 0; k < kScanItems; ++k) {
             o[k] = (uint32_t)run;  // P <= 2^30 is checked before use
             run += c[k];
-            p[k] = DUAL ? (uint32_t)r : c[k];
+            p[k] = DUAL ? r : c[k];
             r += d[k];
         }
 #pragma unroll
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(kScanBlock) scan_onepass_kernel(ScanArgs A) {
         for (int k = 0; k < kScanItems; ++k) {
             if (base + k < (size_t)n) {
                 A.offsets[base + k] = (uint32_t)run;
-                A.coff[base + k] = DUAL ? (uint32_t)r : c[k];
+                A.coff[base + k] = DUAL ? r : c[k];
             }
             run += c[k];
             r += d[k];
@@ -249,13 +250,13 @@ cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint
                               uint64_t *partials, uint64_t *n_pairs, uint64_t *n_cells, uint64_t capacity,
                               uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s) {
     ScanArgs A{};
+    A.chunk_first = chunk_first;
+    A.chunk_cap = chunk_cap;
     A.cc = cc;
     A.perm = perm;
     A.n = n;
     A.offsets = offsets;
     A.coff = coff;
-    A.chunk_first = chunk_first;
-    A.chunk_cap = chunk_cap;
     A.n_pairs = n_pairs;
     A.n_cells = n_cells;
     A.capacity = capacity;

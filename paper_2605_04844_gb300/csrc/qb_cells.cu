@@ -30,9 +30,9 @@
 
 namespace qb {
 
-constexpr int kCellWarps = 8;             // warps per emit block
-constexpr uint32_t kCellChunk = 512;      // emitted entries per warp and step
-constexpr int kCellHistMax = 4096;        // cells a block's histogram holds in shared memory
+constexpr int kCellWarps = 8;          // warps per emit block
+constexpr uint32_t kCellChunk = 512;   // entries per warp and step
+constexpr int kCellHistMax = 4096;     // cells a block's histogram holds in shared memory
 static_assert(kCellChunk % kEmitStride == 0, "a warp's range starts on the scan's chunk table");
 
 CellGeo cell_geo(int W, int H, int digit_bits) {
@@ -44,7 +44,7 @@ CellGeo cell_geo(int W, int H, int digit_bits) {
     g.cells_y = (g.tiles_y + kCellY - 1) / kCellY;
     g.ncells = g.cells_x * g.cells_y;
     g.cell_bits = 0;
-    while ((1 << g.cell_bits) < g.ncells) ++g.cell_bits;
+    while ((1 << g.cell_bits) < g.ncells + 1) ++g.cell_bits;  // id ncells: entries without a tile
     g.digit_bits = digit_bits;
     g.passes = pass_geo(g.cell_bits, g.digit_bits);
     return g;
@@ -52,20 +52,9 @@ CellGeo cell_geo(int W, int H, int digit_bits) {
 
 size_t cell_sort_scratch_bytes(uint64_t pair_capacity, int ncells, int digit_bits) {
     int bits = 1;
-    while ((1 << bits) < ncells) ++bits;
+    while ((1 << bits) < ncells + 1) ++bits;
     return sort_scratch_bytes(pair_capacity, bits, digit_bits);
 }
-
-// A warp's table of the cell-level QPass segments of 32 Gaussians, and their
-// tile rectangles.
-struct CellTable {
-    int32_t start[32 * 7];  // range position of the segment's first entry
-    uint32_t geo[32 * 7];   // first line | first cell << 16
-    uint32_t len[32 * 7];   // cells per line | owner lane << 16 | column flag << 24
-    float inv[32 * 7];      // 1 / cells per line
-    uint32_t gid[32];
-    uint4 rects[32][2];
-};
 
 __device__ __forceinline__ uint64_t cell_value(uint32_t gid, uint32_t bits) { return ((uint64_t)bits << 32) | gid; }
 
@@ -74,97 +63,84 @@ __device__ __forceinline__ uint32_t tiles_in_cell(const uint4 &w0, const uint4 &
            cell_bits_of(unpack_rect(w1.x, w1.y), cx, cy) | cell_bits_of(unpack_rect(w1.z, w1.w), cx, cy);
 }
 
+// 32 Gaussians of a warp: their cells' bounding boxes and tile rectangles.
+struct CellTable {
+    int4 box[32];    // range position of its first entry, first cell x | y << 16, cells per row, Gaussian
+    float2 inv[32];  // 1 / cells per row; entries of a Gaussian that skips cells (cell_entries), else 0
+    uint4 rects[32][2];
+};
+
 // Entries [C, C + L) in emission order, by one warp: the Gaussian whose run
 // holds entry C comes from the scan's table; the following ones are taken 32
-// at a time, each lane decomposing its Gaussian's cells into runs, and the
-// range is produced 32 consecutive entries at a time (lane q finds its run
-// from a ballot of the run starts in its group).
+// at a time, one per lane, and the range is produced 32 consecutive entries at
+// a time: lane q finds the Gaussian of its entry from a ballot of the run
+// starts in its group (every Gaussian with entries comes before those without
+// in depth order, so run starts and lanes correspond), and the entry's cell by
+// a division by its box's width.
 __device__ __forceinline__ void cell_emit_range(const CellBin &b, uint64_t E, uint64_t C, int32_t L, CellTable &S,
                                                 uint32_t *hist) {
     const int lane = threadIdx.x & 31;
     const uint32_t le_mask = lanemask_le();
+    const uint32_t none = (uint32_t)b.geo.ncells;
     int64_t j0 = b.chunk_first[C / kEmitStride];
     int32_t done_to = 0;  // range positions [0, done_to) produced
     while (done_to < L && j0 < b.n) {
         const int64_t j = j0 + lane;
+        // the run of position j, relative to C (none beyond the last one)
+        int64_t rel = (int64_t)E - (int64_t)C, end = rel;
         uint32_t gid = 0;
-        int64_t rel = (int64_t)1 << 40;
         if (j < b.n) {
             gid = b.perm[j];
             rel = (int64_t)b.coff[j] - (int64_t)C;
+            end = j + 1 < b.n ? (int64_t)b.coff[j + 1] - (int64_t)C : end;
         }
-        // the run ends where the next one begins
-        int64_t end = __shfl_down_sync(0xffffffffu, rel, 1);
-        if (lane == 31) end = j + 1 < b.n ? (int64_t)b.coff[j + 1] - (int64_t)C : (int64_t)E - (int64_t)C;
-        if (end == (int64_t)1 << 40) end = (int64_t)E - (int64_t)C;
-        if (j >= b.n) rel = end = (int64_t)E - (int64_t)C;
         const bool relevant = end > rel && rel < L && end > 0;
-        QSeg seg[7];
-#pragma unroll
-        for (int q = 0; q < 7; ++q) seg[q] = QSeg{0, 0, 0, 0};
-        bool columns = false;
         __syncwarp();
         if (relevant) {
             const uint4 w0 = b.rects[2 * (size_t)gid], w1 = b.rects[2 * (size_t)gid + 1];
+            const Rect r[4] = {unpack_rect(w0.x, w0.y), unpack_rect(w0.z, w0.w), unpack_rect(w1.x, w1.y),
+                               unpack_rect(w1.z, w1.w)};
+            const Rect box = cell_box(r);
+            const int bw = box.x1 - box.x0 + 1, cells = bw * (box.y1 - box.y0 + 1);
+            S.box[lane] = make_int4((int32_t)rel, box.x0 | (box.y0 << 16), bw, (int)gid);
+            S.inv[lane] = make_float2(1.0f / (float)bw, cells != (int)(end - rel) ? (float)cells : 0.f);
             S.rects[lane][0] = w0;
             S.rects[lane][1] = w1;
-            const Rect r[4] = {cell_rect(unpack_rect(w0.x, w0.y)), cell_rect(unpack_rect(w0.z, w0.w)),
-                               cell_rect(unpack_rect(w1.x, w1.y)), cell_rect(unpack_rect(w1.z, w1.w))};
-            QPass qp;
-            if (qpass_setup(r, qp)) {
-                qpass_segments(qp, seg);
-                columns = qp.columns;
-            }
         }
-        int ns = 0;
-#pragma unroll
-        for (int q = 0; q < 7; ++q) ns += seg_empty(seg[q]) ? 0 : 1;
-        S.gid[lane] = gid;
-        const int sincl = warp_incl_scan(ns);
-        const int nseg = __shfl_sync(0xffffffffu, sincl, 31);
-        int32_t r0 = (int32_t)(rel > -((int64_t)1 << 30) ? rel : -((int64_t)1 << 30));
-        int k = sincl - ns;  // this lane's first table entry
-#pragma unroll
-        for (int q = 0; q < 7; ++q) {
-            if (seg_empty(seg[q])) continue;
-            S.start[k] = r0;
-            S.geo[k] = (uint32_t)seg[q].s0 | ((uint32_t)seg[q].lo << 16);
-            S.len[k] = (uint32_t)seg[q].len | ((uint32_t)lane << 16) | ((uint32_t)columns << 24);
-            S.inv[k] = 1.0f / (float)seg[q].len;
-            r0 += seg[q].nl * seg[q].len;
-            ++k;
-        }
+        // where the lane's run starts among the positions still to come
+        const int32_t start = relevant && rel > done_to ? (int32_t)rel : INT32_MAX;
+        // the Gaussian of position done_to
+        int cur = __popc(__ballot_sync(0xffffffffu, rel <= done_to)) - 1;
         const int64_t last_end = __shfl_sync(0xffffffffu, end, 31);
         const int32_t batch_end = (int32_t)(last_end < (int64_t)L ? last_end : (int64_t)L);
         __syncwarp();
-        // cur: last segment starting at or before done_to
-        int cur = -1;
-        for (int q = 0; q < nseg; q += 32) {
-            const bool le = q + lane < nseg && S.start[q + lane] <= done_to;
-            cur += __popc(__ballot_sync(0xffffffffu, le));
-        }
         for (int32_t c0 = done_to; c0 < batch_end; c0 += 32) {
-            const int cand = cur + 1 + lane;
-            uint32_t bit = 0u;
-            if (cand < nseg) {
-                const int32_t st = S.start[cand];
-                if (st < c0 + 32) bit = 1u << (st - c0);
-            }
-            const uint32_t M = __reduce_or_sync(0xffffffffu, bit);
+            // runs that start in this group (the first position's is cur already)
+            const uint32_t ahead = (uint32_t)(start - c0);
+            const uint32_t M = __reduce_or_sync(0xffffffffu, ahead < 32u ? 1u << ahead : 0u);
             const int32_t p = c0 + lane;
             if (p < batch_end) {
                 const int idx = cur + __popc(M & le_mask);
-                const uint32_t geo = S.geo[idx], ln = S.len[idx];
+                const int4 B = S.box[idx];
+                const float2 inv = S.inv[idx];
+                const uint4 w0 = S.rects[idx][0], w1 = S.rects[idx][1];
+                uint32_t k = (uint32_t)(p - B.x);
+                const int x0 = B.y & 0xffff, y0 = B.y >> 16;
                 uint32_t q, r;
-                seg_divide((uint32_t)(p - S.start[idx]), ln & 0xffffu, S.inv[idx], q, r);
-                const uint32_t line = (geo & 0xffffu) + q, u = (geo >> 16) + r;
-                const bool cols = (ln >> 24) & 1u;
-                const uint32_t owner = (ln >> 16) & 0xffu;
-                const uint32_t cx = cols ? line : u, cy = cols ? u : line;
-                const uint32_t cell = cy * (uint32_t)b.geo.cells_x + cx;
+                if (inv.y != 0.f) {  // entry k is the k-th of the box's cells that hold a tile
+                    uint32_t c = 0;
+                    for (uint32_t left = k + 1; c < (uint32_t)inv.y; ++c) {
+                        seg_divide(c, (uint32_t)B.z, inv.x, q, r);
+                        if (tiles_in_cell(w0, w1, x0 + (int)r, y0 + (int)q) && --left == 0u) break;
+                    }
+                    k = c;
+                }
+                seg_divide(k, (uint32_t)B.z, inv.x, q, r);
+                const int cx = x0 + (int)r, cy = y0 + (int)q;
+                const uint32_t bits = tiles_in_cell(w0, w1, cx, cy);
+                const uint32_t cell = bits ? (uint32_t)(cy * b.geo.cells_x + cx) : none;
                 b.arr.keys_a[C + p] = cell;
-                b.arr.vals_a[C + p] =
-                    cell_value(S.gid[owner], tiles_in_cell(S.rects[owner][0], S.rects[owner][1], (int)cx, (int)cy));
+                b.arr.vals_a[C + p] = cell_value((uint32_t)B.w, bits);
                 atomicAdd(hist + cell, 1u);
             }
             cur += __popc(M);
@@ -208,16 +184,16 @@ __device__ __forceinline__ void cell_emit_naive(const CellBin &b, int64_t j, uin
 // offsets.  s_dsum has room for 2^kMaxDigitBits digit sums.
 __device__ __forceinline__ void cell_prepare(const CellBin &b, uint32_t *s_dsum) {
     constexpr int U = 4;
-    const int ncells = b.geo.ncells;
+    const int ncells = b.geo.ncells, ids = ncells + 1;  // (id ncells: entries without a tile, no rows)
     uint32_t entries = 0, rows = 0;  // before this step's cells
-    for (int c0 = 0; c0 < ncells; c0 += U * (int)blockDim.x) {
+    for (int c0 = 0; c0 < ids; c0 += U * (int)blockDim.x) {
         uint32_t v[U], sum = 0, rsum = 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int c = c0 + (int)threadIdx.x * U + u;
-            v[u] = c < ncells ? __ldcg(b.arr.count + c) : 0u;
+            v[u] = c < ids ? __ldcg(b.arr.count + c) : 0u;
             sum += v[u];
-            rsum += (v[u] + kCellRow - 1) / kCellRow;
+            rsum += c < ncells ? (v[u] + kCellRow - 1) / kCellRow : 0u;
         }
         uint32_t total, rtotal;
         uint32_t e = entries + block_incl_scan<uint32_t>(sum, &total) - sum;
@@ -225,20 +201,17 @@ __device__ __forceinline__ void cell_prepare(const CellBin &b, uint32_t *s_dsum)
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int c = c0 + (int)threadIdx.x * U + u;
-            if (c < ncells) {
+            if (c < ids) {
                 b.arr.start[c] = e;
-                b.arr.row_start[c] = r;
+                b.arr.row_start[c] = r;  // [ncells]: the rows there are
             }
             e += v[u];
-            r += (v[u] + kCellRow - 1) / kCellRow;
+            r += c < ncells ? (v[u] + kCellRow - 1) / kCellRow : 0u;
         }
         entries += total;
         rows += rtotal;
     }
-    if (threadIdx.x == 0) {
-        b.arr.start[ncells] = entries;
-        b.arr.row_start[ncells] = rows;
-    }
+    if (threadIdx.x == 0) b.arr.start[ids] = entries;
     __threadfence_block();
     __syncthreads();
     uint32_t *table = sort_hist_at(b.sort_scratch);
@@ -246,14 +219,14 @@ __device__ __forceinline__ void cell_prepare(const CellBin &b, uint32_t *s_dsum)
     for (int p = 0; p < b.geo.passes.passes; ++p) {
         const int bits = b.geo.passes.bits[p], sh = b.geo.passes.shift[p];
         const int Rp = 1 << bits, period = Rp << sh;
-        const int runs = Rp * ((ncells + period - 1) / period);
+        const int runs = Rp * ((ids + period - 1) / period);
         for (int d = threadIdx.x; d < Rp; d += blockDim.x) s_dsum[d] = 0u;
         __syncthreads();
         for (int i = threadIdx.x; i < runs; i += blockDim.x) {
             const int d = i & (Rp - 1), u = i >> bits;
             const int c = u * period + (d << sh);
-            if (c >= ncells) continue;
-            const uint32_t v = start[min(ncells, c + (1 << sh))] - start[c];
+            if (c >= ids) continue;
+            const uint32_t v = start[min(ids, c + (1 << sh))] - start[c];
             if (v) atomicAdd(&s_dsum[d], v);
         }
         __syncthreads();
@@ -271,11 +244,16 @@ __device__ __forceinline__ void cell_prepare(const CellBin &b, uint32_t *s_dsum)
     }
 }
 
-// The emit, balanced over the entries (warp w takes the ranges [w C, (w+1) C),
-// w + warps, ...), with a histogram of the cells (in shared memory up to
+// The emit, with a histogram of the cells (in shared memory up to
 // kCellHistMax cells) whose last block makes the cells' offsets.  It also
 // zeroes the look-back words and counters of the sort's passes, sized by the
 // entries there are and not by the capacity.
+//
+// Bound by issue slots.  Decomposing every Gaussian's cells into QPass runs
+// took 41M warp instructions and 79 us for 1M Gaussians at 1080p (2.7M entries);
+// EMITFIG.  (A thread per Gaussian that runs through a small box, and a block's
+// warps sharing the large ones, took 72 us, and 104 instead of 48 for 3M at
+// 1440p seen from inside, where the nearest Gaussians' boxes fill the image.)
 template <bool NAIVE>
 __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -283,14 +261,14 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     uint32_t *s_hist = reinterpret_cast<uint32_t *>(smem + (NAIVE ? 0 : kCellWarps * sizeof(CellTable)));
     __shared__ bool s_last;
     const int tid = threadIdx.x, wid = tid >> 5;
-    const bool in_smem = b.geo.ncells <= kCellHistMax;
+    const bool in_smem = b.geo.ncells < kCellHistMax;
     const uint64_t E = *b.n_cells;
     if (blockIdx.x == 0 && tid == 0) {
         const uint64_t P = *b.n_pairs;
         if (P > b.capacity || (P > 0 && E == 0)) atomicOr(b.err, kErrCapacity);
     }
     if (in_smem)
-        for (int c = tid; c < b.geo.ncells; c += blockDim.x) s_hist[c] = 0u;
+        for (int c = tid; c <= b.geo.ncells; c += blockDim.x) s_hist[c] = 0u;
     const uint64_t threads = (uint64_t)gridDim.x * blockDim.x, gt = (uint64_t)blockIdx.x * blockDim.x + tid;
     for (int p = 0; p < b.geo.passes.passes; ++p) {
         uint32_t *lb = sort_lookback_at(b.sort_scratch, b.capacity, b.geo.digit_bits, p);
@@ -311,14 +289,14 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     }
     if (in_smem) {
         __syncthreads();
-        for (int c = tid; c < b.geo.ncells; c += blockDim.x) {
+        for (int c = tid; c <= b.geo.ncells; c += blockDim.x) {
             const uint32_t v = s_hist[c];
             if (v) atomicAdd(b.arr.count + c, v);
         }
     }
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(b.arr.count + b.geo.ncells, 1u) == gridDim.x - 1;
+    if (tid == 0) s_last = atomicAdd(b.arr.count + b.geo.ncells + 1, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -331,7 +309,7 @@ cudaError_t launch_cell_emit(const CellBin &b, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t hist = b.geo.ncells <= kCellHistMax ? 4 * (size_t)b.geo.ncells : 0;
+    const size_t hist = b.geo.ncells < kCellHistMax ? 4 * ((size_t)b.geo.ncells + 1) : 0;
     const size_t dsum = (size_t)4 << kMaxDigitBits;
     if (b.naive) {
         const size_t smem = std::max(hist, dsum);
@@ -341,10 +319,8 @@ cudaError_t launch_cell_emit(const CellBin &b, cudaStream_t s) {
         return cudaGetLastError();
     }
     const size_t smem = std::max(kCellWarps * sizeof(CellTable) + hist, dsum);
-    e = ensure_dyn_smem((const void *)cell_emit_kernel<false>, kCellWarps * sizeof(CellTable) + 4 * (size_t)kCellHistMax);
-    if (e != cudaSuccess) return e;
     const uint64_t want = (b.n_cells_max + kCellWarps * kCellChunk - 1) / (kCellWarps * kCellChunk);
-    const uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * 4));
+    const uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * 6));
     note_launch("cell_emit_kernel", s), cell_emit_kernel<false><<<(unsigned)blocks, kCellWarps * 32, smem, s>>>(b);
     return cudaGetLastError();
 }
@@ -449,7 +425,7 @@ __global__ void __launch_bounds__(1024) cell_prefix_kernel(CellGeo g, CellArrays
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(a.count + g.ncells + 1, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) s_last = atomicAdd(a.count + g.ncells + 2, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();

@@ -373,6 +373,35 @@ __device__ __forceinline__ uint32_t cell_bits_of(const Rect &r, int cx, int cy) 
     return row * rows;
 }
 
+// The cells of the bounding box of four tile rectangles (not all empty).
+__device__ __forceinline__ Rect cell_box(const Rect r[4]) {
+    Rect box{1 << 30, 1 << 30, -1, -1};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const bool e = rect_empty(r[q]);
+        box.x0 = e ? box.x0 : min(box.x0, r[q].x0);
+        box.y0 = e ? box.y0 : min(box.y0, r[q].y0);
+        box.x1 = e ? box.x1 : max(box.x1, r[q].x1);
+        box.y1 = e ? box.y1 : max(box.y1, r[q].y1);
+    }
+    return cell_rect(box);
+}
+
+// The entries that a Gaussian of `tiles` tiles gets: one per cell of its
+// cells' bounding box, an eighth or so of them without a tile, which the emit
+// files apart.  The few whose bounding box has more cells than they have tiles
+// (two or three tiles around a corner of four cells) get one per cell that
+// holds a tile, so there are never more entries than tiles.
+__device__ __forceinline__ uint32_t cell_entries(const Rect r[4], uint32_t tiles) {
+    if (tiles == 0u) return 0u;
+    const uint32_t cells = (uint32_t)rect_area(cell_box(r));
+    if (cells <= tiles) return cells;
+    Rect c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[q] = cell_rect(r[q]);
+    return union_count(c);
+}
+
 // A Gaussian's four sub-box rectangles in two uint4 (tile coordinates below
 // 2^16), rectangle q in words 2q (x0 | y0 << 16) and 2q + 1 (x1 | y1 << 16).
 __device__ __forceinline__ void pack_rects(const Rect r[4], uint4 out[2]) {

@@ -98,8 +98,8 @@ struct CellGeo {
 
 // Device arrays of the cell binning (qb_cells.cu).
 struct CellArrays {
-    uint32_t *count;       // [ncells] entries per cell, then the two finished-block counters
-    uint32_t *start;       // [ncells + 1] first sorted entry of each cell
+    uint32_t *count;       // [ncells + 1] entries per cell and without a tile, then two finished-block counters
+    uint32_t *start;       // [ncells + 2] first sorted entry of each cell (last: of those without a tile)
     uint32_t *row_start;   // [ncells + 1] first row of each cell
     uint32_t *row_cell;    // [rows]
     uint32_t *row_counts;  // [rows][32] entries per tile; after the prefix, those of the cell's earlier rows
@@ -110,13 +110,13 @@ struct CellArrays {
     uint64_t *vals_a, *vals_b;
 };
 constexpr uint32_t kCellRow = 128;  // sorted entries per row
-inline size_t cell_zero_words(int ncells) { return (size_t)ncells + 2; }
+inline size_t cell_zero_words(int ncells) { return (size_t)ncells + 3; }
 inline size_t cell_rows_max(uint64_t pair_capacity, int ncells) { return (size_t)(pair_capacity / kCellRow) + ncells; }
 
 struct CellBin {
     int n;
     const uint32_t *perm;   // record of each emission position
-    const uint32_t *coff;   // cell offset of each emission position
+    const uint32_t *coff;   // first entry of each emission position
     const uint32_t *chunk_first;
     const uint4 *rects;     // by record
     const uint64_t *n_pairs, *n_cells;

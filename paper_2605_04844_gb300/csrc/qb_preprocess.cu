@@ -92,20 +92,19 @@ __global__ void __launch_bounds__(256, 3) preprocess_kernel(PreArgs a) {
 
     Rect rects[4];
     box_rects(p.mx, p.my, bt.box, bt.r3, bt.orient, a.mode, a.clamp3s, cam.W, cam.H, rects);
-    // tiles, and cells of 8 x 4 tiles, of the QPass traversal
+    // tiles of the QPass traversal, and the entries it gets among the cells of
+    // 8 x 4 tiles: the cells of the bounding box of its tiles (cell_entries)
     uint32_t cnt, ccnt;
-    Rect crects[4];
+    if (a.mode == QB_BIN_QUADBOX_NAIVE) {  // the same set, counted the naive way
+        Rect crects[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) crects[q] = cell_rect(rects[q]);
-    if (a.mode == QB_BIN_AABB3S || a.mode == QB_BIN_ADR) {  // a single box
-        cnt = (uint32_t)rect_area(rects[0]);
-        ccnt = (uint32_t)rect_area(crects[0]);
-    } else if (a.mode == QB_BIN_QUADBOX_NAIVE) {  // the same sets, counted the naive way
+        for (int q = 0; q < 4; ++q) crects[q] = cell_rect(rects[q]);
         cnt = naive_count(rects);
         ccnt = naive_count(crects);
     } else {
-        cnt = union_count(rects);
-        ccnt = union_count(crects);
+        // (a mode of a single box has the others empty)
+        cnt = a.mode == QB_BIN_AABB3S || a.mode == QB_BIN_ADR ? (uint32_t)rect_area(rects[0]) : union_count(rects);
+        ccnt = cell_entries(rects, cnt);
     }
     if (cnt > 0u) {
         uint4 pk[2];

@@ -217,6 +217,12 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
     if (wcount == 32 * kSortItems) rank_items(std::true_type{});
     else rank_items(std::false_type{});
 
+    // the ranks wait in the (still unused) scatter buffer while the look-back
+    // needs the registers; every thread reads back its own
+    uint16_t *s_rank = reinterpret_cast<uint16_t *>(smem) + tid;
+#pragma unroll
+    for (int k = 0; k < kSortItems; ++k) s_rank[k * kSortBlock] = (uint16_t)rank[k];
+
     // ---- look back for the running totals, publish the inclusive prefix ----
     // Each thread walks back for its digits, kLookWindow words at a time
     // (their addresses do not depend on what is read), adding aggregates until
@@ -288,6 +294,8 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
             r += c;
         }
     }
+#pragma unroll
+    for (int k = 0; k < kSortItems; ++k) rank[k] = s_rank[k * kSortBlock];
     __syncthreads();
 
     const uint32_t tcount = min(n - tbase, (uint32_t)kSortTile);
