@@ -78,12 +78,7 @@ bool make_layout(int n, int W, int H, uint64_t cap, Layout &L) {
     L.dkeys1 = take(4 * N);
     L.dvals0 = take(4 * N);
     L.dvals1 = take(4 * N);
-    size_t db = 0;
-    for (int d = 8; d <= kMaxDigitBits; ++d) {
-        size_t b = sort_scratch_bytes(N, kDepthBits, d);
-        if (b > db) db = b;
-    }
-    L.dsort_scratch = take(db);
+    L.dsort_scratch = take(depth_sort_scratch_bytes(N));
     L.ranges = take(8 * (size_t)tiles);
     const int ncells = cell_geo(W, H, 8).ncells;
     L.cell_zero = take(4 * cell_zero_words(ncells));

@@ -129,14 +129,12 @@ bool make_blayout(int n, int n_cams, int group, uint64_t cap, const Geo &g, BLay
     L.coff = take(4 * (size_t)n);
     L.chunk_first = take(4 * chunk_table_size(cap));
     L.scan_part = take(8 * scan_partials_count(n));
-    size_t db = 0, sb = 0;
+    size_t sb = 0;
     for (int d = 8; d <= kMaxDigitBits; ++d) {
-        const size_t b1 = sort_scratch_bytes((uint64_t)n, kDepthBits, d);
         const size_t b2 = cell_sort_scratch_bytes(cap, g.max_cells, d);
-        db = b1 > db ? b1 : db;
         sb = b2 > sb ? b2 : sb;
     }
-    L.dsort = take(db);
+    L.dsort = take(depth_sort_scratch_bytes((uint64_t)n));
     L.sort = take(sb);
     L.n_cells = take(8);
     L.cell_zero = take(4 * cell_zero_words(g.max_cells));

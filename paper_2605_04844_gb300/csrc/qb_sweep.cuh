@@ -21,11 +21,11 @@ namespace qb {
 
 constexpr int kSortBlock = 256;
 constexpr int kSortWarps = kSortBlock / 32;
-constexpr int kSortItems = 16;
+constexpr int kSortItems = 16;  // keys per thread (fewer for short sorts of 32-bit keys: sort_items_u32)
 constexpr int kSortBlocksPerSM = 5;  // resident pass blocks per SM the registers are sized for (32-bit keys)
 constexpr int kSortTile = kSortBlock * kSortItems;  // 4096 keys per block
 constexpr int kSpinLimit = 1 << 22;
-constexpr int kLookWindow = 8;  // status words fetched per look-back step
+constexpr int kLookWindow = 8;  // status words fetched per look-back step (16, 24, 32 measured slower)
 constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagIncl = 2u << 30;
 constexpr uint32_t kCountMask = (1u << 30) - 1u;
@@ -117,14 +117,14 @@ __device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t v, uint32_t *to
 // keys; keys, then values, for 64-bit keys; values and keys side by side for
 // 64-bit values), per-warp digit counters, and per-digit global base, local
 // start and tile count.
-template <typename ValT>
+template <typename ValT, int ITEMS = kSortItems>
 constexpr size_t sweep_stage() {
-    return (size_t)kSortTile * (sizeof(ValT) == 8 ? 12 : 8);
+    return (size_t)kSortBlock * ITEMS * (sizeof(ValT) == 8 ? 12 : 8);
 }
 
-template <int RB, typename ValT = uint32_t>
+template <int RB, typename ValT = uint32_t, int ITEMS = kSortItems>
 constexpr size_t sweep_smem() {
-    return sweep_stage<ValT>() + (size_t)kSortWarps * (1 << RB) * 2 + (size_t)3 * (1 << RB) * 4;
+    return sweep_stage<ValT, ITEMS>() + (size_t)kSortWarps * (1 << RB) * 2 + (size_t)3 * (1 << RB) * 4;
 }
 
 // One pass over the tile `tile` (positions [tbase, tbase + kSortTile) of n) on the
@@ -134,8 +134,8 @@ constexpr size_t sweep_smem() {
 // bucket offsets; lookback: the pass's status words [tiles][2^RB].  Without
 // WRITE_KEYS (the last pass of a sort whose keys its ranges imply) only the
 // values are written.  64-bit values go with 32-bit keys.
-template <int RB, typename KeyT, typename ValT, bool WRITE_KEYS, class ValFn>
-__device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn &&val,
+template <int RB, typename KeyT, typename ValT, bool WRITE_KEYS, int ITEMS, class ValFn>
+__device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val,
                                            uint32_t n, uint32_t tbase, uint32_t tile,
                                            const uint32_t *__restrict__ bin_off, uint32_t *lookback, int shift,
                                            uint32_t mask, uint32_t *err, KeyT *__restrict__ kout,
@@ -143,7 +143,7 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
     static_assert(sizeof(ValT) == 4 || sizeof(KeyT) == 4, "64-bit values go with 32-bit keys");
     constexpr int R = 1 << RB;
     constexpr int PER = (R + kSortBlock - 1) / kSortBlock;
-    uint16_t *s_whist = reinterpret_cast<uint16_t *>(smem + sweep_stage<ValT>());
+    uint16_t *s_whist = reinterpret_cast<uint16_t *>(smem + sweep_stage<ValT, ITEMS>());
     uint32_t *s_gbase = reinterpret_cast<uint32_t *>(s_whist + kSortWarps * R);
     uint32_t *s_lstart = s_gbase + R;
     uint32_t *s_bcount = s_lstart + R;
@@ -152,15 +152,15 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
     for (int j = tid; j < kSortWarps * R / 2; j += kSortBlock) reinterpret_cast<uint32_t *>(s_whist)[j] = 0u;
     for (int j = tid; j < R; j += kSortBlock) s_bcount[j] = 0u;
     __syncthreads();
-    const uint32_t wbase = tbase + (uint32_t)wid * (32 * kSortItems);
+    const uint32_t wbase = tbase + (uint32_t)wid * (32 * ITEMS);
     // items of this warp that exist: item k of lane l is valid when 32 k + l < wcount
-    const int wcount = n > wbase ? (int)min(n - wbase, (uint32_t)(32 * kSortItems)) : 0;
-    uint32_t rank[kSortItems];
+    const int wcount = n > wbase ? (int)min(n - wbase, (uint32_t)(32 * ITEMS)) : 0;
+    uint32_t rank[ITEMS];
     auto dig = [&](int k) { return (uint32_t)(key[k] >> shift) & mask; };
 
     // ---- early digit counts of the tile ----
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k)
+    for (int k = 0; k < ITEMS; ++k)
         if (32 * k + lane < wcount) atomicAdd(&s_bcount[dig(k)], 1u);
     __syncthreads();
 
@@ -196,7 +196,7 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
         constexpr bool FULL = decltype(full_tag)::value;
         constexpr int NB = FULL ? RB : RB + 1;
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             const bool valid = FULL || 32 * k + lane < wcount;
             const uint32_t d = valid ? dig(k) : (uint32_t)R;
             uint32_t peers = 0xffffffffu;
@@ -214,14 +214,14 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
             rank[k] = pre + lower;
         }
     };
-    if (wcount == 32 * kSortItems) rank_items(std::true_type{});
+    if (wcount == 32 * ITEMS) rank_items(std::true_type{});
     else rank_items(std::false_type{});
 
     // the ranks wait in the (still unused) scatter buffer while the look-back
     // needs the registers; every thread reads back its own
     uint16_t *s_rank = reinterpret_cast<uint16_t *>(smem) + tid;
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) s_rank[k * kSortBlock] = (uint16_t)rank[k];
+    for (int k = 0; k < ITEMS; ++k) s_rank[k * kSortBlock] = (uint16_t)rank[k];
 
     // ---- look back for the running totals, publish the inclusive prefix ----
     // Each thread walks back for its digits, kLookWindow words at a time
@@ -295,16 +295,16 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
         }
     }
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) rank[k] = s_rank[k * kSortBlock];
+    for (int k = 0; k < ITEMS; ++k) rank[k] = s_rank[k * kSortBlock];
     __syncthreads();
 
-    const uint32_t tcount = min(n - tbase, (uint32_t)kSortTile);
+    const uint32_t tcount = min(n - tbase, (uint32_t)(kSortBlock * ITEMS));
     if constexpr (sizeof(ValT) == 8) {
         // ---- values and keys to block order in shared memory, then out ----
         ValT *s_val = reinterpret_cast<ValT *>(smem);
-        uint32_t *s_key = reinterpret_cast<uint32_t *>(smem + (size_t)kSortTile * 8);
+        uint32_t *s_key = reinterpret_cast<uint32_t *>(smem + (size_t)kSortBlock * ITEMS * 8);
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             if (32 * k + lane < wcount) {
                 const uint32_t d = dig(k);
                 const uint32_t j = s_lstart[d] + s_whist[wid * R + d] + rank[k];
@@ -314,7 +314,7 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             const uint32_t j = tid + k * kSortBlock;
             if (j < tcount) {
                 const uint32_t kk = s_key[j];
@@ -329,7 +329,7 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
         // ---- (key, value) pairs to block order in shared memory, then out ----
         uint2 *s_pairs = reinterpret_cast<uint2 *>(smem);
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             if (32 * k + lane < wcount) {
                 const uint32_t d = dig(k);
                 s_pairs[s_lstart[d] + s_whist[wid * R + d] + rank[k]] = make_uint2((uint32_t)key[k], val(k));
@@ -337,7 +337,7 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             const uint32_t j = tid + k * kSortBlock;
             if (j < tcount) {
                 const uint2 kv = s_pairs[j];
@@ -354,7 +354,7 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
         KeyT *s_keys = reinterpret_cast<KeyT *>(smem);
         uint32_t *s_vals = reinterpret_cast<uint32_t *>(smem);
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             if (32 * k + lane < wcount) {
                 const uint32_t d = dig(k);
                 const uint32_t lr = s_lstart[d] + s_whist[wid * R + d] + rank[k];
@@ -363,9 +363,9 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
             }
         }
         __syncthreads();
-        uint32_t dest[kSortItems];
+        uint32_t dest[ITEMS];
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             const uint32_t j = tid + k * kSortBlock;
             if (j < tcount) {
                 const KeyT kk = s_keys[j];
@@ -377,11 +377,11 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[kSortItems], ValFn 
         __syncthreads();
         // ---- values through the same permutation ----
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k)
+        for (int k = 0; k < ITEMS; ++k)
             if (32 * k + lane < wcount) s_vals[rank[k]] = val(k);
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
+        for (int k = 0; k < ITEMS; ++k) {
             const uint32_t j = tid + k * kSortBlock;
             if (j < tcount && dest[k] < n) vout[dest[k]] = s_vals[j];
         }
