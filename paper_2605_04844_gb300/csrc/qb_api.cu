@@ -398,19 +398,28 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
     uint32_t *chunk_first = at<uint32_t>(frame, L.chunk_first);
     const uint32_t chunk_cap = (uint32_t)chunk_table_size(frame->pair_capacity);
     if (depth_first) {
-        // emission order = Gaussians sorted by (depth, index)
-        uint32_t *dk0 = at<uint32_t>(frame, L.dkeys0), *dk1 = at<uint32_t>(frame, L.dkeys1);
-        uint32_t *dv0 = at<uint32_t>(frame, L.dvals0), *dv1 = at<uint32_t>(frame, L.dvals1);
-        // (keys and indices in dk0 / dv0 from the preprocess)
-        int passes = 0;
-        if (frame->n > 0)
-            QB_CUDA(sort_pairs(dk0, dv0, dk1, dv1, (uint64_t)frame->n, nullptr, kDepthBits, kDepthDigitBits,
-                               at<void>(frame, L.dsort_scratch), err, s, &passes));
-        frame->depth_in_alt = passes & 1;
-        QB_CUDA(launch_scan_cells(at<uint2>(frame, L.cc), frame->depth_in_alt ? dv1 : dv0, frame->n,
-                                  at<uint32_t>(frame, L.offsets), at<uint32_t>(frame, L.coff), partials, d_np,
-                                  at<uint64_t>(frame, L.state + 16), frame->pair_capacity, err, chunk_first, chunk_cap,
-                                  s));
+        // emission order = Gaussians sorted by (depth, index); keys and indices
+        // from the preprocess
+        OrderArgs o;
+        std::memset(&o, 0, sizeof(o));
+        o.keys = at<uint32_t>(frame, L.dkeys0);
+        o.vals = at<uint32_t>(frame, L.dvals0);
+        o.keys_alt = at<uint32_t>(frame, L.dkeys1);
+        o.vals_alt = at<uint32_t>(frame, L.dvals1);
+        o.sort_scratch = at<void>(frame, L.dsort_scratch);
+        o.cc = at<uint2>(frame, L.cc);
+        o.offsets = at<uint32_t>(frame, L.offsets);
+        o.coff = at<uint32_t>(frame, L.coff);
+        o.chunk_first = chunk_first;
+        o.chunk_cap = chunk_cap;
+        o.partials = partials;
+        o.n_pairs = d_np;
+        o.n_cells = at<uint64_t>(frame, L.state + 16);
+        o.capacity = frame->pair_capacity;
+        o.err = err;
+        bool in_alt = false;
+        QB_CUDA(launch_depth_order(o, frame->n, s, &in_alt));
+        frame->depth_in_alt = in_alt;
     } else {
         QB_CUDA(launch_scan(at<uint32_t>(frame, L.counts), frame->n, at<uint32_t>(frame, L.offsets),
                             at<uint32_t>(frame, L.coff), partials, d_np, err, chunk_first, chunk_cap, s));

@@ -453,18 +453,28 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
             const cudaStream_t cs = nside > 0 ? ss.side[set] : s;
             const size_t so = (size_t)set * L.set_stride;
             const size_t r0 = (size_t)c * n;  // the camera's records within the group
-            uint32_t *dk0 = bat<uint32_t>(b, L.dk0) + r0, *dk1 = bat<uint32_t>(b, L.dk1) + r0;
-            uint32_t *dv0 = bat<uint32_t>(b, L.dv0) + r0, *dv1 = bat<uint32_t>(b, L.dv1) + r0;
-            int passes = 0;
-            if (n > 0)
-                QB_BCUDA(sort_pairs(dk0, dv0, dk1, dv1, (uint64_t)n, nullptr, kDepthBits, kDepthDigitBits,
-                                    bat<void>(b, L.dsort + so), err, cs, &passes));
-            const uint32_t *perm = (passes & 1) ? dv1 : dv0;  // group record indices in depth order
             uint64_t *n_cells = bat<uint64_t>(b, L.n_cells + so);
             uint32_t *coff = bat<uint32_t>(b, L.coff + so), *chunk_first = bat<uint32_t>(b, L.chunk_first + so);
-            QB_BCUDA(launch_scan_cells(a.cc, perm, n, bat<uint32_t>(b, L.offsets + so), coff,
-                                       bat<uint64_t>(b, L.scan_part + so), npairs + k, n_cells, cap, err, chunk_first,
-                                       (uint32_t)chunk_table_size(cap), cs));
+            OrderArgs o;
+            std::memset(&o, 0, sizeof(o));
+            o.keys = bat<uint32_t>(b, L.dk0) + r0;
+            o.vals = bat<uint32_t>(b, L.dv0) + r0;
+            o.keys_alt = bat<uint32_t>(b, L.dk1) + r0;
+            o.vals_alt = bat<uint32_t>(b, L.dv1) + r0;
+            o.sort_scratch = bat<void>(b, L.dsort + so);
+            o.cc = a.cc;
+            o.offsets = bat<uint32_t>(b, L.offsets + so);
+            o.coff = coff;
+            o.chunk_first = chunk_first;
+            o.chunk_cap = (uint32_t)chunk_table_size(cap);
+            o.partials = bat<uint64_t>(b, L.scan_part + so);
+            o.n_pairs = npairs + k;
+            o.n_cells = n_cells;
+            o.capacity = cap;
+            o.err = err;
+            bool in_alt = false;
+            QB_BCUDA(launch_depth_order(o, n, cs, &in_alt));
+            const uint32_t *perm = in_alt ? o.vals_alt : o.vals;  // group record indices in depth order
             CellBin e;
             std::memset(&e, 0, sizeof(e));
             e.n = n;

@@ -241,6 +241,21 @@ cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32
 cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint32_t *offsets, uint32_t *coff,
                               uint64_t *partials, uint64_t *n_pairs, uint64_t *n_cells, uint64_t capacity,
                               uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s);
+// The depth order of n Gaussians (keys and record indices from the
+// preprocess) and the scan in that order.
+struct OrderArgs {
+    uint32_t *keys, *vals, *keys_alt, *vals_alt;
+    void *sort_scratch;  // depth_sort_scratch_bytes(n)
+    const uint2 *cc;     // by record
+    uint32_t *offsets, *coff, *chunk_first;
+    uint32_t chunk_cap;
+    uint64_t *partials;  // as launch_scan_cells
+    uint64_t *n_pairs, *n_cells;
+    uint64_t capacity;
+    uint32_t *err;
+};
+// *in_alt: the order lies in vals_alt.
+cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *in_alt);
 // Output positions per entry of the scan's chunk table (a divisor of every
 // emit kernel's per-warp output range).
 constexpr uint32_t kEmitStride = 256;
