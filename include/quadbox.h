@@ -306,6 +306,10 @@ qb_status qb_render_bwd(qb_frame *frame, const qb_scene *scene, const qb_camera 
 /* One optimisation step around the rasteriser (training integration).       */
 /* ------------------------------------------------------------------------ */
 
+/* Zeroes the five gradient arrays of a scene of n Gaussians (device float32,
+ * shapes as qb_scene) in one launch, before a backward adds to them. */
+qb_status qb_scene_grads_zero(const qb_scene_grads *grads, int32_t n, int32_t sh_degree, qb_stream_t stream);
+
 /* L1 image loss: d_dL[i] = scale * sign(d_img[i] - d_target[i]) (0 where
  * equal), and, when d_loss is non-NULL, *d_loss += scale * sum |img - target|
  * (device double, accumulated; zero it first).  All device float [n].  With

@@ -105,6 +105,7 @@ _SIGS = [
     ("qb_render_fwd_counted", c_i32, [ctypes.POINTER(QbFrame), ctypes.POINTER(c_f), c_vp, c_vp, c_vp]),
     ("qb_render_bwd", c_i32, [ctypes.POINTER(QbFrame), ctypes.POINTER(QbScene), ctypes.POINTER(QbCamera),
                               ctypes.POINTER(c_f), c_vp, ctypes.POINTER(QbSceneGrads), c_vp, c_vp]),
+    ("qb_scene_grads_zero", c_i32, [ctypes.POINTER(QbSceneGrads), c_i32, c_i32, c_vp]),
     ("qb_l1_loss_grad", c_i32, [c_vp, c_vp, c_vp, c_u64, ctypes.c_float, c_vp, c_vp]),
     ("qb_adam_step", c_i32, [c_vp, c_vp, c_vp, c_vp, c_u64, ctypes.c_float, ctypes.c_float, ctypes.c_float,
                              ctypes.c_float, c_i32, c_vp]),
@@ -158,10 +159,28 @@ def check(status: int):
         raise QbError(status, msg)
 
 
-def stream_handle(stream=None):
+def _raw_stream():
+    """The current stream's handle as an int.  Looking it up through
+    torch.cuda.current_stream() builds a Stream object, 3 us of every call."""
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    try:
+        get, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    except AttributeError:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    torch.cuda.init()
+    return lambda: get(device())
+
+
+_current = None
+
+
+def stream_handle(stream=None):
+    global _current
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    if _current is None:
+        _current = _raw_stream()
+    return ctypes.c_void_p(_current())
 
 
 def ptr(t):
@@ -251,6 +270,10 @@ def qb_render_bwd(frame: QbFrame, scene: QbScene, camera: QbCamera, bg, dL_dimg,
                   grad_screen=None, stream=None):
     check(load().qb_render_bwd(ctypes.byref(frame), ctypes.byref(scene), ctypes.byref(camera), _bg(bg),
                                ptr(dL_dimg), ctypes.byref(grads), ptr(grad_screen), stream_handle(stream)))
+
+
+def qb_scene_grads_zero(grads: QbSceneGrads, n, sh_degree, stream=None):
+    check(load().qb_scene_grads_zero(ctypes.byref(grads), n, sh_degree, stream_handle(stream)))
 
 
 def qb_l1_loss_grad(img, target, dL, scale, loss=None, stream=None):

@@ -172,6 +172,42 @@ CamSet frame_camset(const qb_camera &c) {
     return cs;
 }
 
+// A word of mapped host memory per host thread, that the count scan writes P
+// to: a synchronised qb_bin_emit then waits for the stream only, without a
+// device-to-host copy behind the scan.  Freed when the thread ends.
+struct HostWord {
+    volatile uint64_t *host = nullptr;
+    uint64_t *device = nullptr;
+    bool tried = false;
+    bool get() {
+        if (!tried) {
+            tried = true;
+            void *h = nullptr, *d = nullptr;
+            // (an allocation must not disturb a graph capture of another thread)
+            cudaStreamCaptureMode capture = cudaStreamCaptureModeRelaxed;
+            (void)cudaThreadExchangeStreamCaptureMode(&capture);
+            const cudaError_t e = cudaHostAlloc(&h, sizeof(uint64_t), cudaHostAllocPortable | cudaHostAllocMapped);
+            (void)cudaThreadExchangeStreamCaptureMode(&capture);
+            if (e != cudaSuccess) {
+                (void)cudaGetLastError();
+                return false;
+            }
+            if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess || d != h) {  // one address on every device
+                (void)cudaGetLastError();
+                (void)cudaFreeHost(h);
+                return false;
+            }
+            host = static_cast<volatile uint64_t *>(h);
+            device = static_cast<uint64_t *>(d);
+        }
+        return host != nullptr;
+    }
+    ~HostWord() {
+        if (host) (void)cudaFreeHost(const_cast<uint64_t *>(host));
+    }
+};
+thread_local HostWord t_pairs;
+
 qb_status check_frame(const qb_frame *f, Layout &L) {
     if (!f || !f->workspace) return fail(QB_ERR_INVALID_ARG, "frame is NULL or not initialised");
     if (!make_layout(f->n, f->width, f->height, f->pair_capacity, L))
@@ -394,6 +430,7 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
     uint64_t *d_np = at<uint64_t>(frame, L.state);
     uint32_t *err = at<uint32_t>(frame, L.state + 8);
     const bool depth_first = frame->sort_mode != QB_SORT_FULL_KEY;  // Gaussians emitted in depth order
+    const bool mapped = n_pairs_out && frame->n > 0 && t_pairs.get();
     uint64_t *partials = at<uint64_t>(frame, L.scan_part);
     uint32_t *chunk_first = at<uint32_t>(frame, L.chunk_first);
     const uint32_t chunk_cap = (uint32_t)chunk_table_size(frame->pair_capacity);
@@ -414,6 +451,7 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
         o.chunk_cap = chunk_cap;
         o.partials = partials;
         o.n_pairs = d_np;
+        o.n_pairs_host = mapped ? t_pairs.device : nullptr;
         o.n_cells = at<uint64_t>(frame, L.state + 16);
         o.capacity = frame->pair_capacity;
         o.err = err;
@@ -422,13 +460,15 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
         frame->depth_in_alt = in_alt;
     } else {
         QB_CUDA(launch_scan(at<uint32_t>(frame, L.counts), frame->n, at<uint32_t>(frame, L.offsets),
-                            at<uint32_t>(frame, L.coff), partials, d_np, err, chunk_first, chunk_cap, s));
+                            at<uint32_t>(frame, L.coff), partials, d_np, mapped ? t_pairs.device : nullptr, err,
+                            chunk_first, chunk_cap, s));
     }
     frame->n_pairs = UINT64_MAX;
     if (n_pairs_out) {
         uint64_t P = 0;
-        QB_CUDA(cudaMemcpyAsync(&P, d_np, sizeof(P), cudaMemcpyDeviceToHost, s));
+        if (!mapped) QB_CUDA(cudaMemcpyAsync(&P, d_np, sizeof(P), cudaMemcpyDeviceToHost, s));
         QB_CUDA(cudaStreamSynchronize(s));
+        if (mapped) P = *t_pairs.host;
         *n_pairs_out = P;
         if (P > frame->pair_capacity) {
             frame->stage = 1;
@@ -603,6 +643,18 @@ qb_status qb_render_bwd(qb_frame *frame, const qb_scene *scene, const qb_camera 
     p.sh_vec4 = reinterpret_cast<uintptr_t>(scene->sh) % 16 == 0;
     p.gsh_vec4 = reinterpret_cast<uintptr_t>(grads->sh) % 16 == 0;
     QB_CUDA(launch_preprocess_bwd(p, scene->sh_degree, s));
+    return QB_OK;
+}
+
+qb_status qb_scene_grads_zero(const qb_scene_grads *grads, int32_t n, int32_t sh_degree, qb_stream_t stream) {
+    if (n < 0 || sh_degree < 0 || sh_degree > 3) return fail(QB_ERR_INVALID_ARG, "need n >= 0 and sh_degree in 0..3");
+    if (n == 0) return QB_OK;
+    if (!grads || !grads->means || !grads->scales || !grads->quats || !grads->opacities || !grads->sh)
+        return fail(QB_ERR_INVALID_ARG, "grads or a gradient array is NULL");
+    float *const p[5] = {grads->means, grads->scales, grads->quats, grads->opacities, grads->sh};
+    const uint64_t N = (uint64_t)n, K = (uint64_t)(sh_degree + 1) * (sh_degree + 1);
+    const uint64_t len[5] = {3 * N, 3 * N, 4 * N, N, 3 * K * N};
+    QB_CUDA(launch_zero5(p, len, (cudaStream_t)stream));
     return QB_OK;
 }
 

@@ -432,8 +432,8 @@ __device__ __forceinline__ void add_row(float *p, bool vec, const float (&Y)[16]
 // such a Gaussian is listed too: kMetaNonFinite.)  1M Gaussians at 1080p, a
 // sixth of them listed: 188 -> 72 us; 1024 Gaussians per block 80, 256 threads
 // per block 107.  Of several cameras' views nearly every Gaussian is in some,
-// where the list measured slower than a thread per Gaussian that passes over
-// the cameras with zero sums (220 against 156 us, five views of 200k).
+// where the list measured slower than a thread per Gaussian (220 against 166
+// us, five views of 200k).
 constexpr int kBwdSpan = 512, kBwdListThreads = 128;
 struct BwdList {
     uint32_t count;
@@ -497,20 +497,11 @@ __device__ __forceinline__ void preprocess_bwd_one(const PreBwdArgs &a, int i) {
         const size_t rec = (size_t)cam * a.n + i;
         const int meta = a.meta[rec];
         if (!(meta & kMetaVisible)) continue;
-        const double *gsd = a.g_screen + rec * 9;
-        if (!SINGLE) {
-            double g9[9];
-            bool zero = true;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) g9[k] = gsd[k];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) zero = zero && (__double_as_longlong(g9[k]) << 1) == 0;
-            if (zero && !(meta & kMetaNonFinite)) continue;
-        }
         const CamDev &cd = a.cams.cam[cam];
         Proj p;
         if (!project_gaussian(cd, m0, m1, m2, sc0, sc1, sc2, qw, qx, qy, qz, a.raw, p)) continue;
         any = true;
+        const double *gsd = a.g_screen + rec * 9;
         const float gmx = (float)gsd[0], gmy = (float)gsd[1];
         gop += (float)gsd[5];
         const float grgb[3] = {(float)gsd[6], (float)gsd[7], (float)gsd[8]};

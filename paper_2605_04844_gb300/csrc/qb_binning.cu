@@ -68,7 +68,7 @@ struct ScanArgs {
     uint32_t chunk_cap;
     ScanWord *status;  // one per block, zero
     uint32_t *counter;
-    uint64_t *n_pairs, *n_cells;
+    uint64_t *n_pairs, *n_pairs_host, *n_cells;
     uint64_t capacity;
     uint32_t *err;
 };
@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
         if ((int)b == nb - 1) {
             const uint64_t P = acc + ctot, E = accd + dtot;
             *A.n_pairs = P;
+            if (A.n_pairs_host) *A.n_pairs_host = P;
             // (E <= P: cell_entries)
             if (DUAL) *A.n_cells = P <= A.capacity && E <= A.capacity ? E : 0ull;
         }
@@ -233,8 +234,10 @@ static cudaError_t run_scan(ScanArgs A, uint64_t *partials, bool dual, cudaStrea
 }
 
 cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32_t *counts_e, uint64_t *partials,
-                        uint64_t *n_pairs, uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s) {
+                        uint64_t *n_pairs, uint64_t *n_pairs_host, uint32_t *err, uint32_t *chunk_first,
+                        uint32_t chunk_cap, cudaStream_t s) {
     ScanArgs A{};
+    A.n_pairs_host = n_pairs_host;
     A.counts = counts;
     A.n = n;
     A.offsets = offsets;
@@ -247,9 +250,11 @@ cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32
 }
 
 cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint32_t *offsets, uint32_t *coff,
-                              uint64_t *partials, uint64_t *n_pairs, uint64_t *n_cells, uint64_t capacity,
-                              uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s) {
+                              uint64_t *partials, uint64_t *n_pairs, uint64_t *n_pairs_host, uint64_t *n_cells,
+                              uint64_t capacity, uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap,
+                              cudaStream_t s) {
     ScanArgs A{};
+    A.n_pairs_host = n_pairs_host;
     A.chunk_first = chunk_first;
     A.chunk_cap = chunk_cap;
     A.cc = cc;

@@ -235,12 +235,15 @@ cudaError_t launch_preprocess(const PreArgs &a, int deg, cudaStream_t s);
 // the block counter), 16-byte aligned, cleared by the launch; a look-back that
 // waits too long raises kErrTimeout in *err.  launch_scan: the counts in index
 // order (full-key path).  launch_scan_cells: (tiles, cells) in the order perm;
-// *n_cells becomes 0 when the pairs exceed the capacity.
+// *n_cells becomes 0 when the pairs exceed the capacity.  n_pairs_host, when
+// not null, is a device address of mapped host memory that also gets P (n > 0).
 cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32_t *counts_e, uint64_t *partials,
-                        uint64_t *n_pairs, uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s);
+                        uint64_t *n_pairs, uint64_t *n_pairs_host, uint32_t *err, uint32_t *chunk_first,
+                        uint32_t chunk_cap, cudaStream_t s);
 cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint32_t *offsets, uint32_t *coff,
-                              uint64_t *partials, uint64_t *n_pairs, uint64_t *n_cells, uint64_t capacity,
-                              uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap, cudaStream_t s);
+                              uint64_t *partials, uint64_t *n_pairs, uint64_t *n_pairs_host, uint64_t *n_cells,
+                              uint64_t capacity, uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap,
+                              cudaStream_t s);
 // The depth order of n Gaussians (keys and record indices from the
 // preprocess) and the scan in that order.
 struct OrderArgs {
@@ -250,7 +253,7 @@ struct OrderArgs {
     uint32_t *offsets, *coff, *chunk_first;
     uint32_t chunk_cap;
     uint64_t *partials;  // as launch_scan_cells
-    uint64_t *n_pairs, *n_cells;
+    uint64_t *n_pairs, *n_pairs_host, *n_cells;  // n_pairs_host as launch_scan
     uint64_t capacity;
     uint32_t *err;
 };
@@ -283,6 +286,7 @@ cudaError_t launch_render(const RenderArgs &a, cudaStream_t s);
 cudaError_t launch_tile_work(const RenderArgs &a, cudaStream_t s);
 cudaError_t launch_l1_grad(const float *img, const float *target, float *dL, uint64_t n, float scale, double *loss,
                            cudaStream_t s);
+cudaError_t launch_zero5(float *const p[5], const uint64_t n[5], cudaStream_t s);
 cudaError_t launch_adam(float *p, const float *g, float *m, float *v, uint64_t n, float lr, float b1, float b2,
                         float eps, int t, cudaStream_t s);
 cudaError_t launch_render_bwd(const BwdArgs &a, cudaStream_t s);

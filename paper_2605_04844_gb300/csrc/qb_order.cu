@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(kOrderThreads) depth_order_small_kernel(OrderA
     }
     if (rank_cta == 0 && tid == 0) {
         *a.n_pairs = P;
+        if (a.n_pairs_host) *a.n_pairs_host = P;
         *a.n_cells = P <= a.capacity && E <= a.capacity ? E : 0ull;  // (E <= P: cell_entries)
     }
 #pragma unroll
@@ -254,7 +255,7 @@ cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *
     }
     *in_alt = passes & 1;
     return launch_scan_cells(a.cc, *in_alt ? a.vals_alt : a.vals, n, a.offsets, a.coff, a.partials, a.n_pairs,
-                             a.n_cells, a.capacity, a.err, a.chunk_first, a.chunk_cap, s);
+                             a.n_pairs_host, a.n_cells, a.capacity, a.err, a.chunk_first, a.chunk_cap, s);
 }
 
 }  // namespace qb

@@ -90,6 +90,26 @@ __global__ void __launch_bounds__(256) adam_kernel(float *__restrict__ p, const 
     }
 }
 
+// Zeroes five arrays in one launch (the gradients of a scene, before the
+// backward adds to them).
+struct Zero5 {
+    float *p[5];
+    uint64_t n[5];
+};
+__global__ void __launch_bounds__(256) zero5_kernel(Zero5 z) {
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, threads = (uint64_t)gridDim.x * blockDim.x;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        uint64_t i0 = 0;
+        if ((reinterpret_cast<uintptr_t>(z.p[k]) & 15) == 0) {
+            const uint64_t n4 = z.n[k] / 4;
+            for (uint64_t i = t; i < n4; i += threads) reinterpret_cast<float4 *>(z.p[k])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            i0 = 4 * n4;
+        }
+        for (uint64_t i = i0 + t; i < z.n[k]; i += threads) z.p[k][i] = 0.f;
+    }
+}
+
 static unsigned grid_for(uint64_t n) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -102,6 +122,19 @@ cudaError_t launch_l1_grad(const float *img, const float *target, float *dL, uin
                            cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     note_launch("l1_grad_kernel", s), l1_grad_kernel<<<grid_for(n), 256, 0, s>>>(img, target, dL, n, scale, loss);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_zero5(float *const p[5], const uint64_t n[5], cudaStream_t s) {
+    Zero5 z;
+    uint64_t most = 0;
+    for (int k = 0; k < 5; ++k) {
+        z.p[k] = p[k];
+        z.n[k] = n[k];
+        most = n[k] > most ? n[k] : most;
+    }
+    if (most == 0) return cudaSuccess;
+    note_launch("zero5_kernel", s), zero5_kernel<<<grid_for((most + 3) / 4), 256, 0, s>>>(z);
     return cudaGetLastError();
 }
 

@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import math
 
+import numpy as np
 import torch
 
 from . import _native as N
@@ -26,16 +27,19 @@ def mode_id(mode) -> int:
     return int(mode)
 
 
+def _floats(v, n):
+    """n Python floats from an array, tensor or sequence."""
+    if isinstance(v, np.ndarray) and v.size == n:  # without the way through a tensor: 17 us of a call
+        return v.astype(np.float64).ravel().tolist()
+    return [float(x) for x in torch.as_tensor(v, dtype=torch.float64).reshape(n).tolist()]
+
+
 def camera_struct(cam) -> N.QbCamera:
     c = N.QbCamera()
-    vm = [float(v) for v in torch.as_tensor(cam["viewmat"], dtype=torch.float64).reshape(16).tolist()]
-    for i in range(16):
-        c.viewmat[i] = vm[i]
+    c.viewmat[:] = _floats(cam["viewmat"], 16)
     c.fx, c.fy, c.cx, c.cy = float(cam["fx"]), float(cam["fy"]), float(cam["cx"]), float(cam["cy"])
     c.tan_fovx, c.tan_fovy = float(cam["tan_fovx"]), float(cam["tan_fovy"])
-    cp = [float(v) for v in torch.as_tensor(cam["campos"], dtype=torch.float64).reshape(3).tolist()]
-    for i in range(3):
-        c.campos[i] = cp[i]
+    c.campos[:] = _floats(cam["campos"], 3)
     c.width, c.height = int(cam["width"]), int(cam["height"])
     c.znear = float(cam.get("znear", 0.2))
     return c
@@ -221,10 +225,11 @@ class QuadBoxRasterize(torch.autograd.Function):
         means, scales, quats, opacities, sh = ctx.saved_tensors
         scene = {"means": means, "scales": scales, "quats": quats, "opacities": opacities, "sh": sh,
                  "sh_degree": ctx.deg, "raw": 1}
-        g = {k: torch.zeros_like(v) for k, v in scene.items() if isinstance(v, torch.Tensor)}
+        g = {k: torch.empty_like(v) for k, v in scene.items() if isinstance(v, torch.Tensor)}
         gs = N.QbSceneGrads()
         gs.means, gs.scales, gs.quats = g["means"].data_ptr(), g["scales"].data_ptr(), g["quats"].data_ptr()
         gs.opacities, gs.sh = g["opacities"].data_ptr(), g["sh"].data_ptr()
+        N.qb_scene_grads_zero(gs, int(means.shape[0]), ctx.deg, ctx.frame.stream)
         N.qb_render_bwd(ctx.frame.frame, scene_struct(scene), camera_struct(ctx.cam), ctx.bg,
                         grad_img.contiguous(), gs, None, ctx.frame.stream)
         return g["means"], g["scales"], g["quats"], g["opacities"], g["sh"], None, None, None
@@ -378,8 +383,7 @@ class Trainer:
         fr.render(self.bg, self.img)
         self.loss.zero_()
         N.qb_l1_loss_grad(self.img, target, self.dL, 1.0 / self.img.numel(), self.loss, s)
-        for g in self.grads.values():
-            g.zero_()
+        N.qb_scene_grads_zero(self.gs, self.scene_s.n, self.scene_s.sh_degree, s)
         N.qb_render_bwd(fr.frame, self.scene_s, self.cam_s, self.bg, self.dL, self.gs, None, s)
         self.t += 1
         for k in self.KEYS:
