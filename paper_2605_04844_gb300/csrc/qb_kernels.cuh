@@ -19,7 +19,7 @@ struct PreArgs {
     bool raw;
     bool sh_vec4;    // sh rows may be read as float4 (16-byte aligned)
     bool quat_vec4;  // quats may be read as float4 (16-byte aligned)
-    CamSet cams;     // one grid row per camera
+    CamSet cams;
     int mode;
     bool clamp3s;
     float2 *xy;      // [n_cams * n] ...
@@ -198,6 +198,9 @@ struct RenderArgs {
     // tile b; with order_out.cnt set, every tile is filed by its largest
     // last-contributor count (the backward's work)
     TileOrder order, order_out;
+    // with order_known.cnt set every tile is filed there too, as in order_out
+    // (frames whose blocks take the tiles in index order)
+    TileOrder order_known;
 };
 
 struct BwdArgs {
