@@ -184,7 +184,8 @@ typedef struct {
                                    are then undefined (do not render them)  */
     uint32_t *order_counts; /* [2][64] tiles per work bucket, written by the
                                    forward render: [0] the render's order (by
-                                   an estimate of each tile's work), [1] the
+                                   an estimate of each tile's work; on frames
+                                   rendered in index order as [1]), [1] the
                                    backward's (by the tile's largest
                                    n_contrib); bucket j holds work in
                                    [16 (63 - j), 16 (64 - j)), bucket 0 all
@@ -270,11 +271,12 @@ qb_status qb_sort(qb_frame *frame, qb_stream_t stream);
 /* Stage 4 (Sec. 2 "Render", Eq. 2): front-to-back compositing per pixel.
  * bg: host float[3] background colour (NULL = black).  d_img: device
  * float [3][height][width] (planar RGB), fully overwritten.  Also writes the
- * frame's t_final and n_contrib, which qb_render_bwd needs.  The tiles run
- * heaviest first: a first kernel files every tile by an estimate of its work
- * (order_counts[0] / order_lists[0] of qb_frame_arrays), and the render files
- * every tile again by its largest n_contrib for qb_render_bwd (the second
- * order); the image does not depend on the order. */
+ * frame's t_final and n_contrib, which qb_render_bwd needs.  The tiles of a
+ * frame of few tiles run heaviest first: a first kernel files every tile by an
+ * estimate of its work (order_counts[0] / order_lists[0] of qb_frame_arrays);
+ * those of a larger one run in index order, and that order is filed by the
+ * render.  The render files every tile by its largest n_contrib for
+ * qb_render_bwd (the second order); the image does not depend on the order. */
 qb_status qb_render_fwd(qb_frame *frame, const float *bg, float *d_img, qb_stream_t stream);
 
 /* Measurement only: qb_render_fwd (identical outputs) that also adds, over

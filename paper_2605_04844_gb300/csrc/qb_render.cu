@@ -242,21 +242,26 @@ __global__ void __launch_bounds__(kRenderThreads) render_kernel(RenderArgs a) {
         const int m = __reduce_max_sync(0xffffffffu, last);
         if ((threadIdx.x & 31) == 0) s_last[wid] = m;
         __syncthreads();
-        if (threadIdx.x == 0) order_file(a.order_out, a.ts.total_tiles, t, (uint32_t)max(s_last[0], s_last[1]));
+        if (threadIdx.x == 0) {
+            const uint32_t walked = (uint32_t)max(s_last[0], s_last[1]);
+            order_file(a.order_out, a.ts.total_tiles, t, walked);
+            if (a.order_known.cnt) order_file(a.order_known, a.ts.total_tiles, t, walked);
+        }
     }
 }
 
-// A warp per tile walks the tile's list 32 entries at a time for four sample
-// pixels (offsets 3 and 12 in x and y): each lane takes one entry's
+// A warp per tile walks the tile's list 32 entries at a time for two sample
+// pixels (offsets (3, 4) and (12, 11); four measured the same render and a
+// third more here): each lane takes one entry's
 // 1 - alpha at each pixel (the render's accept rules on the plain conic
 // form), a product scan over the lanes gives the transmittance after every
 // entry, and the first entry that takes a pixel below the stop ends that
 // pixel.  The estimate is the largest stop position, or the list length when
 // a pixel has not stopped within kWorkChunks chunks.  The next chunk's
 // records and the one after's indices are loaded while a chunk is scanned.
-constexpr int kWorkPix = 4;  // sample pixels per tile, at these offsets in the tile
-__device__ constexpr int kWorkX[kWorkPix] = {3, 12, 3, 12};
-__device__ constexpr int kWorkY[kWorkPix] = {3, 3, 12, 12};
+constexpr int kWorkPix = 2;  // sample pixels per tile, at these offsets in the tile
+__device__ constexpr int kWorkX[kWorkPix] = {3, 12};
+__device__ constexpr int kWorkY[kWorkPix] = {4, 11};
 constexpr uint32_t kWorkChunks = 32;  // beyond 1024 entries every tile files into the top bucket
 __global__ void __launch_bounds__(256) tile_work_kernel(RenderArgs a) {
     const int lane = threadIdx.x & 31;
