@@ -30,7 +30,8 @@
 //
 // The kernel is bound by latency between dependent packed operations at 20
 // warps per SM (96 registers; issue 65 %, FMA pipe 52 %).  1M Gaussians at
-// 1080p 461 -> 357 us, 5 views of 200k (persistent) 2023 -> 1710; 80 or 88
+// 1080p 461 -> 357 us, 5 views of 200k (persistent) 2023 -> 1710 (with the
+// ellipse test of elongated Gaussians 326 and 1530); 80 or 88
 // registers (12 or 11 blocks per SM) measured 3 to 6 % slower.
 //
 // K8: one thread per Gaussian with any nonzero sum chains the (mu^2D, Sigma2D, o, colour)

@@ -28,10 +28,13 @@
 // barriers and walked the set bits of a mask, a warp of its own needs no
 // barrier, ends with its own pixels, and its compacted list has no bit scan:
 // 1M Gaussians at 1080p 229 -> 181 us, 3M at 1440p seen from inside 1034 ->
-// 911, 1M at 2160p 816 -> 653, 16 views of 1M (persistent) 3340 -> 2670.
+// 911, 1M at 2160p 816 -> 653, 16 views of 1M (persistent) 3340 -> 2670; with
+// the ellipse test of elongated Gaussians too (qb_internal.cuh; in index order)
+// 174, 485, 578 and 2140.
 // Measured slower: 64 registers (32 warps per SM, spills), two entries'
 // exponents ahead of both blends, the next entry's operands loaded ahead
-// (+21 %), T chosen by a select instead of multiplied by 1 - 0.
+// (+21 %), T chosen by a select instead of multiplied by 1 - 0, a blend of the
+// pair of rows that an entry reaches alone (where most reach both).
 #include "qb_stage.cuh"
 
 namespace qb {
@@ -226,11 +229,12 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
     return max(max(P[0].last0, P[0].last1), max(P[1].last0, P[1].last1));
 }
 
-// One block per tile of a single camera, a warp per half; with an order, the
+// One block per tile of a single camera, a warp per half (72 registers, 14
+// blocks per SM; unbounded the compiler takes 77, 12 blocks); with an order, the
 // blocks (which start roughly in index order) take the heaviest tiles first,
 // so that the last blocks to start are short ones.
 template <bool COUNT>
-__global__ void __launch_bounds__(kRenderThreads) render_kernel(RenderArgs a) {
+__global__ void __launch_bounds__(kRenderThreads, COUNT ? 1 : 14) render_kernel(RenderArgs a) {
     __shared__ RenderStage s_stage[2];
     __shared__ int s_last[2];
     const int wid = threadIdx.x >> 5;

@@ -81,7 +81,7 @@ __device__ __forceinline__ int stage_entries(RenderStage &S, bool have, int pos,
         co = S.raw_co[lane];
         rgb = S.raw_rgb[lane];
         skip = skip_threshold(co.w);
-        hit = ellipse_meets_rect(m.x, m.y, co.x, co.y, co.z, skip, sh.y != 0.f, x0, y0, x0 + 15.f, y0 + 7.f);
+        hit = ellipse_meets_rect(m.x, m.y, co.x, co.y, co.z, skip, sh, x0, y0, x0 + 15.f, y0 + 7.f);
     }
     const uint32_t hits = __ballot_sync(0xffffffffu, hit);
     if (hit) {
