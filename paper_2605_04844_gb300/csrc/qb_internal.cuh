@@ -115,9 +115,10 @@ cudaError_t sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint3
 constexpr float kElongatedF2 = 0.01f;  // f < 0.1: aspect ratio above 10 : 1
 
 // Exponents below this give alpha = o e^power < (1/255) e^-0.001: the 1e-3
-// margin is far wider than the float32 error of the alpha test, so skipping
-// them first never changes a decision of that test.
-__device__ __forceinline__ float skip_threshold(float o) { return -logf(255.0f * o) - 1e-3f; }
+// margin is far wider than the float32 error of the alpha test (and of the
+// fast logarithm, 4e-7 absolute here), so skipping them first never changes a
+// decision of that test.
+__device__ __forceinline__ float skip_threshold(float o) { return -__logf(255.0f * o) - 1e-3f; }
 
 // e^x of both lanes as 2^(x log2 e), for the exponents of the compositing
 // (at least skip_threshold, so the result is no subnormal and ex2's
@@ -134,10 +135,11 @@ __device__ __forceinline__ float2 exp2_of(float2 x) {
 // Whether some point of the pixel rectangle [x0, x1] x [y0, y1] can give the
 // Gaussian (mu^2D, conic (a, b, c)) an exponent above t, i.e. whether the
 // rectangle meets the ellipse q(d) = a dx^2 + 2 b dx dy + c dy^2 <= -2t,
-// d = mu^2D - pixel.  q is convex, so its minimum over the rectangle is 0 when
-// mu^2D lies inside and otherwise lies on an edge, where it is the 1D
-// minimiser clamped to the edge.  The test is conservative: the radius gets a
-// 1 % + 0.01 margin, far above the float32 error of q and of the kernels'
+// d = mu^2D - pixel.  q is convex with its minimum at d = 0, so over the
+// rectangle it is smallest on an edge that faces d = 0 (or there, inside): at
+// the 1D minimiser, clamped, on the lines through the rectangle's point
+// nearest to 0 in x and in y.  The test is conservative: the radius gets a 1 %
+// + 0.01 margin, far above the float32 error of q and of the kernels'
 // exponents.  A degenerate conic always meets the rectangle.
 //
 // An elongated conic (shape = (r, -e/2) with r = b / a, e = 1 / Sigma22, not
@@ -154,28 +156,21 @@ __device__ __forceinline__ bool ellipse_meets_rect(float mx, float my, float a, 
     if (!(a > 0.f && c > 0.f)) return true;
     const float r2 = fmaxf(-2.f * t, 0.f) * 1.01f + 1e-2f;
     const float ul = mx - x1, uh = mx - x0, vl = my - y1, vh = my - y0;
-    if (ul <= 0.f && uh >= 0.f && vl <= 0.f && vh >= 0.f) return true;
     const bool elongated = shape.y != 0.f;
-    const float ic = 1.f / c, ir = elongated ? shape.x : b * (1.f / a), e = -2.f * shape.y;
-    float best = INFINITY;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float v = k ? vh : vl;  // horizontal edge: dy fixed
-        const float u = fminf(fmaxf(-ir * v, ul), uh);
-        const float u2 = k ? uh : ul;  // vertical edge: dx fixed
-        const float v2 = fminf(fmaxf(-b * u2 * ic, vl), vh);
-        float q, q2;
-        if (elongated) {
-            const float w = fmaf(ir, v, u), w2 = fmaf(ir, v2, u2);
-            q = fmaf(a * w, w, e * v * v);
-            q2 = fmaf(a * w2, w2, e * v2 * v2);
-        } else {
-            q = fmaf(a * u, u, fmaf(2.f * b * u, v, c * v * v));
-            q2 = fmaf(a * u2, u2, fmaf(2.f * b * u2, v2, c * v2 * v2));
-        }
-        best = fminf(best, fminf(q, q2));
+    const float ir = elongated ? shape.x : __fdividef(b, a);
+    // on the vertical line dx = u1, and on the horizontal line dy = v2
+    const float u1 = fminf(fmaxf(0.f, ul), uh), v1 = fminf(fmaxf(-__fdividef(b, c) * u1, vl), vh);
+    const float v2 = fminf(fmaxf(0.f, vl), vh), u2 = fminf(fmaxf(-ir * v2, ul), uh);
+    float q1, q2;
+    if (elongated) {
+        const float e = -2.f * shape.y, w1 = fmaf(ir, v1, u1), w2 = fmaf(ir, v2, u2);
+        q1 = fmaf(a * w1, w1, e * v1 * v1);
+        q2 = fmaf(a * w2, w2, e * v2 * v2);
+    } else {
+        q1 = fmaf(a * u1, u1, fmaf(2.f * b * u1, v1, c * v1 * v1));
+        q2 = fmaf(a * u2, u2, fmaf(2.f * b * u2, v2, c * v2 * v2));
     }
-    return !(best > r2);
+    return !(fminf(q1, q2) > r2);
 }
 
 struct Rect {
