@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(1024) sort_hist_scan_kernel(uint32_t *hist, Pa
 
 // One digit pass of the pair sort, ITEMS keys per thread.
 template <int RB, typename KeyT, int ITEMS>
-__global__ void __launch_bounds__(kSortBlock, sizeof(KeyT) == 4 ? kSortBlocksPerSM : 3) onesweep_kernel(const KeyT *__restrict__ kin,
+__global__ void __launch_bounds__(kSortBlock, sizeof(KeyT) == 4 ? kSortBlocksPerSM : RB <= 9 ? kSortBlocksPerSM64 : 3) onesweep_kernel(const KeyT *__restrict__ kin,
                                                               const uint32_t *__restrict__ vin,
                                                               KeyT *__restrict__ kout, uint32_t *__restrict__ vout,
                                                               uint64_t n_max, const uint64_t *n_dev,
@@ -161,7 +161,7 @@ template <int RB, typename KeyT, int ITEMS>
 static cudaError_t launch_pass_t(const KeyT *kin, const uint32_t *vin, KeyT *kout, uint32_t *vout, uint64_t n_max,
                                  const uint64_t *n_dev, const uint32_t *bin_off, uint32_t *lookback,
                                  uint32_t *counter, int shift, uint32_t mask, uint32_t *err, cudaStream_t s) {
-    constexpr size_t smem = sweep_smem<RB, uint32_t, ITEMS>();
+    constexpr size_t smem = sweep_smem<RB, KeyT, uint32_t, ITEMS>();
     cudaError_t e = ensure_dyn_smem((const void *)onesweep_kernel<RB, KeyT, ITEMS>, smem);
     if (e != cudaSuccess) return e;
     note_launch("onesweep_kernel", s), onesweep_kernel<RB, KeyT, ITEMS><<<(unsigned)((n_max + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS)), kSortBlock, smem, s>>>(
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kSortBlock, RB <= 8 ? kCellSortBlocksPerSM : 2
 template <int RB, bool WRITE_KEYS>
 static cudaError_t launch_cell_pass(const CellBin &b, int p, const uint32_t *kin, const uint64_t *vin, uint32_t *kout,
                                     uint64_t *vout, cudaStream_t s) {
-    constexpr size_t smem = sweep_smem<RB, uint64_t>();
+    constexpr size_t smem = sweep_smem<RB, uint32_t, uint64_t, kSortItems>();
     cudaError_t e = ensure_dyn_smem((const void *)cell_sort_kernel<RB, WRITE_KEYS>, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;

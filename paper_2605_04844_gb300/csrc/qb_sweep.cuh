@@ -23,6 +23,7 @@ constexpr int kSortBlock = 256;
 constexpr int kSortWarps = kSortBlock / 32;
 constexpr int kSortItems = 16;  // keys per thread (fewer for short sorts of 32-bit keys: sort_items_u32)
 constexpr int kSortBlocksPerSM = 5;  // resident pass blocks per SM the registers are sized for (32-bit keys)
+constexpr int kSortBlocksPerSM64 = 4;  // with 64-bit keys (three: 5 % slower)
 constexpr int kSortTile = kSortBlock * kSortItems;  // 4096 keys per block
 constexpr int kSpinLimit = 1 << 22;
 constexpr int kLookWindow = 8;  // status words fetched per look-back step (16, 24, 32 measured slower)
@@ -113,18 +114,17 @@ __device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t v, uint32_t *to
     return incl - v + before;
 }
 
-// Shared memory of one pass: the scatter buffer ((key, value) pairs for 32-bit
-// keys; keys, then values, for 64-bit keys; values and keys side by side for
-// 64-bit values), per-warp digit counters, and per-digit global base, local
-// start and tile count.
-template <typename ValT, int ITEMS = kSortItems>
+// Shared memory of one pass: the scatter buffer ((key, value) pairs when both
+// have 32 bits; the 64-bit ones, then the 32-bit ones, otherwise), per-warp
+// digit counters, and per-digit global base, local start and tile count.
+template <typename KeyT, typename ValT, int ITEMS>
 constexpr size_t sweep_stage() {
-    return (size_t)kSortBlock * ITEMS * (sizeof(ValT) == 8 ? 12 : 8);
+    return (size_t)kSortBlock * ITEMS * (sizeof(KeyT) + sizeof(ValT));
 }
 
-template <int RB, typename ValT = uint32_t, int ITEMS = kSortItems>
+template <int RB, typename KeyT, typename ValT, int ITEMS>
 constexpr size_t sweep_smem() {
-    return sweep_stage<ValT, ITEMS>() + (size_t)kSortWarps * (1 << RB) * 2 + (size_t)3 * (1 << RB) * 4;
+    return sweep_stage<KeyT, ValT, ITEMS>() + (size_t)kSortWarps * (1 << RB) * 2 + (size_t)3 * (1 << RB) * 4;
 }
 
 // One pass over the tile `tile` (positions [tbase, tbase + kSortTile) of n) on the
@@ -140,10 +140,10 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val
                                            const uint32_t *__restrict__ bin_off, uint32_t *lookback, int shift,
                                            uint32_t mask, uint32_t *err, KeyT *__restrict__ kout,
                                            ValT *__restrict__ vout, uint8_t *smem) {
-    static_assert(sizeof(ValT) == 4 || sizeof(KeyT) == 4, "64-bit values go with 32-bit keys");
+    static_assert(sizeof(KeyT) + sizeof(ValT) <= 12, "64-bit values go with 32-bit keys");
     constexpr int R = 1 << RB;
     constexpr int PER = (R + kSortBlock - 1) / kSortBlock;
-    uint16_t *s_whist = reinterpret_cast<uint16_t *>(smem + sweep_stage<ValT, ITEMS>());
+    uint16_t *s_whist = reinterpret_cast<uint16_t *>(smem + sweep_stage<KeyT, ValT, ITEMS>());
     uint32_t *s_gbase = reinterpret_cast<uint32_t *>(s_whist + kSortWarps * R);
     uint32_t *s_lstart = s_gbase + R;
     uint32_t *s_bcount = s_lstart + R;
@@ -221,7 +221,7 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val
     // buffer while the look-back needs the registers, and every thread reads back
     // its own (a pass 32 -> 30 us; no gain for the other forms)
     uint16_t *s_rank = reinterpret_cast<uint16_t *>(smem) + tid;
-    if constexpr (sizeof(ValT) == 8) {
+    if constexpr (sizeof(KeyT) + sizeof(ValT) == 12) {
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) s_rank[k * kSortBlock] = (uint16_t)rank[k];
     }
@@ -297,23 +297,26 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val
             r += c;
         }
     }
-    if constexpr (sizeof(ValT) == 8) {
+    if constexpr (sizeof(KeyT) + sizeof(ValT) == 12) {
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) rank[k] = s_rank[k * kSortBlock];
     }
     __syncthreads();
 
     const uint32_t tcount = min(n - tbase, (uint32_t)(kSortBlock * ITEMS));
-    if constexpr (sizeof(ValT) == 8) {
-        // ---- values and keys to block order in shared memory, then out ----
-        ValT *s_val = reinterpret_cast<ValT *>(smem);
-        uint32_t *s_key = reinterpret_cast<uint32_t *>(smem + (size_t)kSortBlock * ITEMS * 8);
+    if constexpr (sizeof(KeyT) + sizeof(ValT) == 12) {
+        // ---- keys and values to block order in shared memory, then out ----
+        // (both at once: keys and values in turn through one buffer took a
+        // barrier more and kept every key's destination in a register)
+        constexpr size_t kWide = (size_t)kSortBlock * ITEMS * 8;  // the 64-bit ones come first
+        KeyT *s_key = reinterpret_cast<KeyT *>(smem + (sizeof(KeyT) == 8 ? 0 : kWide));
+        ValT *s_val = reinterpret_cast<ValT *>(smem + (sizeof(KeyT) == 8 ? kWide : 0));
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
             if (32 * k + lane < wcount) {
                 const uint32_t d = dig(k);
                 const uint32_t j = s_lstart[d] + s_whist[wid * R + d] + rank[k];
-                s_key[j] = (uint32_t)key[k];
+                s_key[j] = key[k];
                 s_val[j] = val(k);
             }
         }
@@ -322,15 +325,15 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val
         for (int k = 0; k < ITEMS; ++k) {
             const uint32_t j = tid + k * kSortBlock;
             if (j < tcount) {
-                const uint32_t kk = s_key[j];
-                const uint32_t dest = s_gbase[(kk >> shift) & mask] + j;
+                const KeyT kk = s_key[j];
+                const uint32_t dest = s_gbase[(uint32_t)(kk >> shift) & mask] + j;
                 if (dest < n) {  // dest >= n only after a look-back timeout
-                    if (WRITE_KEYS) kout[dest] = (KeyT)kk;
+                    if (WRITE_KEYS) kout[dest] = kk;
                     vout[dest] = s_val[j];
                 }
             }
         }
-    } else if constexpr (sizeof(KeyT) == 4) {
+    } else {
         // ---- (key, value) pairs to block order in shared memory, then out ----
         uint2 *s_pairs = reinterpret_cast<uint2 *>(smem);
 #pragma unroll
@@ -353,42 +356,6 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val
                     vout[dest] = kv.y;
                 }
             }
-        }
-    } else {
-        // ---- keys: scatter to block order in shared memory, then out ----
-        KeyT *s_keys = reinterpret_cast<KeyT *>(smem);
-        uint32_t *s_vals = reinterpret_cast<uint32_t *>(smem);
-#pragma unroll
-        for (int k = 0; k < ITEMS; ++k) {
-            if (32 * k + lane < wcount) {
-                const uint32_t d = dig(k);
-                const uint32_t lr = s_lstart[d] + s_whist[wid * R + d] + rank[k];
-                s_keys[lr] = key[k];
-                rank[k] = lr;
-            }
-        }
-        __syncthreads();
-        uint32_t dest[ITEMS];
-#pragma unroll
-        for (int k = 0; k < ITEMS; ++k) {
-            const uint32_t j = tid + k * kSortBlock;
-            if (j < tcount) {
-                const KeyT kk = s_keys[j];
-                const uint32_t d = (uint32_t)(kk >> shift) & mask;
-                dest[k] = s_gbase[d] + j;
-                if (WRITE_KEYS && dest[k] < n) kout[dest[k]] = kk;
-            }
-        }
-        __syncthreads();
-        // ---- values through the same permutation ----
-#pragma unroll
-        for (int k = 0; k < ITEMS; ++k)
-            if (32 * k + lane < wcount) s_vals[rank[k]] = val(k);
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < ITEMS; ++k) {
-            const uint32_t j = tid + k * kSortBlock;
-            if (j < tcount && dest[k] < n) vout[dest[k]] = s_vals[j];
         }
     }
 }
