@@ -30,58 +30,43 @@ __global__ void __launch_bounds__(256) sort_hist_kernel(const KeyT *__restrict__
                                                         uint32_t *done) {
     extern __shared__ uint32_t sh[];  // passes x 2^bits[p], packed
     __shared__ bool s_last;
-    int off[kMaxPasses], total = 0;
-    for (int p = 0; p < g.passes; ++p) {
+    int off[kMaxPasses], total = 0;  // (indexed by unrolled loops only: registers)
+#pragma unroll
+    for (int p = 0; p < kMaxPasses; ++p) {
         off[p] = total;
-        total += 1 << g.bits[p];
+        total += p < g.passes ? 1 << g.bits[p] : 0;
     }
     for (int j = threadIdx.x; j < total; j += blockDim.x) sh[j] = 0u;
     __syncthreads();
     const uint64_t n = device_count(n_dev, n_max);
-    // Each thread takes 8 consecutive keys and adds a run of equal digits
-    // once: keys in emission order repeat their high digits (the tiles of
-    // one Gaussian), which would otherwise be conflicting shared atomics.
+    // J keys in flight per thread, consecutive lanes reading consecutive keys.
+    // (Additions of one to the same word by several lanes of a warp are one
+    // operation, so a thread's runs of equal digits are not collected first; that,
+    // and the pass loops unrolled instead of indexing local arrays: 5M 64-bit keys
+    // 39 -> 28 us, 1M 32-bit keys 17 -> 14.)
     constexpr int J = 8;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * J;
-    for (uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * J; i0 < n; i0 += stride) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += J * stride) {
         KeyT k[J];
-        if (sizeof(KeyT) == 4 && i0 + J <= n && (reinterpret_cast<uintptr_t>(keys) & 15) == 0) {
-            // two 16-byte loads (i0 is a multiple of 8; callers' buffers may be unaligned)
-            const uint4 a = reinterpret_cast<const uint4 *>(keys + i0)[0];
-            const uint4 b = reinterpret_cast<const uint4 *>(keys + i0)[1];
-            k[0] = (KeyT)a.x, k[1] = (KeyT)a.y, k[2] = (KeyT)a.z, k[3] = (KeyT)a.w;
-            k[4] = (KeyT)b.x, k[5] = (KeyT)b.y, k[6] = (KeyT)b.z, k[7] = (KeyT)b.w;
-        } else {
 #pragma unroll
-            for (int j = 0; j < J; ++j) k[j] = i0 + j < n ? keys[i0 + j] : KeyT(0);
-        }
-        const int m = (int)(n - i0 < (uint64_t)J ? n - i0 : (uint64_t)J);
-        for (int p = 0; p < g.passes; ++p) {
-            const KeyT msk = (KeyT(1) << g.bits[p]) - 1;
-            const int sh_p = g.shift[p];
-            int run_d = (int)((k[0] >> sh_p) & msk);
-            uint32_t run_c = 1;
+        for (int j = 0; j < J; ++j) k[j] = i0 + j * stride < n ? keys[i0 + j * stride] : KeyT(0);
 #pragma unroll
-            for (int j = 1; j < J; ++j) {
-                if (j >= m) break;
-                const int d = (int)((k[j] >> sh_p) & msk);
-                if (d == run_d) {
-                    ++run_c;
-                } else {
-                    atomicAdd(&sh[off[p] + run_d], run_c);
-                    run_d = d;
-                    run_c = 1;
-                }
-            }
-            atomicAdd(&sh[off[p] + run_d], run_c);
+        for (int j = 0; j < J; ++j) {
+            if (i0 + j * stride >= n) break;
+#pragma unroll
+            for (int p = 0; p < kMaxPasses; ++p)
+                if (p < g.passes) atomicAdd(&sh[off[p] + ((uint32_t)(k[j] >> g.shift[p]) & ((1u << g.bits[p]) - 1u))], 1u);
         }
     }
     __syncthreads();
-    for (int p = 0; p < g.passes; ++p)
+#pragma unroll
+    for (int p = 0; p < kMaxPasses; ++p) {
+        if (p >= g.passes) break;
         for (int d = threadIdx.x; d < (1 << g.bits[p]); d += blockDim.x) {
             const uint32_t v = sh[off[p] + d];
             if (v) atomicAdd(&hist[p * kHistStride + d], v);
         }
+    }
     if (!done) return;
     __threadfence();
     __syncthreads();
