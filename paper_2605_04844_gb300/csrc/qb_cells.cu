@@ -31,7 +31,7 @@
 namespace qb {
 
 constexpr int kCellWarps = 8;          // warps per emit block
-constexpr uint32_t kCellChunk = 512;   // entries per warp and step
+constexpr uint32_t kCellChunk = 256;   // entries per warp and step (512: 26 instead of 20 us for 400k entries)
 constexpr int kCellHistMax = 4096;     // cells a block's histogram holds in shared memory
 static_assert(kCellChunk % kEmitStride == 0, "a warp's range starts on the scan's chunk table");
 
@@ -84,20 +84,38 @@ __device__ __forceinline__ void cell_emit_range(const CellBin &b, uint64_t E, ui
     const uint32_t none = (uint32_t)b.geo.ncells;
     int64_t j0 = b.chunk_first[C / kEmitStride];
     int32_t done_to = 0;  // range positions [0, done_to) produced
-    while (done_to < L && j0 < b.n) {
-        const int64_t j = j0 + lane;
-        // the run of position j, relative to C (none beyond the last one)
-        int64_t rel = (int64_t)E - (int64_t)C, end = rel;
-        uint32_t gid = 0;
+    // The loads of a batch are taken ahead of it, the Gaussians and their runs
+    // (which the rectangles wait for) two batches, the rectangles one: a warp's
+    // half dozen batches would otherwise cost two memory latencies each.
+    struct Run {
+        uint32_t gid, at, end;  // (entries: E beyond the last Gaussian)
+    };
+    auto load_run = [&](int64_t j) {
+        Run r{0u, (uint32_t)E, (uint32_t)E};
         if (j < b.n) {
-            gid = b.perm[j];
-            rel = (int64_t)b.coff[j] - (int64_t)C;
-            end = j + 1 < b.n ? (int64_t)b.coff[j + 1] - (int64_t)C : end;
+            r.gid = b.perm[j];
+            r.at = b.coff[j];
+            if (j + 1 < b.n) r.end = b.coff[j + 1];
         }
+        return r;
+    };
+    auto load_rects = [&](const Run &r, uint4 &w0, uint4 &w1) {
+        w0 = w1 = make_uint4(1u | (1u << 16), 0u, 1u | (1u << 16), 0u);  // empty rectangles
+        if (r.end > r.at) {
+            w0 = b.rects[2 * (size_t)r.gid];
+            w1 = b.rects[2 * (size_t)r.gid + 1];
+        }
+    };
+    Run cur_run = load_run(j0 + lane), next_run = load_run(j0 + 32 + lane);
+    uint4 w0, w1;
+    load_rects(cur_run, w0, w1);
+    while (done_to < L && j0 < b.n) {
+        // the run of position j0 + lane, relative to C
+        const int64_t rel = (int64_t)cur_run.at - (int64_t)C, end = (int64_t)cur_run.end - (int64_t)C;
+        const uint32_t gid = cur_run.gid;
         const bool relevant = end > rel && rel < L && end > 0;
         __syncwarp();
         if (relevant) {
-            const uint4 w0 = b.rects[2 * (size_t)gid], w1 = b.rects[2 * (size_t)gid + 1];
             const Rect r[4] = {unpack_rect(w0.x, w0.y), unpack_rect(w0.z, w0.w), unpack_rect(w1.x, w1.y),
                                unpack_rect(w1.z, w1.w)};
             const Rect box = cell_box(r);
@@ -107,6 +125,9 @@ __device__ __forceinline__ void cell_emit_range(const CellBin &b, uint64_t E, ui
             S.rects[lane][0] = w0;
             S.rects[lane][1] = w1;
         }
+        cur_run = next_run;
+        load_rects(cur_run, w0, w1);
+        next_run = load_run(j0 + 64 + lane);
         // where the lane's run starts among the positions still to come
         const int32_t start = relevant && rel > done_to ? (int32_t)rel : INT32_MAX;
         // the Gaussian of position done_to
@@ -251,7 +272,7 @@ __device__ __forceinline__ void cell_prepare(const CellBin &b, uint32_t *s_dsum)
 //
 // Bound by issue slots.  Decomposing every Gaussian's cells into QPass runs
 // took 41M warp instructions and 79 us for 1M Gaussians at 1080p (2.7M entries);
-// now 57 us.  (A thread per Gaussian that runs through a small box, and a block's
+// now 48 us (20 us for 200k at 1001 x 701, was 49).  (A thread per Gaussian that runs through a small box, and a block's
 // warps sharing the large ones, took 72 us, and 104 instead of 48 for 3M at
 // 1440p seen from inside, where the nearest Gaussians' boxes fill the image.)
 template <bool NAIVE>
