@@ -478,14 +478,22 @@ __global__ void __launch_bounds__(kPrefixThreads, 3) cell_prefix_kernel(CellGeo 
     }
 }
 
+// The stores bound it: each carries a dozen to 20 words of one tile at any
+// alignment, and the memory-side queue is full (the largest stall) at 4.5 TB/s
+// of sectors.  What else goes through that queue is kept small: the 32 tiles'
+// places come from shared memory four at a time, not by 32 shuffles (1M
+// Gaussians at 1080p 81 -> 77 us, with 3-sigma boxes 203 -> 193).  Staging a
+// row's values in shared memory to write whole 128-byte lines was slower (122,
+// 245 us): the values then pass the queue three times.
 __global__ void __launch_bounds__(kRowWarps * 32) cell_expand_kernel(CellGeo g, CellArrays a,
                                                                      const uint64_t *__restrict__ in,
                                                                      const uint2 *__restrict__ ranges,
                                                                      uint32_t *__restrict__ vals) {
-    const int lane = threadIdx.x & 31;
+    __shared__ __align__(16) uint32_t s_base[kRowWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t lt = lanemask_lt();
     const uint32_t rows = a.row_start[g.ncells];
-    for (uint32_t r = blockIdx.x * kRowWarps + (threadIdx.x >> 5); r < rows; r += gridDim.x * kRowWarps) {
+    for (uint32_t r = blockIdx.x * kRowWarps + w; r < rows; r += gridDim.x * kRowWarps) {
         const int cell = (int)a.row_cell[r];
         const uint32_t first = a.start[cell] + (r - a.row_start[cell]) * kCellRow;
         const uint32_t end = min(first + kCellRow, a.start[cell + 1]);
@@ -502,12 +510,19 @@ __global__ void __launch_bounds__(kRowWarps * 32) cell_expand_kernel(CellGeo g, 
         for (int k = 0; k < (int)kCellRow / 32; ++k) {
             if (first + 32 * k >= end) break;  // warp-uniform
             const uint32_t gid = (uint32_t)e[k], bits = (uint32_t)(e[k] >> 32) & have;
+            __syncwarp();  // the places of the 32 entries before have been read
+            s_base[w][lane] = base;
+            __syncwarp();
 #pragma unroll
-            for (int q = 0; q < 32; ++q) {
-                const bool on = (bits >> q) & 1u;
-                const uint32_t m = __ballot_sync(0xffffffffu, on);
-                const uint32_t at = __shfl_sync(0xffffffffu, base, q) + __popc(m & lt);
-                if (on) vals[at] = gid;
+            for (int q = 0; q < 32; q += 4) {
+                const uint4 to4 = *reinterpret_cast<const uint4 *>(&s_base[w][q]);
+                const uint32_t to[4] = {to4.x, to4.y, to4.z, to4.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const bool on = (bits >> (q + j)) & 1u;
+                    const uint32_t m = __ballot_sync(0xffffffffu, on);
+                    if (on) vals[to[j] + __popc(m & lt)] = gid;
+                }
             }
             base += __popc(warp_transpose(bits, lane));
         }
