@@ -92,6 +92,8 @@ bool make_layout(int n, int W, int H, uint64_t cap, Layout &L) {
     L.tfinal = take(4 * (size_t)W * H);
     L.ncontrib = take(4 * (size_t)W * H);
     L.neval = take(4 * (size_t)W * H);
+    L.bwd_list = take(4 * N);
+    L.bwd_count = take(256);  // directly before the sums: one memset clears both
     L.gscreen = take(72 * N);
     L.state = take(256);
     L.total = off;
@@ -612,10 +614,12 @@ qb_status qb_render_bwd(qb_frame *frame, const qb_scene *scene, const qb_camera 
         return fail(QB_ERR_INVALID_ARG, "a gradient array is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     double *gscreen = d_grad_screen;
+    size_t clear = 256;
     if (!gscreen) {
         gscreen = at<double>(frame, L.gscreen);
-        QB_CUDA(cudaMemsetAsync(gscreen, 0, 72 * (size_t)frame->n, s));
+        clear += 72 * (size_t)frame->n;
     }
+    QB_CUDA(cudaMemsetAsync(at<uint32_t>(frame, L.bwd_count), 0, clear, s));
     BwdArgs b;
     std::memset(&b, 0, sizeof(b));
     b.ranges = at<uint2>(frame, L.ranges);
@@ -650,6 +654,8 @@ qb_status qb_render_bwd(qb_frame *frame, const qb_scene *scene, const qb_camera 
     p.cams = frame_camset(*camera);
     p.meta = at<int>(frame, L.meta);
     p.g_screen = gscreen;
+    p.list_count = at<uint32_t>(frame, L.bwd_count);
+    p.list = at<uint32_t>(frame, L.bwd_list);
     p.gm = grads->means;
     p.gs = grads->scales;
     p.gq = grads->quats;

@@ -426,57 +426,66 @@ __device__ __forceinline__ void add_row(float *p, bool vec, const float (&Y)[16]
 
 // The screen-space sums of most Gaussians of a frame are exactly zero (no pixel
 // composited them), and then so is everything they add to the gradients, which
-// is nine tenths of the bytes this kernel would move for them.  So a block
-// first streams the sums of its kBwdSpan Gaussians and lists those with any
-// that is not zero, and its threads then take the listed ones.  (A colour that
-// is not finite makes the direction's gradient NaN even from zero sums, so
-// such a Gaussian is listed too: kMetaNonFinite.)  1M Gaussians at 1080p, a
-// sixth of them listed: 188 -> 72 us; 1024 Gaussians per block 80, 256 threads
-// per block 107.  Of several cameras' views nearly every Gaussian is in some,
-// where the list measured slower than a thread per Gaussian (220 against 166
-// us, five views of 200k).
-constexpr int kBwdSpan = 512, kBwdListThreads = 128;
-struct BwdList {
-    uint32_t count;
-    uint16_t item[kBwdSpan];  // offset in the block's span
-    uint8_t any[kBwdSpan];
-};
-
-__device__ __forceinline__ void list_nonzero(const PreBwdArgs &a, BwdList &L) {
-    const int tid = threadIdx.x, span = min(kBwdSpan, a.n - (int)blockIdx.x * kBwdSpan);
-    const size_t first = (size_t)blockIdx.x * kBwdSpan;
-    if (tid == 0) L.count = 0u;
-    for (int i = tid; i < span; i += blockDim.x) L.any[i] = 0;
+// is nine tenths of the bytes preprocess_bwd would move for them.  So for one
+// camera's view the Gaussians with any sum that is not zero are listed first.
+// (A colour that is not finite makes the direction's gradient NaN even from
+// zero sums, so such a Gaussian is listed too: kMetaNonFinite.)  A kernel of
+// its own, because it is a stream of 76 bytes per Gaussian that wants many
+// loads in flight, and the chain a few dependent loads and 90 registers per
+// listed Gaussian that want full warps: the two in one kernel, each block
+// listing 512 Gaussians for itself, kept a warp or two per block busy.
+// 1M Gaussians at 1080p, a sixth of them listed: 188 us a thread per Gaussian,
+// 70 in one kernel, now 16 + 17 (500k at 1264 x 832: 102, 43, 10 + 18).  The
+// list with 8-byte loads 27, with 256 Gaussians and 128 threads per block 18.
+// Of several cameras' views nearly every Gaussian is in some, where a list
+// measured slower than a thread per Gaussian (220 against 166 us, five views of
+// 200k).
+constexpr int kListSpan = 512, kListThreads = 256;
+__global__ void __launch_bounds__(kListThreads) bwd_list_kernel(PreBwdArgs a) {
+    __shared__ uint8_t s_any[kListSpan];
+    __shared__ uint32_t s_count, s_at;
+    __shared__ uint16_t s_item[kListSpan];
+    const int tid = threadIdx.x, span = min(kListSpan, a.n - (int)blockIdx.x * kListSpan);
+    const size_t first = (size_t)blockIdx.x * kListSpan;
+    if (tid == 0) s_count = 0u;
+    for (int i = tid; i < kListSpan; i += kListThreads) s_any[i] = 0;
     __syncthreads();
-    const unsigned long long *g = reinterpret_cast<const unsigned long long *>(a.g_screen) + first * 9;
+    const double *g = a.g_screen + first * 9;
     const int words = 9 * span;
-    constexpr int U = 9;
-    for (int i0 = tid; i0 < words; i0 += U * blockDim.x) {
-        unsigned long long v[U];
+    if (span == kListSpan && reinterpret_cast<uintptr_t>(g) % 16 == 0) {
+        constexpr int U = 9 * kListSpan / 2 / kListThreads;
+        ulonglong2 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = __ldcs(reinterpret_cast<const ulonglong2 *>(g) + tid + u * kListThreads);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * (int)blockDim.x;
-            v[u] = i < words ? __ldcs(g + i) : 0ull;
+            const int i = 2 * (tid + u * kListThreads);
+            if (v[u].x << 1) s_any[i / 9] = 1;  // not +-0
+            if (v[u].y << 1) s_any[(i + 1) / 9] = 1;
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (v[u] << 1) L.any[(i0 + u * (int)blockDim.x) / 9] = 1;  // not +-0
+    } else {
+        for (int i = tid; i < words; i += kListThreads)
+            if (g[i] != 0.0) s_any[i / 9] = 1;
     }
-    for (int i = tid; i < span; i += blockDim.x)
-        if (a.meta[first + i] & kMetaNonFinite) L.any[i] = 1;
+    for (int i = tid; i < span; i += kListThreads)
+        if (a.meta[first + i] & kMetaNonFinite) s_any[i] = 1;
     __syncthreads();
-    for (int i0 = 0; i0 < span; i0 += blockDim.x) {  // whole warps pass
-        const int i = i0 + tid;
-        const bool on = i < span && L.any[i];
+    for (int i = tid; i < kListSpan; i += kListThreads) {  // whole warps pass
+        const bool on = s_any[i];
         const uint32_t m = __ballot_sync(0xffffffffu, on);
         uint32_t at = 0;
-        if ((tid & 31) == 0 && m) at = atomicAdd(&L.count, (uint32_t)__popc(m));
+        if ((tid & 31) == 0 && m) at = atomicAdd(&s_count, (uint32_t)__popc(m));
         at = __shfl_sync(0xffffffffu, at, 0);
-        if (on) L.item[at + __popc(m & ((1u << (tid & 31)) - 1u))] = (uint16_t)i;
+        if (on) s_item[at + __popc(m & ((1u << (tid & 31)) - 1u))] = (uint16_t)i;
     }
     __syncthreads();
+    const uint32_t count = s_count;
+    if (tid == 0 && count) s_at = atomicAdd(a.list_count, count);
+    __syncthreads();
+    for (uint32_t k = tid; k < count; k += kListThreads) a.list[s_at + k] = (uint32_t)first + s_item[k];
 }
 
+constexpr int kChainThreads = 128;
 // SINGLE: one camera (a frame); the SH gradient Y gcol^T is then written
 // directly instead of being summed over cameras in registers.
 template <int DEG, bool SINGLE>
@@ -641,12 +650,11 @@ __device__ __forceinline__ void preprocess_bwd_one(const PreBwdArgs &a, int i) {
 }
 
 template <int DEG, bool SINGLE>
-__global__ void __launch_bounds__(SINGLE ? kBwdListThreads : 256) preprocess_bwd_kernel(PreBwdArgs a) {
+__global__ void __launch_bounds__(SINGLE ? kChainThreads : 256) preprocess_bwd_kernel(PreBwdArgs a) {
     if constexpr (SINGLE) {
-        __shared__ BwdList s_list;
-        list_nonzero(a, s_list);
-        for (uint32_t k = threadIdx.x; k < s_list.count; k += blockDim.x)
-            preprocess_bwd_one<DEG, SINGLE>(a, (int)blockIdx.x * kBwdSpan + s_list.item[k]);
+        const uint32_t count = *a.list_count;
+        for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x)
+            preprocess_bwd_one<DEG, SINGLE>(a, (int)a.list[k]);
     } else {
         const int i = blockIdx.x * blockDim.x + threadIdx.x;
         if (i < a.n) preprocess_bwd_one<DEG, SINGLE>(a, i);
@@ -655,8 +663,16 @@ __global__ void __launch_bounds__(SINGLE ? kBwdListThreads : 256) preprocess_bwd
 
 template <bool SINGLE>
 static void run_preprocess_bwd(const PreBwdArgs &a, int deg, cudaStream_t s) {
-    const unsigned block = SINGLE ? kBwdListThreads : 256, span = SINGLE ? kBwdSpan : 256;
-    const unsigned grid = ((unsigned)a.n + span - 1) / span;
+    const unsigned block = SINGLE ? kChainThreads : 256;
+    unsigned grid = ((unsigned)a.n + block - 1) / block;
+    if constexpr (SINGLE) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        grid = std::min(grid, (unsigned)sms * 5u);  // the resident blocks; they stride over the list
+        note_launch("bwd_list_kernel", s);
+        bwd_list_kernel<<<((unsigned)a.n + kListSpan - 1) / kListSpan, kListThreads, 0, s>>>(a);
+    }
     note_launch("preprocess_bwd_kernel", s);
     switch (deg) {
     case 0: preprocess_bwd_kernel<0, SINGLE><<<grid, block, 0, s>>>(a); break;

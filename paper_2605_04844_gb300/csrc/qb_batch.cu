@@ -90,6 +90,7 @@ struct BLayout {
     size_t offsets, coff, chunk_first, scan_part, dsort, sort, n_cells;
     size_t cell_zero, cell_start, row_start, row_cell, row_counts, tile_total;
     size_t set_stride;
+    size_t bwd_list, bwd_count;                       // a one-camera group's chain to the parameters
     size_t gscreen;                                   // [n_cams * n][9]
     size_t queue, state;
     size_t total;
@@ -149,6 +150,8 @@ bool make_blayout(int n, int n_cams, int group, uint64_t cap, const Geo &g, BLay
     L.tile_total = take(4 * (size_t)g.max_tiles);
     L.set_stride = off - set0;
     off += (size_t)(batch_sets(group) - 1) * L.set_stride;  // the other sets
+    L.bwd_list = take(4 * (size_t)n);
+    L.bwd_count = take(256);
     L.gscreen = take(72 * recs);
     L.queue = take(256);
     L.state = take(8 * (size_t)n_cams + 256);
@@ -593,6 +596,9 @@ qb_status qb_render_batch_bwd(qb_batch *b, const qb_scene *scene, const qb_camer
         p.cams = v.cs;
         p.meta = bat<int>(b, L.meta) + v.rec0;
         p.g_screen = gscreen + 9 * v.rec0;
+        p.list_count = bat<uint32_t>(b, L.bwd_count);
+        p.list = bat<uint32_t>(b, L.bwd_list);
+        if (v.cs.n_cams == 1) QB_BCUDA(cudaMemsetAsync(p.list_count, 0, 4, s));
         p.gm = grads->means;
         p.gs = grads->scales;
         p.gq = grads->quats;

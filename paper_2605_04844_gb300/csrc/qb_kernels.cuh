@@ -230,6 +230,8 @@ struct PreBwdArgs {
     const int *meta;          // [n_cams * n]
     const double *g_screen;   // [n_cams * n][9]
     float *gm, *gs, *gq, *go, *gsh;
+    uint32_t *list_count;     // one camera: zero before the launch; Gaussians listed
+    uint32_t *list;           // one camera: [n], the Gaussians with a sum that is not zero
     bool sh_vec4, gsh_vec4;   // sh / gsh rows may be accessed as float4 (16-byte aligned)
 };
 
