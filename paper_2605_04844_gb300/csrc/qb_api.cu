@@ -560,30 +560,11 @@ static qb_status render_fwd_impl(qb_frame *frame, const float *bg, float *d_img,
     a.ncontrib = at<int>(frame, L.ncontrib);
     a.neval = at<int>(frame, L.neval);
     a.counts = counts;
-    // A frame of few tiles takes the heaviest first: every tile is filed by a
-    // work estimate, and blocks take the tiles in that order, so that the last
-    // ones to start are short.  With more tiles than two rounds of resident
-    // blocks (kWorkBlocksPerSM, by the render's registers) the tail is a small
-    // part of the kernel and the estimate costs more than it saves: estimate +
-    // render against index order, 2772 tiles 110 : 123 us, 4108 tiles 126 : 124,
-    // 8160 tiles 201 : 196, 14400 tiles 980 : 960, 32400 tiles 690 : 657.
-    // The render files every tile by the backward's work, and in index order
-    // into the first order too.
     const size_t ntiles = a.ts.total_tiles;
     uint32_t *cnt = at<uint32_t>(frame, L.order_cnt), *list = at<uint32_t>(frame, L.order_list);
-    const TileOrder first{cnt, list};
-    a.order_out = TileOrder{cnt + kOrderBuckets, list + (size_t)kOrderBuckets * ntiles};
-    int dev = 0, sms = 0;
-    QB_CUDA(cudaGetDevice(&dev));
-    QB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    constexpr size_t kWorkBlocksPerSM = 14;
+    a.order_out[0] = TileOrder{cnt, list};
+    a.order_out[1] = TileOrder{cnt + kOrderBuckets, list + (size_t)kOrderBuckets * ntiles};
     QB_CUDA(cudaMemsetAsync(cnt, 0, 4 * 2 * (size_t)kOrderBuckets, (cudaStream_t)stream));
-    if (ntiles <= 2 * kWorkBlocksPerSM * (size_t)sms) {
-        a.order = first;
-        QB_CUDA(launch_tile_work(a, (cudaStream_t)stream));
-    } else {
-        a.order_known = first;
-    }
     QB_CUDA(launch_render(a, (cudaStream_t)stream));
     frame->stage = 4;
     return QB_OK;

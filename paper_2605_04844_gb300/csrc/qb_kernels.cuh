@@ -193,14 +193,9 @@ struct RenderArgs {
     int blocks_per_sm;   // persistent blocks per SM (0: occupancy limit)
     unsigned long long *counts;  // measurement only (single frame): [evaluated, power test passed] or null
     const CamTile *cam_table;    // persistent launch over ts.n_cams cameras from this device table, or null (ts.cam)
-    // one block per tile (single frame): with order.cnt set, block b renders
-    // the tile at position b of the tiles by decreasing work (TileOrder), else
-    // tile b; with order_out.cnt set, every tile is filed by its largest
-    // last-contributor count (the backward's work)
-    TileOrder order, order_out;
-    // with order_known.cnt set every tile is filed there too, as in order_out
-    // (frames whose blocks take the tiles in index order)
-    TileOrder order_known;
+    // single frame, with order_out[0].cnt set: every tile is filed in both by
+    // its largest last-contributor count (the backward's work)
+    TileOrder order_out[2];
 };
 
 struct BwdArgs {
@@ -219,7 +214,7 @@ struct BwdArgs {
     int tiles_per_fetch;
     int blocks_per_sm;
     const CamTile *cam_table;  // as RenderArgs::cam_table
-    TileOrder order;           // as RenderArgs::order
+    TileOrder order;           // one block per tile: with cnt set, block b takes the tile at position b, else tile b
 };
 
 struct PreBwdArgs {
@@ -285,10 +280,6 @@ cudaError_t launch_cell_sort(const CellBin &b, cudaStream_t s);
 // *in_b: the sorted values lie in vals_b.
 cudaError_t cell_sort_passes(const CellBin &b, cudaStream_t s, bool *in_b);
 cudaError_t launch_render(const RenderArgs &a, cudaStream_t s);
-// Files every tile of a single frame (a.ts.cam[0]) into a.order by an
-// estimate of the render's work: the entries composited until four sample
-// pixels of the tile stop (the whole list where one does not).
-cudaError_t launch_tile_work(const RenderArgs &a, cudaStream_t s);
 cudaError_t launch_l1_grad(const float *img, const float *target, float *dL, uint64_t n, float scale, double *loss,
                            cudaStream_t s);
 cudaError_t launch_zero5(float *const p[5], const uint64_t n[5], cudaStream_t s);

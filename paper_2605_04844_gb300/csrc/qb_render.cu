@@ -6,12 +6,13 @@
 // A warp renders one half of a tile (rows 0-7 or 8-15) on its own; a thread
 // owns four pixels of one column of the half, rows r, r + 2, r + 4 and r + 6,
 // evaluated as two packed pairs (r, r + 2) and (r + 4, r + 6) that share the
-// column's dx terms.  The warp walks the tile's depth-sorted Gaussian list 32
+// column's dx terms.  (In a frame of few tiles a warp renders a quarter, a
+// thread one pair.)  The warp walks the tile's depth-sorted Gaussian list 32
 // entries at a time: each lane brings in one entry's record (asynchronous
 // copies of the next 32 run during the walk of the current ones), tests its
-// alpha ellipse against the half's 16 x 8 pixels (ellipse_meets_rect), and
+// alpha ellipse against the part's pixels (ellipse_meets_rect), and
 // the entries that reach it are written, compacted, to the warp's staging
-// memory.  An entry left out is one every pixel of the half would reject.
+// memory.  An entry left out is one every pixel of the part would reject.
 // Per entry and pixel (3DGS conventions):
 //   power = -(a dx^2 + 2 b dx dy + c dy^2)/2, skip if it is so low that alpha
 //   is certainly below 1/255 (power > 0 arises only as a float32 rounding of
@@ -39,8 +40,8 @@
 
 namespace qb {
 
-constexpr int kRenderThreads = 64;  // a block of the single-frame kernel: the two halves of a tile
-constexpr int kRenderPairs = 2;     // packed pixel pairs per thread
+constexpr int kRenderThreads = 64;             // the two halves of a tile
+constexpr uint32_t kQuarterBlocksPerSM = 8;    // blocks of four quarters, by registers
 
 // The compositing state of one packed pair of pixels.  A pixel outside the
 // image, or one that has stopped, carries a NaN row npy: its exponent and its
@@ -56,12 +57,12 @@ struct RenderPair {
 // colour and transmittance bit-for-bit unchanged, so the branch-free update
 // composes exactly the entries the per-pixel rules of the header accept.
 // (alpha >= 1/255 implies power >= skip, so the power test needs no second look.)
-template <bool CAP, bool COUNT>
-__device__ __forceinline__ void blend(RenderPair (&P)[kRenderPairs], const float2 (&pw)[kRenderPairs], float2 op,
-                                      float2 cr, float2 cg, float2 cb, int nj) {
-    float2 al[kRenderPairs], tT[kRenderPairs];
+template <bool CAP, bool COUNT, int PAIRS>
+__device__ __forceinline__ void blend(RenderPair (&P)[PAIRS], const float2 (&pw)[PAIRS], float2 op, float2 cr,
+                                      float2 cg, float2 cb, int nj) {
+    float2 al[PAIRS], tT[PAIRS];
 #pragma unroll
-    for (int r = 0; r < kRenderPairs; ++r) {
+    for (int r = 0; r < PAIRS; ++r) {
         RenderPair &q = P[r];
         al[r] = __fmul2_rn(op, exp2_of(pw[r]));
         if (CAP) al[r] = f2(min_nan(kAlphaMax, al[r].x), min_nan(kAlphaMax, al[r].y));
@@ -81,11 +82,14 @@ __device__ __forceinline__ void blend(RenderPair (&P)[kRenderPairs], const float
         q.last1 = ac1 ? nj : q.last1;
     }
     // Once in a pixel's life an accepted alpha takes T below the stop: its row
-    // becomes NaN.  One minimum over the four pixels tells (a NaN loses against
-    // any number in fminf); which of them stopped is looked at only then.
-    if (fminf(fminf(tT[0].x, tT[0].y), fminf(tT[1].x, tT[1].y)) < kTStop) {
+    // becomes NaN.  One minimum over the thread's pixels tells (a NaN loses
+    // against any number in fminf); which of them stopped is looked at only then.
+    float low = fminf(tT[0].x, tT[0].y);
 #pragma unroll
-        for (int r = 0; r < kRenderPairs; ++r) {
+    for (int r = 1; r < PAIRS; ++r) low = fminf(low, fminf(tT[r].x, tT[r].y));
+    if (low < kTStop) {
+#pragma unroll
+        for (int r = 0; r < PAIRS; ++r) {
             const bool st0 = al[r].x >= kAlphaMin && tT[r].x < kTStop, st1 = al[r].y >= kAlphaMin && tT[r].y < kTStop;
             if (st0) P[r].npy.x = kNaN;
             if (st1) P[r].npy.y = kNaN;
@@ -95,24 +99,25 @@ __device__ __forceinline__ void blend(RenderPair (&P)[kRenderPairs], const float
     }
 }
 
-// One half (0: rows 0-7, 1: rows 8-15) of a tile by one warp; returns the
-// largest last-contributor count of the lane's pixels.  COUNT (measurement
-// only) also adds the half's (pixel, entry) evaluations and the evaluations
+// One part of a tile (16 x 4 PAIRS pixels: a half of two pairs per thread, or
+// a quarter of one) by one warp; returns the largest last-contributor count of
+// the lane's pixels.  COUNT (measurement only) also adds the half's (pixel, entry) evaluations and the evaluations
 // whose power test passed to a.counts[0], a.counts[1].
-template <bool COUNT = false>
-__device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, int half, const CamTile &C,
+template <int PAIRS, bool COUNT = false>
+__device__ __forceinline__ int render_part(const RenderArgs &a, uint32_t gtile, int part, const CamTile &C,
                                            RenderStage &S) {
+    constexpr int kRows = 4 * PAIRS;
     const uint32_t lt = gtile - C.tile_base;
     const int tx = (int)(lt % (uint32_t)C.tiles_x), ty = (int)(lt / (uint32_t)C.tiles_x);
     const int lane = threadIdx.x & 31;
     const int px = tx * kTile + (lane & (kTile - 1));
-    const int pyb = ty * kTile + half * 8 + (lane >> kTileShift);
+    const int pyb = ty * kTile + part * kRows + (lane >> kTileShift);
     const float2 npx = f2(-(float)px, -(float)px);
-    // the half's pixels, for the ellipse test
-    const float x0 = (float)(tx * kTile), y0 = (float)(ty * kTile + half * 8);
-    RenderPair P[kRenderPairs];
+    // the part's pixels, for the ellipse test
+    const float x0 = (float)(tx * kTile), y0 = (float)(ty * kTile + part * kRows);
+    RenderPair P[PAIRS];
 #pragma unroll
-    for (int r = 0; r < kRenderPairs; ++r) {
+    for (int r = 0; r < PAIRS; ++r) {
         const int ya = pyb + 4 * r, yb = ya + 2;
         P[r].npy = f2(px < C.W && ya < C.H ? -(float)ya : kNaN, px < C.W && yb < C.H ? -(float)yb : kNaN);
         P[r].T = f2(1.f, 1.f);
@@ -121,7 +126,10 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
     }
     auto stopped = [](float npy) { return npy != npy; };
     auto all_done = [&]() {
-        return stopped(P[0].npy.x) && stopped(P[0].npy.y) && stopped(P[1].npy.x) && stopped(P[1].npy.y);
+        bool d = true;
+#pragma unroll
+        for (int r = 0; r < PAIRS; ++r) d = d && stopped(P[r].npy.x) && stopped(P[r].npy.y);
+        return d;
     };
 
     const uint2 range = a.ranges[gtile];
@@ -134,7 +142,7 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
 
     for (int base = 0; base < total; base += 32) {
         copy_wait();
-        const int cnt = stage_entries<false>(S, base + lane < total, base + lane + 1, x0, y0, lane);
+        const int cnt = stage_entries<false, kRows>(S, base + lane < total, base + lane + 1, x0, y0, lane);
         if (base + 32 + lane < total) {
             stage_copy(S, src, C.rec_base + vnext, lane);
             vnext = base + 64 + lane < total ? vals[base + 64 + lane] : 0u;
@@ -145,14 +153,14 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
             const float4 X = S.sx[j], Q = S.sq[j], K = S.sk[j];
             const uint32_t info = __float_as_uint(K.w);
             const float2 dx = __fadd2_rn(f2(X.x, X.y), npx);
-            float2 pw[kRenderPairs];
+            float2 pw[PAIRS];
             if (!(info & kLongEntry)) {
                 // power = A + dy (B + cc dy), A = ca dx^2, B = cb dx; dx, A and
-                // B are the column's, shared by the thread's four pixels
+                // B are the column's, shared by the thread's pixels
                 const float2 A = __fmul2_rn(__fmul2_rn(f2(Q.x, Q.y), dx), dx);
                 const float2 B = __fmul2_rn(f2(Q.z, Q.w), dx);
 #pragma unroll
-                for (int r = 0; r < kRenderPairs; ++r) {
+                for (int r = 0; r < PAIRS; ++r) {
                     const float2 dy = __fadd2_rn(f2(X.z, X.w), P[r].npy);
                     pw[r] = __ffma2_rn(dy, __ffma2_rn(f2(K.x, K.y), dy, B), A);
                 }
@@ -161,7 +169,7 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
                 // ce dy^2, u = dx + rr dy
                 const float4 E = S.se[j];
 #pragma unroll
-                for (int r = 0; r < kRenderPairs; ++r) {
+                for (int r = 0; r < PAIRS; ++r) {
                     const float2 dy = __fadd2_rn(f2(X.z, X.w), P[r].npy);
                     const float2 u = __ffma2_rn(f2(E.x, E.y), dy, dx);
                     pw[r] = __ffma2_rn(__fmul2_rn(f2(Q.x, Q.y), u), u, __fmul2_rn(__fmul2_rn(f2(E.z, E.w), dy), dy));
@@ -171,18 +179,21 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
             // positive exponent is a float32 rounding of 0 (the conic is
             // positive definite), where alpha = o e^power rounds like o.
             // (A NaN loses against any number in fmaxf.)
-            const bool any = fmaxf(fmaxf(pw[0].x, pw[0].y), fmaxf(pw[1].x, pw[1].y)) >= K.z;
-            if (COUNT)
-                npass += (uint32_t)(pw[0].x >= K.z) + (uint32_t)(pw[0].y >= K.z) + (uint32_t)(pw[1].x >= K.z) +
-                         (uint32_t)(pw[1].y >= K.z);
-            if (!__any_sync(0xffffffffu, any)) continue;
+            float high = fmaxf(pw[0].x, pw[0].y);
+#pragma unroll
+            for (int r = 1; r < PAIRS; ++r) high = fmaxf(high, fmaxf(pw[r].x, pw[r].y));
+            if (COUNT) {
+#pragma unroll
+                for (int r = 0; r < PAIRS; ++r) npass += (uint32_t)(pw[r].x >= K.z) + (uint32_t)(pw[r].y >= K.z);
+            }
+            if (!__any_sync(0xffffffffu, high >= K.z)) continue;
             const float4 C1 = S.s1[j], C2 = S.s2[j];
             // o G can reach the 0.99 cap only for o near it (G <= 1 up to the
             // exponential's rounding); the same for the whole warp
             if (!(info & kSlowEntry))
-                blend<false, COUNT>(P, pw, f2(C1.x, C1.y), f2(C1.z, C1.w), f2(C2.x, C2.y), f2(C2.z, C2.w), (int)info);
+                blend<false, COUNT, PAIRS>(P, pw, f2(C1.x, C1.y), f2(C1.z, C1.w), f2(C2.x, C2.y), f2(C2.z, C2.w), (int)info);
             else
-                blend<true, COUNT>(P, pw, f2(C1.x, C1.y), f2(C1.z, C1.w), f2(C2.x, C2.y), f2(C2.z, C2.w),
+                blend<true, COUNT, PAIRS>(P, pw, f2(C1.x, C1.y), f2(C1.z, C1.w), f2(C2.x, C2.y), f2(C2.z, C2.w),
                                    (int)(info & ~(kSlowEntry | kLongEntry)));
         }
         if (__all_sync(0xffffffffu, all_done())) break;
@@ -192,7 +203,7 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
     float *img = a.img + 3 * C.pix_base;
     unsigned long long ev = 0;
 #pragma unroll
-    for (int r = 0; r < kRenderPairs; ++r) {
+    for (int r = 0; r < PAIRS; ++r) {
         RenderPair &q = P[r];
         // a pixel that never stopped evaluated the whole list
         if (COUNT && !stopped(q.npy.x)) q.n0 = total;
@@ -226,137 +237,50 @@ __device__ __forceinline__ int render_half(const RenderArgs &a, uint32_t gtile, 
             atomicAdd(a.counts + 1, ps);
         }
     }
-    return max(max(P[0].last0, P[0].last1), max(P[1].last0, P[1].last1));
+    int last = 0;
+#pragma unroll
+    for (int r = 0; r < PAIRS; ++r) last = max(last, max(P[r].last0, P[r].last1));
+    return last;
 }
 
-// One block per tile of a single camera, a warp per half (72 registers, 14
-// blocks per SM; unbounded the compiler takes 77, 12 blocks); with an order, the
-// blocks (which start roughly in index order) take the heaviest tiles first,
-// so that the last blocks to start are short ones.
-template <bool COUNT>
-__global__ void __launch_bounds__(kRenderThreads, COUNT ? 1 : 14) render_kernel(RenderArgs a) {
-    __shared__ RenderStage s_stage[2];
-    __shared__ int s_last[2];
+// One block per tile of a single camera.  PAIRS 2: a warp per half, 72
+// registers, 14 blocks per SM (unbounded the compiler takes 77, 12 blocks).
+// PAIRS 1: a warp per quarter, 64 registers, 8 blocks of four warps per SM.
+//
+// Quarters are for frames whose blocks are all resident at once (at most
+// kQuarterBlocksPerSM tiles per SM): such a frame lasts as long as its longest
+// warp, and a quarter's walk is shorter, by the entries that miss it and by
+// half the work per entry.  Halves against quarters, Gaussians: 10k at 256^2
+// (256 tiles) 28 : 23 us, 20k at 333 x 217 (294) 52 : 42, 50k at 400^2 (625)
+// 73 : 55, at 512^2 (1024) 64 : 56, 100k at 640 x 480 (1200) 69 : 65; beyond,
+// the doubled staging costs more: 100k at 800 x 600 (1900 tiles) 78 : 83, 200k
+// at 1001 x 701 (2772) 99 : 110, 500k at 1264 x 832 (4108) 101 : 126.
+// Tiles run in index order.  Heaviest first by an estimate of the work was no
+// faster on any frame, estimate included (100k at 800 x 600 83 : 78 us, 200k
+// 96 : 99, 500k 103 : 101, 1M at 1080p 201 : 196).  order_out files the tiles
+// by the work there was, for the backward.
+template <int PAIRS, bool COUNT>
+__global__ void __launch_bounds__(2 * kRenderThreads / PAIRS, COUNT ? 1 : PAIRS == 1 ? (int)kQuarterBlocksPerSM : 14) render_kernel(RenderArgs a) {
+    constexpr int kParts = 4 / PAIRS;
+    __shared__ RenderStage s_stage[kParts];
+    __shared__ int s_last[kParts];
     const int wid = threadIdx.x >> 5;
-    const uint32_t t = a.order.cnt ? order_pick(a.order, a.ts.total_tiles, blockIdx.x) : (uint32_t)blockIdx.x;
-    const int last = render_half<COUNT>(a, t, wid, a.ts.cam[0], s_stage[wid]);
-    if (a.order_out.cnt) {
+    const uint32_t t = blockIdx.x;
+    const int last = render_part<PAIRS, COUNT>(a, t, wid, a.ts.cam[0], s_stage[wid]);
+    if (a.order_out[0].cnt) {
         // the tile's largest last-contributor count (the backward walks that
         // many entries) files it for the backward
         const int m = __reduce_max_sync(0xffffffffu, last);
         if ((threadIdx.x & 31) == 0) s_last[wid] = m;
         __syncthreads();
         if (threadIdx.x == 0) {
-            const uint32_t walked = (uint32_t)max(s_last[0], s_last[1]);
-            order_file(a.order_out, a.ts.total_tiles, t, walked);
-            if (a.order_known.cnt) order_file(a.order_known, a.ts.total_tiles, t, walked);
+            uint32_t walked = 0;
+#pragma unroll
+            for (int k = 0; k < kParts; ++k) walked = max(walked, (uint32_t)s_last[k]);
+            order_file(a.order_out[0], a.ts.total_tiles, t, walked);
+            order_file(a.order_out[1], a.ts.total_tiles, t, walked);
         }
     }
-}
-
-// A warp per tile walks the tile's list 32 entries at a time for two sample
-// pixels (offsets (3, 4) and (12, 11); four measured the same render and a
-// third more here): each lane takes one entry's
-// 1 - alpha at each pixel (the render's accept rules on the plain conic
-// form), a product scan over the lanes gives the transmittance after every
-// entry, and the first entry that takes a pixel below the stop ends that
-// pixel.  The estimate is the largest stop position, or the list length when
-// a pixel has not stopped within kWorkChunks chunks.  The next chunk's
-// records and the one after's indices are loaded while a chunk is scanned.
-constexpr int kWorkPix = 2;  // sample pixels per tile, at these offsets in the tile
-__device__ constexpr int kWorkX[kWorkPix] = {3, 12};
-__device__ constexpr int kWorkY[kWorkPix] = {4, 11};
-constexpr uint32_t kWorkChunks = 32;  // beyond 1024 entries every tile files into the top bucket
-__global__ void __launch_bounds__(256) tile_work_kernel(RenderArgs a) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t t = blockIdx.x * 8u + (threadIdx.x >> 5);
-    if (t >= a.ts.total_tiles) return;  // warp-uniform
-    const CamTile &C = a.ts.cam[0];
-    const int tx = (int)(t % (uint32_t)C.tiles_x), ty = (int)(t / (uint32_t)C.tiles_x);
-    float sx[kWorkPix], sy[kWorkPix], T[kWorkPix];
-    bool done[kWorkPix];
-#pragma unroll
-    for (int k = 0; k < kWorkPix; ++k) {
-        const int x = tx * kTile + kWorkX[k], y = ty * kTile + kWorkY[k];
-        sx[k] = (float)x;
-        sy[k] = (float)y;
-        T[k] = 1.f;
-        done[k] = x >= C.W || y >= C.H;
-    }
-    const uint2 range = a.ranges[t];
-    const uint32_t total = range.y - range.x;
-    const uint32_t *vals = a.vals + range.x;
-    // records of chunk 0, indices of chunk 1
-    float2 m = make_float2(0.f, 0.f);
-    float4 co = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (lane < total) {
-        const uint32_t g = vals[lane];
-        m = a.xy[g];
-        co = a.conic_o[g];
-    }
-    uint32_t gn = 32 + lane < total ? vals[32 + lane] : 0u;
-    uint32_t work = 0;
-    bool open = true;
-    for (uint32_t c = 0; c < kWorkChunks && 32 * c < total; ++c) {
-        const uint32_t base = 32 * c;
-        const bool have = base + lane < total;
-        const float2 mc = m;
-        const float4 cc = co;
-        if (base + 32 + lane < total) {  // prefetch: records of chunk c + 1, indices of chunk c + 2
-            m = a.xy[gn];
-            co = a.conic_o[gn];
-            gn = base + 64 + lane < total ? vals[base + 64 + lane] : 0u;
-        }
-        float om[kWorkPix];
-#pragma unroll
-        for (int k = 0; k < kWorkPix; ++k) om[k] = 1.f;
-        if (have) {
-            const float skip = skip_threshold(cc.w);
-#pragma unroll
-            for (int k = 0; k < kWorkPix; ++k) {
-                const float dx = mc.x - sx[k], dy = mc.y - sy[k];
-                const float pw = -0.5f * (cc.x * dx * dx + cc.z * dy * dy) - cc.y * dx * dy;
-                if (pw >= skip) {
-                    const float al = fminf(kAlphaMax, cc.w * __expf(pw));
-                    if (al >= kAlphaMin) om[k] = 1.f - al;
-                }
-            }
-        }
-        bool all = true;
-#pragma unroll
-        for (int k = 0; k < kWorkPix; ++k) {
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const float v = __shfl_up_sync(0xffffffffu, om[k], o);
-                if (lane >= o) om[k] *= v;
-            }
-            const float Tl = T[k] * om[k];
-            const uint32_t stop = __ballot_sync(0xffffffffu, Tl < kTStop);
-            if (!done[k] && stop) {
-                done[k] = true;
-                work = max(work, base + (uint32_t)__ffs(stop));
-            }
-            T[k] = __shfl_sync(0xffffffffu, Tl, 31);
-            all = all && done[k];
-        }
-        if (all) {
-            open = false;
-            break;
-        }
-    }
-    if (open) {
-        bool any_open = false;
-#pragma unroll
-        for (int k = 0; k < kWorkPix; ++k) any_open = any_open || !done[k];
-        if (any_open) work = total;
-    }
-    if (lane == 0) order_file(a.order, a.ts.total_tiles, t, work);
-}
-
-cudaError_t launch_tile_work(const RenderArgs &a, cudaStream_t s) {
-    if (a.ts.total_tiles == 0) return cudaSuccess;
-    note_launch("tile_work_kernel", s), tile_work_kernel<<<(a.ts.total_tiles + 7) / 8, 256, 0, s>>>(a);
-    return cudaGetLastError();
 }
 
 // Persistent warps take the halves of tiles_per_fetch consecutive tiles at a
@@ -374,24 +298,27 @@ __global__ void __launch_bounds__(kRenderThreads) render_persistent_kernel(Rende
         for (uint32_t h = h0; h < h1; ++h) {
             const uint32_t t = h >> 1;
             const CamTile C = a.cam_table[camera_in_table(a.cam_table, a.ts.n_cams, t)];
-            render_half(a, t, (int)(h & 1u), C, S);
+            render_part<2>(a, t, (int)(h & 1u), C, S);
         }
     }
 }
 
 cudaError_t launch_render(const RenderArgs &a, cudaStream_t s) {
     if (a.ts.total_tiles == 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (a.queue) {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_persistent_kernel, kRenderThreads, 0);
         if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_sm) per_sm = a.blocks_per_sm;
         note_launch("render_persistent_kernel", s), render_persistent_kernel<<<sms * (per_sm > 0 ? per_sm : 1), kRenderThreads, 0, s>>>(a);
     } else if (a.counts) {
-        note_launch("render_kernel_counted", s), render_kernel<true><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
+        note_launch("render_kernel_counted", s), render_kernel<2, true><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
+    } else if (a.ts.total_tiles <= kQuarterBlocksPerSM * (uint32_t)sms) {
+        note_launch("render_kernel", s), render_kernel<1, false><<<a.ts.total_tiles, 2 * kRenderThreads, 0, s>>>(a);
     } else {
-        note_launch("render_kernel", s), render_kernel<false><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
+        note_launch("render_kernel", s), render_kernel<2, false><<<a.ts.total_tiles, kRenderThreads, 0, s>>>(a);
     }
     return cudaGetLastError();
 }
