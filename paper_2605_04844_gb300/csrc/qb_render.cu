@@ -101,8 +101,9 @@ __device__ __forceinline__ void blend(RenderPair (&P)[PAIRS], const float2 (&pw)
 
 // One part of a tile (16 x 4 PAIRS pixels: a half of two pairs per thread, or
 // a quarter of one) by one warp; returns the largest last-contributor count of
-// the lane's pixels.  COUNT (measurement only) also adds the half's (pixel, entry) evaluations and the evaluations
-// whose power test passed to a.counts[0], a.counts[1].
+// the lane's pixels.  COUNT (measurement only) also adds the part's (pixel,
+// entry) evaluations and the evaluations whose power test passed to
+// a.counts[0], a.counts[1].
 template <int PAIRS, bool COUNT = false>
 __device__ __forceinline__ int render_part(const RenderArgs &a, uint32_t gtile, int part, const CamTile &C,
                                            RenderStage &S) {

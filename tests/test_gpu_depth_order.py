@@ -37,6 +37,11 @@ def test_depth_order_and_prefixes(n, ties):
     np.testing.assert_array_equal(A["vals"], full.arrays()["vals"].cpu().numpy())
 
 
+@pytest.mark.parametrize("n", [24_575, 24_576, 24_577])
+def test_depth_order_around_three_keys_per_thread(n):
+    test_depth_order_and_prefixes(n, False)
+
+
 def test_overflow_of_a_small_scene_writes_nothing():
     import torch
     from paper_2605_04844_gb300 import _native as N
