@@ -481,12 +481,13 @@ def kernel_work(P, n, evals, packed=False):
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per unit of
 # work, from the ncu --set full captures of the 600k-Gaussian 1080p frame
-# (20,633,099 pairs, 398,728,138 evaluations) summarised under profiles/,
+# (20,633,099 pairs, 398,727,914 evaluations) summarised under profiles/,
 # scaled to a launch of this frame by its units; valid for the kernels as
-# captured (kernel -> (unit, bytes per unit)).  A kernel changed since its
-# capture has no entry.
+# captured (kernel -> (unit, bytes per unit)).  tile_sort_pass and
+# tile_sort_pass_values are the pair passes that a frame took before it was
+# binned through cells; a list without them leaves their entries unused.
 TRAFFIC_PER_UNIT = {
-    "render_kernel": ("eval", (13.032192e6 + 0.436224e6) / 398728138),
+    "render_kernel": ("eval", (13.045248e6 + 0.425984e6) / 398727914),
     "tile_sort_pass": ("pair", (165.526528e6 + 34.277120e6) / 20633099),
     "tile_sort_pass_values": ("pair", (82.809600e6 + 35.105536e6) / 20633099),
 }

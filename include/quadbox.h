@@ -269,12 +269,9 @@ qb_status qb_sort(qb_frame *frame, qb_stream_t stream);
 /* Stage 4 (Sec. 2 "Render", Eq. 2): front-to-back compositing per pixel.
  * bg: host float[3] background colour (NULL = black).  d_img: device
  * float [3][height][width] (planar RGB), fully overwritten.  Also writes the
- * frame's t_final and n_contrib, which qb_render_bwd needs.  The tiles of a
- * frame of few tiles run heaviest first: a first kernel files every tile by an
- * estimate of its work (order_counts[0] / order_lists[0] of qb_frame_arrays);
- * those of a larger one run in index order, and that order is filed by the
- * render.  The render files every tile by its largest n_contrib for
- * qb_render_bwd (the second order); the image does not depend on the order. */
+ * frame's t_final and n_contrib, which qb_render_bwd needs, and files every
+ * tile by its largest n_contrib (order_counts, order_lists of
+ * qb_frame_arrays) for qb_render_bwd. */
 qb_status qb_render_fwd(qb_frame *frame, const float *bg, float *d_img, qb_stream_t stream);
 
 /* Measurement only: qb_render_fwd (identical outputs) that also adds, over
@@ -386,7 +383,7 @@ size_t qb_batch_workspace_bytes(int32_t n, int32_t n_cams, const int32_t *widths
 /* Binds a caller-owned, 256-byte aligned device workspace to *batch, writes
  * the render's per-camera table into it (synchronises the stream once) and
  * creates the batch's side streams: inside qb_render_batch the cameras of a
- * group are binned four at a time on side streams forked from the caller's
+ * group are binned up to eight at a time on side streams forked from the caller's
  * stream and joined back to it (captured into a CUDA graph with the rest).
  * Errors: INVALID_ARG for sizes outside the limits above. */
 qb_status qb_batch_init(qb_batch *batch, int32_t n, int32_t n_cams, const int32_t *widths, const int32_t *heights,
@@ -400,8 +397,8 @@ qb_status qb_batch_release(qb_batch *batch);
 /* Forward of every camera of the batch (Sec. 2's pipeline with QuadBox
  * binning, Sec. 3, per camera): per group, one preprocess over all (camera,
  * Gaussian) records; per camera, the depth order of its records, scan, QPass
- * emit with camera-local tile ids, the tile histogram (ranges and bucket
- * offsets) and the stable tile sort into the camera's slot; then one
+ * emit with camera-local cell ids, the stable cell sort, the ranges and the
+ * expansion into the camera's slot; then one
  * persistent render over the tiles of every camera.  cams: host array of
  * n_cams cameras whose sizes match qb_batch_init; tune: host, NULL for
  * defaults; d_images: device floats, total_floats of them.  No host

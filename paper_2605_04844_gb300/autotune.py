@@ -1,10 +1,10 @@
 """Autotuner for the rasteriser's launch parameters.
 
 Times the candidates on the caller's own scene and camera and keeps the
-fastest.  For a frame: the tile sort's radix digit width (8..11 bits, which
-sets the number of onesweep passes), then the render's per-tile batch depth
-(Gaussians staged in shared memory per step).  For a batch of cameras: the
-digit width, batch depth, tiles a persistent render block takes per fetch
+fastest.  For a frame: the cell sort's radix digit width (8..11 bits, which
+sets the number of passes), then render_batch (a field the library accepts
+without effect: a warp stages 32 Gaussians per step).  For a batch of cameras: the
+digit width, render_batch, tiles a persistent render block takes per fetch
 from the global queue and persistent blocks per SM, by coordinate descent.
 Results are cached as JSON under
 $QUADBOX_CACHE_DIR (default ~/.cache/quadbox/tune.json), keyed by GPU name,

@@ -337,7 +337,7 @@ __device__ __forceinline__ void render_bwd_half(const BwdArgs &a, uint32_t gtile
     __syncwarp();
 }
 
-// One block per tile; with an order, the heaviest tiles first (as the forward).
+// One block per tile; with an order, the heaviest tiles first.
 __global__ void __launch_bounds__(kBwdThreads) render_bwd_kernel(BwdArgs a) {
     __shared__ __align__(16) BwdStage s_stage[2];
     const int wid = threadIdx.x >> 5;

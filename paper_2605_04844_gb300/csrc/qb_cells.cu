@@ -21,8 +21,8 @@
 // is the one of the stable sort of all pairs by tile id.
 // One GB300, start of the frame to its sorted values without the depth order:
 // 1M Gaussians at 1080p (34.8M pairs, 2.7M entries), emit + histogram + two
-// pair passes 0.54 ms, now 0.23; 3-sigma boxes (100.8M pairs, 5.0M entries)
-// 1.36 -> 0.39 ms; 3840 x 2160 (126M pairs, 6.4M entries) 1.9 -> 0.54 ms.
+// pair passes 0.54 ms, now 0.21; 3-sigma boxes (100.8M pairs, 5.0M entries)
+// 1.36 -> 0.35 ms; 3840 x 2160 (126M pairs, 6.4M entries) 1.9 -> 0.53 ms.
 #include <algorithm>
 
 #include "qb_scan.cuh"
