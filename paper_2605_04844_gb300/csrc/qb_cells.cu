@@ -31,7 +31,12 @@
 namespace qb {
 
 constexpr int kCellWarps = 8;          // warps per emit block
-constexpr uint32_t kCellChunk = 256;   // entries per warp and step (512: 26 instead of 20 us for 400k entries)
+// Entries per warp and step: at most kCellChunk (512: 26 instead of 20 us for
+// 400k entries), and no more than spread the entries over all warps of the
+// grid, in steps of kEmitStride (10k Gaussians at 256 x 256 15.6 -> 12.7 us,
+// 200k at 1001 x 701 18.8 -> 16.5; steps of 64 10.2 and 17.5, but the scan's
+// larger table cost 3 us of 17 at 3840 x 2160).
+constexpr uint32_t kCellChunk = 256;
 constexpr int kCellHistMax = 4096;     // cells a block's histogram holds in shared memory
 static_assert(kCellChunk % kEmitStride == 0, "a warp's range starts on the scan's chunk table");
 
@@ -304,9 +309,11 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
         if (E > 0)
             for (uint64_t j = gt; j < (uint64_t)b.n; j += threads) cell_emit_naive(b, (int64_t)j, hist);
     } else {
-        const uint64_t step = (uint64_t)gridDim.x * kCellWarps * kCellChunk;
-        for (uint64_t C = ((uint64_t)blockIdx.x * kCellWarps + wid) * kCellChunk; C < E; C += step)
-            cell_emit_range(b, E, C, (int32_t)min((uint64_t)kCellChunk, E - C), s_tab[wid], hist);
+        const uint64_t warps = (uint64_t)gridDim.x * kCellWarps;
+        const uint64_t even = (E + warps * kEmitStride - 1) / (warps * kEmitStride) * kEmitStride;
+        const uint64_t chunk = min((uint64_t)kCellChunk, even);
+        for (uint64_t C = ((uint64_t)blockIdx.x * kCellWarps + wid) * chunk; C < E; C += warps * chunk)
+            cell_emit_range(b, E, C, (int32_t)min(chunk, E - C), s_tab[wid], hist);
     }
     if (in_smem) {
         __syncthreads();
@@ -340,7 +347,7 @@ cudaError_t launch_cell_emit(const CellBin &b, cudaStream_t s) {
         return cudaGetLastError();
     }
     const size_t smem = std::max(kCellWarps * sizeof(CellTable) + hist, dsum);
-    const uint64_t want = (b.n_cells_max + kCellWarps * kCellChunk - 1) / (kCellWarps * kCellChunk);
+    const uint64_t want = (b.n_cells_max + kCellWarps * kEmitStride - 1) / (kCellWarps * kEmitStride);
     const uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * 6));
     note_launch("cell_emit_kernel", s), cell_emit_kernel<false><<<(unsigned)blocks, kCellWarps * 32, smem, s>>>(b);
     return cudaGetLastError();

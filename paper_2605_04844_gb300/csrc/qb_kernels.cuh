@@ -261,7 +261,7 @@ struct OrderArgs {
 cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *in_alt);
 // Output positions per entry of the scan's chunk table (a divisor of every
 // emit kernel's per-warp output range).
-constexpr uint32_t kEmitStride = 256;
+constexpr uint32_t kEmitStride = 128;
 inline uint64_t chunk_table_size(uint64_t pair_capacity) { return pair_capacity / kEmitStride + 1; }
 size_t scan_partials_count(int n);
 cudaError_t launch_emit(const EmitArgs &a, uint64_t *keys, cudaStream_t s);
