@@ -177,10 +177,12 @@ __global__ void __launch_bounds__(kOrderThreads) depth_order_small_kernel(OrderA
             val[k] = kv.y;
         }
     }
-    // the order, and from here thread t takes ITEMS consecutive positions
+    // the order, beside its input: keys and values stay as the preprocess wrote
+    // them, so another emit of the same preprocess finds them again; from here
+    // thread t takes ITEMS consecutive positions
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k)
-        if (local(k) < mine) a.vals[first + local(k)] = val[k];
+        if (local(k) < mine) a.vals_alt[first + local(k)] = val[k];
     const int i0 = tid * ITEMS;
     uint32_t c[ITEMS], e[ITEMS];
     uint64_t csum = 0, esum = 0;
@@ -255,6 +257,7 @@ static cudaError_t launch_small(const OrderArgs &a, int n, int share, cudaStream
 cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *in_alt) {
     *in_alt = false;
     if (n > 0 && n <= kOrderSmall) {
+        *in_alt = true;
         const int share = ((n + kOrderCtas - 1) / kOrderCtas + 31) & ~31;
         if (share <= kOrderThreads) return launch_small<1>(a, n, share, s);
         if (share <= 2 * kOrderThreads) return launch_small<2>(a, n, share, s);
