@@ -116,10 +116,15 @@ cudaError_t sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint3
 constexpr float kElongatedF2 = 0.01f;  // f < 0.1: aspect ratio above 10 : 1
 
 // Exponents below this give alpha = o e^power < (1/255) e^-0.001: the 1e-3
-// margin is far wider than the float32 error of the alpha test (and of the
-// fast logarithm, 4e-7 absolute here), so skipping them first never changes a
-// decision of that test.
-__device__ __forceinline__ float skip_threshold(float o) { return -__logf(255.0f * o) - 1e-3f; }
+// margin is far wider than the float32 error of the alpha test and of the
+// fast logarithm (2^-21.4 absolute near 1, else 3 ulp: 1.5e-6 at o = 1, 6e-6
+// at o = 10^6), so skipping them first never changes a decision of that test.
+// EXACT takes logf itself: the counted render reports how many
+// exponents pass, and a last bit of the threshold can move that number.
+template <bool EXACT = false>
+__device__ __forceinline__ float skip_threshold(float o) {
+    return -(EXACT ? logf(255.0f * o) : __logf(255.0f * o)) - 1e-3f;
+}
 
 // e^x of both lanes as 2^(x log2 e), for the exponents of the compositing
 // (at least skip_threshold, so the result is no subnormal and ex2's

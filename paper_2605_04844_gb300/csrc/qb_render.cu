@@ -143,7 +143,7 @@ __device__ __forceinline__ int render_part(const RenderArgs &a, uint32_t gtile, 
 
     for (int base = 0; base < total; base += 32) {
         copy_wait();
-        const int cnt = stage_entries<false, kRows>(S, base + lane < total, base + lane + 1, x0, y0, lane);
+        const int cnt = stage_entries<false, kRows, COUNT>(S, base + lane < total, base + lane + 1, x0, y0, lane);
         if (base + 32 + lane < total) {
             stage_copy(S, src, C.rec_base + vnext, lane);
             vnext = base + 64 + lane < total ? vals[base + 64 + lane] : 0u;

@@ -65,10 +65,10 @@ __device__ __forceinline__ void stage_copy(RenderStage &S, const StageSource &sr
 // Stages the warp's entries (lane's record copied; `have`: the lane has one,
 // at list position pos - 1) that reach the 16 x ROWS pixels from (x0, y0), in
 // lane order; returns how many.  BACKWARD stores -o instead of o, and the
-// record's index rec in ids.  All lanes pass through the ballot, so the walk
-// of the last entries is over.  The caller synchronises the warp before it
-// reads them.
-template <bool BACKWARD, int ROWS = 8>
+// record's index rec in ids.  COUNT: for the counted render.  All lanes pass
+// through the ballot, so the walk of the last entries is over.  The caller
+// synchronises the warp before it reads them.
+template <bool BACKWARD, int ROWS = 8, bool COUNT = false>
 __device__ __forceinline__ int stage_entries(RenderStage &S, bool have, int pos, float x0, float y0, int lane,
                                              uint32_t rec = 0u, uint32_t *ids = nullptr) {
     bool hit = false;
@@ -80,7 +80,7 @@ __device__ __forceinline__ int stage_entries(RenderStage &S, bool have, int pos,
         sh = S.raw_sh[lane];
         co = S.raw_co[lane];
         rgb = S.raw_rgb[lane];
-        skip = skip_threshold(co.w);
+        skip = skip_threshold<COUNT>(co.w);
         hit = ellipse_meets_rect(m.x, m.y, co.x, co.y, co.z, skip, sh, x0, y0, x0 + 15.f, y0 + (float)(ROWS - 1));
     }
     const uint32_t hits = __ballot_sync(0xffffffffu, hit);
