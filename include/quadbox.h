@@ -176,12 +176,17 @@ typedef struct {
     uint64_t *n_pairs;  /* [1]     P on the device                          */
     uint32_t *err_flags;/* [2]     [0]: bit0 capacity, bit1 timeout.  [1]:
                                    test-only, zero after qb_frame_init; a test
-                                   may set it to k > 0 to exercise a bounded
-                                   spin-wait: the second tile of the last
-                                   (values-only) cell-sort pass then finds its
-                                   predecessor unpublished, gives up after k
-                                   polls and raises TIMEOUT; the sorted values
-                                   are then undefined (do not render them)  */
+                                   may set it to exercise the bounded
+                                   spin-waits.  k in 1 .. 2^29 - 1: the second
+                                   tile of the last (values-only) cell-sort pass
+                                   finds its predecessor unpublished, gives up
+                                   after k polls and raises TIMEOUT.  Bit 30: the
+                                   same tile of every other sort pass, bit 29: the
+                                   second block of the count scan, ends as after
+                                   such a wait.  A frame whose binning timed out
+                                   has no pairs in its lists (every range is
+                                   empty, vals is undefined): rendered, it shows
+                                   the background                            */
     uint32_t *order_counts; /* [2][64] tiles per work bucket, written by the
                                    forward render, both rows by the tile's
                                    largest n_contrib (the backward takes its

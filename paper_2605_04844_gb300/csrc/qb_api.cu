@@ -151,6 +151,7 @@ CellBin frame_cells(const qb_frame *f, const Layout &L) {
     b.rects = at<uint4>(f, L.rects);
     b.n_pairs = at<uint64_t>(f, L.state);
     b.n_cells = at<uint64_t>(f, L.state + 16);
+    b.scan_failed = depth_order_failed(at<uint64_t>(f, L.scan_part), f->n);
     b.n_cells_max = f->n_pairs != UINT64_MAX ? f->n_pairs : f->pair_capacity;
     b.capacity = f->pair_capacity;
     b.naive = (f->bin_mode & 0xff) == QB_BIN_QUADBOX_NAIVE;
@@ -494,6 +495,7 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
         a.vals = at<uint32_t>(frame, L.vals0);
         a.n_pairs = d_np;
         a.n_pairs_host = frame->n_pairs;
+        a.failed = scan_failed(partials, frame->n);
         a.capacity = frame->pair_capacity;
         a.mode = frame->bin_mode & 0xff;
         a.err = err;
@@ -529,7 +531,9 @@ qb_status qb_sort(qb_frame *frame, qb_stream_t stream) {
                            at<void>(frame, L.sort_scratch), at<uint32_t>(frame, L.state + 8), s, &passes));
         frame->sorted_in_alt = passes & 1;
         const uint64_t *sorted = at<uint64_t>(frame, frame->sorted_in_alt ? L.keys1 : L.keys0);
-        QB_CUDA(launch_ranges(sorted, n_max, n_dev, at<uint2>(frame, L.ranges), frame->tiles_x * frame->tiles_y, s));
+        QB_CUDA(launch_ranges(sorted, n_max, n_dev, at<uint2>(frame, L.ranges), frame->tiles_x * frame->tiles_y,
+                              scan_failed(at<uint64_t>(frame, L.scan_part), frame->n),
+                              at<void>(frame, L.sort_scratch), s));
     }
     frame->stage = 3;
     return QB_OK;

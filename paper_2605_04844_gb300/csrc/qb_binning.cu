@@ -38,6 +38,9 @@ constexpr int kScanChunk = kScanBlock * kScanItems;
 // instead of 16 give twice the blocks, and all resident blocks reach their
 // look-back at about the same time, so it reads 256 words at once instead of
 // 32 (a chain of two or three loads where there were up to a dozen).
+//
+// A look-back that runs out leaves offsets that do not belong together: the
+// failure word beside the block counter then keeps the emits from using them.
 constexpr uint64_t kScanAgg = 1ull << 63, kScanIncl = 1ull << 62, kScanCount = kScanIncl - 1;
 
 struct ScanWord {
@@ -67,7 +70,8 @@ struct ScanArgs {
     uint32_t *offsets, *coff, *chunk_first;
     uint32_t chunk_cap;
     ScanWord *status;  // one per block, zero
-    uint32_t *counter;
+    uint32_t *counter;  // block counter, then the scan's failure word (zero): set when a look-back runs out
+    const uint32_t *order_failed;  // DUAL, or null: the failure word of the sort that made perm
     uint64_t *n_pairs, *n_pairs_host, *n_cells;
     uint64_t capacity;
     uint32_t *err;
@@ -82,6 +86,8 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
     __syncthreads();
     const uint32_t b = s_block;
     const int n = A.n;
+    // (an order with gaps is not gathered through: every count reads as zero)
+    const size_t n_in = DUAL && A.order_failed && *A.order_failed ? 0 : (size_t)n;
     const int nb = (n + kScanChunk - 1) / kScanChunk;
     const size_t base = (size_t)b * kScanChunk + (size_t)tid * kScanItems;
     const bool whole = base + kScanItems <= (size_t)n;
@@ -90,7 +96,7 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
         uint32_t g[kScanItems];
         // 16-byte loads where perm allows them (a batch camera's order starts at a
         // multiple of n records, which need not be one of four)
-        if (whole && (reinterpret_cast<uintptr_t>(A.perm) & 15) == 0) {
+        if (base + kScanItems <= n_in && (reinterpret_cast<uintptr_t>(A.perm) & 15) == 0) {
 #pragma unroll
             for (int q = 0; q < kScanItems / 4; ++q) {
                 const uint4 v = reinterpret_cast<const uint4 *>(A.perm + base)[q];
@@ -98,11 +104,11 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
             }
         } else {
 #pragma unroll
-            for (int k = 0; k < kScanItems; ++k) g[k] = base + k < (size_t)n ? A.perm[base + k] : 0u;
+            for (int k = 0; k < kScanItems; ++k) g[k] = base + k < n_in ? A.perm[base + k] : 0u;
         }
 #pragma unroll
         for (int k = 0; k < kScanItems; ++k) {
-            const uint2 v = base + k < (size_t)n ? A.cc[g[k]] : make_uint2(0u, 0u);
+            const uint2 v = base + k < n_in ? A.cc[g[k]] : make_uint2(0u, 0u);
             c[k] = v.x;
             d[k] = v.y;
         }
@@ -155,10 +161,20 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
         t -= used;
         if (used == 0) {  // the nearest earlier block has not published yet
             if (++spins > kSpinLimit) {
-                if (tid == 0) atomicOr(A.err, kErrTimeout);
+                if (tid == 0) {
+                    atomicOr(A.err, kErrTimeout);
+                    A.counter[1] = 1u;
+                }
                 break;
             }
             __nanosleep(64);
+        }
+    }
+    if (b == 1 && (ld_relaxed(A.err + 1) & kTestScan)) {  // test-only (stall_test)
+        acc = accd = 0;
+        if (tid == 0) {
+            atomicOr(A.err, kErrTimeout);
+            A.counter[1] = 1u;
         }
     }
     if (tid == 0) {
@@ -213,8 +229,13 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
     }
 }
 
-// 64-bit words of scratch: the blocks' status words, then the block counter
+// 64-bit words of scratch: the blocks' status words, then the block counter and the failure word
 size_t scan_partials_count(int n) { return 2 * (size_t)((n + kScanChunk - 1) / kScanChunk) + 2; }
+
+const uint32_t *scan_failed(const uint64_t *partials, int n) {
+    if (n == 0) return nullptr;
+    return reinterpret_cast<const uint32_t *>(partials + 2 * ((n + kScanChunk - 1) / kScanChunk)) + 1;
+}
 
 static cudaError_t run_scan(ScanArgs A, uint64_t *partials, bool dual, cudaStream_t s) {
     if (A.n == 0) {
@@ -251,9 +272,10 @@ cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32
 
 cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint32_t *offsets, uint32_t *coff,
                               uint64_t *partials, uint64_t *n_pairs, uint64_t *n_pairs_host, uint64_t *n_cells,
-                              uint64_t capacity, uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap,
-                              cudaStream_t s) {
+                              uint64_t capacity, uint32_t *err, const uint32_t *order_failed, uint32_t *chunk_first,
+                              uint32_t chunk_cap, cudaStream_t s) {
     ScanArgs A{};
+    A.order_failed = order_failed;
     A.n_pairs_host = n_pairs_host;
     A.chunk_first = chunk_first;
     A.chunk_cap = chunk_cap;
@@ -398,6 +420,7 @@ __global__ void __launch_bounds__(kEmitWarps * 32) emit_warp_kernel(EmitArgs a, 
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t P = *a.n_pairs;
     const uint64_t warp_id = (uint64_t)blockIdx.x * kEmitWarps + wid;
+    if (*a.failed) return;
     if (P > a.capacity) {
         if (warp_id == 0 && lane == 0) atomicOr(a.err, kErrCapacity);
         return;
@@ -419,7 +442,7 @@ __global__ void __launch_bounds__(kEmitWarps * 32) emit_warp_kernel(EmitArgs a, 
 // skips tiles an earlier sub-box already holds.
 __global__ void __launch_bounds__(256) emit_naive_kernel(EmitArgs a, uint64_t *__restrict__ keys) {
     const size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= (size_t)a.n) return;
+    if (j >= (size_t)a.n || *a.failed) return;
     if (*a.n_pairs > a.capacity) {
         if (j == 0) atomicOr(a.err, kErrCapacity);
         return;
@@ -461,11 +484,13 @@ cudaError_t launch_emit(const EmitArgs &a, uint64_t *keys, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// K5: tile boundaries of the sorted keys; ranges must be zero on entry.
+// K5: tile boundaries of the sorted keys; ranges must be zero on entry, and
+// stay so when the scan or the sort before it failed.
 __device__ __forceinline__ uint32_t tile_of(uint64_t k) { return (uint32_t)(k >> kDepthBits); }
 
 __global__ void ranges_kernel(const uint64_t *keys, uint64_t n_max, const uint64_t *n_dev, uint2 *ranges,
-                              uint32_t ntiles) {
+                              uint32_t ntiles, const uint32_t *scan_fail, const uint32_t *sort_fail) {
+    if ((scan_fail && *scan_fail) || *sort_fail) return;
     uint64_t n = n_dev ? (*n_dev > n_max ? 0 : *n_dev) : n_max;  // overflow (flagged by the emit): no pairs
     for (uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
          idx += (uint64_t)gridDim.x * blockDim.x) {
@@ -477,12 +502,12 @@ __global__ void ranges_kernel(const uint64_t *keys, uint64_t n_max, const uint64
 }
 
 cudaError_t launch_ranges(const uint64_t *keys, uint64_t n_max, const uint64_t *n_dev, uint2 *ranges, int ntiles,
-                          cudaStream_t s) {
+                          const uint32_t *scan_fail, void *sort_scratch, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(ranges, 0, sizeof(uint2) * (size_t)ntiles, s);
     if (e != cudaSuccess || n_max == 0) return e;
     uint64_t blocks = (n_max + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    note_launch("ranges_kernel", s), ranges_kernel<<<(unsigned)blocks, 256, 0, s>>>(keys, n_max, n_dev, ranges, (uint32_t)ntiles);
+    note_launch("ranges_kernel", s), ranges_kernel<<<(unsigned)blocks, 256, 0, s>>>(keys, n_max, n_dev, ranges, (uint32_t)ntiles, scan_fail, sort_failed_at(sort_scratch));
     return cudaGetLastError();
 }
 

@@ -181,7 +181,7 @@ __device__ __forceinline__ void cell_emit_range(const CellBin &b, uint64_t E, ui
 __device__ __forceinline__ void cell_emit_naive(const CellBin &b, int64_t j, uint32_t *hist) {
     const uint32_t gid = b.perm[j];
     const uint32_t off = b.coff[j];
-    const uint32_t end = j + 1 < b.n ? b.coff[j + 1] : (uint32_t)*b.n_cells;
+    const uint32_t end = j + 1 < b.n ? b.coff[j + 1] : (uint32_t)*b.n_cells;  // (only where no scan failed)
     if (end == off) return;
     const uint4 w0 = b.rects[2 * (size_t)gid], w1 = b.rects[2 * (size_t)gid + 1];
     const Rect r[4] = {cell_rect(unpack_rect(w0.x, w0.y)), cell_rect(unpack_rect(w0.z, w0.w)),
@@ -288,11 +288,11 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     __shared__ bool s_last;
     const int tid = threadIdx.x, wid = tid >> 5;
     const bool in_smem = b.geo.ncells < kCellHistMax;
-    const uint64_t E = *b.n_cells;
-    if (blockIdx.x == 0 && tid == 0) {
-        const uint64_t P = *b.n_pairs;
-        if (P > b.capacity || (P > 0 && E == 0)) atomicOr(b.err, kErrCapacity);
-    }
+    // after a scan that failed its offsets and counts do not belong together:
+    // no entries
+    const bool failed = b.scan_failed && *b.scan_failed;
+    const uint64_t E = failed ? 0ull : *b.n_cells;
+    if (blockIdx.x == 0 && tid == 0 && *b.n_pairs > b.capacity) atomicOr(b.err, kErrCapacity);
     if (in_smem)
         for (int c = tid; c <= b.geo.ncells; c += blockDim.x) s_hist[c] = 0u;
     const uint64_t threads = (uint64_t)gridDim.x * blockDim.x, gt = (uint64_t)blockIdx.x * blockDim.x + tid;
@@ -303,6 +303,7 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
         for (uint64_t i = gt; i < words; i += threads) lb[i] = 0u;
         if (gt == 0) *sort_counter_at(b.sort_scratch, p) = 0u;
     }
+    if (gt == 0) *sort_failed_at(b.sort_scratch) = 0u;
     __syncthreads();
     uint32_t *hist = in_smem ? s_hist : b.arr.count;
     if constexpr (NAIVE) {
@@ -328,6 +329,7 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     __syncthreads();
     if (!s_last) return;
     __threadfence();
+    if (failed && tid == 0) *b.n_cells = 0ull;  // (every block has read it)
     cell_prepare(b, reinterpret_cast<uint32_t *>(smem));  // the table and histogram are no longer needed
 }
 
@@ -418,7 +420,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) cell_count_kernel(CellGeo g, C
 // block scans the totals into the ranges ([0, 0) for an empty tile).
 constexpr int kPrefixThreads = 512;
 __global__ void __launch_bounds__(kPrefixThreads, 3) cell_prefix_kernel(CellGeo g, CellArrays a, uint2 *__restrict__ ranges,
-                                                           const uint64_t *n_pairs, const uint64_t *n_cells) {
+                                                           const uint64_t *n_pairs, const uint64_t *n_cells,
+                                                           const uint32_t *sort_failed) {
     __shared__ uint32_t s_part[kPrefixThreads / 32][32];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -477,9 +480,10 @@ __global__ void __launch_bounds__(kPrefixThreads, 3) cell_prefix_kernel(CellGeo 
         }
         before += tot;
     }
-    // After a look-back time-out the sorted entries are undefined: unless the
-    // tiles' totals add up to the pairs there are, nothing is expanded.
-    if (*n_cells > 0 && before != *n_pairs) {
+    // After a look-back time-out the sorted entries are undefined, and some of
+    // them whatever the buffer held: nothing is expanded.  (Nor if the tiles'
+    // totals did not add up to the pairs there are.)
+    if (*sort_failed || (*n_cells > 0 && before != *n_pairs)) {
         for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) ranges[t] = make_uint2(0u, 0u);
         if (threadIdx.x == 0) a.row_start[g.ncells] = 0u;
     }
@@ -549,7 +553,8 @@ cudaError_t launch_cell_sort(const CellBin &b, cudaStream_t s) {
     note_launch("cell_count_kernel", s),
         cell_count_kernel<<<(unsigned)blocks, kRowWarps * 32, 0, s>>>(b.geo, b.arr, sorted);
     note_launch("cell_prefix_kernel", s),
-        cell_prefix_kernel<<<b.geo.ncells, kPrefixThreads, 0, s>>>(b.geo, b.arr, b.ranges, b.n_pairs, b.n_cells);
+        cell_prefix_kernel<<<b.geo.ncells, kPrefixThreads, 0, s>>>(b.geo, b.arr, b.ranges, b.n_pairs, b.n_cells,
+                                                                sort_failed_at(b.sort_scratch));
     note_launch("cell_expand_kernel", s),
         cell_expand_kernel<<<(unsigned)blocks, kRowWarps * 32, 0, s>>>(b.geo, b.arr, sorted, b.ranges, b.vals);
     return cudaGetLastError();

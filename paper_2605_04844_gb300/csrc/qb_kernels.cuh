@@ -85,6 +85,7 @@ struct EmitArgs {
     uint64_t capacity;
     int mode;
     uint32_t *err;
+    const uint32_t *failed;  // the scan's failure word: nothing is emitted when it is set
     uint32_t tiles_x;
 };
 
@@ -119,7 +120,9 @@ struct CellBin {
     const uint32_t *coff;   // first entry of each emission position
     const uint32_t *chunk_first;
     const uint4 *rects;     // by record
-    const uint64_t *n_pairs, *n_cells;
+    const uint64_t *n_pairs;
+    uint64_t *n_cells;      // set to 0 when the scan failed
+    const uint32_t *scan_failed;  // the scan's failure word, or null (depth_order_failed)
     uint64_t n_cells_max;   // bound on *n_cells (the capacity, or P where the host knows it)
     uint64_t capacity;
     bool naive;             // emit by nested loops (QB_BIN_QUADBOX_NAIVE)
@@ -242,8 +245,11 @@ cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32
                         uint32_t chunk_cap, cudaStream_t s);
 cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint32_t *offsets, uint32_t *coff,
                               uint64_t *partials, uint64_t *n_pairs, uint64_t *n_pairs_host, uint64_t *n_cells,
-                              uint64_t capacity, uint32_t *err, uint32_t *chunk_first, uint32_t chunk_cap,
-                              cudaStream_t s);
+                              uint64_t capacity, uint32_t *err, const uint32_t *order_failed, uint32_t *chunk_first,
+                              uint32_t chunk_cap, cudaStream_t s);
+// The word of a scan's scratch that is not zero after a look-back ran out (the
+// offsets are then of no use), or null for n = 0.
+const uint32_t *scan_failed(const uint64_t *partials, int n);
 // The depth order of n Gaussians (keys and record indices from the
 // preprocess) and the scan in that order.
 struct OrderArgs {
@@ -259,6 +265,8 @@ struct OrderArgs {
 };
 // *in_alt: the order lies in vals_alt.
 cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *in_alt);
+// The failure word of its scan, or null where n is so small that none runs.
+const uint32_t *depth_order_failed(const uint64_t *partials, int n);
 // Output positions per entry of the scan's chunk table (a divisor of every
 // emit kernel's per-warp output range).
 constexpr uint32_t kEmitStride = 128;
@@ -266,8 +274,9 @@ inline uint64_t chunk_table_size(uint64_t pair_capacity) { return pair_capacity 
 size_t scan_partials_count(int n);
 cudaError_t launch_emit(const EmitArgs &a, uint64_t *keys, cudaStream_t s);
 cudaError_t launch_expand_ranges(const uint2 *ranges, int ntiles, uint32_t *out, uint64_t n_out, cudaStream_t s);
+// scan_fail: the failure word of the pairs' scan, or null; sort_scratch: of their sort.
 cudaError_t launch_ranges(const uint64_t *keys, uint64_t n_max, const uint64_t *n_dev, uint2 *ranges, int ntiles,
-                          cudaStream_t s);
+                          const uint32_t *scan_fail, void *sort_scratch, cudaStream_t s);
 // The depth-first binning after the depth order and the scan: the emit of
 // (cell, Gaussian, tile bits) entries; then their sort by cell and the
 // expansion to the sorted values and ranges.

@@ -272,7 +272,12 @@ cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *
     }
     *in_alt = passes & 1;
     return launch_scan_cells(a.cc, *in_alt ? a.vals_alt : a.vals, n, a.offsets, a.coff, a.partials, a.n_pairs,
-                             a.n_pairs_host, a.n_cells, a.capacity, a.err, a.chunk_first, a.chunk_cap, s);
+                             a.n_pairs_host, a.n_cells, a.capacity, a.err, n > 0 ? sort_failed_at(a.sort_scratch) : nullptr,
+                             a.chunk_first, a.chunk_cap, s);
+}
+
+const uint32_t *depth_order_failed(const uint64_t *partials, int n) {
+    return n > kOrderSmall ? scan_failed(partials, n) : nullptr;
 }
 
 }  // namespace qb

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kSortBlock, sizeof(KeyT) == 4 ? kSortBlocksPer
                                                               uint64_t n_max, const uint64_t *n_dev,
                                                               const uint32_t *__restrict__ bin_off,
                                                               uint32_t *lookback, uint32_t *counter, int shift,
-                                                              uint32_t mask, uint32_t *err) {
+                                                              uint32_t mask, uint32_t *err, uint32_t *failed) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ uint32_t s_tile;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -138,19 +138,20 @@ __global__ void __launch_bounds__(kSortBlock, sizeof(KeyT) == 4 ? kSortBlocksPer
         key[k] = idx < n ? __ldcs(kin + idx) : KeyT(0);
     }
     auto val = [&](int k) -> uint32_t { return __ldcs(vin + wbase + 32 * k + lane); };
-    sweep_tile<RB, KeyT, uint32_t, true, ITEMS>(key, val, n, tbase, tile, bin_off, lookback, shift, mask, err, kout,
-                                                vout, smem);
+    sweep_tile<RB, KeyT, uint32_t, true, ITEMS>(key, val, n, tbase, tile, bin_off, lookback, shift, mask, err, failed,
+                                                kout, vout, smem);
 }
 
 template <int RB, typename KeyT, int ITEMS>
 static cudaError_t launch_pass_t(const KeyT *kin, const uint32_t *vin, KeyT *kout, uint32_t *vout, uint64_t n_max,
                                  const uint64_t *n_dev, const uint32_t *bin_off, uint32_t *lookback,
-                                 uint32_t *counter, int shift, uint32_t mask, uint32_t *err, cudaStream_t s) {
+                                 uint32_t *counter, int shift, uint32_t mask, uint32_t *err, uint32_t *failed,
+                                 cudaStream_t s) {
     constexpr size_t smem = sweep_smem<RB, KeyT, uint32_t, ITEMS>();
     cudaError_t e = ensure_dyn_smem((const void *)onesweep_kernel<RB, KeyT, ITEMS>, smem);
     if (e != cudaSuccess) return e;
     note_launch("onesweep_kernel", s), onesweep_kernel<RB, KeyT, ITEMS><<<(unsigned)((n_max + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS)), kSortBlock, smem, s>>>(
-        kin, vin, kout, vout, n_max, n_dev, bin_off, lookback, counter, shift, mask, err);
+        kin, vin, kout, vout, n_max, n_dev, bin_off, lookback, counter, shift, mask, err, failed);
     return cudaGetLastError();
 }
 
@@ -158,11 +159,12 @@ static cudaError_t launch_pass_t(const KeyT *kin, const uint32_t *vin, KeyT *kou
 template <typename KeyT>
 static cudaError_t launch_pass(const KeyT *kin, const uint32_t *vin, KeyT *kout, uint32_t *vout, uint64_t n_max,
                                const uint64_t *n_dev, const uint32_t *bin_off, uint32_t *lookback,
-                               uint32_t *counter, int shift, int bits, uint32_t *err, int items,
+                               uint32_t *counter, int shift, int bits, uint32_t *err, uint32_t *failed, int items,
                                cudaStream_t s) {
     const uint32_t mask = (1u << bits) - 1u;
 #define QB_PASS_RUN(RB, ITEMS)                                                                                     \
-    launch_pass_t<RB, KeyT, ITEMS>(kin, vin, kout, vout, n_max, n_dev, bin_off, lookback, counter, shift, mask, err, s)
+    launch_pass_t<RB, KeyT, ITEMS>(kin, vin, kout, vout, n_max, n_dev, bin_off, lookback, counter, shift, mask, err,   \
+                                   failed, s)
 #define QB_PASS_CASE(RB)                                                                                           \
     case RB:                                                                                                       \
         if constexpr (sizeof(KeyT) == 4 && RB >= 7 && RB <= 8) {                                                   \
@@ -230,7 +232,7 @@ static cudaError_t sort_impl(KeyT *keys, uint32_t *vals, KeyT *keys_alt, uint32_
     for (int p = 0; p < g.passes; ++p) {
         e = launch_pass<KeyT>(kin, vin, kout, vout, n_max, n_dev, hist + p * kHistStride,
                               sort_lookback_at(scratch, 0, digit_bits, 0) + p * pass_words,
-                              sort_counter_at(scratch, p), g.shift[p], g.bits[p], err, items, s);
+                              sort_counter_at(scratch, p), g.shift[p], g.bits[p], err, sort_failed_at(scratch), items, s);
         if (e != cudaSuccess) return e;
         std::swap(kin, kout);
         std::swap(vin, vout);
@@ -259,7 +261,7 @@ template <int RB, bool WRITE_KEYS>
 __global__ void __launch_bounds__(kSortBlock, RB <= 8 ? kCellSortBlocksPerSM : 2) cell_sort_kernel(
     const uint32_t *__restrict__ kin, const uint64_t *__restrict__ vin, uint32_t *__restrict__ kout,
     uint64_t *__restrict__ vout, const uint64_t *n_dev, const uint32_t *__restrict__ bin_off, uint32_t *lookback,
-    uint32_t *counter, int shift, uint32_t mask, uint32_t *err) {
+    uint32_t *counter, int shift, uint32_t mask, uint32_t *err, uint32_t *failed) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ uint32_t s_tile;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -280,7 +282,7 @@ __global__ void __launch_bounds__(kSortBlock, RB <= 8 ? kCellSortBlocksPerSM : 2
         }
         auto val = [&](int k) -> uint64_t { return __ldcs(vin + wbase + 32 * k + lane); };
         sweep_tile<RB, uint32_t, uint64_t, WRITE_KEYS, kSortItems>(key, val, n, tbase, tile, bin_off, lookback, shift, mask, err,
-                                                       kout, vout, smem);
+                                                       failed, kout, vout, smem);
         __syncthreads();  // shared memory is taken again
     }
 }
@@ -301,7 +303,7 @@ static cudaError_t launch_cell_pass(const CellBin &b, int p, const uint32_t *kin
         cell_sort_kernel<RB, WRITE_KEYS><<<(unsigned)blocks, kSortBlock, smem, s>>>(
             kin, vin, kout, vout, b.n_cells, sort_hist_at(b.sort_scratch) + p * kHistStride,
             sort_lookback_at(b.sort_scratch, b.capacity, b.geo.digit_bits, p), sort_counter_at(b.sort_scratch, p),
-            b.geo.passes.shift[p], (1u << bits) - 1u, b.err);
+            b.geo.passes.shift[p], (1u << bits) - 1u, b.err, sort_failed_at(b.sort_scratch));
     return cudaGetLastError();
 }
 

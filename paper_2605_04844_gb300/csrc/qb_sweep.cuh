@@ -10,7 +10,11 @@
 // digits leave as contiguous stores.  Tile indices are taken from an atomic
 // counter in launch order, so every earlier tile belongs to a block that is
 // already running.  Every look-back spin is bounded; on expiry it raises
-// kErrTimeout and still publishes, so no block waits forever.
+// kErrTimeout and still publishes, so no block waits forever.  The output then
+// has gaps (whatever the buffer held) and is no order any more: the sort's own
+// word sort_failed_at tells the kernels after it, which must not gather through
+// it (the count scan, the cell prefix and the full-key ranges then give an
+// empty frame).
 #pragma once
 
 #include <type_traits>
@@ -32,7 +36,7 @@ constexpr uint32_t kFlagIncl = 2u << 30;
 constexpr uint32_t kCountMask = (1u << 30) - 1u;
 constexpr int kHistStride = 1 << kMaxDigitBits;  // per-pass stride of the histogram table
 // scratch: [bucket offset table: kMaxPasses x kHistStride u32][tile counters:
-// kMaxPasses u32, padded to 256 B][look-back words: passes x tiles x 2^RB u32]
+// kMaxPasses u32, the histogram's block counter, the failure word, padded to 256 B][look-back words: passes x tiles x 2^RB u32]
 constexpr size_t kSortCounters = (size_t)kMaxPasses * kHistStride * 4;
 constexpr size_t kSortHeader = kSortCounters + 256;
 
@@ -62,15 +66,23 @@ __device__ __forceinline__ void st_relaxed(uint32_t *p, uint32_t v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Not zero after a sort one of whose look-backs ran out (zeroed with the
+// counters before the sort's first pass).
+__host__ __device__ inline uint32_t *sort_failed_at(void *scratch) { return sort_counter_at(scratch, kMaxPasses + 1); }
+
 // The error word err[0] is followed by a test-only word, zero in normal use:
-// when err[1] > 0, the block of tile 1 of every values-only pass (the last
-// pass of a tile sort, whose output only the render reads) finds tile 0's
-// status words unpublished and gives up after err[1] polls, so its wait runs
-// out deterministically and raises kErrTimeout.  Its scatter positions then
-// fall short of the true ones but stay inside [0, n); the sorted values are
-// undefined.  Other waits keep the kSpinLimit bound.
+// when 0 < err[1] < kTestScan, the block of tile 1 of every values-only pass
+// (the last pass of a cell sort, whose output only the expansion reads) finds
+// tile 0's status words unpublished and gives up after err[1] polls, so its
+// wait runs out deterministically and raises kErrTimeout.  Its scatter
+// positions then fall short of the true ones but stay inside [0, n); the sorted
+// values are undefined.  With kTestKeyed the same block of every other pass,
+// with kTestScan block 1 of the count scan, ends its walk as if the wait had run
+// out before the first word.  Other waits keep the kSpinLimit bound.
+constexpr uint32_t kTestScan = 1u << 29, kTestKeyed = 1u << 30;
 __device__ __forceinline__ uint32_t stall_test(const uint32_t *err, uint32_t tile) {
-    return tile == 1 ? ld_relaxed(err + 1) : 0u;
+    const uint32_t k = tile == 1 ? ld_relaxed(err + 1) : 0u;
+    return k < kTestScan ? k : 0u;
 }
 
 // Elements to sort: the device count when given, treated as zero when it
@@ -133,13 +145,14 @@ constexpr size_t sweep_smem() {
 // values late and keep fewer registers live).  bin_off: the pass's exclusive
 // bucket offsets; lookback: the pass's status words [tiles][2^RB].  Without
 // WRITE_KEYS (the last pass of a sort whose keys its ranges imply) only the
-// values are written.  64-bit values go with 32-bit keys.
+// values are written.  64-bit values go with 32-bit keys.  failed: set when the
+// look-back runs out.
 template <int RB, typename KeyT, typename ValT, bool WRITE_KEYS, int ITEMS, class ValFn>
 __device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val,
                                            uint32_t n, uint32_t tbase, uint32_t tile,
                                            const uint32_t *__restrict__ bin_off, uint32_t *lookback, int shift,
-                                           uint32_t mask, uint32_t *err, KeyT *__restrict__ kout,
-                                           ValT *__restrict__ vout, uint8_t *smem) {
+                                           uint32_t mask, uint32_t *err, uint32_t *failed,
+                                           KeyT *__restrict__ kout, ValT *__restrict__ vout, uint8_t *smem) {
     static_assert(sizeof(KeyT) + sizeof(ValT) <= 12, "64-bit values go with 32-bit keys");
     constexpr int R = 1 << RB;
     constexpr int PER = (R + kSortBlock - 1) / kSortBlock;
@@ -275,9 +288,15 @@ __device__ __forceinline__ void sweep_tile(const KeyT (&key)[ITEMS], ValFn &&val
                     }
                     if (spins > limit) {
                         atomicOr(err, kErrTimeout);
+                        *failed = 1u;
                         break;
                     }
                 }
+            }
+            if (WRITE_KEYS && tile == 1 && (ld_relaxed(err + 1) & kTestKeyed)) {  // test-only
+                acc = 0;
+                atomicOr(err, kErrTimeout);
+                *failed = 1u;
             }
             st_relaxed(lb + d, kFlagIncl | ((acc + cnt[j]) & kCountMask));
         }
