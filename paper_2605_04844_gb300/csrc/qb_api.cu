@@ -175,41 +175,71 @@ CamSet frame_camset(const qb_camera &c) {
     return cs;
 }
 
-// A word of mapped host memory per host thread, that the count scan writes P
-// to: a synchronised qb_bin_emit then waits for the stream only, without a
-// device-to-host copy behind the scan.  Freed when the thread ends.
-struct HostWord {
-    volatile uint64_t *host = nullptr;
-    uint64_t *device = nullptr;
-    bool tried = false;
-    bool get() {
-        if (!tried) {
-            tried = true;
-            void *h = nullptr, *d = nullptr;
-            // (an allocation must not disturb a graph capture of another thread)
-            cudaStreamCaptureMode capture = cudaStreamCaptureModeRelaxed;
-            (void)cudaThreadExchangeStreamCaptureMode(&capture);
-            const cudaError_t e = cudaHostAlloc(&h, sizeof(uint64_t), cudaHostAllocPortable | cudaHostAllocMapped);
-            (void)cudaThreadExchangeStreamCaptureMode(&capture);
-            if (e != cudaSuccess) {
-                (void)cudaGetLastError();
-                return false;
-            }
-            if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess || d != h) {  // one address on every device
-                (void)cudaGetLastError();
-                (void)cudaFreeHost(h);
-                return false;
-            }
-            host = static_cast<volatile uint64_t *>(h);
-            device = static_cast<uint64_t *>(d);
+// Words of mapped host memory that the count scan writes P to: a synchronised
+// qb_bin_emit then waits for the stream only, without a device-to-host copy
+// behind the scan.  One page of kSlots words per CUDA context, kept until the
+// context ends (which frees it); a call takes a word and gives it back after its
+// synchronisation, so threads and streams never share one.  Without a free word
+// (or in a 17th context) the count is copied.  The word of a call that failed
+// before it synchronised stays taken: a kernel may still write it.  Nothing is
+// freed when a host thread ends, which could be during another's graph capture.
+class PairWords {
+public:
+    struct Word {
+        volatile uint64_t *host = nullptr;  // the device's address too
+        int page = 0, slot = 0;
+    };
+    Word take() {
+        Word w;
+        const uint64_t id = context_id();
+        if (id == 0) return w;
+        std::lock_guard<std::mutex> lock(mu_);
+        int p = 0;
+        while (p < n_ && pages_[p].context != id) ++p;
+        if (p == kPages) return w;
+        if (p == n_) pages_[n_++] = Page{id, allocate(), ~0ull};
+        if (!pages_[p].words || pages_[p].free == 0) return w;
+        w.page = p;
+        w.slot = __builtin_ctzll(pages_[p].free);
+        w.host = pages_[p].words + w.slot * kStride;
+        pages_[p].free &= pages_[p].free - 1;
+        return w;
+    }
+    void give_back(const Word &w) {
+        std::lock_guard<std::mutex> lock(mu_);
+        pages_[w.page].free |= 1ull << w.slot;
+    }
+
+private:
+    static constexpr int kSlots = 64, kStride = 8;  // a cache line each
+    static constexpr int kPages = 16;
+    struct Page {
+        uint64_t context;
+        uint64_t *words;  // null: could not be allocated
+        uint64_t free;
+    };
+    static uint64_t *allocate() {
+        void *h = nullptr, *d = nullptr;
+        // (neither call may disturb a graph capture of another thread)
+        cudaStreamCaptureMode capture = cudaStreamCaptureModeRelaxed;
+        (void)cudaThreadExchangeStreamCaptureMode(&capture);
+        if (cudaHostAlloc(&h, sizeof(uint64_t) * kSlots * kStride, cudaHostAllocPortable | cudaHostAllocMapped) !=
+            cudaSuccess) {
+            h = nullptr;
+            (void)cudaGetLastError();
+        } else if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess || d != h) {  // one address on every device
+            (void)cudaGetLastError();
+            (void)cudaFreeHost(h);
+            h = nullptr;
         }
-        return host != nullptr;
+        (void)cudaThreadExchangeStreamCaptureMode(&capture);
+        return static_cast<uint64_t *>(h);
     }
-    ~HostWord() {
-        if (host) (void)cudaFreeHost(const_cast<uint64_t *>(host));
-    }
+    std::mutex mu_;
+    Page pages_[kPages] = {};
+    int n_ = 0;
 };
-thread_local HostWord t_pairs;
+PairWords g_pair_words;
 
 qb_status check_frame(const qb_frame *f, Layout &L) {
     if (!f || !f->workspace) return fail(QB_ERR_INVALID_ARG, "frame is NULL or not initialised");
@@ -248,6 +278,28 @@ void note_launch(const char *kernel, cudaStream_t s) {
     g_launches.fetch_add(1, std::memory_order_relaxed);
     const qb_launch_hook h = g_hook.load(std::memory_order_acquire);
     if (h) h(kernel, (qb_stream_t)s, g_hook_user.load(std::memory_order_relaxed));
+}
+
+uint64_t context_id() {
+    using GetId = int (*)(void *, unsigned long long *);  // cuCtxGetId
+    static const GetId get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<GetId>(f);
+    }();
+    unsigned long long id = 0;
+    if (!get) return 0;
+    if (get(nullptr, &id) == 0) return id;
+    // no current context yet (a new thread, or after a reset): the runtime makes
+    // one (by a call that no graph capture of another thread forbids)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) (void)cudaGetLastError();
+    return get(nullptr, &id) == 0 ? id : 0;
 }
 
 cudaError_t ensure_dyn_smem(const void *func, size_t bytes) {
@@ -433,7 +485,9 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
     uint64_t *d_np = at<uint64_t>(frame, L.state);
     uint32_t *err = at<uint32_t>(frame, L.state + 8);
     const bool depth_first = frame->sort_mode != QB_SORT_FULL_KEY;  // Gaussians emitted in depth order
-    const bool mapped = n_pairs_out && frame->n > 0 && t_pairs.get();
+    PairWords::Word word;
+    if (n_pairs_out && frame->n > 0) word = g_pair_words.take();
+    uint64_t *const host_word = const_cast<uint64_t *>(word.host);
     uint64_t *partials = at<uint64_t>(frame, L.scan_part);
     uint32_t *chunk_first = at<uint32_t>(frame, L.chunk_first);
     const uint32_t chunk_cap = (uint32_t)chunk_table_size(frame->pair_capacity);
@@ -454,7 +508,7 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
         o.chunk_cap = chunk_cap;
         o.partials = partials;
         o.n_pairs = d_np;
-        o.n_pairs_host = mapped ? t_pairs.device : nullptr;
+        o.n_pairs_host = host_word;
         o.n_cells = at<uint64_t>(frame, L.state + 16);
         o.capacity = frame->pair_capacity;
         o.err = err;
@@ -463,15 +517,18 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
         frame->depth_in_alt = in_alt;
     } else {
         QB_CUDA(launch_scan(at<uint32_t>(frame, L.counts), frame->n, at<uint32_t>(frame, L.offsets),
-                            at<uint32_t>(frame, L.coff), partials, d_np, mapped ? t_pairs.device : nullptr, err,
+                            at<uint32_t>(frame, L.coff), partials, d_np, host_word, err,
                             chunk_first, chunk_cap, s));
     }
     frame->n_pairs = UINT64_MAX;
     if (n_pairs_out) {
         uint64_t P = 0;
-        if (!mapped) QB_CUDA(cudaMemcpyAsync(&P, d_np, sizeof(P), cudaMemcpyDeviceToHost, s));
+        if (!host_word) QB_CUDA(cudaMemcpyAsync(&P, d_np, sizeof(P), cudaMemcpyDeviceToHost, s));
         QB_CUDA(cudaStreamSynchronize(s));
-        if (mapped) P = *t_pairs.host;
+        if (host_word) {
+            P = *word.host;
+            g_pair_words.give_back(word);
+        }
         *n_pairs_out = P;
         if (P > frame->pair_capacity) {
             frame->stage = 1;

@@ -66,6 +66,10 @@ void set_last_error(const char *msg);
 // Counts one kernel launch of the library (qb_kernel_launches) and reports
 // it to the launch hook, if one is set, just before the launch on stream s.
 void note_launch(const char *kernel, cudaStream_t s);
+// A number of the calling thread's CUDA context that no other context of the
+// process has or had (a cudaDeviceReset makes a new one), or 0 if it cannot be
+// told.  What is kept from one call for the next is kept under it.
+uint64_t context_id();
 // Raises kernel func's dynamic shared-memory limit on the current device to
 // at least bytes; the limit set is remembered per (kernel, device), and the
 // calls are safe from several host threads.
