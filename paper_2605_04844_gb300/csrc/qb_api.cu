@@ -304,14 +304,12 @@ uint64_t context_id() {
 
 cudaError_t ensure_dyn_smem(const void *func, size_t bytes) {
     static std::mutex mu;
-    static std::map<std::pair<const void *, int>, size_t> set;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
+    static std::map<std::pair<const void *, uint64_t>, size_t> set;
+    const uint64_t id = context_id();
     std::lock_guard<std::mutex> lock(mu);
-    size_t &have = set[{func, dev}];
+    size_t none = 0, &have = id ? set[{func, id}] : none;
     if (bytes <= have) return cudaSuccess;
-    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) have = bytes;
     return e;
 }

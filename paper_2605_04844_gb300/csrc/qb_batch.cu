@@ -163,6 +163,7 @@ bool make_blayout(int n, int n_cams, int group, uint64_t cap, const Geo &g, BLay
 // qb_batch_init and destroyed by qb_batch_release.
 struct SideStreams {
     int device;
+    uint64_t context;  // (those of a context that has been reset are gone)
     cudaStream_t side[kBatchStreams];
     cudaEvent_t fork, join[kBatchStreams];
 };
@@ -175,13 +176,15 @@ cudaError_t side_create(const void *ws, SideStreams &out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (it != g_side.end() && it->second.device == dev) {
+    const uint64_t context = context_id();
+    if (it != g_side.end() && it->second.device == dev && it->second.context == context) {
         out = it->second;
         return cudaSuccess;
     }
     SideStreams ss;
     std::memset(&ss, 0, sizeof(ss));
     ss.device = dev;
+    ss.context = context;
     for (int i = 0; i < kBatchStreams && e == cudaSuccess; ++i) {
         e = cudaStreamCreateWithFlags(&ss.side[i], cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.join[i], cudaEventDisableTiming);
@@ -381,7 +384,7 @@ qb_status qb_batch_release(qb_batch *batch) {
             g_side.erase(it);
         }
     }
-    if (found) {
+    if (found && ss.context == context_id()) {
         for (int i = 0; i < kBatchStreams; ++i) {
             QB_BCUDA(cudaStreamSynchronize(ss.side[i]));
             QB_BCUDA(cudaStreamDestroy(ss.side[i]));

@@ -70,8 +70,8 @@ void note_launch(const char *kernel, cudaStream_t s);
 // process has or had (a cudaDeviceReset makes a new one), or 0 if it cannot be
 // told.  What is kept from one call for the next is kept under it.
 uint64_t context_id();
-// Raises kernel func's dynamic shared-memory limit on the current device to
-// at least bytes; the limit set is remembered per (kernel, device), and the
+// Raises kernel func's dynamic shared-memory limit in the current context to
+// at least bytes; the limit set is remembered per (kernel, context), and the
 // calls are safe from several host threads.
 cudaError_t ensure_dyn_smem(const void *func, size_t bytes);
 
