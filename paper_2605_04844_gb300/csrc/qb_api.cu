@@ -1,4 +1,5 @@
 // qb_api.cu -- the extern "C" entry points of libquadbox (include/quadbox.h).
+#include <algorithm>
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
@@ -66,7 +67,13 @@ bool make_layout(int n, int W, int H, uint64_t cap, Layout &L) {
     L.keys0 = take(8 * cap);
     L.keys1 = take(8 * cap);
     L.vals0 = take(4 * cap);
-    L.vals1 = take(4 * cap);
+    // the rows of the cell binning lie in vals1: its sort has read the cell ids
+    // there when the first row is written (frame_cells)
+    const int ncells = cell_geo(W, H, 8).ncells;
+    const size_t rows = cell_rows_max(cap, ncells), row_cell_bytes = align256(4 * rows);
+    L.vals1 = take(std::max<size_t>(4 * cap, row_cell_bytes + 128 * rows));
+    L.row_cell = L.vals1;
+    L.row_counts = L.vals1 + row_cell_bytes;
     size_t sb = 0;
     for (int d = 8; d <= kMaxDigitBits; ++d) {
         size_t b = sort_scratch_bytes(cap, key_bits, d);
@@ -80,12 +87,9 @@ bool make_layout(int n, int W, int H, uint64_t cap, Layout &L) {
     L.dvals1 = take(4 * N);
     L.dsort_scratch = take(depth_sort_scratch_bytes(N));
     L.ranges = take(8 * (size_t)tiles);
-    const int ncells = cell_geo(W, H, 8).ncells;
     L.cell_zero = take(4 * cell_zero_words(ncells));
     L.cell_start = take(4 * ((size_t)ncells + 2));
     L.row_start = take(4 * ((size_t)ncells + 1));
-    L.row_cell = take(4 * cell_rows_max(cap, ncells));
-    L.row_counts = take(128 * cell_rows_max(cap, ncells));
     L.tile_total = take(4 * (size_t)tiles);
     L.order_cnt = take(4 * 2 * (size_t)kOrderBuckets);
     L.order_list = take(4 * 2 * (size_t)kOrderBuckets * tiles);
@@ -140,7 +144,8 @@ TileSet frame_tileset(const qb_frame *f) {
 
 // The depth-first binning of a frame.  The cell entries' buffers are those
 // that the full-key path uses for its pairs: there are at most as many entries
-// as pairs, and vals0 receives the sorted values after the last entry is read.
+// as pairs, and vals0 receives the sorted values after the last entry is read
+// (vals1 the rows, after the sort).
 CellBin frame_cells(const qb_frame *f, const Layout &L) {
     CellBin b;
     std::memset(&b, 0, sizeof(b));

@@ -16,6 +16,7 @@
 // values, the ranges and the per-pixel state of every camera stay in the
 // workspace for qb_render_batch_bwd, whose render backward is one persistent
 // launch over all cameras' tiles as well.
+#include <algorithm>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -73,23 +74,40 @@ bool make_geo(int n_cams, const int32_t *W, const int32_t *H, Geo &g) {
 // joined before the next one), so one camera's small, latency-bound kernels
 // overlap another's.
 // Eight against four: 16 views of 1M 5198 -> 5092 us, five views of 200k (one
-// round instead of two) 2873 -> 2715.  A batch of smaller groups has as many
-// sets as its group has cameras.
+// round instead of two) 2873 -> 2715.  A batch has as many sets as its groups
+// have cameras, at most eight, and no more than its workspace bears (below).
 constexpr int kBatchStreams = 8;
-inline int batch_sets(int group) { return group < kBatchStreams ? group : kBatchStreams; }
 
+// What only the binning of a group needs (group scratch and sets) shares its
+// memory with what the render and the backward write later in the call: the
+// pixels' state, the screen-space sums and their list.
+//
+// A set holds two buffers of 8 bytes per pair of capacity (as many entries as
+// pairs, though a twelfth is usual: a Gaussian may have a cell per tile), the
+// sort's look-back words (a quarter byte at 1080p) and a few bytes per
+// Gaussian.  The entries' cell ids lie in the camera's slot, which receives its
+// values after the sort has read them; with more cells than a pass of 8 bits
+// sorts there are 4 bytes more for the ids between two passes; the rows lie in
+// the value buffer that the sorted entries are not in.
 struct BLayout {
-    size_t xy, shape, conic_o, rgbd, box, r3, meta, counts;  // [n_cams * n] records
+    size_t xy, shape, conic_o, rgbd, meta;            // [n_cams * n] records
     size_t cam_table;                                 // [n_cams] CamTile
     size_t slots;                                     // [n_cams][cap] sorted values per camera
     size_t ranges;                                    // [total tiles]
-    size_t tfinal, ncontrib, neval;                   // [total pixels]
-    size_t rects, cc, dk0, dk1, dv0, dv1;             // [group * n] group scratch
-    // one camera's binning scratch, batch_sets sets set_stride bytes apart:
-    size_t keysA, valsA, valsB;                       // [cap] cell entries
+    size_t rects, cc, dk0, dv0;                       // [group * n] group scratch
+    // records that the preprocess writes and nothing of a batch reads: [group * n],
+    // where the sets come to lie
+    size_t box, r3, counts;
+    // one camera's binning scratch, sets of them set_stride bytes apart:
+    int sets;
+    size_t dk1, dv1;                                  // [n] the depth order's other buffers
+    size_t keysB;                                     // [cap] cell ids (two passes)
+    size_t valsA, valsB;                              // [cap] cell entries
+    size_t row_counts;                                // of the rows, within the value buffer
     size_t offsets, coff, chunk_first, scan_part, dsort, sort, n_cells;
-    size_t cell_zero, cell_start, row_start, row_cell, row_counts, tile_total;
+    size_t cell_zero, cell_start, row_start, tile_total;
     size_t set_stride;
+    size_t tfinal, ncontrib;                          // [total pixels]
     size_t bwd_list, bwd_count;                       // a one-camera group's chain to the parameters
     size_t gscreen;                                   // [n_cams * n][9]
     size_t queue, state;
@@ -110,49 +128,57 @@ bool make_blayout(int n, int n_cams, int group, uint64_t cap, const Geo &g, BLay
     L.shape = take(8 * recs);
     L.conic_o = take(16 * recs);
     L.rgbd = take(16 * recs);
-    L.box = take(16 * recs);
-    L.r3 = take(4 * recs);
     L.meta = take(4 * recs);
-    L.counts = take(4 * recs);
     L.cam_table = take(sizeof(CamTile) * (size_t)n_cams);
     L.slots = take(4 * (size_t)n_cams * cap);
     L.ranges = take(8 * g.tile_base[n_cams]);
-    L.tfinal = take(4 * g.pix_base[n_cams]);
-    L.ncontrib = take(4 * g.pix_base[n_cams]);
-    L.neval = take(4 * g.pix_base[n_cams]);
+    const size_t shared0 = off;
     L.rects = take(32 * grecs);
     L.cc = take(8 * grecs);
     L.dk0 = take(4 * grecs);
-    L.dk1 = take(4 * grecs);
     L.dv0 = take(4 * grecs);
-    L.dv1 = take(4 * grecs);
     const size_t set0 = off;
-    L.keysA = take(4 * cap);
-    L.valsA = take(8 * cap);
-    L.valsB = take(8 * cap);
+    L.box = take(16 * grecs);
+    L.r3 = take(4 * grecs);
+    L.counts = take(4 * grecs);
+    const size_t unread = off;
+    off = set0;
+    const size_t rows = cell_rows_max(cap, g.max_cells);
+    L.row_counts = align256(4 * rows);
+    const size_t entries = std::max<size_t>(8 * cap, L.row_counts + 128 * rows);
+    L.dk1 = take(4 * (size_t)n);
+    L.dv1 = take(4 * (size_t)n);
+    L.keysB = take(g.max_cells + 1 > 1 << 8 ? 4 * cap : 0);
+    L.valsA = take(entries);
+    L.valsB = take(entries);
     L.offsets = take(4 * (size_t)n);
     L.coff = take(4 * (size_t)n);
     L.chunk_first = take(4 * chunk_table_size(cap));
     L.scan_part = take(8 * scan_partials_count(n));
-    size_t sb = 0;
-    for (int d = 8; d <= kMaxDigitBits; ++d) {
-        const size_t b2 = cell_sort_scratch_bytes(cap, g.max_cells, d);
-        sb = b2 > sb ? b2 : sb;
-    }
     L.dsort = take(depth_sort_scratch_bytes((uint64_t)n));
-    L.sort = take(sb);
+    L.sort = take(cell_sort_scratch_bytes(cap, g.max_cells));
     L.n_cells = take(8);
     L.cell_zero = take(4 * cell_zero_words(g.max_cells));
     L.cell_start = take(4 * ((size_t)g.max_cells + 2));
     L.row_start = take(4 * ((size_t)g.max_cells + 1));
-    L.row_cell = take(4 * cell_rows_max(cap, g.max_cells));
-    L.row_counts = take(128 * cell_rows_max(cap, g.max_cells));
     L.tile_total = take(4 * (size_t)g.max_tiles);
     L.set_stride = off - set0;
-    off += (size_t)(batch_sets(group) - 1) * L.set_stride;  // the other sets
+    // As many sets as keep the shared memory within what four sets of 16 bytes
+    // per pair (14 of few tiles) would take beside the rest instead of sharing
+    // with it.  16 views of 1M at 1080p and 35M pairs: all eight, 8.5 GB; of 1M at
+    // 1440p and 60M pairs, where the ids take two passes: five, 11.7 GB.
+    const size_t pix = g.pix_base[n_cams];
+    const size_t bound = 96 * recs + 80 * grecs + 12 * pix + 4 * (g.max_tiles > 2048 ? 16 : 14) * cap + 64 * (size_t)n;
+    const size_t fit = set0 - shared0 < bound ? (bound - (set0 - shared0)) / L.set_stride : 0;
+    L.sets = (int)std::max<size_t>(1, std::min<size_t>(fit, (size_t)std::min(group, kBatchStreams)));
+    const size_t binning_end = std::max(unread, set0 + (size_t)L.sets * L.set_stride);
+    off = shared0;
+    L.tfinal = take(4 * pix);
+    L.ncontrib = take(4 * pix);
     L.bwd_list = take(4 * (size_t)n);
     L.bwd_count = take(256);
     L.gscreen = take(72 * recs);
+    off = std::max(off, binning_end);
     L.queue = take(256);
     L.state = take(8 * (size_t)n_cams + 256);
     L.total = off;
@@ -441,18 +467,18 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
         a.shape = bat<float2>(b, L.shape) + v.rec0;
         a.conic_o = bat<float4>(b, L.conic_o) + v.rec0;
         a.rgbd = bat<float4>(b, L.rgbd) + v.rec0;
-        a.box = bat<float4>(b, L.box) + v.rec0;
-        a.r3 = bat<float>(b, L.r3) + v.rec0;
+        a.box = bat<float4>(b, L.box);
+        a.r3 = bat<float>(b, L.r3);
         a.meta = bat<int>(b, L.meta) + v.rec0;
-        a.counts = bat<uint32_t>(b, L.counts) + v.rec0;
+        a.counts = bat<uint32_t>(b, L.counts);
         a.rects = bat<uint4>(b, L.rects);
         a.cc = bat<uint2>(b, L.cc);
         a.depth_keys = bat<uint32_t>(b, L.dk0);  // the depth-order sort's keys and record indices
         a.depth_vals = bat<uint32_t>(b, L.dv0);
         QB_BCUDA(launch_preprocess(a, scene->sh_degree, s));
         // ---- each camera binned like a frame, into its own slot; camera c on
-        // side stream c % kBatchStreams with that stream's scratch set ----
-        const int nside = forked ? batch_sets(v.ncam) : 0;
+        // side stream c % nside with that stream's scratch set ----
+        const int nside = forked ? std::min(v.ncam, L.sets) : 0;
         if (nside > 0) {
             QB_BCUDA(cudaEventRecord(ss.fork, s));
             for (int i = 0; i < nside; ++i) QB_BCUDA(cudaStreamWaitEvent(ss.side[i], ss.fork, 0));
@@ -469,8 +495,8 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
             std::memset(&o, 0, sizeof(o));
             o.keys = bat<uint32_t>(b, L.dk0) + r0;
             o.vals = bat<uint32_t>(b, L.dv0) + r0;
-            o.keys_alt = bat<uint32_t>(b, L.dk1) + r0;
-            o.vals_alt = bat<uint32_t>(b, L.dv1) + r0;
+            o.keys_alt = bat<uint32_t>(b, L.dk1 + so);
+            o.vals_alt = bat<uint32_t>(b, L.dv1 + so);
             o.sort_scratch = bat<void>(b, L.dsort + so);
             o.cc = a.cc;
             o.offsets = bat<uint32_t>(b, L.offsets + so);
@@ -501,13 +527,13 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
             e.err = err;
             e.sort_scratch = bat<void>(b, L.sort + so);
             e.geo = cell_geo(b->widths[k], b->heights[k], rb);
-            // (the slot holds the cell ids of a second pass until the expansion writes the values)
             uint32_t *slot = bat<uint32_t>(b, L.slots) + (size_t)k * cap;
+            uint8_t *rows = bat<uint8_t>(b, (e.geo.passes.passes & 1 ? L.valsA : L.valsB) + so);
             e.arr = CellArrays{bat<uint32_t>(b, L.cell_zero + so), bat<uint32_t>(b, L.cell_start + so),
-                               bat<uint32_t>(b, L.row_start + so), bat<uint32_t>(b, L.row_cell + so),
-                               bat<uint32_t>(b, L.row_counts + so), bat<uint32_t>(b, L.tile_total + so),
-                               bat<uint32_t>(b, L.keysA + so), slot, bat<uint64_t>(b, L.valsA + so),
-                               bat<uint64_t>(b, L.valsB + so)};
+                               bat<uint32_t>(b, L.row_start + so), reinterpret_cast<uint32_t *>(rows),
+                               reinterpret_cast<uint32_t *>(rows + L.row_counts),
+                               bat<uint32_t>(b, L.tile_total + so), slot, bat<uint32_t>(b, L.keysB + so),
+                               bat<uint64_t>(b, L.valsA + so), bat<uint64_t>(b, L.valsB + so)};
             e.ranges = bat<uint2>(b, L.ranges) + geo.tile_base[k];
             e.vals = slot;
             QB_BCUDA(launch_cell_emit(e, cs));
@@ -532,7 +558,6 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
     r.img = d_images;
     r.tfinal = bat<float>(b, L.tfinal);
     r.ncontrib = bat<int>(b, L.ncontrib);
-    r.neval = bat<int>(b, L.neval);
     r.ts = batch_tileset(b, geo);
     r.cam_table = bat<CamTile>(b, L.cam_table);
     r.queue = bat<uint32_t>(b, L.queue);

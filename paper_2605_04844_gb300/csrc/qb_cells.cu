@@ -50,15 +50,19 @@ CellGeo cell_geo(int W, int H, int digit_bits) {
     g.ncells = g.cells_x * g.cells_y;
     g.cell_bits = 0;
     while ((1 << g.cell_bits) < g.ncells + 1) ++g.cell_bits;  // id ncells: entries without a tile
-    g.digit_bits = digit_bits;
-    g.passes = pass_geo(g.cell_bits, g.digit_bits);
+    g.passes = pass_geo(g.cell_bits, digit_bits);
+    g.digit_bits = std::max(g.passes.bits[0], 4);  // (a pass of fewer than 4 bits runs with 16 digits)
     return g;
 }
 
-size_t cell_sort_scratch_bytes(uint64_t pair_capacity, int ncells, int digit_bits) {
-    int bits = 1;
-    while ((1 << bits) < ncells + 1) ++bits;
-    return sort_scratch_bytes(pair_capacity, bits, digit_bits);
+size_t cell_sort_scratch_bytes(uint64_t pair_capacity, int max_cells) {
+    size_t words = 0;  // look-back words per tile of the passes together
+    for (int bits = 1; bits == 1 || (1 << (bits - 1)) < max_cells + 1; ++bits)
+        for (int d = 8; d <= kMaxDigitBits; ++d) {
+            const PassGeo g = pass_geo(bits, d);
+            words = std::max(words, (size_t)g.passes << std::max(g.bits[0], 4));
+        }
+    return align256(kSortHeader + sort_tiles(pair_capacity) * words * 4);
 }
 
 __device__ __forceinline__ uint64_t cell_value(uint32_t gid, uint32_t bits) { return ((uint64_t)bits << 32) | gid; }

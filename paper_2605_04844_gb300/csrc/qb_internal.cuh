@@ -50,7 +50,7 @@ struct Layout {
     size_t dkeys0, dkeys1, dvals0, dvals1, dsort_scratch;  // depth order of the Gaussians
     size_t ranges, tfinal, ncontrib, neval;
     size_t cell_zero;    // cell counts and finished-block counters (CellLayout)
-    size_t cell_start, row_start, row_cell, row_counts, tile_total;  // CellArrays
+    size_t cell_start, row_start, row_cell, row_counts, tile_total;  // CellArrays (the rows inside vals1)
     size_t order_cnt;   // [2][kOrderBuckets]: tile orders by the backward's work (TileOrder)
     size_t order_list;  // [2][kOrderBuckets][tiles]
     size_t bwd_list, bwd_count;  // Gaussians with a screen-space gradient; their number (just before gscreen)

@@ -93,7 +93,7 @@ struct EmitArgs {
 // their ids.
 struct CellGeo {
     int tiles_x, tiles_y, cells_x, cells_y, ncells, ntiles;
-    int cell_bits, digit_bits;  // digit_bits: of a pass at most (sort scratch layout)
+    int cell_bits, digit_bits;  // digit_bits: of the widest pass (sort scratch layout)
     PassGeo passes;
 };
 
@@ -281,7 +281,8 @@ cudaError_t launch_ranges(const uint64_t *keys, uint64_t n_max, const uint64_t *
 // (cell, Gaussian, tile bits) entries; then their sort by cell and the
 // expansion to the sorted values and ranges.
 CellGeo cell_geo(int W, int H, int digit_bits);
-size_t cell_sort_scratch_bytes(uint64_t pair_capacity, int ncells, int digit_bits);
+// Scratch of the cell sort for images of at most max_cells cells and any digit width.
+size_t cell_sort_scratch_bytes(uint64_t pair_capacity, int max_cells);
 cudaError_t launch_cell_emit(const CellBin &b, cudaStream_t s);
 cudaError_t launch_cell_sort(const CellBin &b, cudaStream_t s);
 // Sorts b's entries by cell (bucket offsets already in the scratch's table,
