@@ -158,20 +158,19 @@ __device__ __forceinline__ float2 exp2_of(float2 x) {
 // at most 3 x 2^-24 (|dx| + |r dy|) here and in the kernels' exponent together.
 // It counts by sqrt(a) and sqrt(a) |r| <= sqrt(c), each at most 1 / sqrt(0.3)
 // (Sigma's eigenvalues are at least the dilation): the Mahalanobis distance is
-// off by less than 3.3e-7 (|dx| + |dy|).  The margin covers 0.0099 (where the
-// radius is 1; more elsewhere), that is 30000 pixels from mu^2D; entries farther
-// than half of that, kEllipseFar, always meet the rectangle.  (Images are up to
-// 32768 pixels and mu^2D may lie any distance outside; at 10^7 pixels 2 % of the
-// rectangles that a needle reaches would be missed.)  The edge minimisers'
-// rounding, below 0.01 pixels there, enters q squared.
+// off by less than d = 3.3e-7 D, D = |dx| + |dy|.  (R + d)^2 <= 1.01 R^2 +
+// 101 d^2 for every radius R, so 1.2e-11 D^2 more in the squared radius covers it:
+// 0.01 at 30000 pixels from mu^2D, everything from 10^6 on.  (Images are up to
+// 32768 pixels and mu^2D may lie any distance outside; with the margin alone, 2 %
+// of the rectangles that a needle reaches were missed at 10^7 pixels.)  The edge
+// minimisers' rounding enters q squared, relative to D, and is far smaller.
 // Before elongated conics were tested they met every rectangle: of the 19.4M
 // entries staged for 3M Gaussians at 1440p seen from inside, where thin ones
 // abound, 16.9M were walked and 2.8M reached a running pixel.
-constexpr float kEllipseFar = 16384.f;
 __device__ __forceinline__ bool ellipse_meets_rect(float mx, float my, float a, float b, float c, float t,
                                                    float2 shape, float x0, float y0, float x1, float y1) {
     if (!(a > 0.f && c > 0.f)) return true;
-    const float r2 = fmaxf(-2.f * t, 0.f) * 1.01f + 1e-2f;
+    float r2 = fmaxf(-2.f * t, 0.f) * 1.01f + 1e-2f;
     const float ul = mx - x1, uh = mx - x0, vl = my - y1, vh = my - y0;
     const bool elongated = shape.y != 0.f;
     const float ir = elongated ? shape.x : __fdividef(b, a);
@@ -180,7 +179,8 @@ __device__ __forceinline__ bool ellipse_meets_rect(float mx, float my, float a, 
     const float v2 = fminf(fmaxf(0.f, vl), vh), u2 = fminf(fmaxf(-ir * v2, ul), uh);
     float q1, q2;
     if (elongated) {
-        if (fabsf(u1) + fabsf(v2) > kEllipseFar) return true;
+        const float D = fabsf(u1) + fabsf(v2);
+        r2 = fmaf(D * 1.2e-11f, D, r2);
         const float e = -2.f * shape.y, w1 = fmaf(ir, v1, u1), w2 = fmaf(ir, v2, u2);
         q1 = fmaf(a * w1, w1, e * v1 * v1);
         q2 = fmaf(a * w2, w2, e * v2 * v2);
