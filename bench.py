@@ -157,8 +157,7 @@ def run_ours(args, rank, world, local_rank):
     scene_s, cam_s = R.scene_struct(sd), R.camera_struct(cam)
     bg = (0.0, 0.0, 0.0)
 
-    # autotuned sort digit width and render batch depth unless the digit
-    # width is given
+    # autotuned sort digit width unless it is given
     digit_bits = args.digit_bits
     render_batch = 128
     tune = None

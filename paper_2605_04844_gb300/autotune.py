@@ -2,11 +2,11 @@
 
 Times the candidates on the caller's own scene and camera and keeps the
 fastest.  For a frame: the cell sort's radix digit width (8..11 bits, which
-sets the number of passes), then render_batch (a field the library accepts
-without effect: a warp stages 32 Gaussians per step).  For a batch of cameras: the
-digit width, render_batch, tiles a persistent render block takes per fetch
-from the global queue and persistent blocks per SM, by coordinate descent.
-Results are cached as JSON under
+sets the number of passes).  For a batch of cameras: the digit width, tiles a
+persistent render block takes per fetch from the global queue and persistent
+blocks per SM, by coordinate descent.  render_batch, which the library accepts
+without effect (a warp stages 32 Gaussians per step), is not searched: a result
+carries its default.  Results are cached as JSON under
 $QUADBOX_CACHE_DIR (default ~/.cache/quadbox/tune.json), keyed by GPU name,
 Gaussian count, image size and binning mode.
 """
@@ -20,7 +20,7 @@ import torch
 from . import rasterizer as R
 
 DIGIT_CANDIDATES = (8, 9, 10, 11)
-RENDER_BATCH_CANDIDATES = (64, 128, 256)
+RENDER_BATCH = 128
 
 
 def _cache_path():
@@ -57,8 +57,8 @@ def _time(fn, reps):
 
 
 def tune_frame(scene, cam, mode="quadbox", reps=5, use_cache=True):
-    """Pick the sort digit width (timing preprocess, emit and sort), then the
-    render's batch depth (timing the render), for this scene and camera."""
+    """Pick the sort digit width (timing preprocess, emit and sort) for this
+    scene and camera, and time the render."""
     n = int(scene["means"].shape[0])
     W, H = int(cam["width"]), int(cam["height"])
     key = f"{torch.cuda.get_device_name()}|frame2|n={n}|{W}x{H}|{mode}"
@@ -83,16 +83,12 @@ def tune_frame(scene, cam, mode="quadbox", reps=5, use_cache=True):
     fr.bin_emit(sync=False)
     fr.sort()
     img = torch.empty((3, H, W), dtype=torch.float32, device=fr.ws.device)
-    rtimes = {}
-    for rb in RENDER_BATCH_CANDIDATES:
-        fr.set_tuning(render_batch=rb)
-        fr.render(None, img)
-        rtimes[rb] = _time(lambda: fr.render(None, img), reps)
+    fr.render(None, img)
+    render_ms = _time(lambda: fr.render(None, img), reps)
     fr.check()
-    best_rb = min(rtimes, key=rtimes.get)
-    res = {"digit_bits": int(best), "render_batch": int(best_rb),
+    res = {"digit_bits": int(best), "render_batch": RENDER_BATCH,
            "ms": {str(k): round(v, 4) for k, v in timings.items()},
-           "render_ms": {str(k): round(v, 4) for k, v in rtimes.items()}}
+           "render_ms": {str(RENDER_BATCH): round(render_ms, 4)}}
     if use_cache:
         db[key] = res
         _save(db)
@@ -101,7 +97,6 @@ def tune_frame(scene, cam, mode="quadbox", reps=5, use_cache=True):
 
 BATCH_SPACE = {
     "sort_digit_bits": (8, 10, 11),
-    "render_batch": (64, 128, 256),
     "tiles_per_fetch": (1, 2, 4),
     "blocks_per_sm": (0, 2, 4),
 }
@@ -109,15 +104,14 @@ BATCH_SPACE = {
 
 def tune_batch(batch, scene, cams, mode="quadbox", reps=2, use_cache=True):
     """Coordinate descent over the batched path's launch parameters (sort
-    digit width, staging batch depth, tiles per queue fetch, persistent
-    blocks per SM), timing qb_render_batch on the caller's scene and cameras."""
+    digit width, tiles per queue fetch, persistent blocks per SM), timing qb_render_batch on the caller's scene and cameras."""
     key = (f"{torch.cuda.get_device_name()}|batch|n={batch.n}|cams={batch.n_cams}|group={batch.group}|"
            f"{'-'.join(f'{w}x{h}' for w, h in zip(batch.widths, batch.heights))[:200]}|{mode}")
     db = _load() if use_cache else {}
     if key in db:
         return dict(db[key], cached=True)
     scene_s, cams_arr = R.scene_struct(scene), R.camera_array(cams)
-    best = {"sort_digit_bits": 8, "render_batch": 128, "tiles_per_fetch": 2, "blocks_per_sm": 0}
+    best = {"sort_digit_bits": 8, "render_batch": RENDER_BATCH, "tiles_per_fetch": 2, "blocks_per_sm": 0}
     timings = {}
     for name, values in BATCH_SPACE.items():
         res = {}
