@@ -388,8 +388,10 @@ size_t qb_batch_workspace_bytes(int32_t n, int32_t n_cams, const int32_t *widths
 /* Binds a caller-owned, 256-byte aligned device workspace to *batch, writes
  * the render's per-camera table into it (synchronises the stream once) and
  * creates the batch's side streams: inside qb_render_batch the cameras of a
- * group are binned up to eight at a time on side streams forked from the caller's
- * stream and joined back to it (captured into a CUDA graph with the rest).
+ * group are binned up to eight at a time (fewer where their scratch would make
+ * the workspace large) on side streams forked from the caller's stream and joined
+ * back to it (captured into a CUDA graph with the rest).  A forward overwrites
+ * what the backward of the one before it needs.
  * Errors: INVALID_ARG for sizes outside the limits above. */
 qb_status qb_batch_init(qb_batch *batch, int32_t n, int32_t n_cams, const int32_t *widths, const int32_t *heights,
                         int32_t group, uint64_t pair_capacity, void *d_workspace, size_t workspace_bytes,

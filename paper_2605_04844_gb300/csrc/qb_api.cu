@@ -520,7 +520,7 @@ qb_status qb_bin_emit(qb_frame *frame, uint64_t *n_pairs_out, qb_stream_t stream
         frame->depth_in_alt = in_alt;
     } else {
         QB_CUDA(launch_scan(at<uint32_t>(frame, L.counts), frame->n, at<uint32_t>(frame, L.offsets),
-                            at<uint32_t>(frame, L.coff), partials, d_np, host_word, err,
+                            partials, d_np, host_word, err,
                             chunk_first, chunk_cap, s));
     }
     frame->n_pairs = UINT64_MAX;

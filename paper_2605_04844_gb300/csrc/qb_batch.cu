@@ -46,7 +46,9 @@ struct Geo {  // per-camera geometry of a batch
     int max_tiles, max_cells;
 };
 
-constexpr int kMaxCameraTiles = 24576;  // accepted tiles of one camera
+// Accepted tiles of one camera (quadbox.h): a limit of the interface, which the
+// binning through cells does not need.
+constexpr int kMaxCameraTiles = 24576;
 
 bool make_geo(int n_cams, const int32_t *W, const int32_t *H, Geo &g) {
     if (n_cams < 1 || n_cams > QB_MAX_CAMERAS || !W || !H) return false;
@@ -170,7 +172,7 @@ bool make_blayout(int n, int n_cams, int group, uint64_t cap, const Geo &g, BLay
     const size_t pix = g.pix_base[n_cams];
     const size_t bound = 96 * recs + 80 * grecs + 12 * pix + 4 * (g.max_tiles > 2048 ? 16 : 14) * cap + 64 * (size_t)n;
     const size_t fit = set0 - shared0 < bound ? (bound - (set0 - shared0)) / L.set_stride : 0;
-    L.sets = (int)std::max<size_t>(1, std::min<size_t>(fit, (size_t)std::min(group, kBatchStreams)));
+    L.sets = (int)std::max<size_t>(1, std::min<size_t>(fit, (size_t)std::min({group, n_cams, kBatchStreams})));
     const size_t binning_end = std::max(unread, set0 + (size_t)L.sets * L.set_stride);
     off = shared0;
     L.tfinal = take(4 * pix);
@@ -274,35 +276,21 @@ CamTile cam_tile(const qb_batch *b, const Geo &g, int k) {
     return t;
 }
 
-// A group of cameras: camera set for the preprocess, and a tile set whose
-// cameras all start at tile 0 (each camera is binned on its own tiles).
+// A group of cameras.
 struct GroupView {
     int k0, k1, ncam;
     uint64_t rec0;  // first record
     CamSet cs;
-    TileSet ts;
 };
 
-void group_view(const qb_batch *b, const Geo &g, const qb_camera *cams, int gi, GroupView &v) {
+void group_view(const qb_batch *b, const qb_camera *cams, int gi, GroupView &v) {
     std::memset(&v, 0, sizeof(v));
     v.k0 = gi * b->group;
     v.k1 = v.k0 + b->group < b->n_cams ? v.k0 + b->group : b->n_cams;
     v.ncam = v.k1 - v.k0;
     v.rec0 = (uint64_t)v.k0 * b->n;
     v.cs.n_cams = v.ncam;
-    v.ts.n_cams = v.ncam;
-    for (int c = 0; c < v.ncam; ++c) {
-        const int k = v.k0 + c;
-        if (cams) v.cs.cam[c] = cam_dev(cams[k]);
-        v.ts.cam[c].W = b->widths[k];
-        v.ts.cam[c].H = b->heights[k];
-        v.ts.cam[c].tiles_x = g.tx[k];
-        v.ts.cam[c].tiles_y = g.ty[k];
-        v.ts.cam[c].tile_base = 0;
-        v.ts.cam[c].pix_base = g.pix_base[k];
-        v.ts.total_tiles = v.ts.total_tiles > (uint32_t)(g.tx[k] * g.ty[k]) ? v.ts.total_tiles
-                                                                           : (uint32_t)(g.tx[k] * g.ty[k]);
-    }
+    for (int c = 0; c < v.ncam; ++c) v.cs.cam[c] = cam_dev(cams[v.k0 + c]);
 }
 
 // The whole batch as one tile set for the persistent render and backward
@@ -447,7 +435,7 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
     const bool forked = side_find(b->workspace, ss);
     for (int gi = 0; gi < b->n_groups; ++gi) {
         GroupView v;
-        group_view(b, geo, cams, gi, v);
+        group_view(b, cams, gi, v);
         // ---- preprocess over the group's (camera, Gaussian) records ----
         PreArgs a;
         std::memset(&a, 0, sizeof(a));
@@ -612,7 +600,7 @@ qb_status qb_render_batch_bwd(qb_batch *b, const qb_scene *scene, const qb_camer
     // ---- the chain to the scene parameters, one launch per group ----
     for (int gi = 0; gi < b->n_groups; ++gi) {
         GroupView v;
-        group_view(b, geo, cams, gi, v);
+        group_view(b, cams, gi, v);
         PreBwdArgs p;
         std::memset(&p, 0, sizeof(p));
         p.n = n;

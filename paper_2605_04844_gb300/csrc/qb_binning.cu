@@ -23,12 +23,12 @@ constexpr int kScanChunk = kScanBlock * kScanItems;
 //
 // DUAL (depth-first): entry j is the pair cc[perm[j]] = (tiles, cells) of the
 // j-th Gaussian in depth order; offsets gets the tiles' exclusive prefix,
-// coff the cells'.  Otherwise entry j is counts[j], offsets its prefix and
-// coff the count itself (the emit reads it in order).  chunk_first[c] becomes
-// the position whose outputs (cell entries or pairs) hold output c
-// kEmitStride, so the emit's warps find their first Gaussian with one load
-// instead of a search.  The last block writes P, and for DUAL the number of cell entries,
-// 0 when P exceeds the capacity (then nothing downstream writes).
+// coff the cells'.  Otherwise entry j is counts[j] and offsets its prefix (coff
+// is not used).  chunk_first[c] becomes the position whose outputs (cell entries
+// or pairs) hold output c kEmitStride, so the emit's warps find their first
+// Gaussian with one load instead of a search.  The last block writes P, and for
+// DUAL the number of cell entries, 0 when P exceeds the capacity (then nothing
+// downstream writes).
 //
 // Status of a block: two 64-bit words stored and loaded as one 128-bit word,
 // flag (bit 63: sum of the block, bit 62: total through the block) and a
@@ -208,20 +208,20 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
         for (int k = 0; k < kScanItems; ++k) {
             o[k] = (uint32_t)run;  // P <= 2^30 is checked before use
             run += c[k];
-            p[k] = DUAL ? r : c[k];
+            p[k] = r;
             r += d[k];
         }
 #pragma unroll
         for (int q = 0; q < kScanItems / 4; ++q) {
             reinterpret_cast<uint4 *>(A.offsets + base)[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-            reinterpret_cast<uint4 *>(A.coff + base)[q] = make_uint4(p[4 * q], p[4 * q + 1], p[4 * q + 2], p[4 * q + 3]);
+            if (DUAL) reinterpret_cast<uint4 *>(A.coff + base)[q] = make_uint4(p[4 * q], p[4 * q + 1], p[4 * q + 2], p[4 * q + 3]);
         }
     } else {
 #pragma unroll
         for (int k = 0; k < kScanItems; ++k) {
             if (base + k < (size_t)n) {
                 A.offsets[base + k] = (uint32_t)run;
-                A.coff[base + k] = DUAL ? r : c[k];
+                if (DUAL) A.coff[base + k] = r;
             }
             run += c[k];
             r += d[k];
@@ -254,7 +254,7 @@ static cudaError_t run_scan(ScanArgs A, uint64_t *partials, bool dual, cudaStrea
     return cudaGetLastError();
 }
 
-cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32_t *counts_e, uint64_t *partials,
+cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint64_t *partials,
                         uint64_t *n_pairs, uint64_t *n_pairs_host, uint32_t *err, uint32_t *chunk_first,
                         uint32_t chunk_cap, cudaStream_t s) {
     ScanArgs A{};
@@ -262,7 +262,6 @@ cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32
     A.counts = counts;
     A.n = n;
     A.offsets = offsets;
-    A.coff = counts_e;
     A.chunk_first = chunk_first;
     A.chunk_cap = chunk_cap;
     A.n_pairs = n_pairs;

@@ -42,7 +42,7 @@ struct Layout {
     size_t xy, shape, conic_o, rgbd, box, r3, meta, counts, offsets;
     size_t rects;  // [n] packed sub-box tile rectangles (pack_rects)
     size_t cc;     // [n] (tile count, cell count)
-    size_t coff;   // [n] counts (FULL_KEY) or cell offsets (DEPTH_FIRST) in emission order
+    size_t coff;   // [n] cell offsets in emission order (DEPTH_FIRST)
     size_t chunk_first;  // the emit's chunk table
     size_t scan_part;
     size_t keys0, keys1, vals0, vals1;

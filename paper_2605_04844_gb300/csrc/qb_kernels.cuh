@@ -65,13 +65,6 @@ struct TileSet {
     CamTile cam[kMaxGroupCams];
 };
 
-__device__ __forceinline__ int camera_of(const TileSet &ts, uint32_t gtile) {
-    int c = 0;
-#pragma unroll 1
-    for (int k = 1; k < ts.n_cams; ++k) c = gtile >= ts.cam[k].tile_base ? k : c;
-    return c;
-}
-
 // The full-key emit (a single frame, index order).
 struct EmitArgs {
     int n;
@@ -240,7 +233,7 @@ cudaError_t launch_preprocess(const PreArgs &a, int deg, cudaStream_t s);
 // order (full-key path).  launch_scan_cells: (tiles, cells) in the order perm;
 // *n_cells becomes 0 when the pairs exceed the capacity.  n_pairs_host, when
 // not null, is a device address of mapped host memory that also gets P (n > 0).
-cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint32_t *counts_e, uint64_t *partials,
+cudaError_t launch_scan(const uint32_t *counts, int n, uint32_t *offsets, uint64_t *partials,
                         uint64_t *n_pairs, uint64_t *n_pairs_host, uint32_t *err, uint32_t *chunk_first,
                         uint32_t chunk_cap, cudaStream_t s);
 cudaError_t launch_scan_cells(const uint2 *cc, const uint32_t *perm, int n, uint32_t *offsets, uint32_t *coff,

@@ -139,6 +139,11 @@ class Frame:
         return self.ws[off:off + nbytes].view(dtype).view(*shape)
 
     def arrays(self, n_pairs=None):
+        """Views of the frame's device arrays (qb_frame_arrays).  In depth_first
+        mode vals, keys and tile_keys hold the emitted cell entries' scratch
+        between bin_emit and sort; after sort vals holds the sorted pairs and
+        tile_keys is made from the ranges.  The pairs as emitted are there in
+        full_key mode only."""
         a = N.qb_frame_arrays_get(self.frame)
         n, H, W = self.n, self.height, self.width
         P = n_pairs if n_pairs is not None else (self.n_pairs or 0)
