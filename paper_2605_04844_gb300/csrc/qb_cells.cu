@@ -488,6 +488,7 @@ __global__ void __launch_bounds__(kPrefixThreads, 3) cell_prefix_kernel(CellGeo 
     // them whatever the buffer held: nothing is expanded.  (Nor if the tiles'
     // totals did not add up to the pairs there are.)
     if (*sort_failed || (*n_cells > 0 && before != *n_pairs)) {
+        __syncthreads();  // the ranges above were written by other threads
         for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) ranges[t] = make_uint2(0u, 0u);
         if (threadIdx.x == 0) a.row_start[g.ncells] = 0u;
     }
