@@ -86,7 +86,8 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
     __syncthreads();
     const uint32_t b = s_block;
     const int n = A.n;
-    // (an order with gaps is not gathered through: every count reads as zero)
+    // (an order with gaps is not gathered through: every count reads as zero; the
+    // order itself is read meanwhile, so that its loads do not wait for this one)
     const size_t n_in = DUAL && A.order_failed && *A.order_failed ? 0 : (size_t)n;
     const int nb = (n + kScanChunk - 1) / kScanChunk;
     const size_t base = (size_t)b * kScanChunk + (size_t)tid * kScanItems;
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
         uint32_t g[kScanItems];
         // 16-byte loads where perm allows them (a batch camera's order starts at a
         // multiple of n records, which need not be one of four)
-        if (base + kScanItems <= n_in && (reinterpret_cast<uintptr_t>(A.perm) & 15) == 0) {
+        if (whole && (reinterpret_cast<uintptr_t>(A.perm) & 15) == 0) {
 #pragma unroll
             for (int q = 0; q < kScanItems / 4; ++q) {
                 const uint4 v = reinterpret_cast<const uint4 *>(A.perm + base)[q];
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
             }
         } else {
 #pragma unroll
-            for (int k = 0; k < kScanItems; ++k) g[k] = base + k < n_in ? A.perm[base + k] : 0u;
+            for (int k = 0; k < kScanItems; ++k) g[k] = base + k < (size_t)n ? A.perm[base + k] : 0u;
         }
 #pragma unroll
         for (int k = 0; k < kScanItems; ++k) {

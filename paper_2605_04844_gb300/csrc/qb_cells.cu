@@ -294,8 +294,9 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     const bool in_smem = b.geo.ncells < kCellHistMax;
     // after a scan that failed its offsets and counts do not belong together:
     // no entries
+    const uint64_t cells = *b.n_cells;
     const bool failed = b.scan_failed && *b.scan_failed;
-    const uint64_t E = failed ? 0ull : *b.n_cells;
+    const uint64_t E = failed ? 0ull : cells;
     if (blockIdx.x == 0 && tid == 0 && *b.n_pairs > b.capacity) atomicOr(b.err, kErrCapacity);
     if (in_smem)
         for (int c = tid; c <= b.geo.ncells; c += blockDim.x) s_hist[c] = 0u;
@@ -430,6 +431,7 @@ __global__ void __launch_bounds__(kPrefixThreads, 3) cell_prefix_kernel(CellGeo 
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int cell = blockIdx.x;
+    const bool failed = *sort_failed != 0u;
     const uint32_t r0 = a.row_start[cell], nr = a.row_start[cell + 1] - r0;
     const uint32_t per = (nr + nw - 1) / nw;
     const uint32_t w0 = min(nr, wid * per), w1 = min(nr, w0 + per);
@@ -487,7 +489,7 @@ __global__ void __launch_bounds__(kPrefixThreads, 3) cell_prefix_kernel(CellGeo 
     // After a look-back time-out the sorted entries are undefined, and some of
     // them whatever the buffer held: nothing is expanded.  (Nor if the tiles'
     // totals did not add up to the pairs there are.)
-    if (*sort_failed || (*n_cells > 0 && before != *n_pairs)) {
+    if (failed || (*n_cells > 0 && before != *n_pairs)) {
         __syncthreads();  // the ranges above were written by other threads
         for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) ranges[t] = make_uint2(0u, 0u);
         if (threadIdx.x == 0) a.row_start[g.ncells] = 0u;
