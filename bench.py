@@ -482,9 +482,10 @@ def kernel_work(P, n, evals, packed=False):
 # work, from the ncu --set full captures of the 600k-Gaussian 1080p frame
 # (20,633,099 pairs, 398,727,914 evaluations) summarised under profiles/,
 # scaled to a launch of this frame by its units; valid for the kernels as
-# captured (kernel -> (unit, bytes per unit)).  tile_sort_pass and
-# tile_sort_pass_values are the pair passes that a frame took before it was
-# binned through cells; a list without them leaves their entries unused.
+# captured (kernel -> (unit, bytes per unit)).  No frame launches tile_sort_pass
+# and tile_sort_pass_values (a radix sort of all pairs by tile id, for lists of an
+# earlier library); the cell binning's kernels have no row, except the expansion,
+# since the number of entries is not read back.
 TRAFFIC_PER_UNIT = {
     "render_kernel": ("eval", (13.045248e6 + 0.425984e6) / 398727914),
     "tile_sort_pass": ("pair", (165.526528e6 + 34.277120e6) / 20633099),
@@ -830,8 +831,9 @@ KERNEL_TIMING_SPIN_CYCLES = 8_000_000
 # Algorithmic bytes of the preprocess per Gaussian: read 44 B of parameters and
 # 192 B of SH coefficients (degree 3), write mu^2D 8, conic+o 16, colour+depth
 # 16, box 16, 3-sigma radius 4, meta 4, count 4, depth-sort key and index 8
-# (76 B).  The QPass run records (16 to 64 B per visible Gaussian) are left
-# out, which understates the kernel's fraction slightly.
+# (76 B).  The tile rectangles (32 B per Gaussian with tiles), the shape pair and
+# the tile and cell counts (8 B each) are left out, which understates the
+# kernel's fraction slightly.
 PREPROCESS_BYTES = 236 + 76
 
 # FP32 arithmetic of Eq. 2's per-pixel loop (an FMA counts 2, comparisons
@@ -840,6 +842,9 @@ PREPROCESS_BYTES = 236 + 76
 # (3 mul + 2 FMA) = 9.  An entry whose power test passes also takes alpha =
 # o exp(power) (exp 1 + its argument scaling 1 + mul 1), T' = T (1 - alpha)
 # (sub 1 + mul 1), the weight alpha T (mul 1) and three colour FMAs (6) = 12.
+# The rate is one of this arithmetic, not of the ALU's: the evaluations are the
+# list positions up to a pixel's stop, those among them that the render's ellipse
+# test drops for a whole half tile ahead of any per-pixel operation.
 RENDER_FLOPS_POWER_TEST = 9
 RENDER_FLOPS_PASSED = 12
 
