@@ -156,7 +156,6 @@ CellBin frame_cells(const qb_frame *f, const Layout &L) {
     b.rects = at<uint4>(f, L.rects);
     b.n_pairs = at<uint64_t>(f, L.state);
     b.n_cells = at<uint64_t>(f, L.state + 16);
-    b.scan_failed = depth_order_failed(at<uint64_t>(f, L.scan_part), f->n);
     b.n_cells_max = f->n_pairs != UINT64_MAX ? f->n_pairs : f->pair_capacity;
     b.capacity = f->pair_capacity;
     b.naive = (f->bin_mode & 0xff) == QB_BIN_QUADBOX_NAIVE;

@@ -508,7 +508,6 @@ qb_status qb_render_batch(qb_batch *b, const qb_scene *scene, const qb_camera *c
             e.rects = a.rects;
             e.n_pairs = npairs + k;
             e.n_cells = n_cells;
-            e.scan_failed = depth_order_failed(o.partials, n);
             e.n_cells_max = cap;
             e.capacity = cap;
             e.naive = base_mode == QB_BIN_QUADBOX_NAIVE;

@@ -40,7 +40,8 @@ constexpr int kScanChunk = kScanBlock * kScanItems;
 // 32 (a chain of two or three loads where there were up to a dozen).
 //
 // A look-back that runs out leaves offsets that do not belong together: the
-// failure word beside the block counter then keeps the emits from using them.
+// number of cell entries is then 0, and the full-key emit is kept from using
+// them by the failure word beside the block counter.
 constexpr uint64_t kScanAgg = 1ull << 63, kScanIncl = 1ull << 62, kScanCount = kScanIncl - 1;
 
 struct ScanWord {
@@ -76,6 +77,24 @@ struct ScanArgs {
     uint64_t capacity;
     uint32_t *err;
 };
+
+__device__ __forceinline__ void set_cells(const ScanArgs &A, uint64_t v) {
+    atomicExch(reinterpret_cast<unsigned long long *>(A.n_cells), (unsigned long long)v);
+}
+
+// A block's look-back ran out.  DUAL: the number of cell entries ends as 0,
+// whichever comes later, this or the last block's writing it: each writes its
+// word, fences, and then the last block reads the failure word and this one
+// writes the number, so that one of the two sees the other.
+template <bool DUAL>
+__device__ __forceinline__ void scan_gave_up(const ScanArgs &A) {
+    atomicOr(A.err, kErrTimeout);
+    atomicExch(A.counter + 1, 1u);
+    if (DUAL) {
+        __threadfence();
+        set_cells(A, 0ull);
+    }
+}
 
 template <bool DUAL>
 __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A) {
@@ -162,10 +181,7 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
         t -= used;
         if (used == 0) {  // the nearest earlier block has not published yet
             if (++spins > kSpinLimit) {
-                if (tid == 0) {
-                    atomicOr(A.err, kErrTimeout);
-                    A.counter[1] = 1u;
-                }
+                if (tid == 0) scan_gave_up<DUAL>(A);
                 break;
             }
             __nanosleep(64);
@@ -173,10 +189,7 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
     }
     if (b == 1 && (ld_relaxed(A.err + 1) & kTestScan)) {  // test-only (stall_test)
         acc = accd = 0;
-        if (tid == 0) {
-            atomicOr(A.err, kErrTimeout);
-            A.counter[1] = 1u;
-        }
+        if (tid == 0) scan_gave_up<DUAL>(A);
     }
     if (tid == 0) {
         if (b > 0) st_status(A.status + b, ScanWord{kScanIncl | ((acc + ctot) & kScanCount), accd + dtot});
@@ -185,7 +198,11 @@ __global__ void __launch_bounds__(kScanBlock, 4) scan_onepass_kernel(ScanArgs A)
             *A.n_pairs = P;
             if (A.n_pairs_host) *A.n_pairs_host = P;
             // (E <= P: cell_entries)
-            if (DUAL) *A.n_cells = P <= A.capacity && E <= A.capacity ? E : 0ull;
+            if (DUAL) {
+                set_cells(A, P <= A.capacity && E <= A.capacity ? E : 0ull);
+                __threadfence();  // (scan_gave_up)
+                if (ld_relaxed(A.counter + 1)) set_cells(A, 0ull);
+            }
         }
     }
     uint64_t run = acc + cincl - csum;

@@ -185,7 +185,7 @@ __device__ __forceinline__ void cell_emit_range(const CellBin &b, uint64_t E, ui
 __device__ __forceinline__ void cell_emit_naive(const CellBin &b, int64_t j, uint32_t *hist) {
     const uint32_t gid = b.perm[j];
     const uint32_t off = b.coff[j];
-    const uint32_t end = j + 1 < b.n ? b.coff[j + 1] : (uint32_t)*b.n_cells;  // (only where no scan failed)
+    const uint32_t end = j + 1 < b.n ? b.coff[j + 1] : (uint32_t)*b.n_cells;
     if (end == off) return;
     const uint4 w0 = b.rects[2 * (size_t)gid], w1 = b.rects[2 * (size_t)gid + 1];
     const Rect r[4] = {cell_rect(unpack_rect(w0.x, w0.y)), cell_rect(unpack_rect(w0.z, w0.w)),
@@ -292,11 +292,7 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     __shared__ bool s_last;
     const int tid = threadIdx.x, wid = tid >> 5;
     const bool in_smem = b.geo.ncells < kCellHistMax;
-    // after a scan that failed its offsets and counts do not belong together:
-    // no entries
-    const uint64_t cells = *b.n_cells;
-    const bool failed = b.scan_failed && *b.scan_failed;
-    const uint64_t E = failed ? 0ull : cells;
+    const uint64_t E = *b.n_cells;  // (0 after a scan that failed)
     if (blockIdx.x == 0 && tid == 0 && *b.n_pairs > b.capacity) atomicOr(b.err, kErrCapacity);
     if (in_smem)
         for (int c = tid; c <= b.geo.ncells; c += blockDim.x) s_hist[c] = 0u;
@@ -334,7 +330,6 @@ __global__ void __launch_bounds__(kCellWarps * 32) cell_emit_kernel(CellBin b) {
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    if (failed && tid == 0) *b.n_cells = 0ull;  // (every block has read it)
     cell_prepare(b, reinterpret_cast<uint32_t *>(smem));  // the table and histogram are no longer needed
 }
 

@@ -113,9 +113,7 @@ struct CellBin {
     const uint32_t *coff;   // first entry of each emission position
     const uint32_t *chunk_first;
     const uint4 *rects;     // by record
-    const uint64_t *n_pairs;
-    uint64_t *n_cells;      // set to 0 when the scan failed
-    const uint32_t *scan_failed;  // the scan's failure word, or null (depth_order_failed)
+    const uint64_t *n_pairs, *n_cells;  // (n_cells 0: too many pairs, or the scan failed)
     uint64_t n_cells_max;   // bound on *n_cells (the capacity, or P where the host knows it)
     uint64_t capacity;
     bool naive;             // emit by nested loops (QB_BIN_QUADBOX_NAIVE)
@@ -258,8 +256,6 @@ struct OrderArgs {
 };
 // *in_alt: the order lies in vals_alt.
 cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *in_alt);
-// The failure word of its scan, or null where n is so small that none runs.
-const uint32_t *depth_order_failed(const uint64_t *partials, int n);
 // Output positions per entry of the scan's chunk table (a divisor of every
 // emit kernel's per-warp output range).
 constexpr uint32_t kEmitStride = 128;

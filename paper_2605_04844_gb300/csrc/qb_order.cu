@@ -276,8 +276,4 @@ cudaError_t launch_depth_order(const OrderArgs &a, int n, cudaStream_t s, bool *
                              a.chunk_first, a.chunk_cap, s);
 }
 
-const uint32_t *depth_order_failed(const uint64_t *partials, int n) {
-    return n > kOrderSmall ? scan_failed(partials, n) : nullptr;
-}
-
 }  // namespace qb
